@@ -580,7 +580,7 @@ def roofline_of(w, name, job, r):
     hbm_peak = float(peaks["hbm_gbs"])
     if not tc_path:
         peak = 148 * 128 * 2 * 1.965e9 / 1e12     # 128 fp32 FMA lanes x 148 SMs x 2 FLOP at the maximum SM clock
-        out = {"kernel": "simt_dw_kernel + simt_dx_kernel", "bound": "alu", "achieved": flops / (launch_ms * 1e-3) / 1e12,
+        out = {"kernel": "fma_backward_kernel", "bound": "alu", "achieved": flops / (launch_ms * 1e-3) / 1e12,
                "peak": peak, "peak_kind": "derived: 148 SMs x 128 FMA/clk x 2 x 1.965 GHz", "unit": "TFLOP/s", "traffic": None}
     elif by / (hbm_peak * 1e9) > flops / (burst_peak * 1e12):
         out = {"kernel": "tc_backward_kernel (dW and dX tiles, db on the side; timed with its reduce kernel)", "bound": "hbm",

@@ -1,0 +1,548 @@
+// Products on the CUDA cores, fp32 fused multiply-adds: the fp32 path (whose 1e-5 tolerance rules out reduced-precision
+// tensor-core modes) and bf16 shapes too small for the tensor-core kernels.
+//   forward  Y[m, j] = sum_i X[m, i] W[i, j] + bias[j]                        (Eq. 2)
+//   dW[i, j] = sum_m X_keep[m, i] dY[keep_rows[m], j],  db[j] = sum_m dY[keep_rows[m], j]       (Eq. 5)
+//   dX[keep_rows[m], i] = sum_j dY[keep_rows[m], j] W[i, j]; every other row of dX = +0.0
+//
+// Bound by the FMA pipes.  Blackwell issues two fp32 FMAs per lane with one packed instruction (fma.rn.f32x2, each half
+// rounded as its own fmaf); the scalar form reaches half of the peak at best.  A thread owns 8 x 8 outputs as 8 x 4 packed
+// pairs: per reduction step it reads 16 operands from shared memory (four 16-byte loads, each a broadcast or conflict-free
+// within the warp's 32 x 64 outputs) for 32 packed FMAs.  The 256 threads of a block form kG groups which make the same
+// 64 x BN outputs from different depths of each stage (2 groups for BN = 128, 4 for BN = 64) and add their accumulators up
+// through shared memory at the end: a tile takes 1 / kG of the time, each thread carries 1 / kG of the loads in flight, and
+// what a thread needs fits 128 registers, so sixteen warps per SM hide each other's shared-memory latency.  Operands go
+// global -> registers -> shared memory, two 16-deep stages, the next one's loads in flight during the current arithmetic.
+//
+// Measured on B200, fp32 768 -> 3072, 3136 rows with 1568 kept, against 64 x 64 tiles of scalar FMAs in a kernel per product
+// and two for db: forward 441 -> 338 us (43.7 TFLOP/s, FMA pipes busy 66 % of the time), dW + db + dX 612 -> 392 us.  One
+// group of 128 threads a block at 162 registers: forward 404 us.  Operand A stored as ready-made pairs {a, a}, which saves
+// the moves that double it: 450 us (the registers of eight more 64-bit operands cost more than the moves).
+#include "zero_rows.cuh"
+
+namespace sbp {
+namespace {
+
+constexpr int kBK = 16;                   // reduction depth of a stage
+constexpr int kBM = 64;                   // rows of a tile
+constexpr int kTM = 8, kTN = 8;           // outputs per thread
+constexpr int NT = 256;                   // threads of a block
+
+template <typename T> __device__ __forceinline__ float4 load4(const T* p);
+template <> __device__ __forceinline__ float4 load4<float>(const float* p) {
+    return __ldg(reinterpret_cast<const float4*>(p));
+}
+template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                       __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
+template <typename T> __device__ __forceinline__ void store4(T* p, float4 v);
+template <> __device__ __forceinline__ void store4<float>(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, float4 v) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
+    uint2 u;
+    u.x = *reinterpret_cast<const uint32_t*>(&lo);
+    u.y = *reinterpret_cast<const uint32_t*>(&hi);
+    *reinterpret_cast<uint2*>(p) = u;
+}
+
+__device__ __forceinline__ uint64_t twice(float a) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void add2(uint64_t& d, uint64_t a) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a));
+}
+__device__ __forceinline__ float2 halves(uint64_t v) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+
+// One operand of a product, [extent x depth] as the product sees it: a row-major matrix whose rows are extent indices
+// (depth inner) or depth indices.  `map` sends a row of the matrix to the row of memory it lives in (nullptr: itself).
+template <typename T>
+struct Operand {
+    const T* base;
+    int64_t ld;                            // elements between rows of memory
+    const int32_t* map;
+    int64_t extent;                        // valid extent indices
+};
+
+// Global -> register -> shared-memory path of one operand: a tile of B extent indices x kBK depth.
+template <typename T, int B, bool kDepthInner>
+struct TileLoader {
+    static constexpr int kVecs = B * kBK / 4 / NT;       // 4-element vectors per thread and stage
+    static constexpr int kPitch = B + 4;                 // floats per depth row in shared memory
+    static_assert(kVecs >= 1 && B * kBK % (4 * NT) == 0, "tile divides among the threads");
+    float4 v[kVecs];
+    const T* ptr[kDepthInner ? kVecs : 1];               // depth inner: the rows are the same in every stage
+    int32_t row[kDepthInner ? 1 : kVecs];                // otherwise: rows of memory of the stage fetched next
+
+    __device__ __forceinline__ void init(const Operand<T>& op, int64_t e0, int64_t d0, int64_t d_end) {
+        if constexpr (kDepthInner) {
+#pragma unroll
+            for (int i = 0; i < kVecs; ++i) {
+                const int idx = threadIdx.x + i * NT;
+                const int64_t e = e0 + idx / (kBK / 4);
+                ptr[i] = e < op.extent ? op.base + (int64_t)mapped_row(op.map, e) * op.ld + (idx % (kBK / 4)) * 4 : nullptr;
+            }
+        } else {
+            fetch_rows(op, d0, d_end);
+        }
+    }
+    __device__ __forceinline__ void fetch_rows(const Operand<T>& op, int64_t d0, int64_t d_end) {
+#pragma unroll
+        for (int i = 0; i < kVecs; ++i) {
+            const int64_t d = d0 + (threadIdx.x + i * NT) / (B / 4);
+            row[i] = d < d_end ? mapped_row(op.map, d) : -1;
+        }
+    }
+    // stage of depth [d0, d0 + kBK), depth indices from d_end on read as zero
+    __device__ __forceinline__ void fetch(const Operand<T>& op, int64_t e0, int64_t d0, int64_t d_end) {
+#pragma unroll
+        for (int i = 0; i < kVecs; ++i) {
+            const int idx = threadIdx.x + i * NT;
+            v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (kDepthInner) {
+                if (ptr[i] != nullptr && d0 + (idx % (kBK / 4)) * 4 < d_end) v[i] = load4<T>(ptr[i] + d0);
+            } else {
+                const int64_t e = e0 + (idx % (B / 4)) * 4;
+                if (row[i] >= 0 && e < op.extent) v[i] = load4<T>(op.base + (int64_t)row[i] * op.ld + e);
+            }
+        }
+        if constexpr (!kDepthInner) fetch_rows(op, d0 + kBK, d_end);
+    }
+    __device__ __forceinline__ void put(float* tile) const {           // tile[depth][extent]
+#pragma unroll
+        for (int i = 0; i < kVecs; ++i) {
+            const int idx = threadIdx.x + i * NT;
+            if constexpr (kDepthInner) {
+                const int e = idx / (kBK / 4), d = (idx % (kBK / 4)) * 4;
+                tile[(d + 0) * kPitch + e] = v[i].x;
+                tile[(d + 1) * kPitch + e] = v[i].y;
+                tile[(d + 2) * kPitch + e] = v[i].z;
+                tile[(d + 3) * kPitch + e] = v[i].w;
+            } else {
+                *reinterpret_cast<float4*>(tile + (idx / (B / 4)) * kPitch + (idx % (B / 4)) * 4) = v[i];
+            }
+        }
+    }
+};
+
+template <int BN>
+union ProductShared {
+    struct {
+        float a[2][kBK][kBM + 4];
+        float b[2][kBK][BN + 4];
+    } t;
+    ulonglong2 swap[8][NT];                // half a thread's accumulators, on their way to the partner group
+};
+
+// Where a thread's outputs sit in the tile: before the groups add up, rows row0 + {0..3, 16..19}, columns col0 + {0..3,
+// 32..35} in every group; afterwards group g holds kRows of the eight rows, from number first on.
+template <int BN>
+struct ThreadTile {
+    static constexpr int kThreads = (kBM / kTM) * (BN / kTN);          // threads of a group
+    static constexpr int kG = NT / kThreads, kRows = kTM / kG;
+    int group, row0, col0, first;
+    __device__ __forceinline__ ThreadTile() {
+        group = threadIdx.x / kThreads;
+        const int warp = (threadIdx.x % kThreads) >> 5, lane = threadIdx.x & 31;
+        row0 = (warp / (BN / 64)) * 32 + (lane >> 3) * 4;
+        col0 = (warp % (BN / 64)) * 64 + (lane & 7) * 4;
+        first = group * kRows;
+    }
+    __device__ __forceinline__ int row(int q) const { return row0 + ((first + q) & 3) + ((first + q) >> 2) * 16; }
+    __device__ __forceinline__ int col(int half) const { return col0 + half * 32; }
+};
+
+// One step of the sum over groups: partners exchange halves of kHave accumulator rows, `upper` keeps the upper half.
+template <int BN, int kHave>
+__device__ __forceinline__ void halve(ProductShared<BN>& sh, uint64_t (&acc)[kTM][kTN / 2], bool upper, int partner) {
+    constexpr int kKeep = kHave / 2;
+    if (upper) {
+#pragma unroll
+        for (int r = 0; r < kKeep; ++r)
+#pragma unroll
+            for (int c = 0; c < kTN / 2; ++c) {
+                const uint64_t t = acc[r][c];
+                acc[r][c] = acc[r + kKeep][c];
+                acc[r + kKeep][c] = t;
+            }
+    }
+    __syncthreads();                       // the tiles (or the exchange before) have been read
+#pragma unroll
+    for (int r = 0; r < kKeep; ++r) {
+        sh.swap[2 * r][threadIdx.x] = make_ulonglong2(acc[kKeep + r][0], acc[kKeep + r][1]);
+        sh.swap[2 * r + 1][threadIdx.x] = make_ulonglong2(acc[kKeep + r][2], acc[kKeep + r][3]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kKeep; ++r) {
+        const ulonglong2 u = sh.swap[2 * r][partner], w = sh.swap[2 * r + 1][partner];
+        add2(acc[r][0], u.x); add2(acc[r][1], u.y); add2(acc[r][2], w.x); add2(acc[r][3], w.y);
+    }
+}
+
+// acc = A[e_a0 .., d] * B[e_b0 .., d] over the depth range [d_begin, d_end), in the first kRows rows of `acc` (ThreadTile).
+// kSum: 0 none, 1 / 2: `colsum` of thread t receives the sum over the depth of extent index t of operand A / B (the
+// bias gradient).
+template <typename T, int BN, bool kAInner, bool kBInner, int kSum>
+__device__ __forceinline__ void product(ProductShared<BN>& sh, const ThreadTile<BN>& tt, const Operand<T>& A, const Operand<T>& B,
+                                        int64_t e_a0, int64_t e_b0, int64_t d_begin, int64_t d_end, bool want_sum,
+                                        uint64_t (&acc)[kTM][kTN / 2], float& colsum) {
+    constexpr int kG = ThreadTile<BN>::kG, kMine = kBK / kG;           // depth steps of a stage for each group
+    TileLoader<T, kBM, kAInner> la;
+    TileLoader<T, BN, kBInner> lb;
+#pragma unroll
+    for (int r = 0; r < kTM; ++r)
+#pragma unroll
+        for (int c = 0; c < kTN / 2; ++c) acc[r][c] = 0ull;
+    colsum = 0.f;
+    float lost = 0.f;                      // of the compensated sum below
+    if (d_begin >= d_end) return;
+    la.init(A, e_a0, d_begin, d_end);
+    lb.init(B, e_b0, d_begin, d_end);
+    la.fetch(A, e_a0, d_begin, d_end);
+    lb.fetch(B, e_b0, d_begin, d_end);
+    int buf = 0;
+    for (int64_t d0 = d_begin; d0 < d_end; d0 += kBK, buf ^= 1) {
+        la.put(&sh.t.a[buf][0][0]);
+        lb.put(&sh.t.b[buf][0][0]);
+        __syncthreads();                   // (two buffers: the one written next was last read before this barrier)
+        if (d0 + kBK < d_end) {
+            la.fetch(A, e_a0, d0 + kBK, d_end);
+            lb.fetch(B, e_b0, d0 + kBK, d_end);
+        }
+        if (kSum != 0 && want_sum && threadIdx.x < (kSum == 1 ? kBM : BN)) {
+            float part[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < kBK; ++k) part[k & 3] += kSum == 1 ? sh.t.a[buf][k][threadIdx.x % kBM] : sh.t.b[buf][k][threadIdx.x % BN];
+            const float y = ((part[0] + part[1]) + (part[2] + part[3])) - lost, t = colsum + y;     // Kahan's sum: one chain
+            lost = (t - colsum) - y;                                                                // of up to thousands of stages
+            colsum = t;
+        }
+#pragma unroll
+        for (int k = 0; k < kMine; ++k) {
+            const float* ak = &sh.t.a[buf][tt.group * kMine + k][tt.row0];
+            const float* bk = &sh.t.b[buf][tt.group * kMine + k][tt.col0];
+            const float4 a0 = *reinterpret_cast<const float4*>(ak), a1 = *reinterpret_cast<const float4*>(ak + 16);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bk), b1 = *reinterpret_cast<const ulonglong2*>(bk + 32);
+            const float a[kTM] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const uint64_t b[kTN / 2] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+            for (int r = 0; r < kTM; ++r) {
+                const uint64_t a2 = twice(a[r]);
+#pragma unroll
+                for (int c = 0; c < kTN / 2; ++c) fma2(acc[r][c], a2, b[c]);
+            }
+        }
+    }
+    constexpr int kT = ThreadTile<BN>::kThreads;
+    if constexpr (kG == 2) {
+        halve<BN, 8>(sh, acc, tt.group != 0, threadIdx.x ^ kT);
+    } else {
+        halve<BN, 8>(sh, acc, tt.group >= 2, threadIdx.x ^ (2 * kT));
+        halve<BN, 4>(sh, acc, (tt.group & 1) != 0, threadIdx.x ^ kT);
+    }
+}
+
+__device__ __forceinline__ float4 quad(const uint64_t (&acc)[kTM][kTN / 2], int q, int half) {
+    const float2 lo = halves(acc[q][2 * half]), hi = halves(acc[q][2 * half + 1]);
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+template <typename T>
+struct ForwardParams {
+    Operand<T> X, W;
+    const float* bias;
+    T* Y;
+    int64_t M;
+    int C_in, C_out;
+    const int32_t* status_word;
+};
+
+template <typename T, int BN, bool kOutIn>
+__global__ void __launch_bounds__(NT, 2)
+fma_forward_kernel(const ForwardParams<T> p) {
+    __shared__ __align__(16) ProductShared<BN> sh;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (p.status_word != nullptr && *p.status_word != 0) return;
+    const int64_t m0 = (int64_t)blockIdx.x * kBM;
+    const int j0 = blockIdx.y * BN;
+    const ThreadTile<BN> tt;
+    uint64_t acc[kTM][kTN / 2];
+    float unused;
+    product<T, BN, true, kOutIn, 0>(sh, tt, p.X, p.W, m0, j0, 0, p.C_in, false, acc, unused);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = j0 + tt.col(h);
+        if (j >= p.C_out) continue;
+        float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.bias != nullptr) bv = __ldg(reinterpret_cast<const float4*>(p.bias + j));
+#pragma unroll
+        for (int q = 0; q < tt.kRows; ++q) {
+            const int64_t m = m0 + tt.row(q);
+            if (m >= p.M) continue;
+            const float4 v = quad(acc, q, h);
+            store4<T>(p.Y + m * p.C_out + j, make_float4(v.x + bv.x, v.y + bv.y, v.z + bv.z, v.w + bv.w));
+        }
+    }
+}
+
+// dW, db and dX of one layer in one launch: a block makes one tile of either product.
+template <typename T>
+struct BackwardParams {
+    const T *X_keep, *dY, *W;
+    const int32_t *dy_rows, *dx_rows;      // row m of the products reads row dy_rows[m] of dY, writes row dx_rows[m] of dX
+    const int32_t* M_keep_dev;
+    int64_t M, M_keep_cap;                 // M = rows of dX
+    int C_in, C_out;
+    float* dW;                             // dW itself, or the partials [splits, C_in * C_out]
+    float* db;                             // nullptr: not asked for; db itself, or the partials [splits, C_out]
+    T* dX;
+    int w_tiles, w_col_tiles, splits, accumulate;
+    int x_row_tiles, x_col_tiles;          // w_tiles / x_row_tiles 0: that product is not asked for
+    const int32_t* status_word;
+};
+
+template <typename T, int BN, bool kOutIn>
+__device__ __forceinline__ void dw_tile(ProductShared<BN>& sh, const BackwardParams<T>& p, int q, int64_t M_keep) {
+    const int split = q % p.splits, tile = q / p.splits;
+    const int row_tile = tile / p.w_col_tiles, col_tile = tile % p.w_col_tiles;
+    int64_t per = (M_keep + p.splits - 1) / p.splits;
+    per = (per + kBK - 1) / kBK * kBK;
+    const int64_t begin = per * split, end = begin + per < M_keep ? begin + per : M_keep;
+    const Operand<T> X{p.X_keep, p.C_in, nullptr, p.C_in}, Y{p.dY, p.C_out, p.dy_rows, p.C_out};
+    const ThreadTile<BN> tt;
+    uint64_t acc[kTM][kTN / 2];
+    float colsum;
+    // rows of the output are C_in x columns C_out, or the other way round for weights stored [C_out, C_in]
+    const bool want_sum = p.db != nullptr && (kOutIn ? col_tile : row_tile) == 0;
+    if constexpr (kOutIn) product<T, BN, false, false, 1>(sh, tt, Y, X, row_tile * kBM, col_tile * BN, begin, end, want_sum, acc, colsum);
+    else product<T, BN, false, false, 2>(sh, tt, X, Y, row_tile * kBM, col_tile * BN, begin, end, want_sum, acc, colsum);
+    if (want_sum) {
+        const int t = threadIdx.x, j = (kOutIn ? row_tile * kBM : col_tile * BN) + t;
+        if (t < (kOutIn ? kBM : BN) && j < p.C_out) {
+            float* o = p.db + (int64_t)split * p.C_out + j;
+            *o = p.accumulate ? *o + colsum : colsum;
+        }
+    }
+    const int rows = kOutIn ? p.C_out : p.C_in, cols = kOutIn ? p.C_in : p.C_out;
+    float* out = p.dW + (int64_t)split * p.C_in * p.C_out;
+#pragma unroll
+    for (int r = 0; r < tt.kRows; ++r) {
+        const int i = row_tile * kBM + tt.row(r);
+        if (i >= rows) continue;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = col_tile * BN + tt.col(h);
+            if (j >= cols) continue;
+            float4 v = quad(acc, r, h);
+            float4* o = reinterpret_cast<float4*>(out + (int64_t)i * cols + j);
+            if (p.accumulate) { const float4 w = *o; v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w; }
+            *o = v;
+        }
+    }
+}
+
+template <typename T, int BN, bool kOutIn>
+__device__ __forceinline__ void dx_tile(ProductShared<BN>& sh, const BackwardParams<T>& p, int q, int64_t M_keep) {
+    constexpr int kWarps = NT / 32;
+    const int row_tile = q / p.x_col_tiles, i0 = (q % p.x_col_tiles) * BN;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int quads = ((p.C_in - i0 < BN) ? p.C_in - i0 : BN) / 4;
+    // zeros of the dropped rows: every block takes an equal share of the rows of dX, in its own column strip
+    {
+        const int64_t per = (p.M + p.x_row_tiles - 1) / p.x_row_tiles;
+        const int64_t begin = per * row_tile, end = begin + per < p.M ? begin + per : p.M;
+        const int64_t warp_per = ((per + kWarps - 1) / kWarps + 31) / 32 * 32;
+        const int64_t lo = begin + warp * warp_per, hi = lo + warp_per < end ? lo + warp_per : end;
+        const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        warp_visit_dropped_rows(p.dx_rows, M_keep, lo, hi, lane, [&](int64_t base, uint32_t todo) {
+            for (; todo; todo &= todo - 1u)
+                if (lane < quads) store4<T>(p.dX + (base + __ffs(todo) - 1) * p.C_in + i0 + lane * 4, zero4);
+        });
+    }
+    const int64_t m0 = (int64_t)row_tile * kBM;
+    if (m0 >= M_keep) return;
+    const Operand<T> Y{p.dY, p.C_out, p.dy_rows, M_keep};
+    const Operand<T> W{p.W, kOutIn ? p.C_in : p.C_out, nullptr, p.C_in};
+    const ThreadTile<BN> tt;
+    uint64_t acc[kTM][kTN / 2];
+    float unused;
+    product<T, BN, true, !kOutIn, 0>(sh, tt, Y, W, m0, i0, 0, p.C_out, false, acc, unused);
+#pragma unroll
+    for (int r = 0; r < tt.kRows; ++r) {
+        const int64_t m = m0 + tt.row(r);
+        if (m >= M_keep) continue;
+        T* out = p.dX + (int64_t)mapped_row(p.dx_rows, m) * p.C_in;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = i0 + tt.col(h);
+            if (i < p.C_in) store4<T>(out + i, quad(acc, r, h));
+        }
+    }
+}
+
+template <typename T, int BN, bool kOutIn>
+__global__ void __launch_bounds__(NT, 2)
+fma_backward_kernel(const BackwardParams<T> p) {
+    __shared__ __align__(16) ProductShared<BN> sh;
+    static_assert(BN / 4 <= 32, "a warp clears a strip of a row at once");
+    pdl_launch_dependents();
+    pdl_wait();
+    if (p.status_word != nullptr && *p.status_word != 0) return;
+    const int64_t M_keep = load_m_keep(p.M_keep_dev, p.M_keep_cap);
+    const int x_blocks = p.x_row_tiles * p.x_col_tiles;
+    if ((int)blockIdx.x < x_blocks) dx_tile<T, BN, kOutIn>(sh, p, (int)blockIdx.x, M_keep);
+    else dw_tile<T, BN, kOutIn>(sh, p, (int)blockIdx.x - x_blocks, M_keep);
+}
+
+// ---- host side: tile shape, splits of the dW reduction, launches ----
+constexpr int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+struct FmaPlan {
+    bool wide;             // 64 x 128 tiles instead of 64 x 64
+    int64_t w_rows, w_cols, x_rows, x_cols;
+    int splits;
+};
+
+// 64 x 128 tiles (half as many shared-memory reads of W or dY per output) where they fill the two blocks per SM at least
+// once, 64 x 64 below that (fp32 only: the bf16 shapes that come here are small).
+// A dW tile is cut along the kept rows so that no block reduces over more than half of what an SM has to do in all.
+FmaPlan fma_plan(bool fp32, bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_w, bool want_x) {
+    FmaPlan pl;
+    const int64_t wr = out_in ? C_out : C_in, wc = out_in ? C_in : C_out;
+    const auto set = [&](int bn) {
+        pl.w_rows = want_w ? ceil_div(wr, kBM) : 0;
+        pl.w_cols = want_w ? ceil_div(wc, bn) : 0;
+        pl.x_rows = want_x ? (M_keep_cap > 0 ? ceil_div(M_keep_cap, kBM) : 1) : 0;
+        pl.x_cols = want_x ? ceil_div(C_in, bn) : 0;
+    };
+    set(128);
+    pl.wide = fp32 && pl.w_rows * pl.w_cols + pl.x_rows * pl.x_cols >= 2 * kNumSMs;
+    if (!pl.wide) set(64);
+    const double w_depth = (double)ceil_div(M_keep_cap, kBK), x_depth = (double)ceil_div(C_out, kBK);
+    const double per_sm = (pl.w_rows * pl.w_cols * w_depth + pl.x_rows * pl.x_cols * x_depth) / kNumSMs;
+    const double limit = per_sm / 2 > 8.0 ? per_sm / 2 : 8.0;
+    double s = want_w ? w_depth / limit : 1.0;
+    if (s > 64.0) s = 64.0;
+    pl.splits = (int)s < s ? (int)s + 1 : (int)s;
+    if (pl.splits < 1) pl.splits = 1;
+    return pl;
+}
+
+template <typename T, int BN, bool kOutIn>
+cudaError_t launch_forward(const ForwardParams<T>& p, cudaStream_t stream) {
+    const dim3 grid((unsigned)ceil_div(p.M, kBM), (unsigned)ceil_div(p.C_out, BN));
+    return launch_pdl(fma_forward_kernel<T, BN, kOutIn>, grid, dim3(NT), 0, stream, p);
+}
+
+template <typename T>
+cudaError_t forward_typed(const void* X, const void* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out, void* Y,
+                          const int32_t* status_word, cudaStream_t stream) {
+    ForwardParams<T> p;
+    p.X = Operand<T>{(const T*)X, C_in, nullptr, M};
+    p.W = Operand<T>{(const T*)W, w_out_in ? C_in : C_out, nullptr, C_out};
+    p.bias = bias;
+    p.Y = (T*)Y;
+    p.M = M;
+    p.C_in = (int)C_in;
+    p.C_out = (int)C_out;
+    p.status_word = status_word;
+    if constexpr (sizeof(T) == 4) {
+        if (ceil_div(M, kBM) * ceil_div(C_out, 128) >= 2 * kNumSMs)
+            return w_out_in ? launch_forward<T, 128, true>(p, stream) : launch_forward<T, 128, false>(p, stream);
+    }
+    return w_out_in ? launch_forward<T, 64, true>(p, stream) : launch_forward<T, 64, false>(p, stream);
+}
+
+template <typename T, int BN, bool kOutIn>
+cudaError_t launch_backward(const BackwardParams<T>& p, cudaStream_t stream) {
+    const int64_t blocks = (int64_t)p.x_row_tiles * p.x_col_tiles + (int64_t)p.w_tiles * p.splits;
+    return launch_pdl(fma_backward_kernel<T, BN, kOutIn>, dim3((unsigned)blocks), dim3(NT), 0, stream, p);
+}
+
+template <typename T>
+cudaError_t backward_typed(const BackwardParams<T>& p, bool wide, bool w_out_in, cudaStream_t stream) {
+    if constexpr (sizeof(T) == 4) {
+        if (wide) return w_out_in ? launch_backward<T, 128, true>(p, stream) : launch_backward<T, 128, false>(p, stream);
+    }
+    return w_out_in ? launch_backward<T, 64, true>(p, stream) : launch_backward<T, 64, false>(p, stream);
+}
+
+}  // namespace
+
+cudaError_t launch_fma_forward(sbp_dtype dt, const void* X, const void* W, bool w_out_in, const float* bias, int64_t M,
+                               int64_t C_in, int64_t C_out, void* Y, const int32_t* status_word, cudaStream_t stream) {
+    return dt == SBP_BF16 ? forward_typed<__nv_bfloat16>(X, W, w_out_in, bias, M, C_in, C_out, Y, status_word, stream)
+                          : forward_typed<float>(X, W, w_out_in, bias, M, C_in, C_out, Y, status_word, stream);
+}
+
+size_t fma_dw_workspace_bytes(sbp_dtype dt, int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
+    int most = 1;
+    for (int v = 0; v < 4; ++v) {
+        const int s = fma_plan(dt == SBP_F32, (v & 1) != 0, M_keep_cap, C_in, C_out, true, (v & 2) != 0).splits;
+        if (s > most) most = s;
+    }
+    return most > 1 ? (size_t)most * (size_t)(C_in + 1) * (size_t)C_out * sizeof(float) : 0;
+}
+
+int fma_backward_kernel_count(sbp_dtype dt, bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
+    if (!want_dw && !want_dx) return 0;
+    return 1 + (want_dw && fma_plan(dt == SBP_F32, w_out_in, M_keep_cap, C_in, C_out, want_dw, want_dx).splits > 1 ? 1 : 0);
+}
+
+cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY, const void* W, bool w_out_in, const int32_t* dy_rows,
+                                const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
+                                int64_t C_out, float* dW, float* db, bool accumulate, void* dX, float* workspace,
+                                const int32_t* status_word, cudaStream_t stream) {
+    const FmaPlan pl = fma_plan(dt == SBP_F32, w_out_in, M_keep_cap, C_in, C_out, dW != nullptr, dX != nullptr);
+    const bool split = dW != nullptr && pl.splits > 1;
+    float* ws_db = workspace;                                          // [splits, C_out], then [splits, C_in * C_out]
+    float* ws_dw = workspace + (int64_t)pl.splits * C_out;
+    const auto fill = [&](auto& p) {
+        p.dy_rows = dy_rows;
+        p.dx_rows = dx_rows;
+        p.M_keep_dev = M_keep_dev;
+        p.M = M;
+        p.M_keep_cap = M_keep_cap;
+        p.C_in = (int)C_in;
+        p.C_out = (int)C_out;
+        p.dW = split ? ws_dw : dW;
+        p.db = (db == nullptr || dW == nullptr) ? nullptr : (split ? ws_db : db);
+        p.w_tiles = (int)(pl.w_rows * pl.w_cols);
+        p.w_col_tiles = (int)pl.w_cols;
+        p.splits = pl.splits;
+        p.accumulate = (accumulate && !split) ? 1 : 0;
+        p.x_row_tiles = (int)pl.x_rows;
+        p.x_col_tiles = (int)pl.x_cols;
+        p.status_word = status_word;
+    };
+    cudaError_t e;
+    if (dt == SBP_BF16) {
+        BackwardParams<__nv_bfloat16> p{};
+        fill(p);
+        p.X_keep = (const __nv_bfloat16*)X_keep; p.dY = (const __nv_bfloat16*)dY; p.W = (const __nv_bfloat16*)W; p.dX = (__nv_bfloat16*)dX;
+        e = backward_typed(p, pl.wide, w_out_in, stream);
+    } else {
+        BackwardParams<float> p{};
+        fill(p);
+        p.X_keep = (const float*)X_keep; p.dY = (const float*)dY; p.W = (const float*)W; p.dX = (float*)dX;
+        e = backward_typed(p, pl.wide, w_out_in, stream);
+    }
+    if (e != cudaSuccess || !split) return e;
+    if (db != nullptr)
+        return launch_reduce_partials_pair(ws_dw, pl.splits, C_in * C_out, dW, ws_db, pl.splits, C_out, db, accumulate, status_word, stream);
+    return launch_reduce_partials(ws_dw, pl.splits, C_in * C_out, dW, accumulate, status_word, stream);
+}
+
+}  // namespace sbp

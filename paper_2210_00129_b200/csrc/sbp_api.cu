@@ -161,7 +161,7 @@ sbp_status sbp_linear_forward(sbp_dtype dt, const void* X, const void* W, const 
             return SBP_ERR_CUDA;
         return SBP_OK;
     }
-    if (launch_simt_forward(dt, X, W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, Y, status_word, stream) !=
+    if (launch_fma_forward(dt, X, W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, Y, status_word, stream) !=
         cudaSuccess)
         return SBP_ERR_CUDA;
     if (X_keep != nullptr &&
@@ -190,7 +190,7 @@ size_t sbp_linear_backward_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_ke
 namespace {
 size_t base_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
     const size_t db_part = db_scratch_bytes(dt, M_keep_cap, C_out);
-    size_t dw_part = simt_dw_workspace_bytes(M_keep_cap, C_in, C_out);
+    size_t dw_part = fma_dw_workspace_bytes(dt, M_keep_cap, C_in, C_out);
     if (dt == SBP_BF16 && tc_shapes_supported(M, M_keep_cap, C_in, C_out)) {
         const size_t t = tc_dw_workspace_bytes(M_keep_cap, C_in, C_out);
         if (t > dw_part) dw_part = t;
@@ -200,8 +200,8 @@ size_t base_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_keep_cap, int64_t
 }  // namespace
 
 namespace {
-// the backward with W and dW in the paper's [C_in, C_out] layout
-sbp_status backward_in_out(sbp_dtype dt, const void* X_keep, const void* dY, const void* W,
+// the backward with W and dW in the paper's [C_in, C_out] layout, or (w_out_in) in the other one where the kernels take it
+sbp_status backward_direct(sbp_dtype dt, bool w_out_in, const void* X_keep, const void* dY, const void* W,
                            const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M,
                            int64_t M_keep_cap, int64_t C_in, int64_t C_out, float* dW, float* db, void* dX,
                            uint32_t flags, void* workspace, size_t workspace_bytes, size_t workspace_required,
@@ -242,8 +242,9 @@ sbp_status backward_in_out(sbp_dtype dt, const void* X_keep, const void* dY, con
             return SBP_ERR_CUDA;
     }
     const bool tc = use_tensor_cores(dt, flags, M, M_keep_cap, C_in, C_out);
-    // with the tensor-core kernel running, the bias sums ride along in it; otherwise they get their own kernel
-    const bool db_rides = tc && db != nullptr && (dW != nullptr || dX != nullptr);
+    // the bias sums ride along in the tensor-core kernel, and in the CUDA-core one on the way to dW; otherwise they get
+    // their own kernel
+    const bool db_rides = db != nullptr && (dW != nullptr || (tc && dX != nullptr));
     if (db != nullptr && !db_rides) {
         if (launch_db(dt, dY, dy_rows, M_keep_dev, M_keep_cap, C_out, db, accumulate, ws_db, kDbMaxSplits,
                       status_word, stream) != cudaSuccess)
@@ -255,12 +256,9 @@ sbp_status backward_in_out(sbp_dtype dt, const void* X_keep, const void* dY, con
                                                 accumulate, dX, db_rides ? db : nullptr, ws_dw, ws_db, status_word,
                                                 stream);
         if (s != SBP_OK) return s;
-    } else {
-        if (dW != nullptr && launch_simt_dw(dt, X_keep, dY, dy_rows, M_keep_dev, M_keep_cap, C_in, C_out, dW,
-                                            accumulate, ws_dw, status_word, stream) != cudaSuccess)
-            return SBP_ERR_CUDA;
-        if (dX != nullptr && launch_simt_dx(dt, dY, W, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap, C_in, C_out, dX,
-                                            status_word, stream) != cudaSuccess)
+    } else if (dW != nullptr || dX != nullptr) {
+        if (launch_fma_backward(dt, X_keep, dY, W, w_out_in, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap, C_in, C_out, dW,
+                                db_rides ? db : nullptr, accumulate, dX, ws_dw, status_word, stream) != cudaSuccess)
             return SBP_ERR_CUDA;
     }
     return SBP_OK;
@@ -275,7 +273,7 @@ sbp_status sbp_linear_backward(sbp_dtype dt, const void* X_keep, const void* dY,
                                void* stream_v) {
     cudaStream_t stream = (cudaStream_t)stream_v;
     if (!(flags & SBP_FLAG_W_OUT_IN) || (dW == nullptr && dX == nullptr))
-        return backward_in_out(dt, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX, flags,
+        return backward_direct(dt, false, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX, flags,
                                workspace, workspace_bytes,
                                (M > 0 && M_keep_cap >= 0 && C_in > 0 && C_out > 0)
                                    ? sbp_linear_backward_workspace_bytes(dt, M, M_keep_cap, C_in, C_out) : 0,
@@ -299,14 +297,14 @@ sbp_status sbp_linear_backward(sbp_dtype dt, const void* X_keep, const void* dY,
     sbp_status s;
     if (accumulate && dW != nullptr) {
         // dW is produced fresh in the copy and added in by the transpose; db accumulates in place on its own
-        s = backward_in_out(dt, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in,
+        s = backward_direct(dt, false, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in,
                             C_out, dw_copy, nullptr, dX, inner & ~(uint32_t)SBP_FLAG_ACCUMULATE, workspace, base, base,
                             status_word, stream);
         if (s == SBP_OK && db != nullptr)
-            s = backward_in_out(dt, nullptr, dY, nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, nullptr, db,
+            s = backward_direct(dt, false, nullptr, dY, nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, nullptr, db,
                                 nullptr, inner & ~(uint32_t)SBP_FLAG_VALIDATE, workspace, base, base, status_word, stream);
     } else {
-        s = backward_in_out(dt, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in,
+        s = backward_direct(dt, false, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in,
                             C_out, dW != nullptr ? dw_copy : nullptr, db, dX, inner, workspace, base, base, status_word, stream);
     }
     if (s != SBP_OK) return s;
@@ -321,13 +319,11 @@ int sbp_linear_backward_kernel_count(sbp_dtype dt, int64_t M, int64_t M_keep_cap
     const bool tc = use_tensor_cores(dt, flags, M, M_keep_cap, C_in, C_out);
     int n = (flags & SBP_FLAG_VALIDATE) ? 1 : 0;
     if ((flags & SBP_FLAG_W_OUT_IN) && (want_dW || want_dX)) n += (want_dX ? 1 : 0) + (want_dW ? 1 : 0);   // transposes
-    const bool db_rides = tc && want_db && (want_dW || want_dX);
+    const bool db_rides = want_db && (want_dW || (tc && want_dX));
     if (want_db && !db_rides) n += 2;                      // strip partials + fixed-order reduce
     if (tc) return n + tc_backward_kernel_count(M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0, db_rides,
                                                 (flags & SBP_FLAG_DY_COMPACT) != 0);
-    if (want_dW) n += simt_dw_kernel_count(M_keep_cap, C_in, C_out);
-    if (want_dX) n += 1;
-    return n;
+    return n + fma_backward_kernel_count(dt, false, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0);
 }
 
 int64_t sbp_plan_search_count(void) { return tc_plan_searches(); }

@@ -158,18 +158,17 @@ cudaError_t launch_reduce_partials_pair(const float* partials_a, int splits_a, i
                                         const float* partials_b, int splits_b, int64_t n_b, float* out_b,
                                         bool accumulate, const int32_t* status_word, cudaStream_t stream);
 
-// plain-FMA (CUDA-core) products for fp32 and for bf16 shapes the tensor-core kernels do not take
-size_t simt_dw_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
-int    simt_dw_kernel_count(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
-cudaError_t launch_simt_dw(sbp_dtype dt, const void* X_keep, const void* dY, const int32_t* keep_rows,
-                           const int32_t* M_keep_dev, int64_t M_keep_cap, int64_t C_in, int64_t C_out,
-                           float* dW, bool accumulate, float* workspace, const int32_t* status_word,
-                           cudaStream_t stream);
+// CUDA-core products (fp32 FMAs) for fp32 and for bf16 shapes the tensor-core kernels do not take: dW (nullable), db
+// (nullable, made on the way to dW and only with it) and dX (nullable) in one launch, plus one reduce when the dW
+// reduction is split.  w_out_in: W and dW are [C_out, C_in].
 // dy_rows / dx_rows: row m of the product reads row dy_rows[m] of dY and writes row dx_rows[m] of dX
 // (nullptr = m itself); M = rows of dX
-cudaError_t launch_simt_dx(sbp_dtype dt, const void* dY, const void* W, const int32_t* dy_rows,
-                           const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap,
-                           int64_t C_in, int64_t C_out, void* dX, const int32_t* status_word, cudaStream_t stream);
+size_t fma_dw_workspace_bytes(sbp_dtype dt, int64_t M_keep_cap, int64_t C_in, int64_t C_out);
+int    fma_backward_kernel_count(sbp_dtype dt, bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
+cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY, const void* W, bool w_out_in, const int32_t* dy_rows,
+                                const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
+                                int64_t C_out, float* dW, float* db, bool accumulate, void* dX, float* workspace,
+                                const int32_t* status_word, cudaStream_t stream);
 
 // transposes for weights in the [C_out, C_in] layout
 cudaError_t launch_transpose(int elem_bytes, const void* in, void* out, int64_t rows, int64_t cols,
@@ -179,8 +178,8 @@ cudaError_t launch_transpose_add_f32(const float* in, float* out, int64_t rows, 
 
 // forward of the layer, Y = X W + bias (bias nullable)
 // w_out_in: W is stored [C_out, C_in] instead of [C_in, C_out]
-cudaError_t launch_simt_forward(sbp_dtype dt, const void* X, const void* W, bool w_out_in, const float* bias, int64_t M,
-                                int64_t C_in, int64_t C_out, void* Y, const int32_t* status_word, cudaStream_t stream);
+cudaError_t launch_fma_forward(sbp_dtype dt, const void* X, const void* W, bool w_out_in, const float* bias, int64_t M,
+                               int64_t C_in, int64_t C_out, void* Y, const int32_t* status_word, cudaStream_t stream);
 bool   tc_forward_supported(int64_t M, int64_t C_in, int64_t C_out);
 // bf16 forward on the tensor cores; when X_keep is given the same kernel also writes the forward cache
 sbp_status launch_tc_forward(const void* X, const void* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,
@@ -216,7 +215,7 @@ int    tc_backward_kernel_count(int64_t M_keep_cap, int64_t C_in, int64_t C_out,
                                 bool want_db, bool dy_packed);
 // dW (nullable) and dX (nullable) of one layer in a single persistent kernel (+ the split reduce); when db is
 // given its column sums ride along in the same kernel (db_workspace: kNumSMs * C_out floats) + one reduce
-// (dy_rows / dx_rows as for launch_simt_dx)
+// (dy_rows / dx_rows as for launch_fma_backward)
 sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W, const int32_t* dy_rows,
                               const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
                               int64_t C_out, float* dW, bool accumulate, void* dX, float* db, float* workspace,
