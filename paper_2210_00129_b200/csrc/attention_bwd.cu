@@ -1,35 +1,39 @@
 // SBP backward of scaled dot-product attention on token subsets (Sec. 4, "How to apply SBP on MHSA?"; supplementary,
 // "Gradient Calculation of Attention Layers"), bf16 on the tensor cores (tcgen05 / TMEM), head dimension 64.
 //
-// One (sample, head) problem at a time per block (persistent blocks, one per SM).  With Zq the kept query tokens and Zk
-// the kept key / value tokens of the sample (at most 256 each):
+// One (sample, head) problem at a time per block.  With Zq the kept query tokens and Zk the kept key / value tokens of the
+// sample (at most 256 each):
 //     S  = softmax_j(q_i . k_j / sqrt(d))  over j in Zk          (recomputed here: no n x n map is cached at all)
 //     dS = dA V^T,   dM = S * (dS - rowsum(S * dS)) / sqrt(d)
 //     dV = S^T dA,   dK = dM^T Q,   dQ = dM K
 // All five products run as tcgen05.mma on operands staged once in shared memory (128-byte swizzle): a row-major
 // [tokens x 64] tile serves as the K-major operand of Q K^T / dA V^T and, unchanged, as the MN-major operand of the
-// three gradient products.  A first pass over the query tiles finds each row's softmax statistics (maximum, sum,
-// rowsum(S * dS)) from S and dS in tensor memory; the second pass recomputes 128 x 128 blocks of S and dS, turns them
-// into bf16 blocks of S and dM in shared memory, and accumulates dV, dK (per key tile) and dQ (per query tile) in
-// tensor memory: 128 + 128 + 64 + 64 + 2 * 64 = 512 columns.  Rows of the outputs outside the token sets are zeroed
-// by a small kernel of their own.  Every wait is bounded and reports through the status word.
+// three gradient products.
+//
+// Bound by memory at the paper's sizes, and in practice by the length of a problem's chain (copies, two products, softmax,
+// three products, read-out), which the layout below keeps short:
+//  - A row of S is shared by G threads of one TMEM lane quadrant, 64 columns each (G = 2: up to 128 tokens a side, two blocks
+//    of 256 threads per SM; G = 4: up to 256, one block of 512).  Each thread keeps its 64 numbers of S in registers and
+//    turns them into e^(s - own maximum) once; one exchange of (maximum, sum, sum of e dS) among the G threads gives the
+//    row's statistics.
+//  - S and dM go to shared-memory blocks of their own where these fit, so the three gradient products run back to back
+//    (G = 2: the second half of dM takes the place of V, which is dead by then); otherwise dM waits in registers and
+//    overwrites S once dV is done.
+//  - Buffers are sized by the rows in use (token bound rounded up to 16), not by 128 or 256.
+//  - The next problem's rows are copied as soon as the last product has read the operands, under the read-out and the
+//    stores of this one.
+// Query tiles of 128 rows follow one another (dV and dK stay in tensor memory); with two of them S and dS share columns.
+// Rows outside the token sets are zeroed here too, while the first products run.  Every wait is bounded and reports through
+// the status word.
 #include "tc_ptx.cuh"
 
 namespace sbp {
 namespace {
 
-constexpr int kAttnThreads = 256;
 constexpr int kD = 64;                          // head dimension (one 128-byte swizzle row of bf16)
 constexpr int kMaxTok = 256;                    // most kept tokens of a sample on either side
 constexpr uint32_t kRowB = 128;
-constexpr uint32_t kTokBytes = kMaxTok * kRowB;             // 32 KB: one [256 x 64] operand
-constexpr uint32_t kBlkBytes = 128 * kRowB;                 // 16 KB: [128 rows x 64 columns]
-constexpr uint32_t kAttnSmem = 4 * kTokBytes + 2 * 2 * kBlkBytes + 1024;   // Q, K, V, dA + S block + dM block (+ alignment slack)
-static_assert(kAttnSmem <= 227 * 1024, "shared memory per block");
-
-// tensor-memory columns
-constexpr uint32_t kColS = 0, kColDS = 128, kColDV = 256, kColDK = 320, kColDQ = 384;   // second pass
-constexpr uint32_t kColS1 = 0, kColDS1 = 256;                                            // first pass: up to 256 keys each
+constexpr uint32_t kTileB = 128 * kRowB;        // a 128-row tile of an operand
 
 struct AttnParams {
     const __nv_bfloat16 *Q, *K, *V, *dA;
@@ -39,16 +43,12 @@ struct AttnParams {
     __nv_bfloat16 *dQ, *dK, *dV;
     float scale;
     int zero_fill;                // 1: the rows of a sample that its list leaves out are written as zeros
+    int rq, rk;                   // rows of the query-side and key-side buffers: the token bounds rounded up to 16
+    uint32_t block_bytes;         // one 64-key block of S: 128 bytes for each query row of a tile
+    uint32_t off_dm, dm_stride;   // dM blocks (separate: next to S; otherwise the S blocks themselves)
+    uint32_t off_q, off_da, off_k, off_v;
+    int separate;                 // dM has blocks of its own
     int32_t* status_word;
-};
-
-struct AttnShared {
-    uint64_t bar_s, bar_o;
-    uint32_t tmem_slot;
-    int abort_flag;
-    float part[2][128][3];        // per column half: running maximum, sum, sum of e^(s-m) * dS
-    float stat[kMaxTok][3];       // per query row: -maximum (base 2, scaled), 1 / sum, -rowsum(S * dS) / sqrt(d)
-    int32_t q_glob[kMaxTok], k_glob[kMaxTok];   // global row of every query / key of the problem (-1: none)
 };
 
 __device__ __forceinline__ uint32_t swz(uint32_t row, uint32_t chunk) { return row * kRowB + ((chunk ^ (row & 7u)) << 4); }
@@ -93,58 +93,78 @@ __device__ __forceinline__ void zero_unlisted_rows(const AttnParams& p, int prob
     if (p.k_rows != nullptr) zero_gap_rows(p.dK, p.dV, p.ld_out, col0, k_glob, nk, b * p.N, p.N, t, threads);
 }
 
-// What a thread needs to know about a problem before it can start its copies: the token counts, the global rows
-// (t / 8 + 32 i) whose 16-byte chunk t % 8 it copies on the query and on the key side, and the global rows of query
-// and key number t (for the read-out).  Fetched one problem ahead, so that these dependent index loads never sit in
-// front of the copies.
-struct BigMeta {
-    int nq, nk;
-    int32_t qid[8], kid[8];       // -1: no such token (the row is zero-filled)
-    int32_t q_glob, k_glob;
+
+template <int G>
+struct AttnShared {
+    static constexpr int kTok = G == 2 ? 128 : kMaxTok;
+    uint64_t bar_s, bar_o;
+    uint32_t tmem_slot;
+    int abort_flag;
+    float part[G][128][3];        // per 64 columns of a row: maximum, sum of e = 2^((s - maximum) log2 e / sqrt(d)), sum of e dS
+    int32_t q_glob[2][kTok], k_glob[2][kTok];   // global rows of the listed tokens: of this problem and of the next one
 };
-__device__ __forceinline__ BigMeta fetch_big_meta(const AttnParams& p, int prob) {
-    BigMeta mt;
-    mt.nq = mt.nk = 0;
-    if (prob >= p.B * p.heads) return mt;
-    const int b = prob / p.heads;
-    const int base_row = b * p.N;
+
+// Token counts of a problem and the global rows of its query and key number t.
+struct Meta { int nq, nk; int32_t q, k; };
+__device__ __forceinline__ Meta fetch_meta(const AttnParams& p, int prob, int t) {
+    Meta m{0, 0, 0, 0};
+    if (prob >= p.B * p.heads) return m;
+    const int b = prob / p.heads, base_row = b * p.N;
     const int q0 = p.q_rows ? __ldg(p.q_offs + b) : 0, k0 = p.k_rows ? __ldg(p.k_offs + b) : 0;
-    mt.nq = p.q_rows ? __ldg(p.q_offs + b + 1) - q0 : p.N;
-    mt.nk = p.k_rows ? __ldg(p.k_offs + b + 1) - k0 : p.N;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = (threadIdx.x >> 3) + 32 * i;
-        mt.qid[i] = r < mt.nq ? (p.q_rows ? __ldg(p.q_rows + q0 + r) : base_row + r) : -1;
-        mt.kid[i] = r < mt.nk ? (p.k_rows ? __ldg(p.k_rows + k0 + r) : base_row + r) : -1;
-    }
-    const int r = threadIdx.x;
-    mt.q_glob = r < mt.nq ? (p.q_rows ? __ldg(p.q_rows + q0 + r) : base_row + r) : -1;
-    mt.k_glob = r < mt.nk ? (p.k_rows ? __ldg(p.k_rows + k0 + r) : base_row + r) : -1;
-    return mt;
+    m.nq = p.q_rows ? __ldg(p.q_offs + b + 1) - q0 : p.N;
+    m.nk = p.k_rows ? __ldg(p.k_offs + b + 1) - k0 : p.N;
+    if (m.nq > p.rq) m.nq = p.rq;           // lists longer than the stated bound stay inside the buffers
+    if (m.nk > p.rk) m.nk = p.rk;
+    if (t < m.nq) m.q = p.q_rows ? __ldg(p.q_rows + q0 + t) : base_row + t;
+    if (t < m.nk) m.k = p.k_rows ? __ldg(p.k_rows + k0 + t) : base_row + t;
+    return m;
 }
-// rows past `count` (up to the next multiple of 16, which is as far as the products step) become zeros
-__device__ __forceinline__ void load_rows_big(uint32_t dst, const __nv_bfloat16* src, int64_t ld, const int32_t (&id)[8], int count, int col0) {
+
+// Copies one operand's rows (64 columns from col0 on) into its swizzled tile; rows past `count`, up to the next multiple
+// of 16 (as far as the products step), become zeros.
+template <int kThreads>
+__device__ __forceinline__ void load_rows(uint32_t dst, const __nv_bfloat16* src, int64_t ld, const int32_t* glob, int count, int col0) {
     const uint32_t chunk = threadIdx.x & 7u;
     const int padded = (count + 15) & ~15;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = (threadIdx.x >> 3) + 32 * i;
-        if (r < padded)
-            ptx::cp_async_16(dst + swz((uint32_t)r, chunk), src + (id[i] >= 0 ? (int64_t)id[i] * ld + col0 + chunk * 8 : 0), id[i] >= 0 ? 16u : 0u);
+    for (int r = threadIdx.x >> 3; r < padded; r += kThreads / 8) {
+        const bool live = r < count;
+        ptx::cp_async_16(dst + swz((uint32_t)r, chunk), src + (live ? (int64_t)glob[r] * ld + col0 + chunk * 8 : 0), live ? 16u : 0u);
     }
 }
 
-__global__ void __launch_bounds__(kAttnThreads, 1) attention_bwd_kernel(const AttnParams p) {
+__device__ __forceinline__ uint4 pack8(const float* f) {
+    return make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
+}
+// 32 accumulator columns of this thread's row to chunks [chunk0, chunk0 + 4) of a staged [rows x 64] output
+__device__ __forceinline__ void stage32(uint8_t* stage, int row, uint32_t chunk0, const float (&v)[32]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(stage + swz((uint32_t)row, chunk0 + q)) = pack8(v + q * 8);
+}
+// staged rows [0, count) to the rows glob[] of an output, whole 128-byte rows
+template <int kThreads>
+__device__ __forceinline__ void store_rows(__nv_bfloat16* out, int64_t ld, int col0, const uint8_t* stage, const int32_t* glob, int count) {
+    const uint32_t chunk = threadIdx.x & 7u;
+    for (int r = threadIdx.x >> 3; r < count; r += kThreads / 8) {
+        const uint4 pk = *reinterpret_cast<const uint4*>(stage + swz((uint32_t)r, chunk));
+        ptx::st_global_v4(out + (int64_t)glob[r] * ld + col0 + chunk * 8, pk.x, pk.y, pk.z, pk.w);
+    }
+}
+
+// kSeparate: dM has blocks of its own
+template <int G, bool kSeparate>
+__global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(const AttnParams p) {
+    constexpr int kThreads = 128 * G;
+    constexpr uint32_t kTmemCols = G == 2 ? 256 : 512;
+    // tensor-memory columns.  G = 2: S and dS side by side, then dV, dK, dQ in their place.  G = 4: S (dQ later); dS in the
+    // upper half, or, when two query tiles keep dV and dK there, in the place of S
+    constexpr uint32_t kColDV = G == 2 ? 0 : 256, kColDK = G == 2 ? 64 : 384, kColDQ = G == 2 ? 128 : 0;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ AttnShared sh;
+    __shared__ AttnShared<G> sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t raw = ptx::smem_addr(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* gen = smem_raw + (base - raw);                 // generic pointer to the same place
-    const uint32_t sQ = base, sK = base + kTokBytes, sV = base + 2 * kTokBytes, sDA = base + 3 * kTokBytes;
-    const uint32_t sP = base + 4 * kTokBytes, sDM = sP + 2 * kBlkBytes;     // [2 blocks of 64 keys][128 query rows][128 B]
-    uint8_t* gP = gen + 4 * kTokBytes;
-    uint8_t* gDM = gP + 2 * kBlkBytes;
+    const uint32_t sP = base, sDM = base + p.off_dm, sQ = base + p.off_q, sDA = base + p.off_da, sK = base + p.off_k, sV = base + p.off_v;
 
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
@@ -153,10 +173,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_bwd_kernel(const At
         sh.abort_flag = 0;
         ptx::fence_mbar_init();
     }
-    if (warp == 0) ptx::tmem_alloc(ptx::smem_addr(&sh.tmem_slot), 512);
-    // operand rows a problem does not fill are still read by the products (they only reach accumulator rows nobody
-    // stores), so they must hold finite numbers: clear everything once
-    for (uint32_t w = threadIdx.x; w < (4 * kTokBytes + 4 * kBlkBytes) / 16; w += kAttnThreads) reinterpret_cast<uint4*>(gen)[w] = make_uint4(0u, 0u, 0u, 0u);
+    if (warp == 0) ptx::tmem_alloc(ptx::smem_addr(&sh.tmem_slot), kTmemCols);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
@@ -165,550 +182,355 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attention_bwd_kernel(const At
     pdl_wait();
     const bool skip_all = p.status_word != nullptr && *reinterpret_cast<volatile int32_t*>(p.status_word) != 0;
 
-    const int q4 = warp & 3, half = warp >> 2;              // TMEM lane quadrant of this warp; which half of the columns it takes
-    const int row = q4 * 32 + lane;                         // accumulator row (query row, or key row in the dV / dK read-out)
-    const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-    const float sl2 = p.scale * 1.4426950408889634f;        // scores are kept in base 2: e^(x) = 2^(x log2 e)
+    const int quad = warp & 3, g = warp >> 2;               // TMEM lane quadrant of this warp; which 64 key columns it takes
+    const int row = quad * 32 + lane;                       // accumulator row: a query, or a key in the dV / dK read-out
+    const int key0 = g * 64;
+    const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
+    const float sl2 = p.scale * 1.4426950408889634f;        // scores are kept in base 2: e^x = 2^(x log2 e)
+    const int problems = p.B * p.heads;
     uint32_t n_s = 0, n_o = 0;                              // completed uses of the two barriers
     bool ok = !skip_all;
-    BigMeta cur = fetch_big_meta(p, ok ? (int)blockIdx.x : p.B * p.heads);
+    int buf = 0;                                            // which half of q_glob / k_glob holds this problem's rows
 
-    for (int prob = blockIdx.x; ok && prob < p.B * p.heads; prob += gridDim.x) {
+    // rows of problem `prob` into buffer half `b`, then its copies (after a barrier: the rows come from shared memory)
+    auto begin_problem = [&](const Meta& m, int prob, int b) {
+        if (threadIdx.x < AttnShared<G>::kTok) {
+            sh.q_glob[b][threadIdx.x] = m.q;
+            sh.k_glob[b][threadIdx.x] = m.k;
+        }
+        __syncthreads();
+        if (m.nq <= 0 || m.nk <= 0) return;
+        const int col0 = (prob % p.heads) * kD;
+        load_rows<kThreads>(sQ, p.Q, p.ld_qkv, sh.q_glob[b], m.nq, col0);
+        load_rows<kThreads>(sK, p.K, p.ld_qkv, sh.k_glob[b], m.nk, col0);
+        load_rows<kThreads>(sDA, p.dA, p.ld_da, sh.q_glob[b], m.nq, col0);
+        load_rows<kThreads>(sV, p.V, p.ld_qkv, sh.k_glob[b], m.nk, col0);
+    };
+    // every thread of the block waits for a commit; false (for all of them) when any wait gave up
+    auto wait_products = [&](uint64_t* bar, uint32_t& n) {
+        bool good = ptx::mbar_wait(ptx::smem_addr(bar), n & 1u, abort_flag, p.status_word);
+        ++n;
+        good = !__syncthreads_or(!good);
+        ptx::tc_fence_after_sync();
+        return good;
+    };
+
+    Meta cur = fetch_meta(p, ok ? (int)blockIdx.x : problems, (int)threadIdx.x);
+    if (ok && (int)blockIdx.x < problems) begin_problem(cur, (int)blockIdx.x, 0);
+
+    for (int prob = blockIdx.x; ok && prob < problems; prob += gridDim.x, buf ^= 1) {
         const int nq = cur.nq, nk = cur.nk;
         const int col0 = (prob % p.heads) * kD;
-        if (nq > 0 && nk > 0) {
-            load_rows_big(sQ, p.Q, p.ld_qkv, cur.qid, nq, col0);
-            load_rows_big(sK, p.K, p.ld_qkv, cur.kid, nk, col0);
-            load_rows_big(sDA, p.dA, p.ld_da, cur.qid, nq, col0);
-            load_rows_big(sV, p.V, p.ld_qkv, cur.kid, nk, col0);
-        }
-        sh.q_glob[threadIdx.x] = cur.q_glob;
-        sh.k_glob[threadIdx.x] = cur.k_glob;
-        cur = fetch_big_meta(p, prob + (int)gridDim.x);      // the next problem's indices travel while this one computes
+        const int next = prob + (int)gridDim.x;
+        cur = fetch_meta(p, next, (int)threadIdx.x);        // travels while this problem computes
+        const int32_t *q_glob = sh.q_glob[buf], *k_glob = sh.k_glob[buf];
         if (nq <= 0 || nk <= 0) {                            // nothing to compute: only the zeros of the unlisted rows
-            __syncthreads();
-            zero_unlisted_rows(p, prob, nq, nk, sh.q_glob, sh.k_glob, (int)threadIdx.x, kAttnThreads);
-            __syncthreads();
+            zero_unlisted_rows(p, prob, nq, nk, q_glob, k_glob, (int)threadIdx.x, kThreads);
+            if (next < problems) begin_problem(cur, next, buf ^ 1);
             continue;
         }
-        const int QT = (nq + 127) >> 7, KT = (nk + 127) >> 7;
-        const int keys_pad = (nk + 15) & ~15;               // accumulator columns of the first pass (a multiple of 16)
+        const int QT = G == 2 ? 1 : (nq + 127) >> 7;
+        const bool shared_cols = G == 4 && QT > 1;           // dS takes the place of S
+        const uint32_t col_ds = G == 2 ? 128u : shared_cols ? 0u : 256u;
+        const uint32_t k_steps = (uint32_t)(nk + 15) >> 4;
+        const int n_keys = (int)k_steps * 16;                // accumulator columns computed
         ptx::cp_async_wait_all();
         ptx::fence_async_proxy();
         __syncthreads();
 
-        // ---- first pass: softmax statistics of every query row (S and dS over all keys: up to 256 columns each) ----
-        for (int qt = 0; qt < QT && ok; ++qt) {
+        for (int qt = 0; qt < QT; ++qt) {
+            const int q_here = nq - qt * 128 < 128 ? nq - qt * 128 : 128;
+            const uint32_t q_steps = (uint32_t)(q_here + 15) >> 4;
+            const uint32_t idesc_s = ptx::umma_idesc_bf16(128, n_keys, false, false);
             if (threadIdx.x == 0) {
                 ptx::tc_fence_after_sync();
-                const uint32_t idesc = ptx::umma_idesc_bf16(128, keys_pad, false, false);
 #pragma unroll
-                for (uint32_t u = 0; u < 4; ++u) {          // the two products alternate: they fill different accumulators
-                    ptx::umma_bf16(tmem + kColS1, ptx::umma_desc_sw128(sQ + qt * kBlkBytes + u * 32, 16, 1024),
-                                   ptx::umma_desc_sw128(sK + u * 32, 16, 1024), idesc, u != 0);
-                    ptx::umma_bf16(tmem + kColDS1, ptx::umma_desc_sw128(sDA + qt * kBlkBytes + u * 32, 16, 1024),
-                                   ptx::umma_desc_sw128(sV + u * 32, 16, 1024), idesc, u != 0);
+                for (uint32_t u = 0; u < 4; ++u) {           // the two products alternate: they fill different accumulators
+                    ptx::umma_bf16(tmem, ptx::umma_desc_sw128(sQ + qt * kTileB + u * 32, 16, 1024), ptx::umma_desc_sw128(sK + u * 32, 16, 1024), idesc_s, u != 0);
+                    if (!shared_cols)
+                        ptx::umma_bf16(tmem + col_ds, ptx::umma_desc_sw128(sDA + qt * kTileB + u * 32, 16, 1024), ptx::umma_desc_sw128(sV + u * 32, 16, 1024), idesc_s, u != 0);
                 }
                 ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
             }
-            if (qt == 0) zero_unlisted_rows(p, prob, nq, nk, sh.q_glob, sh.k_glob, (int)threadIdx.x, kAttnThreads);
-            ok = ptx::mbar_wait(ptx::smem_addr(&sh.bar_s), n_s & 1u, abort_flag, p.status_word);
-            ++n_s;
-            ok = !__syncthreads_or(!ok);
+            if (qt == 0) zero_unlisted_rows(p, prob, nq, nk, q_glob, k_glob, (int)threadIdx.x, kThreads);
+            ok = wait_products(&sh.bar_s, n_s);
             if (!ok) break;
-            ptx::tc_fence_after_sync();
-            // this thread: row `row`, columns [128 half, 128 half + 128) below keys_pad; two sweeps (maximum; sums)
-            const int cbeg = half * 128, cend = keys_pad < cbeg + 128 ? keys_pad : cbeg + 128;
-            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // four interleaved chains, not one long one
-            for (int c = cbeg; c < cend; c += 32) {
-                float s[32];
-                ptx::tmem_ld_32x32(tmem + kColS1 + (uint32_t)c + lane_off, s);
+            // ---- this thread's 64 columns of its row.  Columns from nk on (padding keys, stale columns past n_keys) are masked ----
+            float e[2][32];
+            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four interleaved chains, not one of 64 links
+            if (key0 < n_keys) {
+                ptx::tmem_ld_32x32(tmem + (uint32_t)key0 + lane_off, e[0]);
+                if (key0 + 32 < n_keys) ptx::tmem_ld_32x32(tmem + (uint32_t)key0 + 32u + lane_off, e[1]);
                 ptx::tmem_ld_wait();
-                if (c + 32 <= nk) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], s[j]);
-                } else {
+                for (int j = 0; j < 64; ++j) {
+                    if (key0 + 64 > nk && key0 + j >= nk) e[j >> 5][j & 31] = -INFINITY;
+                    mx4[j & 3] = fmaxf(mx4[j & 3], e[j >> 5][j & 31]);
+                }
+            }
+            if (shared_cols) {
+                ptx::tc_fence_before_sync();
+                __syncthreads();                             // S has been read by every warp
+                if (threadIdx.x == 0) {
+                    ptx::tc_fence_after_sync();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], (c + j < nk) ? s[j] : -INFINITY);
+                    for (uint32_t u = 0; u < 4; ++u)
+                        ptx::umma_bf16(tmem, ptx::umma_desc_sw128(sDA + qt * kTileB + u * 32, 16, 1024), ptx::umma_desc_sw128(sV + u * 32, 16, 1024), idesc_s, u != 0);
+                    ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
                 }
             }
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
             float l4[4] = {0.f, 0.f, 0.f, 0.f}, u4[4] = {0.f, 0.f, 0.f, 0.f};
-            if (mx > -INFINITY) {
-                const float nm = -mx * sl2;
-                for (int c = cbeg; c < cend; c += 32) {
-                    float s[32], ds[32];
-                    ptx::tmem_ld_32x32(tmem + kColS1 + (uint32_t)c + lane_off, s);
-                    ptx::tmem_ld_32x32(tmem + kColDS1 + (uint32_t)c + lane_off, ds);
+            if (key0 < n_keys) {
+                const float nm = mx > -INFINITY ? -mx * sl2 : 0.f;
+#pragma unroll
+                for (int j = 0; j < 64; ++j) {
+                    e[j >> 5][j & 31] = ex2(fmaf(e[j >> 5][j & 31], sl2, nm));          // masked columns: 2^-inf = 0
+                    l4[j & 3] += e[j >> 5][j & 31];
+                }
+            }
+            if (shared_cols) {
+                ok = wait_products(&sh.bar_s, n_s);
+                if (!ok) break;
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (key0 + c * 32 < n_keys) {
+                    float ds[32];
+                    ptx::tmem_ld_32x32(tmem + col_ds + (uint32_t)(key0 + c * 32) + lane_off, ds);
                     ptx::tmem_ld_wait();
-                    const bool whole = c + 32 <= nk;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {           // a stale column may hold anything, NaN included
+                        const float d = (key0 + 64 > nk && key0 + c * 32 + j >= nk) ? 0.f : ds[j];
+                        u4[j & 3] = fmaf(e[c][j], d, u4[j & 3]);
+                    }
+                }
+            }
+            sh.part[g][row][0] = mx;
+            sh.part[g][row][1] = (l4[0] + l4[1]) + (l4[2] + l4[3]);
+            sh.part[g][row][2] = (u4[0] + u4[1]) + (u4[2] + u4[3]);
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + quad), "n"(32 * G) : "memory");   // the G warps of this quadrant
+            float mm = sh.part[0][row][0];
+#pragma unroll
+            for (int i = 1; i < G; ++i) mm = fmaxf(mm, sh.part[i][row][0]);
+            float L = 0.f, U = 0.f;
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                const float f = ex2((sh.part[i][row][0] - mm) * sl2);                   // an empty share: 2^-inf = 0
+                L = fmaf(sh.part[i][row][1], f, L);
+                U = fmaf(sh.part[i][row][2], f, U);
+            }
+            const float inv_l = 1.f / L;
+            const float mine = ex2((mx - mm) * sl2) * inv_l;
+            const float nds = -U * inv_l * p.scale;          // -rowsum(S dS) / sqrt(d)
+            uint32_t dm[32];                                 // dM waits here when its blocks are those of S
+            uint8_t* blkP = gen + (uint32_t)g * p.block_bytes;
+            uint8_t* blkM = gen + p.off_dm + (uint32_t)g * p.dm_stride;
+            const bool row_fits = (uint32_t)row * kRowB < p.block_bytes;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (key0 + c * 32 < n_keys) {
+                    float ds[32];
+                    ptx::tmem_ld_32x32(tmem + col_ds + (uint32_t)(key0 + c * 32) + lane_off, ds);
+                    ptx::tmem_ld_wait();
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
-                        float e = ex2(fmaf(s[j], sl2, nm)), g = ds[j];
-                        if (!whole) {                        // a stale column may hold anything, NaN included
-                            e = (c + j < nk) ? e : 0.f;
-                            g = (c + j < nk) ? g : 0.f;
+                        const float d = (key0 + 64 > nk && key0 + c * 32 + j >= nk) ? 0.f : ds[j];
+                        e[c][j] *= mine;                     // S
+                        ds[j] = e[c][j] * fmaf(d, p.scale, nds);                        // dM / sqrt(d)
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (row_fits) *reinterpret_cast<uint4*>(blkP + swz((uint32_t)row, (uint32_t)(c * 4 + q))) = pack8(&e[c][q * 8]);
+                        const uint4 w = pack8(ds + q * 8);
+                        if (kSeparate) {
+                            if (row_fits) *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 4 + q))) = w;
+                        } else {
+                            dm[c * 16 + q * 4] = w.x; dm[c * 16 + q * 4 + 1] = w.y; dm[c * 16 + q * 4 + 2] = w.z; dm[c * 16 + q * 4 + 3] = w.w;
                         }
-                        l4[j & 3] += e;
-                        u4[j & 3] = fmaf(e, g, u4[j & 3]);
                     }
                 }
             }
-            const float l = (l4[0] + l4[1]) + (l4[2] + l4[3]), u_acc = (u4[0] + u4[1]) + (u4[2] + u4[3]);
-            sh.part[half][row][0] = mx; sh.part[half][row][1] = l; sh.part[half][row][2] = u_acc;
+            ptx::fence_async_proxy();                        // the blocks are read by the tensor core
             ptx::tc_fence_before_sync();
-            __syncthreads();
-            if (half == 0) {                                 // the two halves of a row, rescaled to their common maximum
-                const float m0 = sh.part[0][row][0], m1 = sh.part[1][row][0];
-                const float mm = fmaxf(m0, m1);
-                const float f0 = (m0 > -INFINITY) ? ex2((m0 - mm) * sl2) : 0.f, f1 = (m1 > -INFINITY) ? ex2((m1 - mm) * sl2) : 0.f;
-                const float ll = sh.part[0][row][1] * f0 + sh.part[1][row][1] * f1;
-                const float uu = sh.part[0][row][2] * f0 + sh.part[1][row][2] * f1;
-                const float inv_l = 1.f / ll;
-                sh.stat[qt * 128 + row][0] = -mm * sl2;
-                sh.stat[qt * 128 + row][1] = inv_l;
-                sh.stat[qt * 128 + row][2] = -uu * inv_l * p.scale;      // -rowsum(S dS) / sqrt(d)
-            }
-            __syncthreads();
-        }
-        if (!ok) break;
-
-        // ---- second pass: 128 x 128 blocks of S and dM, and the three gradient products ----
-        for (int kt = 0; kt < KT && ok; ++kt) {
-            const int kb = keys_pad - kt * 128 < 128 ? keys_pad - kt * 128 : 128;      // key columns of this tile (a multiple of 16)
-            const uint32_t k_steps = (uint32_t)kb >> 4;
-            for (int qt = 0; qt < QT && ok; ++qt) {
-                const int q_rows_here = nq - qt * 128 < 128 ? nq - qt * 128 : 128;
-                const uint32_t q_steps = (uint32_t)(q_rows_here + 15) >> 4;
+            __syncthreads();                                 // S and dS in tensor memory are dead from here on
+            // ---- the gradient products; only the 16-row steps that hold tokens run, accumulators take turns ----
+            const uint32_t id_t = ptx::umma_idesc_bf16(128, 64, true, true);             // dV, dK: both operands MN-major
+            const uint32_t id_q = ptx::umma_idesc_bf16(128, 64, false, true);            // dQ: dM K-major, K MN-major
+            const int KT = G == 2 ? 1 : (nk + 127) >> 7;
+            auto issue_dv = [&](uint32_t u) {
+                for (int kt = 0; kt < KT; ++kt)
+                    ptx::umma_bf16(tmem + kColDV + (uint32_t)kt * 64u, ptx::umma_desc_sw128(sP + (uint32_t)kt * 2u * p.block_bytes + u * 2048, p.block_bytes, 1024),
+                                   ptx::umma_desc_sw128(sDA + qt * kTileB + u * 2048, kTileB, 1024), id_t, (qt | (int)u) != 0);
+            };
+            auto issue_dk = [&](uint32_t u) {
+                for (int kt = 0; kt < KT; ++kt)
+                    ptx::umma_bf16(tmem + kColDK + (uint32_t)kt * 64u, ptx::umma_desc_sw128(sDM + (uint32_t)kt * 2u * p.dm_stride + u * 2048, p.dm_stride, 1024),
+                                   ptx::umma_desc_sw128(sQ + qt * kTileB + u * 2048, kTileB, 1024), id_t, (qt | (int)u) != 0);
+            };
+            auto issue_dq = [&](uint32_t u) {
+                ptx::umma_bf16(tmem + kColDQ, ptx::umma_desc_sw128(sDM + (u >> 2) * p.dm_stride + (u & 3u) * 32, 16, 1024),
+                               ptx::umma_desc_sw128(sK + u * 2048, kTileB, 1024), id_q, u != 0);
+            };
+            const uint32_t steps = q_steps > k_steps ? q_steps : k_steps;
+            if (!kSeparate) {
                 if (threadIdx.x == 0) {
                     ptx::tc_fence_after_sync();
-                    const uint32_t idesc = ptx::umma_idesc_bf16(128, kb, false, false);
-#pragma unroll
-                    for (uint32_t u = 0; u < 4; ++u) {
-                        ptx::umma_bf16(tmem + kColS, ptx::umma_desc_sw128(sQ + qt * kBlkBytes + u * 32, 16, 1024),
-                                       ptx::umma_desc_sw128(sK + kt * kBlkBytes + u * 32, 16, 1024), idesc, u != 0);
-                        ptx::umma_bf16(tmem + kColDS, ptx::umma_desc_sw128(sDA + qt * kBlkBytes + u * 32, 16, 1024),
-                                       ptx::umma_desc_sw128(sV + kt * kBlkBytes + u * 32, 16, 1024), idesc, u != 0);
-                    }
-                    ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
-                }
-                ok = ptx::mbar_wait(ptx::smem_addr(&sh.bar_s), n_s & 1u, abort_flag, p.status_word);
-                ++n_s;
-                ok = !__syncthreads_or(!ok);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const float nm = sh.stat[qt * 128 + row][0], inv_l = sh.stat[qt * 128 + row][1], nds = sh.stat[qt * 128 + row][2];
-#pragma unroll
-                for (int c = 0; c < 64; c += 32) {
-                    const int cc = half * 64 + c;           // column within the tile
-                    if (cc < kb) {
-                        float s[32], ds[32];
-                        ptx::tmem_ld_32x32(tmem + kColS + (uint32_t)cc + lane_off, s);
-                        ptx::tmem_ld_32x32(tmem + kColDS + (uint32_t)cc + lane_off, ds);
-                        ptx::tmem_ld_wait();
-                        const bool whole = kt * 128 + cc + 32 <= nk;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            float e = ex2(fmaf(s[j], sl2, nm)), g = ds[j];
-                            if (!whole) {
-                                e = (kt * 128 + cc + j < nk) ? e : 0.f;
-                                g = (kt * 128 + cc + j < nk) ? g : 0.f;
-                            }
-                            const float pj = e * inv_l;
-                            s[j] = pj;
-                            ds[j] = pj * fmaf(g, p.scale, nds);      // dM / sqrt(d)
-                        }
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint32_t off = (uint32_t)half * kBlkBytes + swz((uint32_t)row, (uint32_t)(c / 8 + q));
-                            *reinterpret_cast<uint4*>(gP + off) =
-                                make_uint4(pack2(s[q * 8], s[q * 8 + 1]), pack2(s[q * 8 + 2], s[q * 8 + 3]), pack2(s[q * 8 + 4], s[q * 8 + 5]), pack2(s[q * 8 + 6], s[q * 8 + 7]));
-                            *reinterpret_cast<uint4*>(gDM + off) =
-                                make_uint4(pack2(ds[q * 8], ds[q * 8 + 1]), pack2(ds[q * 8 + 2], ds[q * 8 + 3]), pack2(ds[q * 8 + 4], ds[q * 8 + 5]), pack2(ds[q * 8 + 6], ds[q * 8 + 7]));
-                        }
-                    }
-                }
-                ptx::fence_async_proxy();                    // the blocks are read by the tensor core
-                ptx::tc_fence_before_sync();
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    ptx::tc_fence_after_sync();
-                    const uint32_t id_t = ptx::umma_idesc_bf16(128, 64, true, true);     // dV, dK: both operands MN-major
-                    const uint32_t id_q = ptx::umma_idesc_bf16(128, 64, false, true);    // dQ: dM K-major, K MN-major
-                    const uint32_t steps = q_steps > k_steps ? q_steps : k_steps;
-                    for (uint32_t u = 0; u < steps; ++u) {   // three accumulators take turns; only the 16-row steps that hold tokens run
-                        if (u < q_steps) {                   // reductions over the query rows of the tile
-                            ptx::umma_bf16(tmem + kColDV, ptx::umma_desc_sw128(sP + u * 2048, kBlkBytes, 1024),
-                                           ptx::umma_desc_sw128(sDA + qt * kBlkBytes + u * 2048, kBlkBytes, 1024), id_t, (qt | (int)u) != 0);
-                            ptx::umma_bf16(tmem + kColDK, ptx::umma_desc_sw128(sDM + u * 2048, kBlkBytes, 1024),
-                                           ptx::umma_desc_sw128(sQ + qt * kBlkBytes + u * 2048, kBlkBytes, 1024), id_t, (qt | (int)u) != 0);
-                        }
-                        if (u < k_steps)                     // reduction over the keys of the tile: two 64-key blocks x four steps
-                            ptx::umma_bf16(tmem + kColDQ + (uint32_t)qt * 64u, ptx::umma_desc_sw128(sDM + (u >> 2) * kBlkBytes + (u & 3u) * 32, 16, 1024),
-                                           ptx::umma_desc_sw128(sK + kt * kBlkBytes + u * 2048, kBlkBytes, 1024), id_q, (kt | (int)u) != 0);
-                    }
+                    for (uint32_t u = 0; u < q_steps; ++u) issue_dv(u);
                     ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
                 }
-                ok = ptx::mbar_wait(ptx::smem_addr(&sh.bar_o), n_o & 1u, abort_flag, p.status_word);
-                ++n_o;
-                ok = !__syncthreads_or(!ok);
+                ok = wait_products(&sh.bar_o, n_o);
+                if (!ok) break;
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    if (key0 + c * 32 < n_keys && row_fits) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 4 + q))) =
+                                make_uint4(dm[c * 16 + q * 4], dm[c * 16 + q * 4 + 1], dm[c * 16 + q * 4 + 2], dm[c * 16 + q * 4 + 3]);
+                    }
+                ptx::fence_async_proxy();
+                ptx::tc_fence_before_sync();
+                __syncthreads();
             }
+            if (threadIdx.x == 0) {
+                ptx::tc_fence_after_sync();
+                for (uint32_t u = 0; u < steps; ++u) {
+                    if (u < q_steps) {
+                        if (kSeparate) issue_dv(u);
+                        issue_dk(u);
+                    }
+                    if (u < k_steps) issue_dq(u);
+                }
+                ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
+            }
+            ok = wait_products(&sh.bar_o, n_o);
             if (!ok) break;
-            // ---- dV and dK of this key tile: accumulator row = key; through shared memory (the S and dM blocks are free)
-            //      so that every store instruction writes whole 128-byte rows ----
-            ptx::tc_fence_after_sync();
-#pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                float v[32];
-                ptx::tmem_ld_32x32(tmem + (which ? kColDK : kColDV) + (uint32_t)(half * 32) + lane_off, v);
+            // the operands have been read: the next problem's rows may come in (the read-out stages in the S and dM blocks,
+            // of which G = 2 leaves V's place alone)
+            if (qt + 1 == QT && next < problems) begin_problem(cur, next, buf ^ 1);
+            if constexpr (G == 4) {                          // dQ of this query tile, 16 columns a group
+                float v[16];
+                ptx::tmem_ld_32x16(tmem + kColDQ + (uint32_t)(g * 16) + lane_off, v);
                 ptx::tmem_ld_wait();
-                uint8_t* stage = which ? gDM : gP;
+                if (row_fits) {
+                    *reinterpret_cast<uint4*>(gen + swz((uint32_t)row, (uint32_t)(g * 2))) = pack8(v);
+                    *reinterpret_cast<uint4*>(gen + swz((uint32_t)row, (uint32_t)(g * 2 + 1))) = pack8(v + 8);
+                }
+                ptx::tc_fence_before_sync();
+                __syncthreads();
+                store_rows<kThreads>(p.dQ, p.ld_out, col0, gen, q_glob + qt * 128, q_here);
+                __syncthreads();                             // the stage becomes S blocks (or another stage) again
+            }
+        }
+        if (!ok) break;
+        // ---- read-out: a thread holds one accumulator row, but a store that touches 32 rows costs 32 transactions, so rows
+        //      go through shared memory and leave as whole 128-byte lines ----
+        if constexpr (G == 2) {
+            const uint32_t stage_b = p.block_bytes;          // three stages: the two S blocks and the first dM block
+            float v[32];
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    *reinterpret_cast<uint4*>(stage + swz((uint32_t)row, (uint32_t)(half * 4 + q))) =
-                        make_uint4(pack2(v[q * 8], v[q * 8 + 1]), pack2(v[q * 8 + 2], v[q * 8 + 3]), pack2(v[q * 8 + 4], v[q * 8 + 5]), pack2(v[q * 8 + 6], v[q * 8 + 7]));
+            for (int which = 0; which < 3; ++which) {
+                if (which == 2 && !kSeparate) break;
+                ptx::tmem_ld_32x32(tmem + (uint32_t)(which * 64 + g * 32) + lane_off, v);
+                ptx::tmem_ld_wait();
+                if ((uint32_t)row * kRowB < stage_b) stage32(gen + which * stage_b, row, (uint32_t)(g * 4), v);
+            }
+            if (!kSeparate) {                               // (two stages only)
+                ptx::tmem_ld_32x32(tmem + (uint32_t)(128 + g * 32) + lane_off, v);
+                ptx::tmem_ld_wait();
+            }
+            ptx::tc_fence_before_sync();
+            __syncthreads();
+            store_rows<kThreads>(p.dV, p.ld_out, col0, gen, k_glob, nk);
+            store_rows<kThreads>(p.dK, p.ld_out, col0, gen + stage_b, k_glob, nk);
+            if (!kSeparate) {
+                __syncthreads();
+                if ((uint32_t)row * kRowB < stage_b) stage32(gen, row, (uint32_t)(g * 4), v);
+                __syncthreads();
+            }
+            store_rows<kThreads>(p.dQ, p.ld_out, col0, kSeparate ? gen + 2 * stage_b : gen, q_glob, nq);
+        } else {
+            // group g takes dV (g even) or dK (g odd) of key tile g / 2
+            const int kt = g >> 1;
+            if (kt * 128 < nk) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    float v[32];
+                    ptx::tmem_ld_32x32(tmem + ((g & 1) ? kColDK : kColDV) + (uint32_t)(kt * 64 + half * 32) + lane_off, v);
+                    ptx::tmem_ld_wait();
+                    stage32(gen + (uint32_t)g * kTileB, row, (uint32_t)(half * 4), v);
+                }
             }
             ptx::tc_fence_before_sync();
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int idx = threadIdx.x + kAttnThreads * i;          // 2 outputs x 128 rows x 8 chunks
-                const int which = idx >> 10, r = (idx >> 3) & 127, ch = idx & 7;
-                const int32_t g = sh.k_glob[kt * 128 + r];
-                if (kt * 128 + r < nk && g >= 0) {
-                    const uint4 pk = *reinterpret_cast<const uint4*>((which ? gDM : gP) + swz((uint32_t)r, (uint32_t)ch));
-                    ptx::st_global_v4((which ? p.dK : p.dV) + (int64_t)g * p.ld_out + col0 + ch * 8, pk.x, pk.y, pk.z, pk.w);
-                }
-            }
-            __syncthreads();                                 // the stages become S / dM blocks again
-        }
-        if (!ok) break;
-        // ---- dQ of every query tile ----
-        ptx::tc_fence_after_sync();
-        for (int qt = 0; qt < QT; ++qt) {
-            float v[32];
-            ptx::tmem_ld_32x32(tmem + kColDQ + (uint32_t)(qt * 64 + half * 32) + lane_off, v);
-            ptx::tmem_ld_wait();
-            uint8_t* stage = qt ? gDM : gP;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                *reinterpret_cast<uint4*>(stage + swz((uint32_t)row, (uint32_t)(half * 4 + q))) =
-                    make_uint4(pack2(v[q * 8], v[q * 8 + 1]), pack2(v[q * 8 + 2], v[q * 8 + 3]), pack2(v[q * 8 + 4], v[q * 8 + 5]), pack2(v[q * 8 + 6], v[q * 8 + 7]));
-        }
-        ptx::tc_fence_before_sync();
-        __syncthreads();
-        for (int i = 0; i < 4 * QT; ++i) {
-            const int idx = threadIdx.x + kAttnThreads * i;              // QT tiles x 128 rows x 8 chunks
-            const int qt = idx >> 10, r = (idx >> 3) & 127, ch = idx & 7;
-            const int32_t g = sh.q_glob[qt * 128 + r];
-            if (qt * 128 + r < nq && g >= 0) {
-                const uint4 pk = *reinterpret_cast<const uint4*>((qt ? gDM : gP) + swz((uint32_t)r, (uint32_t)ch));
-                ptx::st_global_v4(p.dQ + (int64_t)g * p.ld_out + col0 + ch * 8, pk.x, pk.y, pk.z, pk.w);
+            for (int i = 0; i < 4; ++i) {
+                const int first = (i >> 1) * 128;
+                if (first < nk)
+                    store_rows<kThreads>((i & 1) ? p.dK : p.dV, p.ld_out, col0, gen + (uint32_t)i * kTileB, k_glob + first, nk - first < 128 ? nk - first : 128);
             }
         }
-        ptx::tc_fence_before_sync();
-        __syncthreads();                                     // operands, stages and accumulators are free for the next problem
+        // (the barrier in front of the next problem's products keeps its writers off stages still being stored)
     }
+    ptx::cp_async_wait_all();
     ptx::tc_fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, 512);
+        ptx::tmem_dealloc(tmem, kTmemCols);
     }
 }
 
-// ---------------------------------------------------------------------------------------------
-// At most 128 kept tokens on both sides (keep ratios up to 0.5 on 14 x 14 maps, the paper's setting): one 128 x 128
-// tile per problem, so S and dS are computed once, the statistics and the blocks come from the same accumulators, and
-// the block is small enough for two per SM (96 KB of operands, 256 tensor-memory columns, 128 threads): while one block
-// waits for its loads or its products, the other computes.  Each thread owns one query row: it keeps the row's dM as
-// packed bf16 in registers while the S block feeds dV, then writes dM over the S block for dK and dQ.
-// ---------------------------------------------------------------------------------------------
-constexpr int kSmallThreads = 128;
-constexpr uint32_t kSmallSmem = 4 * kBlkBytes + 2 * kBlkBytes + 1024;      // Q, K, V, dA + one S / dM block (+ alignment slack)
+// ---- host side: buffer layout and launch ----
+int round16(int64_t v) { return (int)((v + 15) / 16 * 16); }
 
-struct SmallShared {
-    uint64_t bar_s, bar_o;
-    uint32_t tmem_slot;
-    int abort_flag;
-    int32_t q_glob[kSmallThreads], k_glob[kSmallThreads];   // global row of every query / key of the problem (-1: none)
-};
-
-// What a thread needs to know about a problem before it can start its copies: the token counts, the global rows
-// (t / 8 + 16 i) whose 16-byte chunk t % 8 it copies on the query and on the key side, and the rows whose results it
-// stores.  Fetched one problem ahead, so that these dependent index loads never sit in front of the copies.
-struct SmallMeta {
-    int nq, nk;
-    int32_t qid[8], kid[8];       // -1: no such token (the row is zero-filled)
-    int32_t q_out, k_out;         // global row of query / key number threadIdx.x, -1 if there is none
-};
-__device__ __forceinline__ SmallMeta fetch_meta(const AttnParams& p, int prob) {
-    SmallMeta mt;
-    mt.nq = mt.nk = 0;
-    if (prob >= p.B * p.heads) return mt;
-    const int b = prob / p.heads;
-    const int base_row = b * p.N;
-    const int q0 = p.q_rows ? __ldg(p.q_offs + b) : 0, k0 = p.k_rows ? __ldg(p.k_offs + b) : 0;
-    mt.nq = p.q_rows ? __ldg(p.q_offs + b + 1) - q0 : p.N;
-    mt.nk = p.k_rows ? __ldg(p.k_offs + b + 1) - k0 : p.N;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = (threadIdx.x >> 3) + 16 * i;
-        mt.qid[i] = r < mt.nq ? (p.q_rows ? __ldg(p.q_rows + q0 + r) : base_row + r) : -1;
-        mt.kid[i] = r < mt.nk ? (p.k_rows ? __ldg(p.k_rows + k0 + r) : base_row + r) : -1;
-    }
-    const int r = threadIdx.x;
-    mt.q_out = r < mt.nq ? (p.q_rows ? __ldg(p.q_rows + q0 + r) : base_row + r) : -1;
-    mt.k_out = r < mt.nk ? (p.k_rows ? __ldg(p.k_rows + k0 + r) : base_row + r) : -1;
-    return mt;
-}
-// rows past `count` (up to the next multiple of 16, which is as far as the products step) become zeros
-__device__ __forceinline__ void load_rows_small(uint32_t dst, const __nv_bfloat16* src, int64_t ld, const int32_t (&id)[8], int count, int col0) {
-    const uint32_t chunk = threadIdx.x & 7u;
-    const int padded = (count + 15) & ~15;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = (threadIdx.x >> 3) + 16 * i;
-        if (r < padded)
-            ptx::cp_async_16(dst + swz((uint32_t)r, chunk), src + (id[i] >= 0 ? (int64_t)id[i] * ld + col0 + chunk * 8 : 0), id[i] >= 0 ? 16u : 0u);
-    }
-}
-__global__ void __launch_bounds__(kSmallThreads, 2) attention_bwd_small_kernel(const AttnParams p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ SmallShared sh;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t raw = ptx::smem_addr(smem_raw);
-    const uint32_t base = (raw + 1023u) & ~1023u;
-    uint8_t* gen = smem_raw + (base - raw);
-    const uint32_t sQ = base, sK = base + kBlkBytes, sV = base + 2 * kBlkBytes, sDA = base + 3 * kBlkBytes;
-    const uint32_t sP = base + 4 * kBlkBytes;              // [2 blocks of 64 keys][128 query rows][128 B]: S, later dM
-    uint8_t* gP = gen + 4 * kBlkBytes;
-    uint8_t* gV = gen + 2 * kBlkBytes;
-
-    pdl_launch_dependents();
-    if (threadIdx.x == 0) {
-        ptx::mbar_init(ptx::smem_addr(&sh.bar_s), 1);
-        ptx::mbar_init(ptx::smem_addr(&sh.bar_o), 1);
-        sh.abort_flag = 0;
-        ptx::fence_mbar_init();
-    }
-    if (warp == 0) ptx::tmem_alloc(ptx::smem_addr(&sh.tmem_slot), 256);
-    // operand rows that a problem does not fill are still read by the products (they only reach accumulator rows nobody
-    // stores), so they must hold finite numbers: clear everything once
-    for (uint32_t w = threadIdx.x; w < 6 * kBlkBytes / 16; w += kSmallThreads) reinterpret_cast<uint4*>(gen)[w] = make_uint4(0u, 0u, 0u, 0u);
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&sh.tmem_slot);
-    volatile int* abort_flag = &sh.abort_flag;
-    pdl_wait();
-    const bool skip_all = p.status_word != nullptr && *reinterpret_cast<volatile int32_t*>(p.status_word) != 0;
-
-    const int row = threadIdx.x;                            // accumulator row of this thread: a query, or a key in the dV / dK read-out
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
-    const float sl2 = p.scale * 1.4426950408889634f;        // scores in base 2: e^x = 2^(x log2 e)
-    uint32_t n_s = 0, n_o = 0;
-    bool ok = !skip_all;
-    SmallMeta cur = fetch_meta(p, ok ? (int)blockIdx.x : p.B * p.heads);
-
-    for (int prob = blockIdx.x; ok && prob < p.B * p.heads; prob += gridDim.x) {
-        const int nq = cur.nq, nk = cur.nk;
-        const int col0 = (prob % p.heads) * kD;
-        const int32_t q_out = cur.q_out, k_out = cur.k_out;
-        if (nq > 0 && nk > 0) {
-            load_rows_small(sQ, p.Q, p.ld_qkv, cur.qid, nq, col0);
-            load_rows_small(sK, p.K, p.ld_qkv, cur.kid, nk, col0);
-            load_rows_small(sDA, p.dA, p.ld_da, cur.qid, nq, col0);
-            load_rows_small(sV, p.V, p.ld_qkv, cur.kid, nk, col0);
-        }
-        if (p.zero_fill) {
-            sh.q_glob[threadIdx.x] = q_out;
-            sh.k_glob[threadIdx.x] = k_out;
-        }
-        cur = fetch_meta(p, prob + (int)gridDim.x);          // the next problem's indices travel while this one computes
-        if (nq <= 0 || nk <= 0) {                            // nothing to compute: only the zeros of the unlisted rows
-            __syncthreads();
-            zero_unlisted_rows(p, prob, nq, nk, sh.q_glob, sh.k_glob, (int)threadIdx.x, kSmallThreads);
-            __syncthreads();
-            continue;
-        }
-        const uint32_t q_steps = (uint32_t)(nq + 15) >> 4, k_steps = (uint32_t)(nk + 15) >> 4;   // 16-row steps that hold tokens
-        const uint32_t n_keys = k_steps * 16u;              // accumulator columns computed (a multiple of 16)
-        ptx::cp_async_wait_all();
-        ptx::fence_async_proxy();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            ptx::tc_fence_after_sync();
-            const uint32_t idesc = ptx::umma_idesc_bf16(128, (int)n_keys, false, false);
-#pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) {              // the two products alternate: they fill different accumulators
-                ptx::umma_bf16(tmem, ptx::umma_desc_sw128(sQ + u * 32, 16, 1024), ptx::umma_desc_sw128(sK + u * 32, 16, 1024), idesc, u != 0);
-                ptx::umma_bf16(tmem + 128u, ptx::umma_desc_sw128(sDA + u * 32, 16, 1024), ptx::umma_desc_sw128(sV + u * 32, 16, 1024), idesc, u != 0);
-            }
-            ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
-        }
-        zero_unlisted_rows(p, prob, nq, nk, sh.q_glob, sh.k_glob, (int)threadIdx.x, kSmallThreads);
-        ok = ptx::mbar_wait(ptx::smem_addr(&sh.bar_s), n_s & 1u, abort_flag, p.status_word);
-        ++n_s;
-        ok = !__syncthreads_or(!ok);
-        if (!ok) break;
-        ptx::tc_fence_after_sync();
-        // ---- this thread's row of S and dS, three sweeps over the accumulators: the maximum; the sum and
-        //      rowsum(e^(s - m) dS); then the S block to shared memory with dM kept in registers.  Columns from nk on
-        //      (padding keys, stale columns past n_keys) are masked; only the chunk holding column nk pays for it. ----
-        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // four interleaved chains, not one of n_keys links
-        for (uint32_t c = 0; c < n_keys; c += 32) {
-            float s[32];
-            ptx::tmem_ld_32x32(tmem + c + lane_off, s);
-            ptx::tmem_ld_wait();
-            if ((int)c + 32 <= nk) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], s[j]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], ((int)c + j < nk) ? s[j] : -INFINITY);
-            }
-        }
-        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-        const float nm = -mx * sl2;
-        float l4[4] = {0.f, 0.f, 0.f, 0.f}, u4[4] = {0.f, 0.f, 0.f, 0.f};
-        for (uint32_t c = 0; c < n_keys; c += 32) {
-            float s[32], ds[32];
-            ptx::tmem_ld_32x32(tmem + c + lane_off, s);
-            ptx::tmem_ld_32x32(tmem + 128u + c + lane_off, ds);
-            ptx::tmem_ld_wait();
-            const bool whole = (int)c + 32 <= nk;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                float e = ex2(fmaf(s[j], sl2, nm)), g = ds[j];
-                if (!whole) {                                // a stale column may hold anything, NaN included
-                    e = ((int)c + j < nk) ? e : 0.f;
-                    g = ((int)c + j < nk) ? g : 0.f;
-                }
-                l4[j & 3] += e;
-                u4[j & 3] = fmaf(e, g, u4[j & 3]);
-            }
-        }
-        const float l = (l4[0] + l4[1]) + (l4[2] + l4[3]), u_acc = (u4[0] + u4[1]) + (u4[2] + u4[3]);
-        const float inv_l = 1.f / l;
-        const float nds = -u_acc * inv_l * p.scale;         // -rowsum(S dS) / sqrt(d)
-        uint32_t dm[64];
-#pragma unroll
-        for (uint32_t c = 0; c < 128; c += 32) {
-            if (c < n_keys) {
-                float s[32], ds[32];
-                ptx::tmem_ld_32x32(tmem + c + lane_off, s);
-                ptx::tmem_ld_32x32(tmem + 128u + c + lane_off, ds);
-                ptx::tmem_ld_wait();
-                const bool whole = (int)c + 32 <= nk;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float e = ex2(fmaf(s[j], sl2, nm)), g = ds[j];
-                    if (!whole) {
-                        e = ((int)c + j < nk) ? e : 0.f;
-                        g = ((int)c + j < nk) ? g : 0.f;
-                    }
-                    const float pj = e * inv_l;
-                    s[j] = pj;
-                    ds[j] = pj * fmaf(g, p.scale, nds);      // dM / sqrt(d)
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    *reinterpret_cast<uint4*>(gP + (c >> 6) * kBlkBytes + swz((uint32_t)row, ((c & 63u) >> 3) + q)) =
-                        make_uint4(pack2(s[q * 8], s[q * 8 + 1]), pack2(s[q * 8 + 2], s[q * 8 + 3]), pack2(s[q * 8 + 4], s[q * 8 + 5]), pack2(s[q * 8 + 6], s[q * 8 + 7]));
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) dm[(c >> 1) + q * 4 + e] = pack2(ds[q * 8 + 2 * e], ds[q * 8 + 2 * e + 1]);
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) dm[(c >> 1) + e] = 0u;
-            }
-        }
-        ptx::fence_async_proxy();
-        ptx::tc_fence_before_sync();
-        __syncthreads();                                     // S and dS in tensor memory are dead from here on
-        if (threadIdx.x == 0) {
-            ptx::tc_fence_after_sync();
-            const uint32_t id_t = ptx::umma_idesc_bf16(128, 64, true, true);
-            for (uint32_t u = 0; u < q_steps; ++u)           // dV = S^T dA over the query rows
-                ptx::umma_bf16(tmem, ptx::umma_desc_sw128(sP + u * 2048, kBlkBytes, 1024), ptx::umma_desc_sw128(sDA + u * 2048, kBlkBytes, 1024), id_t, u != 0);
-            ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
-        }
-        ok = ptx::mbar_wait(ptx::smem_addr(&sh.bar_o), n_o & 1u, abort_flag, p.status_word);
-        ++n_o;
-        ok = !__syncthreads_or(!ok);
-        if (!ok) break;
-        // ---- dM over the S block ----
-#pragma unroll
-        for (uint32_t c = 0; c < 128; c += 8)
-            if (c < n_keys)
-                *reinterpret_cast<uint4*>(gP + (c >> 6) * kBlkBytes + swz((uint32_t)row, (c & 63u) >> 3)) =
-                    make_uint4(dm[c >> 1], dm[(c >> 1) + 1], dm[(c >> 1) + 2], dm[(c >> 1) + 3]);
-        ptx::fence_async_proxy();
-        ptx::tc_fence_before_sync();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            ptx::tc_fence_after_sync();
-            const uint32_t id_t = ptx::umma_idesc_bf16(128, 64, true, true), id_q = ptx::umma_idesc_bf16(128, 64, false, true);
-            const uint32_t steps = q_steps > k_steps ? q_steps : k_steps;
-            for (uint32_t u = 0; u < steps; ++u) {           // dK = dM^T Q over the query rows, dQ = dM K over the keys, alternating
-                if (u < q_steps)
-                    ptx::umma_bf16(tmem + 64u, ptx::umma_desc_sw128(sP + u * 2048, kBlkBytes, 1024), ptx::umma_desc_sw128(sQ + u * 2048, kBlkBytes, 1024), id_t, u != 0);
-                if (u < k_steps)
-                    ptx::umma_bf16(tmem + 128u, ptx::umma_desc_sw128(sP + (u >> 2) * kBlkBytes + (u & 3u) * 32, 16, 1024),
-                                   ptx::umma_desc_sw128(sK + u * 2048, kBlkBytes, 1024), id_q, u != 0);
-            }
-            ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
-        }
-        ok = ptx::mbar_wait(ptx::smem_addr(&sh.bar_o), n_o & 1u, abort_flag, p.status_word);
-        ++n_o;
-        ok = !__syncthreads_or(!ok);
-        if (!ok) break;
-        ptx::tc_fence_after_sync();
-        // ---- read-out.  A thread holds one accumulator row (a key for dV and dK, a query for dQ), but a store that
-        //      touches 32 rows costs 32 transactions: each warp passes its 32 rows through shared memory (the S block's
-        //      two halves and the V operand are free by now) and writes four whole 128-byte rows per instruction. ----
-#pragma unroll
-        for (int which = 0; which < 3; ++which) {
-            uint8_t* stage = which == 0 ? gP : which == 1 ? gP + kBlkBytes : gV;
-#pragma unroll
-            for (int c = 0; c < 64; c += 32) {
-                float v[32];
-                ptx::tmem_ld_32x32(tmem + (uint32_t)(which * 64 + c) + lane_off, v);
-                ptx::tmem_ld_wait();
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    *reinterpret_cast<uint4*>(stage + swz((uint32_t)row, (uint32_t)(c / 8 + q))) =
-                        make_uint4(pack2(v[q * 8], v[q * 8 + 1]), pack2(v[q * 8 + 2], v[q * 8 + 3]), pack2(v[q * 8 + 4], v[q * 8 + 5]), pack2(v[q * 8 + 6], v[q * 8 + 7]));
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int which = 0; which < 3; ++which) {
-            const uint8_t* stage = which == 0 ? gP : which == 1 ? gP + kBlkBytes : gV;
-            __nv_bfloat16* out = (which == 0 ? p.dV : which == 1 ? p.dK : p.dQ) + col0 + (lane & 7) * 8;
-            const int32_t mine = which == 2 ? q_out : k_out;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int r = i * 4 + (lane >> 3);                                   // row within this warp's 32
-                const int32_t g = __shfl_sync(0xffffffffu, mine, r);
-                const uint4 pk = *reinterpret_cast<const uint4*>(stage + swz((uint32_t)(warp * 32 + r), (uint32_t)(lane & 7)));
-                if (g >= 0) ptx::st_global_v4(out + (int64_t)g * p.ld_out, pk.x, pk.y, pk.z, pk.w);
-            }
-        }
-        ptx::tc_fence_before_sync();
-        __syncthreads();                                     // operands, stages and accumulators are free for the next problem
-    }
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 0) {
-        ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, 256);
-    }
+template <int G, bool kSeparate>
+cudaError_t launch_attention_kernel(const AttnParams& prm, uint32_t bytes, int most_bytes, cudaStream_t stream) {
+    const cudaError_t opt = opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate>>(most_bytes);
+    if (opt != cudaSuccess) return opt;
+    const int64_t problems = (int64_t)prm.B * prm.heads, resident = G == 2 ? 2 * kNumSMs : kNumSMs;
+    return launch_pdl(attention_bwd_kernel<G, kSeparate>, dim3((unsigned)(problems < resident ? problems : resident)), dim3(128 * G), bytes,
+                      stream, prm);
 }
 
-// rows of an output [M, ld] (columns [0, cols)) that are not in its ascending list rows[0 .. *total) become +0.0:
-// entry m of the list owns the gap in front of it, one extra worker the tail; blockIdx.y picks the output
+template <int G>
+cudaError_t launch_attention(AttnParams& prm, int64_t q_most, int64_t k_most, cudaStream_t stream) {
+    // most shared memory a block may ask for: half of an SM's (G = 2) or a block's limit, less the static part, the 1 KB the
+    // system keeps per block and the alignment slack
+    constexpr uint32_t kLimit = (G == 2 ? 233472u / 2 - 1024u : 232448u) - (uint32_t)sizeof(AttnShared<G>) - 64u - 1024u;
+    prm.rq = round16(q_most);
+    prm.rk = round16(k_most);
+    if (G == 2) prm.rq = prm.rk = prm.rq > prm.rk ? prm.rq : prm.rk;      // one size for all: the stages hold queries or keys
+    const uint32_t tile_rows = prm.rq < 128 ? (uint32_t)prm.rq : 128u;
+    prm.block_bytes = tile_rows * kRowB;
+    const uint32_t blocks = G == 2 ? 2u : (uint32_t)(prm.rk + 63) / 64u;
+    uint32_t s_bytes = blocks * prm.block_bytes;
+    if (G == 4 && s_bytes < 4 * kTileB) s_bytes = 4 * kTileB;             // the read-out stages four tiles there
+    const uint32_t q_bytes = (uint32_t)prm.rq * kRowB, k_bytes = (uint32_t)prm.rk * kRowB;
+    // S | dM | Q | dA | K | V: what the products read 128 rows of, whatever it holds, is followed by other buffers
+    const auto layout = [&](uint32_t dm_bytes) {
+        prm.off_dm = dm_bytes ? s_bytes : 0u;
+        prm.off_q = s_bytes + dm_bytes;
+        prm.off_da = prm.off_q + q_bytes;
+        prm.off_k = prm.off_da + q_bytes;
+        prm.off_v = prm.off_k + k_bytes;
+        prm.dm_stride = (G == 2 && dm_bytes) ? prm.off_v - prm.off_dm : prm.block_bytes;
+        prm.separate = dm_bytes ? 1 : 0;
+        return prm.off_v + k_bytes;
+    };
+    uint32_t bytes = layout(G == 2 ? prm.block_bytes : blocks * prm.block_bytes);
+    if (bytes > kLimit) bytes = layout(0u);
+    // The products read 128 rows of every query tile and of every dM block (of V's place too, with G = 2), whatever the rows
+    // past the tokens hold: those reads end inside the buffers that follow, or in room added here.
+    const uint32_t q_tiles = (uint32_t)(prm.rq + 127) / 128u;
+    const uint32_t ends[2] = {prm.off_da + q_tiles * kTileB, G == 2 && prm.separate ? prm.off_v + kTileB : 0u};
+    for (uint32_t end : ends) bytes = bytes < end ? end : bytes;
+    if (bytes > kLimit) return cudaErrorInvalidValue;
+    return prm.separate ? launch_attention_kernel<G, true>(prm, bytes + 1024u, (int)kLimit + 1024, stream)
+                        : launch_attention_kernel<G, false>(prm, bytes + 1024u, (int)kLimit + 1024, stream);
+}
+
 }  // namespace
 
 bool attention_supported(sbp_dtype dt, int64_t head_dim) { return dt == SBP_BF16 && head_dim == kD; }
@@ -716,7 +538,7 @@ int64_t attention_max_tokens() { return kMaxTok; }
 
 cudaError_t launch_attention_backward(const void* Q, const void* K, const void* V, int64_t ld_qkv, const void* dA, int64_t ld_da,
                                       const int32_t* q_rows, const int32_t* q_offs, const int32_t* k_rows, const int32_t* k_offs,
-                                      int64_t B, int64_t N, int64_t heads, int64_t most_tokens, void* dQ, void* dK, void* dV,
+                                      int64_t B, int64_t N, int64_t heads, int64_t q_most, int64_t k_most, void* dQ, void* dK, void* dV,
                                       int64_t ld_out, bool zero_other_rows, int32_t* status_word, cudaStream_t stream) {
     AttnParams prm;
     prm.Q = static_cast<const __nv_bfloat16*>(Q); prm.K = static_cast<const __nv_bfloat16*>(K);
@@ -727,19 +549,9 @@ cudaError_t launch_attention_backward(const void* Q, const void* K, const void* 
     prm.dQ = static_cast<__nv_bfloat16*>(dQ); prm.dK = static_cast<__nv_bfloat16*>(dK); prm.dV = static_cast<__nv_bfloat16*>(dV);
     prm.scale = 1.0f / sqrtf((float)kD);
     prm.status_word = status_word;
-    const int64_t problems = B * heads;
     // the zeros for the rows outside the lists are written by the same kernel, between a problem's copies and its products
     prm.zero_fill = (zero_other_rows && (q_rows != nullptr || k_rows != nullptr)) ? 1 : 0;
-    if (most_tokens <= 128) {
-        const cudaError_t opt = opt_in_dynamic_smem<attention_bwd_small_kernel>((int)kSmallSmem);
-        if (opt != cudaSuccess) return opt;
-        const dim3 grid((unsigned)(problems < 2 * kNumSMs ? problems : 2 * kNumSMs));
-        return launch_pdl(attention_bwd_small_kernel, grid, dim3(kSmallThreads), kSmallSmem, stream, prm);
-    }
-    const cudaError_t opt = opt_in_dynamic_smem<attention_bwd_kernel>((int)kAttnSmem);
-    if (opt != cudaSuccess) return opt;
-    const dim3 grid((unsigned)(problems < kNumSMs ? problems : kNumSMs));
-    return launch_pdl(attention_bwd_kernel, grid, dim3(kAttnThreads), kAttnSmem, stream, prm);
+    return q_most <= 128 && k_most <= 128 ? launch_attention<2>(prm, q_most, k_most, stream) : launch_attention<4>(prm, q_most, k_most, stream);
 }
 
 }  // namespace sbp

@@ -420,10 +420,10 @@ sbp_status sbp_attention_backward(sbp_dtype dt, const void* Q, const void* K, co
     const bool any_all = q_rows == nullptr || k_rows == nullptr;
     const bool any_list = q_rows != nullptr || k_rows != nullptr;
     if (any_list && (max_kept <= 0 || max_kept > N)) return SBP_ERR_INVALID_ARG;
-    const int64_t most = any_all ? N : max_kept;
-    if (most > attention_max_tokens()) return SBP_ERR_UNSUPPORTED;
-    const cudaError_t e = launch_attention_backward(Q, K, V, ld_qkv, dA, ld_da, q_rows, q_offsets, k_rows, k_offs, B, N, heads, most,
-                                                    dQ, dK, dV, ld_out, (flags & SBP_FLAG_ATTN_KEPT_ROWS_ONLY) == 0, status_word,
+    if ((any_all ? N : max_kept) > attention_max_tokens()) return SBP_ERR_UNSUPPORTED;
+    const int64_t q_most = q_rows != nullptr ? max_kept : N, k_most = k_rows != nullptr ? max_kept : N;
+    const cudaError_t e = launch_attention_backward(Q, K, V, ld_qkv, dA, ld_da, q_rows, q_offsets, k_rows, k_offs, B, N, heads, q_most,
+                                                    k_most, dQ, dK, dV, ld_out, (flags & SBP_FLAG_ATTN_KEPT_ROWS_ONLY) == 0, status_word,
                                                     (cudaStream_t)stream);
     return e == cudaSuccess ? SBP_OK : SBP_ERR_CUDA;
 }

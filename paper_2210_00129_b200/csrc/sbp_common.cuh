@@ -199,12 +199,12 @@ cudaError_t launch_patch_scatter(const void* dXp, int64_t B, int64_t H, int64_t 
                                  int32_t* slot, const int32_t* status_word, cudaStream_t stream);
 
 // SBP attention backward on token subsets (bf16, head dimension 64, at most attention_max_tokens() kept tokens per sample
-// and side); null row lists mean every token of the sample
+// and side); null row lists mean every token of the sample; q_most / k_most = most tokens a sample brings to either side
 bool    attention_supported(sbp_dtype dt, int64_t head_dim);
 int64_t attention_max_tokens();
 cudaError_t launch_attention_backward(const void* Q, const void* K, const void* V, int64_t ld_qkv, const void* dA, int64_t ld_da,
                                       const int32_t* q_rows, const int32_t* q_offs, const int32_t* k_rows, const int32_t* k_offs,
-                                      int64_t B, int64_t N, int64_t heads, int64_t most_tokens, void* dQ, void* dK, void* dV,
+                                      int64_t B, int64_t N, int64_t heads, int64_t q_most, int64_t k_most, void* dQ, void* dK, void* dV,
                                       int64_t ld_out, bool zero_other_rows, int32_t* status_word, cudaStream_t stream);
 
 // tcgen05 / TMEM bf16 products
