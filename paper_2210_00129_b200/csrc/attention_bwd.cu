@@ -22,6 +22,11 @@
 //  - Buffers are sized by the rows in use (token bound rounded up to 16), not by 128 or 256.
 //  - The next problem's rows are copied as soon as the last product has read the operands, under the read-out and the
 //    stores of this one.
+// Measured on B200, ViT-B/16 heads (12 x 64, 196 tokens), whole pass with the sampler: Drop QKV, half of the tokens, B = 128:
+// 99 us with a thread a row and copies behind the read-out, now 75 us; Drop Query only, B = 64: 94 -> 84 us.  What is left of a
+// problem's chain, some 20000 clocks with two blocks on an SM: copies and zero rows 5500 (all SMs load, then all store, so
+// memory is busy a quarter of the time on average), softmax 6000, products 4500, read-out 2500.  Copies and zeros by four warps
+// of their own did not pay: the computing warps need more registers than setmaxnreg could then give them (76 us).
 // Query tiles of 128 rows follow one another (dV and dK stay in tensor memory); with two of them S and dS share columns.
 // Rows outside the token sets are zeroed here too, while the first products run.  Every wait is bounded and reports through
 // the status word.
@@ -37,7 +42,7 @@ constexpr uint32_t kTileB = 128 * kRowB;        // a 128-row tile of an operand
 
 struct AttnParams {
     const __nv_bfloat16 *Q, *K, *V, *dA;
-    int64_t ld_qkv, ld_da, ld_out;
+    uint32_t ld_qkv, ld_da, ld_out;                       // row strides in 16-byte vectors
     const int32_t *q_rows, *q_offs, *k_rows, *k_offs;     // null rows = every token of the sample
     int B, N, heads;
     __nv_bfloat16 *dQ, *dK, *dV;
@@ -65,43 +70,52 @@ __device__ __forceinline__ float ex2(float x) {
 }
 
 // Zeros for one head's 64 columns in the rows of sample b that an ascending token list leaves out.  `glob` holds the
-// global row of every listed token of the sample (shared memory, filled by the block before the barrier in front of
-// this call).  Eight threads share a row (one 128-byte line, 16 bytes each, so that a warp's store covers four whole
-// lines); such a group takes the runs of rows in front of listed token g, g + groups, ..., the run behind the last
-// token counting as one more.  Rows are clamped to the sample, so that a list that breaks the ascending order cannot
-// send a store anywhere else.  The stores are fire and forget: issued while the first products run.
-__device__ __forceinline__ void zero_gap_rows(__nv_bfloat16* out0, __nv_bfloat16* out1, int64_t ld, int col0, const int32_t* glob,
-                                              int count, int base_row, int N, int t, int threads) {
-    const int end = base_row + N;
-    const int chunk = (t & 7) * 8;
-    for (int g = t >> 3; g <= count; g += threads >> 3) {
-        int lo = g > 0 ? glob[g - 1] + 1 : base_row;
-        int hi = g < count ? glob[g] : end;
-        lo = lo < base_row ? base_row : lo;
-        hi = hi > end ? end : hi;
-        for (int r = lo; r < hi; ++r) {
-            ptx::st_global_v4(out0 + (int64_t)r * ld + col0 + chunk, 0u, 0u, 0u, 0u);
-            if (out1 != nullptr) ptx::st_global_v4(out1 + (int64_t)r * ld + col0 + chunk, 0u, 0u, 0u, 0u);
+// global row of every listed token of the sample (shared memory).  The z-th unlisted row lies behind g listed ones, with g
+// the first list position whose token has more than z unlisted rows in front of it: a search of at most eight steps.  Every
+// lane of a warp searches for a row of its own; then eight lanes at a time clear one 128-byte line, 16 bytes each, so that a
+// warp's store covers four whole lines.  (Walking the gaps between listed tokens, a group of eight lanes each, gave the warps
+// very different amounts of work: 3000 - 4700 clocks a problem.)  Rows are clamped to the sample, so that a list that breaks the
+// ascending order cannot send a store anywhere else.
+__device__ __forceinline__ void zero_unlisted_rows(__nv_bfloat16* out0, __nv_bfloat16* out1, __nv_bfloat16* out2, uint32_t ld, int col0,
+                                                   const int32_t* glob, int count, int base_row, int N, int warp, int warps, int lane) {
+    const int unlisted = N - count;
+    int per = ((unlisted + warps - 1) / warps + 3) & ~3;     // rows of a warp's turn: an equal share, at most one for each lane
+    per = per < 32 ? per : 32;
+    for (int z0 = warp * per; z0 < unlisted; z0 += warps * per) {
+        const int want = z0 + lane + base_row;
+        int g = 0;                                           // tokens with glob[i] - i <= want are in front of the row
+#pragma unroll
+        for (int step = 128; step > 0; step >>= 1)
+            if (g + step <= count && glob[g + step - 1] - (g + step - 1) <= want) g += step;
+        if (g < count && glob[g] - g <= want) ++g;           // (lists of 256 tokens)
+        int r = z0 + lane + g;
+        r = base_row + (r < N ? r : N - 1);
+        const int here = unlisted - z0 < per ? unlisted - z0 : per;
+#pragma unroll 2
+        for (int i = 0; i < here; i += 4) {
+            const int row = __shfl_sync(0xffffffffu, r, i + (lane >> 3));
+            if (i + (lane >> 3) < here) {
+                const int64_t at = (int64_t)((uint64_t)(uint32_t)row * ld * 8u) + col0 + (lane & 7) * 8;
+                if (out0 != nullptr) ptx::st_global_v4(out0 + at, 0u, 0u, 0u, 0u);
+                if (out1 != nullptr) ptx::st_global_v4(out1 + at, 0u, 0u, 0u, 0u);
+                if (out2 != nullptr) ptx::st_global_v4(out2 + at, 0u, 0u, 0u, 0u);
+            }
         }
     }
 }
-__device__ __forceinline__ void zero_unlisted_rows(const AttnParams& p, int prob, int nq, int nk, const int32_t* q_glob,
-                                                   const int32_t* k_glob, int t, int threads) {
-    if (!p.zero_fill) return;
-    const int b = prob / p.heads, col0 = (prob % p.heads) * kD;
-    if (p.q_rows != nullptr) zero_gap_rows(p.dQ, nullptr, p.ld_out, col0, q_glob, nq, b * p.N, p.N, t, threads);
-    if (p.k_rows != nullptr) zero_gap_rows(p.dK, p.dV, p.ld_out, col0, k_glob, nk, b * p.N, p.N, t, threads);
-}
 
+__device__ __forceinline__ void prefetch_row(const __nv_bfloat16* p, int32_t row, uint32_t ld) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const uint4*>(p) + (uint64_t)(uint32_t)row * ld));
+}
 
 template <int G>
 struct AttnShared {
     static constexpr int kTok = G == 2 ? 128 : kMaxTok;
-    uint64_t bar_s, bar_o;
+    uint64_t bar_s, bar_o;        // products of S and dS; gradient products
     uint32_t tmem_slot;
     int abort_flag;
     float part[G][128][3];        // per 64 columns of a row: maximum, sum of e = 2^((s - maximum) log2 e / sqrt(d)), sum of e dS
-    int32_t q_glob[2][kTok], k_glob[2][kTok];   // global rows of the listed tokens: of this problem and of the next one
+    int32_t q_glob[2][kTok], k_glob[2][kTok];   // global rows of the listed tokens (0 past the last): this problem's, the next one's
 };
 
 // Token counts of a problem and the global rows of its query and key number t.
@@ -120,16 +134,67 @@ __device__ __forceinline__ Meta fetch_meta(const AttnParams& p, int prob, int t)
     return m;
 }
 
-// Copies one operand's rows (64 columns from col0 on) into its swizzled tile; rows past `count`, up to the next multiple
-// of 16 (as far as the products step), become zeros.
+// Copies the rows of one side's two operands (64 columns each) into their swizzled tiles; rows past `count`, up to the next
+// multiple of 16 (as far as the products step), become zeros.  Up to four rows at a time, their ids read together; a thread's
+// rows are a multiple of 8 apart, so that its place in the swizzle is the same in all of them.
 template <int kThreads>
-__device__ __forceinline__ void load_rows(uint32_t dst, const __nv_bfloat16* src, int64_t ld, const int32_t* glob, int count, int col0) {
-    const uint32_t chunk = threadIdx.x & 7u;
+__device__ __forceinline__ void load_rows(uint32_t dst0, uint32_t dst1, const __nv_bfloat16* src0, uint32_t ld0, const __nv_bfloat16* src1,
+                                          uint32_t ld1, const int32_t* glob, int count, int t) {
+    const uint32_t chunk = t & 7u;
+    const uint4* s0 = reinterpret_cast<const uint4*>(src0) + chunk;
+    const uint4* s1 = reinterpret_cast<const uint4*>(src1) + chunk;
+    constexpr int kStep = kThreads / 8;
     const int padded = (count + 15) & ~15;
-    for (int r = threadIdx.x >> 3; r < padded; r += kThreads / 8) {
-        const bool live = r < count;
-        ptx::cp_async_16(dst + swz((uint32_t)r, chunk), src + (live ? (int64_t)glob[r] * ld + col0 + chunk * 8 : 0), live ? 16u : 0u);
+    uint32_t at = swz(t >> 3, chunk);
+    for (int r = t >> 3; r < padded; r += 4 * kStep, at += 4 * kStep * kRowB) {
+        uint32_t id[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) id[i] = (r + i * kStep < padded) ? (uint32_t)glob[r + i * kStep] : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (r + i * kStep < padded) {
+                const uint32_t bytes = r + i * kStep < count ? 16u : 0u;
+                ptx::cp_async_16(dst0 + at + i * kStep * kRowB, s0 + (uint64_t)id[i] * ld0, bytes);
+                ptx::cp_async_16(dst1 + at + i * kStep * kRowB, s1 + (uint64_t)id[i] * ld1, bytes);
+            }
+        }
     }
+}
+
+// Operand descriptor (128-byte swizzle, 1024 bytes between eight-row groups) whose low word holds the address and the
+// leading-dimension offset, both in 16-byte units: stepping through an operand is one 32-bit addition for the issuing thread.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) { return (saddr >> 4) | ((lbo_bytes >> 4) << 16); }
+__device__ __forceinline__ uint64_t desc(uint32_t lo) {
+    constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "n"(hi));
+    return d;
+}
+
+__device__ __forceinline__ uint64_t pair(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 halves(uint64_t v) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
 __device__ __forceinline__ uint4 pack8(const float* f) {
@@ -140,13 +205,24 @@ __device__ __forceinline__ void stage32(uint8_t* stage, int row, uint32_t chunk0
 #pragma unroll
     for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(stage + swz((uint32_t)row, chunk0 + q)) = pack8(v + q * 8);
 }
-// staged rows [0, count) to the rows glob[] of an output, whole 128-byte rows
+// staged rows [0, count) to the rows glob[] of an output, whole 128-byte rows, four in flight per thread
 template <int kThreads>
-__device__ __forceinline__ void store_rows(__nv_bfloat16* out, int64_t ld, int col0, const uint8_t* stage, const int32_t* glob, int count) {
+__device__ __forceinline__ void store_rows(__nv_bfloat16* out, uint32_t ld, int col0, const uint8_t* stage, const int32_t* glob, int count) {
     const uint32_t chunk = threadIdx.x & 7u;
-    for (int r = threadIdx.x >> 3; r < count; r += kThreads / 8) {
-        const uint4 pk = *reinterpret_cast<const uint4*>(stage + swz((uint32_t)r, chunk));
-        ptx::st_global_v4(out + (int64_t)glob[r] * ld + col0 + chunk * 8, pk.x, pk.y, pk.z, pk.w);
+    uint4* to = reinterpret_cast<uint4*>(out + col0) + chunk;
+    for (int r0 = threadIdx.x >> 3; r0 < count; r0 += 4 * (kThreads / 8)) {
+        const uint8_t* from = stage + swz((uint32_t)r0, chunk);            // (rows a multiple of 8 apart: the same place in the swizzle)
+        int32_t id[4];
+        uint4 pk[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (r0 + i * (kThreads / 8) < count) {
+                id[i] = glob[r0 + i * (kThreads / 8)];
+                pk[i] = *reinterpret_cast<const uint4*>(from + i * (kThreads / 8) * kRowB);
+            }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (r0 + i * (kThreads / 8) < count) ptx::st_global_v4(to + (uint64_t)(uint32_t)id[i] * ld, pk[i].x, pk[i].y, pk[i].z, pk[i].w);
     }
 }
 
@@ -194,21 +270,33 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
 
     // rows of problem `prob` into buffer half `b`, then its copies (after a barrier: the rows come from shared memory)
     auto begin_problem = [&](const Meta& m, int prob, int b) {
-        if (threadIdx.x < AttnShared<G>::kTok) {
-            sh.q_glob[b][threadIdx.x] = m.q;
-            sh.k_glob[b][threadIdx.x] = m.k;
+        const int t = (int)threadIdx.x;
+        if (t < AttnShared<G>::kTok) {
+            sh.q_glob[b][t] = m.q;
+            sh.k_glob[b][t] = m.k;
         }
         __syncthreads();
         if (m.nq <= 0 || m.nk <= 0) return;
         const int col0 = (prob % p.heads) * kD;
-        load_rows<kThreads>(sQ, p.Q, p.ld_qkv, sh.q_glob[b], m.nq, col0);
-        load_rows<kThreads>(sK, p.K, p.ld_qkv, sh.k_glob[b], m.nk, col0);
-        load_rows<kThreads>(sDA, p.dA, p.ld_da, sh.q_glob[b], m.nq, col0);
-        load_rows<kThreads>(sV, p.V, p.ld_qkv, sh.k_glob[b], m.nk, col0);
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side)                  // (one loop body: copies of it cost registers)
+            load_rows<kThreads>(side ? sK : sQ, side ? sV : sDA, (side ? p.K : p.Q) + col0, p.ld_qkv, (side ? p.V : p.dA) + col0,
+                                side ? p.ld_qkv : p.ld_da, side ? sh.k_glob[b] : sh.q_glob[b], side ? m.nk : m.nq, t);
     };
-    // every thread of the block waits for a commit; false (for all of them) when any wait gave up
+    // zeros for the rows of problem `prob` outside its lists
+    auto zero_rows = [&](int prob, int nq, int nk, const int32_t* q_glob, const int32_t* k_glob) {
+        if (!p.zero_fill) return;
+        const int b = prob / p.heads, col0 = (prob % p.heads) * kD;
+        const bool same = p.q_rows == p.k_rows && p.q_offs == p.k_offs;
+        if (p.q_rows != nullptr)
+            zero_unlisted_rows(p.dQ, same ? p.dK : nullptr, same ? p.dV : nullptr, p.ld_out, col0, q_glob, nq, b * p.N, p.N, warp, kThreads / 32, lane);
+        if (p.k_rows != nullptr && !same)
+            zero_unlisted_rows(nullptr, p.dK, p.dV, p.ld_out, col0, k_glob, nk, b * p.N, p.N, warp, kThreads / 32, lane);
+    };
+    // every thread of the block waits for a commit (one polls); false for all of them when the wait gave up
     auto wait_products = [&](uint64_t* bar, uint32_t& n) {
-        bool good = ptx::mbar_wait(ptx::smem_addr(bar), n & 1u, abort_flag, p.status_word);
+        bool good = true;
+        if (threadIdx.x == 0) good = ptx::mbar_wait(ptx::smem_addr(bar), n & 1u, abort_flag, p.status_word);
         ++n;
         good = !__syncthreads_or(!good);
         ptx::tc_fence_after_sync();
@@ -225,7 +313,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         cur = fetch_meta(p, next, (int)threadIdx.x);        // travels while this problem computes
         const int32_t *q_glob = sh.q_glob[buf], *k_glob = sh.k_glob[buf];
         if (nq <= 0 || nk <= 0) {                            // nothing to compute: only the zeros of the unlisted rows
-            zero_unlisted_rows(p, prob, nq, nk, q_glob, k_glob, (int)threadIdx.x, kThreads);
+            zero_rows(prob, nq, nk, q_glob, k_glob);
             if (next < problems) begin_problem(cur, next, buf ^ 1);
             continue;
         }
@@ -242,73 +330,104 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             const int q_here = nq - qt * 128 < 128 ? nq - qt * 128 : 128;
             const uint32_t q_steps = (uint32_t)(q_here + 15) >> 4;
             const uint32_t idesc_s = ptx::umma_idesc_bf16(128, n_keys, false, false);
+            const uint32_t dQ0 = desc_lo(sQ + qt * kTileB, 16), dDA0 = desc_lo(sDA + qt * kTileB, 16), dK0 = desc_lo(sK, 16), dV0 = desc_lo(sV, 16);
             if (threadIdx.x == 0) {
                 ptx::tc_fence_after_sync();
 #pragma unroll
                 for (uint32_t u = 0; u < 4; ++u) {           // the two products alternate: they fill different accumulators
-                    ptx::umma_bf16(tmem, ptx::umma_desc_sw128(sQ + qt * kTileB + u * 32, 16, 1024), ptx::umma_desc_sw128(sK + u * 32, 16, 1024), idesc_s, u != 0);
-                    if (!shared_cols)
-                        ptx::umma_bf16(tmem + col_ds, ptx::umma_desc_sw128(sDA + qt * kTileB + u * 32, 16, 1024), ptx::umma_desc_sw128(sV + u * 32, 16, 1024), idesc_s, u != 0);
+                    ptx::umma_bf16(tmem, desc(dQ0 + u * 2), desc(dK0 + u * 2), idesc_s, u != 0);
+                    if (!shared_cols) ptx::umma_bf16(tmem + col_ds, desc(dDA0 + u * 2), desc(dV0 + u * 2), idesc_s, u != 0);
                 }
                 ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
             }
-            if (qt == 0) zero_unlisted_rows(p, prob, nq, nk, q_glob, k_glob, (int)threadIdx.x, kThreads);
+            if (qt == 0) zero_rows(prob, nq, nk, q_glob, k_glob);
             ok = wait_products(&sh.bar_s, n_s);
             if (!ok) break;
-            // ---- this thread's 64 columns of its row.  Columns from nk on (padding keys, stale columns past n_keys) are masked ----
-            float e[2][32];
+            // ---- this thread's 64 columns of its row, in two chunks of 32 which are skipped past n_keys.  Columns from nk on
+            //      (padding keys) are masked; stale columns may hold anything, NaN included ----
+            uint64_t e[2][16];                               // S, then e^(s - own maximum), packed in pairs
             float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four interleaved chains, not one of 64 links
-            if (key0 < n_keys) {
-                ptx::tmem_ld_32x32(tmem + (uint32_t)key0 + lane_off, e[0]);
-                if (key0 + 32 < n_keys) ptx::tmem_ld_32x32(tmem + (uint32_t)key0 + 32u + lane_off, e[1]);
-                ptx::tmem_ld_wait();
 #pragma unroll
-                for (int j = 0; j < 64; ++j) {
-                    if (key0 + 64 > nk && key0 + j >= nk) e[j >> 5][j & 31] = -INFINITY;
-                    mx4[j & 3] = fmaxf(mx4[j & 3], e[j >> 5][j & 31]);
+            for (int c = 0; c < 2; ++c) {
+                const int first = key0 + c * 32;
+                if (first >= n_keys) break;
+                float v[32];
+                ptx::tmem_ld_32x32(tmem + (uint32_t)first + lane_off, v);
+                ptx::tmem_ld_wait();
+                if (first + 32 > nk) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = first + j < nk ? v[j] : -INFINITY;
                 }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], v[j]);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) e[c][j] = pair(v[2 * j], v[2 * j + 1]);
             }
             if (shared_cols) {
                 ptx::tc_fence_before_sync();
-                __syncthreads();                             // S has been read by every warp
+                __syncthreads();                              // S has been read by every warp
                 if (threadIdx.x == 0) {
                     ptx::tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t u = 0; u < 4; ++u)
-                        ptx::umma_bf16(tmem, ptx::umma_desc_sw128(sDA + qt * kTileB + u * 32, 16, 1024), ptx::umma_desc_sw128(sV + u * 32, 16, 1024), idesc_s, u != 0);
+                        ptx::umma_bf16(tmem, desc(dDA0 + u * 2), desc(dV0 + u * 2), idesc_s, u != 0);
                     ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
                 }
             }
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-            float l4[4] = {0.f, 0.f, 0.f, 0.f}, u4[4] = {0.f, 0.f, 0.f, 0.f};
-            if (key0 < n_keys) {
-                const float nm = mx > -INFINITY ? -mx * sl2 : 0.f;
+            uint64_t l2[2] = {0ull, 0ull}, u2[2] = {0ull, 0ull};
+            const float nm = mx > -INFINITY ? -mx * sl2 : 0.f;
+            const uint64_t sl22 = pair(sl2, sl2), nm2 = pair(nm, nm);
 #pragma unroll
-                for (int j = 0; j < 64; ++j) {
-                    e[j >> 5][j & 31] = ex2(fmaf(e[j >> 5][j & 31], sl2, nm));          // masked columns: 2^-inf = 0
-                    l4[j & 3] += e[j >> 5][j & 31];
+            for (int c = 0; c < 2; ++c) {
+                if (key0 + c * 32 >= n_keys) break;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const float2 x = halves(fma2(e[c][j], sl22, nm2));       // masked columns: 2^-inf = 0
+                    e[c][j] = pair(ex2(x.x), ex2(x.y));
+                    l2[j & 1] = add2(l2[j & 1], e[c][j]);
                 }
             }
             if (shared_cols) {
                 ok = wait_products(&sh.bar_s, n_s);
                 if (!ok) break;
             }
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                if (key0 + c * 32 < n_keys) {
-                    float ds[32];
-                    ptx::tmem_ld_32x32(tmem + col_ds + (uint32_t)(key0 + c * 32) + lane_off, ds);
-                    ptx::tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {           // a stale column may hold anything, NaN included
-                        const float d = (key0 + 64 > nk && key0 + c * 32 + j >= nk) ? 0.f : ds[j];
-                        u4[j & 3] = fmaf(e[c][j], d, u4[j & 3]);
-                    }
+            // the next problem's rows on their way into L2, a query's and a key's two lines a thread
+            if (qt == 0 && next < problems) {
+                const int next_col0 = (next % p.heads) * kD;
+                if ((int)threadIdx.x < cur.nq) {
+                    prefetch_row(p.Q + next_col0, cur.q, p.ld_qkv);
+                    prefetch_row(p.dA + next_col0, cur.q, p.ld_da);
+                }
+                if ((int)threadIdx.x < cur.nk) {
+                    prefetch_row(p.K + next_col0, cur.k, p.ld_qkv);
+                    prefetch_row(p.V + next_col0, cur.k, p.ld_qkv);
                 }
             }
+            // 16 columns of dS from column `first` on, in pairs
+            auto load_ds = [&](int first, uint64_t (&d)[8]) {
+                float v[16];
+                ptx::tmem_ld_32x16(tmem + col_ds + (uint32_t)first + lane_off, v);
+                ptx::tmem_ld_wait();
+                if (first + 16 > nk) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = first + j < nk ? v[j] : 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) d[j] = pair(v[2 * j], v[2 * j + 1]);
+            };
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (key0 + c * 16 >= n_keys) break;
+                uint64_t d[8];
+                load_ds(key0 + c * 16, d);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) u2[j & 1] = fma2(e[c >> 1][(c & 1) * 8 + j], d[j], u2[j & 1]);
+            }
+            const float2 lx = halves(add2(l2[0], l2[1])), ux = halves(add2(u2[0], u2[1]));
             sh.part[g][row][0] = mx;
-            sh.part[g][row][1] = (l4[0] + l4[1]) + (l4[2] + l4[3]);
-            sh.part[g][row][2] = (u4[0] + u4[1]) + (u4[2] + u4[3]);
+            sh.part[g][row][1] = lx.x + lx.y;
+            sh.part[g][row][2] = ux.x + ux.y;
             asm volatile("bar.sync %0, %1;" ::"r"(1 + quad), "n"(32 * G) : "memory");   // the G warps of this quadrant
             float mm = sh.part[0][row][0];
 #pragma unroll
@@ -323,54 +442,56 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             const float inv_l = 1.f / L;
             const float mine = ex2((mx - mm) * sl2) * inv_l;
             const float nds = -U * inv_l * p.scale;          // -rowsum(S dS) / sqrt(d)
+            const uint64_t mine2 = pair(mine, mine), nds2 = pair(nds, nds), scale2 = pair(p.scale, p.scale);
             uint32_t dm[32];                                 // dM waits here when its blocks are those of S
             uint8_t* blkP = gen + (uint32_t)g * p.block_bytes;
             uint8_t* blkM = gen + p.off_dm + (uint32_t)g * p.dm_stride;
             const bool row_fits = (uint32_t)row * kRowB < p.block_bytes;
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                if (key0 + c * 32 < n_keys) {
-                    float ds[32];
-                    ptx::tmem_ld_32x32(tmem + col_ds + (uint32_t)(key0 + c * 32) + lane_off, ds);
-                    ptx::tmem_ld_wait();
+            for (int c = 0; c < 4; ++c) {
+                if (key0 + c * 16 >= n_keys) break;
+                uint64_t d[8];
+                load_ds(key0 + c * 16, d);
+                uint32_t w[8];
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float d = (key0 + 64 > nk && key0 + c * 32 + j >= nk) ? 0.f : ds[j];
-                        e[c][j] *= mine;                     // S
-                        ds[j] = e[c][j] * fmaf(d, p.scale, nds);                        // dM / sqrt(d)
-                    }
+                for (int j = 0; j < 8; ++j) {
+                    const uint64_t s2 = mul2(e[c >> 1][(c & 1) * 8 + j], mine2);        // S
+                    const float2 sf = halves(s2), mf = halves(mul2(s2, fma2(d[j], scale2, nds2)));   // dM / sqrt(d)
+                    w[j] = pack2(sf.x, sf.y);
+                    dm[c * 8 + j] = pack2(mf.x, mf.y);
+                }
+                if (row_fits) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if (row_fits) *reinterpret_cast<uint4*>(blkP + swz((uint32_t)row, (uint32_t)(c * 4 + q))) = pack8(&e[c][q * 8]);
-                        const uint4 w = pack8(ds + q * 8);
-                        if (kSeparate) {
-                            if (row_fits) *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 4 + q))) = w;
-                        } else {
-                            dm[c * 16 + q * 4] = w.x; dm[c * 16 + q * 4 + 1] = w.y; dm[c * 16 + q * 4 + 2] = w.z; dm[c * 16 + q * 4 + 3] = w.w;
-                        }
+                    for (int q = 0; q < 2; ++q) {
+                        *reinterpret_cast<uint4*>(blkP + swz((uint32_t)row, (uint32_t)(c * 2 + q))) = make_uint4(w[q * 4], w[q * 4 + 1], w[q * 4 + 2], w[q * 4 + 3]);
+                        if (kSeparate)
+                            *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 2 + q))) =
+                                make_uint4(dm[c * 8 + q * 4], dm[c * 8 + q * 4 + 1], dm[c * 8 + q * 4 + 2], dm[c * 8 + q * 4 + 3]);
                     }
                 }
             }
             ptx::fence_async_proxy();                        // the blocks are read by the tensor core
             ptx::tc_fence_before_sync();
-            __syncthreads();                                 // S and dS in tensor memory are dead from here on
+            __syncthreads();                                  // S and dS in tensor memory are dead from here on
             // ---- the gradient products; only the 16-row steps that hold tokens run, accumulators take turns ----
             const uint32_t id_t = ptx::umma_idesc_bf16(128, 64, true, true);             // dV, dK: both operands MN-major
             const uint32_t id_q = ptx::umma_idesc_bf16(128, 64, false, true);            // dQ: dM K-major, K MN-major
             const int KT = G == 2 ? 1 : (nk + 127) >> 7;
+            // 16 rows of a token tile are 2048 bytes; 16 columns of a block 32 bytes.  (N = 64 is one block: the leading-dimension
+            // offset of the B operands plays no part.)
+            const uint32_t dP = desc_lo(sP, p.block_bytes), dMt = desc_lo(sDM, p.dm_stride), dMk = desc_lo(sDM, 16);
             auto issue_dv = [&](uint32_t u) {
-                for (int kt = 0; kt < KT; ++kt)
-                    ptx::umma_bf16(tmem + kColDV + (uint32_t)kt * 64u, ptx::umma_desc_sw128(sP + (uint32_t)kt * 2u * p.block_bytes + u * 2048, p.block_bytes, 1024),
-                                   ptx::umma_desc_sw128(sDA + qt * kTileB + u * 2048, kTileB, 1024), id_t, (qt | (int)u) != 0);
+                ptx::umma_bf16(tmem + kColDV, desc(dP + u * 128u), desc(dDA0 + u * 128u), id_t, (qt | (int)u) != 0);
+                if (G == 4 && KT > 1)
+                    ptx::umma_bf16(tmem + kColDV + 64u, desc(dP + (p.block_bytes >> 3) + u * 128u), desc(dDA0 + u * 128u), id_t, (qt | (int)u) != 0);
             };
             auto issue_dk = [&](uint32_t u) {
-                for (int kt = 0; kt < KT; ++kt)
-                    ptx::umma_bf16(tmem + kColDK + (uint32_t)kt * 64u, ptx::umma_desc_sw128(sDM + (uint32_t)kt * 2u * p.dm_stride + u * 2048, p.dm_stride, 1024),
-                                   ptx::umma_desc_sw128(sQ + qt * kTileB + u * 2048, kTileB, 1024), id_t, (qt | (int)u) != 0);
+                ptx::umma_bf16(tmem + kColDK, desc(dMt + u * 128u), desc(dQ0 + u * 128u), id_t, (qt | (int)u) != 0);
+                if (G == 4 && KT > 1)
+                    ptx::umma_bf16(tmem + kColDK + 64u, desc(dMt + (p.dm_stride >> 3) + u * 128u), desc(dQ0 + u * 128u), id_t, (qt | (int)u) != 0);
             };
             auto issue_dq = [&](uint32_t u) {
-                ptx::umma_bf16(tmem + kColDQ, ptx::umma_desc_sw128(sDM + (u >> 2) * p.dm_stride + (u & 3u) * 32, 16, 1024),
-                               ptx::umma_desc_sw128(sK + u * 2048, kTileB, 1024), id_q, u != 0);
+                ptx::umma_bf16(tmem + kColDQ, desc(dMk + (u >> 2) * (p.dm_stride >> 4) + (u & 3u) * 2u), desc(dK0 + u * 128u), id_q, u != 0);
             };
             const uint32_t steps = q_steps > k_steps ? q_steps : k_steps;
             if (!kSeparate) {
@@ -382,13 +503,9 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 ok = wait_products(&sh.bar_o, n_o);
                 if (!ok) break;
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
-                    if (key0 + c * 32 < n_keys && row_fits) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 4 + q))) =
-                                make_uint4(dm[c * 16 + q * 4], dm[c * 16 + q * 4 + 1], dm[c * 16 + q * 4 + 2], dm[c * 16 + q * 4 + 3]);
-                    }
+                for (int c = 0; c < 8; ++c)
+                    if (key0 + (c >> 1) * 16 < n_keys && row_fits)
+                        *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)c)) = make_uint4(dm[c * 4], dm[c * 4 + 1], dm[c * 4 + 2], dm[c * 4 + 3]);
                 ptx::fence_async_proxy();
                 ptx::tc_fence_before_sync();
                 __syncthreads();
@@ -442,14 +559,16 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             }
             ptx::tc_fence_before_sync();
             __syncthreads();
-            store_rows<kThreads>(p.dV, p.ld_out, col0, gen, k_glob, nk);
-            store_rows<kThreads>(p.dK, p.ld_out, col0, gen + stage_b, k_glob, nk);
+#pragma unroll 1
+            for (int which = 0; which < (kSeparate ? 3 : 2); ++which)      // (one loop body: copies of it cost registers)
+                store_rows<kThreads>(which == 0 ? p.dV : which == 1 ? p.dK : p.dQ, p.ld_out, col0, gen + which * stage_b,
+                                     which == 2 ? q_glob : k_glob, which == 2 ? nq : nk);
             if (!kSeparate) {
                 __syncthreads();
                 if ((uint32_t)row * kRowB < stage_b) stage32(gen, row, (uint32_t)(g * 4), v);
                 __syncthreads();
+                store_rows<kThreads>(p.dQ, p.ld_out, col0, gen, q_glob, nq);
             }
-            store_rows<kThreads>(p.dQ, p.ld_out, col0, kSeparate ? gen + 2 * stage_b : gen, q_glob, nq);
         } else {
             // group g takes dV (g even) or dK (g odd) of key tile g / 2
             const int kt = g >> 1;
@@ -464,14 +583,15 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             }
             ptx::tc_fence_before_sync();
             __syncthreads();
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < 4; ++i) {
                 const int first = (i >> 1) * 128;
                 if (first < nk)
                     store_rows<kThreads>((i & 1) ? p.dK : p.dV, p.ld_out, col0, gen + (uint32_t)i * kTileB, k_glob + first, nk - first < 128 ? nk - first : 128);
             }
         }
-        // (the barrier in front of the next problem's products keeps its writers off stages still being stored)
+        // (the barrier at the next problem's start keeps its writers off stages still being stored)
+        ptx::tc_fence_before_sync();
     }
     ptx::cp_async_wait_all();
     ptx::tc_fence_before_sync();
@@ -543,7 +663,7 @@ cudaError_t launch_attention_backward(const void* Q, const void* K, const void* 
     AttnParams prm;
     prm.Q = static_cast<const __nv_bfloat16*>(Q); prm.K = static_cast<const __nv_bfloat16*>(K);
     prm.V = static_cast<const __nv_bfloat16*>(V); prm.dA = static_cast<const __nv_bfloat16*>(dA);
-    prm.ld_qkv = ld_qkv; prm.ld_da = ld_da; prm.ld_out = ld_out;
+    prm.ld_qkv = (uint32_t)(ld_qkv / 8); prm.ld_da = (uint32_t)(ld_da / 8); prm.ld_out = (uint32_t)(ld_out / 8);
     prm.q_rows = q_rows; prm.q_offs = q_offs; prm.k_rows = k_rows; prm.k_offs = k_offs;
     prm.B = (int)B; prm.N = (int)N; prm.heads = (int)heads;
     prm.dQ = static_cast<__nv_bfloat16*>(dQ); prm.dK = static_cast<__nv_bfloat16*>(dK); prm.dV = static_cast<__nv_bfloat16*>(dV);
