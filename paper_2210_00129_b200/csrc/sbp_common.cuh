@@ -215,10 +215,10 @@ int    tc_backward_kernel_count(int64_t M_keep_cap, int64_t C_in, int64_t C_out,
                                 bool want_db, bool dy_packed);
 // dW (nullable) and dX (nullable) of one layer in a single persistent kernel (+ the split reduce); when db is
 // given its column sums ride along in the same kernel (db_workspace: kNumSMs * C_out floats) + one reduce
-// (dy_rows / dx_rows as for launch_fma_backward)
+// (dy_rows / dx_rows as for launch_fma_backward; w_out_in: W and dW are [C_out, C_in])
 sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W, const int32_t* dy_rows,
                               const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
-                              int64_t C_out, float* dW, bool accumulate, void* dX, float* db, float* workspace,
+                              int64_t C_out, float* dW, bool accumulate, void* dX, float* db, bool w_out_in, float* workspace,
                               float* db_workspace, int32_t* status_word, cudaStream_t stream);
 
 }  // namespace sbp

@@ -1,7 +1,6 @@
-// Matrix transposes for weights kept in the [C_out, C_in] layout (SBP_FLAG_W_OUT_IN): the backward kernels work
-// on W [C_in, C_out] (the paper's convention, Sec. 3.2.1), so such a W is transposed into the workspace before
-// them and dW is transposed (or transpose-added) out of the workspace after them.  32 x 32 tiles through
-// shared memory, both sides coalesced; HBM-bound and small next to the products.
+// Matrix transposes for small weights kept in the [C_out, C_in] layout (SBP_FLAG_W_OUT_IN): such a W is transposed into the
+// workspace before the backward kernels and dW is transposed (or transpose-added) out of the workspace after them; larger
+// weights are read and written in place.  32 x 32 tiles through shared memory, both sides coalesced; bound by their launches.
 #include "sbp_common.cuh"
 
 namespace sbp {
