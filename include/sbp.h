@@ -201,9 +201,10 @@ size_t sbp_linear_backward_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_ke
  *
  * Weight layout.  The paper writes Y = X W with W [C_in, C_out] (Sec. 3.2.1), and that
  * is the native layout here.  With SBP_FLAG_W_OUT_IN both W and dW are [C_out, C_in]
- * (dW[j, i] as above with the indices swapped): W is transposed into the workspace
- * before the products and dW is transposed out of it after them (two small extra
- * launches); the results are the same numbers.
+ * (dW[j, i] as above with the indices swapped) and the results are the same numbers.
+ * From 131072 weights on both are read and written in place; smaller ones are
+ * transposed into the workspace before the products and out of it after them (two
+ * small extra launches).
  *
  * SBP_BF16: inputs bf16, products accumulated in fp32 on the tensor cores, dX
  * rounded to bf16 (nearest even).  SBP_F32: plain fp32 FMA arithmetic.
@@ -269,7 +270,7 @@ sbp_status sbp_act_backward(sbp_dtype dt, sbp_activation act, const void* Z_keep
  *   sbp_patch_scatter   dX[b, stride*ho + dh, stride*wo + dw, c] = dX_patches[m, (dh, dw, c)] for kept m; every
  *                       other input position (dropped patches, positions no patch covers) = +0.0.  Every element
  *                       of dX is written exactly once.  workspace: sbp_patch_scatter_workspace_bytes(...) bytes,
- *                       256-byte aligned (one int32 per output position).
+ *                       256-byte aligned (one int32 per output position; checked, and at present not used).
  * C * sizeof(element) must be a multiple of 16 (else SBP_ERR_UNSUPPORTED); stride < k, k larger than the map and
  * other bad sizes or pointers give SBP_ERR_INVALID_ARG; a short workspace SBP_ERR_WORKSPACE.  M_keep is
  * *M_keep_dev when given, else M_keep_cap.  Bit-exact copies; deterministic.

@@ -8,85 +8,135 @@
 //   patch scatter: the packed input gradient [M_keep, k * k * C] back into dX [B, H, W, C]; every input position
 //                  outside the kept patches (dropped positions, positions no patch covers when s > k) gets +0.0
 // Both move 16-byte vectors and are HBM-bound.
-#include "sbp_common.cuh"
+#include "row_copy.cuh"
+#include "zero_rows.cuh"
 
 namespace sbp {
 namespace {
 
-constexpr int kPatchThreads = 256;
-
 struct PatchGeom {
     int H, W, Ho, Wo, k, s;
+    int Hc, Wc;                     // cells of s x s input positions (cut short at the map's edges): output position
+                                    // (ho, wo) owns cell (ho, wo), cells past the output grid belong to none
     uint32_t vec_c;                 // 16-byte vectors per input position (C * element size / 16)
+    FastDiv row;                    // vectors of a patch row (k * k positions)
+    FastDiv seg;                    // ... of one of its k pieces
+    FastDiv map, line;              // output positions of a sample, of a row of the output map
+    FastDiv cell;                   // vectors of a whole cell
+    FastDiv cell_line;              // ... of one of its s rows
+    int cells_per_block;
+    uint32_t slice;                 // vectors of its cells that a block writes (large cells: several blocks per cell)
 };
 
-__device__ __forceinline__ uint4 ld_stream16(const uint4* p) {
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-
-__global__ void __launch_bounds__(kPatchThreads)
+// A block writes 1024 consecutive vectors of the patch rows.  Four 64-bit divisions a vector held it at 3.2 TB/s: 25088 patch
+// rows of 512 bf16 16.0 -> 9.4 us (5.5 TB/s).
+__global__ void __launch_bounds__(kCopyThreads)
 patch_gather_kernel(const uint4* __restrict__ X, const PatchGeom g, const int32_t* __restrict__ keep_rows,
                     const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, uint4* __restrict__ X_keep) {
     pdl_wait();
     const int64_t M_keep = load_m_keep(M_keep_dev, M_keep_cap);
-    const uint32_t vec_seg = (uint32_t)g.k * g.vec_c;                  // one piece: k positions of a row of the patch
-    const uint32_t vec_row = (uint32_t)g.k * vec_seg;                  // one patch row
-    const int64_t total = M_keep_cap * (int64_t)vec_row;
-    const int64_t stride = (int64_t)gridDim.x * kPatchThreads;
-    for (int64_t i = (int64_t)blockIdx.x * kPatchThreads + threadIdx.x; i < total; i += stride) {
-        const int64_t m = i / vec_row;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);                          // rows past M_keep are cleared
+    const int64_t begin = (int64_t)blockIdx.x * kCopySpan, total = M_keep_cap * (int64_t)g.row.d;
+    const SpanRows span(begin, g.row.d);
+    int64_t src[kCopyUnroll];
+    uint4 v[kCopyUnroll];
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) {
+        uint32_t q;
+        const uint32_t in_row = span.place(threadIdx.x + u * kCopyThreads, g.row, &q);
+        const int64_t m = span.first + q;
+        src[u] = -1;                                                   // rows past M_keep are cleared
         if (m < M_keep) {
-            const uint32_t in_row = (uint32_t)(i - m * vec_row);
-            const uint32_t dh = in_row / vec_seg, off = in_row - dh * vec_seg;
-            const int64_t pos = __ldg(keep_rows + m);
-            const int64_t b = pos / ((int64_t)g.Ho * g.Wo);
-            const int rem = (int)(pos - b * (int64_t)g.Ho * g.Wo);
-            const int ho = rem / g.Wo, wo = rem - ho * g.Wo;
-            const int64_t pix = (b * g.H + (int64_t)g.s * ho + dh) * g.W + (int64_t)g.s * wo;
-            v = ld_stream16(X + pix * g.vec_c + off);
+            const uint32_t dh = g.seg(in_row), off = in_row - dh * g.seg.d;
+            const uint32_t pos = (uint32_t)__ldg(keep_rows + m);
+            const uint32_t b = g.map(pos), rem = pos - b * g.map.d;
+            const uint32_t ho = g.line(rem), wo = rem - ho * g.line.d;
+            const int64_t pix = ((int64_t)b * g.H + (int64_t)g.s * ho + dh) * g.W + (int64_t)g.s * wo;
+            src[u] = pix * g.vec_c + off;
         }
-        X_keep[i] = v;
+    }
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) v[u] = (src[u] >= 0) ? ld_stream(X + src[u]) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) {
+        const int64_t i = begin + threadIdx.x + u * kCopyThreads;
+        if (i < total) X_keep[i] = v[u];
     }
     pdl_launch_dependents();
 }
 
-// slot[pos] = m for the kept output positions (the slots were set to -1 beforehand)
-__global__ void patch_slots_kernel(const int32_t* __restrict__ keep_rows, const int32_t* __restrict__ M_keep_dev,
-                                   int64_t M_keep_cap, int32_t* __restrict__ slot, const int32_t* status_word) {
+// A block writes the input positions of `cells_per_block` consecutive cells.  Which packed row covers a cell comes from the
+// block's stretch of the ascending keep_rows list, found by search: one launch, where a map from output positions to packed
+// rows in global memory took a memset, a launch to fill it and a look-up for every vector.  [64, 56, 56, 128] bf16 from 25088
+// packed rows: memset + 3.3 + 26.3 us -> 18.2 us (77 MB; a third of it the search's dependent loads, which eight blocks an
+// SM overlap only in part).
+constexpr int kMaxCells = 128;
+__global__ void __launch_bounds__(kCopyThreads)
+patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int32_t* __restrict__ keep_rows,
+                     const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, int64_t cells, uint4* __restrict__ dX,
+                     const int32_t* status_word) {
+    __shared__ int32_t row_of[kMaxCells];          // packed row of each cell, -1: none
+    __shared__ int32_t pixel_of[kMaxCells];        // first input position of each cell
+    __shared__ int2 room[kMaxCells];               // rows of the cell inside the map, vectors of such a row
     pdl_launch_dependents();
     pdl_wait();
     if (status_word != nullptr && *reinterpret_cast<const volatile int32_t*>(status_word) != 0) return;
     const int64_t M_keep = load_m_keep(M_keep_dev, M_keep_cap);
-    for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < M_keep; m += (int64_t)gridDim.x * blockDim.x)
-        slot[__ldg(keep_rows + m)] = (int32_t)m;
-}
-
-__global__ void __launch_bounds__(kPatchThreads)
-patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int32_t* __restrict__ slot, int64_t positions,
-                     uint4* __restrict__ dX, const int32_t* status_word) {
-    pdl_launch_dependents();
-    pdl_wait();
-    if (status_word != nullptr && *reinterpret_cast<const volatile int32_t*>(status_word) != 0) return;
-    const int64_t total = positions * (int64_t)g.vec_c;               // every 16-byte vector of dX is written exactly once
-    const uint32_t vec_seg = (uint32_t)g.k * g.vec_c, vec_row = (uint32_t)g.k * vec_seg;
-    const int64_t stride = (int64_t)gridDim.x * kPatchThreads;
-    for (int64_t i = (int64_t)blockIdx.x * kPatchThreads + threadIdx.x; i < total; i += stride) {
-        const int64_t pix = i / g.vec_c;
-        const uint32_t c = (uint32_t)(i - pix * g.vec_c);
-        const int w = (int)(pix % g.W);
-        const int64_t bh = pix / g.W;
-        const int h = (int)(bh % g.H);
-        const int64_t b = bh / g.H;
-        const int ho = h / g.s, dh = h - ho * g.s, wo = w / g.s, dw = w - wo * g.s;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (dh < g.k && dw < g.k && ho < g.Ho && wo < g.Wo) {
-            const int32_t m = __ldg(slot + (b * g.Ho + ho) * g.Wo + wo);
-            if (m >= 0) v = ld_stream16(dXp + (int64_t)m * vec_row + (uint32_t)dh * vec_seg + (uint32_t)dw * g.vec_c + c);
+    const int64_t c0 = (int64_t)blockIdx.x * g.cells_per_block;
+    const int n = cells - c0 < g.cells_per_block ? (int)(cells - c0) : g.cells_per_block;
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < kMaxCells) row_of[threadIdx.x] = -1;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        // output positions in front of cell c, and the cell of an output position, by the two grids' sizes
+        const auto positions_before = [&](int64_t c) {
+            const int64_t b = c / ((int64_t)g.Hc * g.Wc);
+            const int rem = (int)(c - b * ((int64_t)g.Hc * g.Wc)), hc = rem / g.Wc, wc = rem - hc * g.Wc;
+            const int64_t in_map = hc < g.Ho ? (int64_t)hc * g.Wo + (wc < g.Wo ? wc : g.Wo) : (int64_t)g.Ho * g.Wo;
+            return b * g.Ho * g.Wo + in_map;
+        };
+        const int64_t begin = positions_before(c0), end = positions_before(c0 + n);
+        for (int64_t m = warp_lower_bound(keep_rows, M_keep, begin, lane) + lane;; m += 32) {
+            const int64_t pos = m < M_keep ? (int64_t)__ldg(keep_rows + m) : end;
+            if (pos >= begin && pos < end) {
+                const uint32_t b = g.map((uint32_t)pos), rem = (uint32_t)pos - b * g.map.d;
+                const uint32_t ho = g.line(rem), wo = rem - ho * g.line.d;
+                row_of[((int64_t)b * g.Hc + ho) * g.Wc + wo - c0] = (int32_t)m;
+            }
+            if (__any_sync(0xffffffffu, pos >= end)) break;
         }
-        dX[i] = v;
+    } else if (threadIdx.x >= 128) {
+        for (int i = threadIdx.x - 128; i < n; i += kCopyThreads - 128) {
+            const int64_t c = c0 + i, bh = c / g.Wc, b = bh / g.Hc;
+            const int wc = (int)(c - bh * g.Wc), hc = (int)(bh - b * g.Hc);
+            pixel_of[i] = (int32_t)((b * g.H + (int64_t)hc * g.s) * g.W + (int64_t)wc * g.s);
+            const int rows = g.H - hc * g.s < g.s ? g.H - hc * g.s : g.s, cols = g.W - wc * g.s < g.s ? g.W - wc * g.s : g.s;
+            room[i] = make_int2(rows, cols * (int)g.vec_c);
+        }
+    }
+    __syncthreads();
+    const uint32_t all = (uint32_t)n * g.cell.d, slice0 = blockIdx.y * g.slice;
+    const uint32_t vectors = all - slice0 < g.slice ? all : slice0 + g.slice;
+    for (uint32_t base = slice0 + threadIdx.x; base < vectors; base += kCopySpan) {
+        uint4 v[kCopyUnroll];
+        int64_t dst[kCopyUnroll];
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u) {
+            const uint32_t i = base + u * kCopyThreads;
+            dst[u] = -1;
+            v[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < vectors) {
+                const uint32_t c = g.cell(i), in_cell = i - c * g.cell.d;
+                const uint32_t dh = g.cell_line(in_cell), off = in_cell - dh * g.cell_line.d;
+                if ((int)dh < room[c].x && (int)off < room[c].y) {
+                    dst[u] = ((int64_t)pixel_of[c] + (int64_t)dh * g.W) * g.vec_c + off;
+                    const int32_t m = row_of[c];
+                    if (m >= 0 && (int)dh < g.k && off < g.seg.d) v[u] = ld_stream(dXp + (int64_t)m * g.row.d + dh * g.seg.d + off);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u)
+            if (dst[u] >= 0) dX[dst[u]] = v[u];
     }
 }
 
@@ -94,15 +144,13 @@ PatchGeom geom(int64_t H, int64_t W, int64_t k, int64_t s, int64_t pos_bytes) {
     PatchGeom g;
     g.H = (int)H; g.W = (int)W; g.k = (int)k; g.s = (int)s;
     g.Ho = (int)((H - k) / s + 1); g.Wo = (int)((W - k) / s + 1);
+    g.Hc = (int)((H + s - 1) / s); g.Wc = (int)((W + s - 1) / s);
     g.vec_c = (uint32_t)(pos_bytes / 16);
+    g.seg = FastDiv((uint32_t)k * g.vec_c);
+    g.row = FastDiv((uint32_t)k * g.seg.d);
+    g.map = FastDiv((uint32_t)((int64_t)g.Ho * g.Wo));
+    g.line = FastDiv((uint32_t)g.Wo);
     return g;
-}
-
-unsigned blocks_for(int64_t vectors) {
-    int64_t blocks = (vectors + kPatchThreads * 4 - 1) / (kPatchThreads * 4);
-    if (blocks < 1) blocks = 1;
-    if (blocks > (int64_t)kNumSMs * 16) blocks = (int64_t)kNumSMs * 16;
-    return (unsigned)blocks;
 }
 
 }  // namespace
@@ -111,27 +159,32 @@ cudaError_t launch_patch_gather(const void* X, int64_t H, int64_t W, int64_t pos
                                 const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M_keep_cap, void* X_keep,
                                 cudaStream_t stream) {
     const PatchGeom g = geom(H, W, k, s, pos_bytes);
-    const int64_t total = M_keep_cap * k * k * (int64_t)g.vec_c;
+    const int64_t total = M_keep_cap * (int64_t)g.row.d;
     if (total == 0) return cudaSuccess;
-    return launch_pdl(patch_gather_kernel, dim3(blocks_for(total)), dim3(kPatchThreads), 0, stream, (const uint4*)X, g, keep_rows,
-                      M_keep_dev, M_keep_cap, (uint4*)X_keep);
+    return launch_pdl(patch_gather_kernel, dim3((unsigned)copy_blocks(total)), dim3(kCopyThreads), 0, stream, (const uint4*)X, g,
+                      keep_rows, M_keep_dev, M_keep_cap, (uint4*)X_keep);
 }
 
 cudaError_t launch_patch_scatter(const void* dXp, int64_t B, int64_t H, int64_t W, int64_t pos_bytes, int64_t k, int64_t s,
                                  const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M_keep_cap, void* dX,
-                                 int32_t* slot, const int32_t* status_word, cudaStream_t stream) {
-    const PatchGeom g = geom(H, W, k, s, pos_bytes);
-    const int64_t outputs = B * (int64_t)g.Ho * g.Wo;
-    cudaError_t e = cudaMemsetAsync(slot, 0xFF, (size_t)outputs * sizeof(int32_t), stream);     // every slot -1
-    if (e != cudaSuccess) return e;
-    int64_t blocks = (M_keep_cap + 255) / 256;
-    if (blocks < 1) blocks = 1;
-    if (blocks > kNumSMs * 8) blocks = kNumSMs * 8;
-    e = launch_pdl(patch_slots_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, keep_rows, M_keep_dev, M_keep_cap, slot, status_word);
-    if (e != cudaSuccess) return e;
-    const int64_t positions = B * H * W;
-    return launch_pdl(patch_scatter_kernel, dim3(blocks_for(positions * g.vec_c)), dim3(kPatchThreads), 0, stream, (const uint4*)dXp, g,
-                      (const int32_t*)slot, positions, (uint4*)dX, status_word);
+                                 const int32_t* status_word, cudaStream_t stream) {
+    PatchGeom g = geom(H, W, k, s, pos_bytes);
+    const int64_t cells = B * g.Hc * g.Wc;
+    const uint32_t cell_w = (uint32_t)(s < W ? s : W), cell_h = (uint32_t)(s < H ? s : H);
+    g.cell_line = FastDiv(cell_w * g.vec_c);
+    g.cell = FastDiv(cell_h * g.cell_line.d);
+    // About 2048 vectors (32 KB) a block: eight blocks of an SM then hide each other's search, and small maps still spread.
+    constexpr uint32_t kTarget = 2048;
+    const uint32_t n = kTarget / g.cell.d;
+    g.cells_per_block = (int)(n < 1 ? 1 : n > (uint32_t)kMaxCells ? (uint32_t)kMaxCells : n);
+    const uint32_t per_block = (uint32_t)g.cells_per_block * g.cell.d;
+    uint32_t slices = (per_block + kTarget - 1) / kTarget;
+    if (slices > 65535u) slices = 65535u;
+    g.slice = (per_block + slices - 1) / slices;
+    slices = (per_block + g.slice - 1) / g.slice;
+    const dim3 grid((unsigned)((cells + g.cells_per_block - 1) / g.cells_per_block), slices);
+    return launch_pdl(patch_scatter_kernel, grid, dim3(kCopyThreads), 0, stream, (const uint4*)dXp, g, keep_rows, M_keep_dev, M_keep_cap,
+                      cells, (uint4*)dX, status_word);
 }
 
 }  // namespace sbp

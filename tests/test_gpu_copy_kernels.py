@@ -1,0 +1,67 @@
+"""The copy kernels (forward cache, patch cache, patch scatter) where their spans, cells and slices end: rows of one vector,
+rows around a span's length, strides beyond the kernel and beyond the map, cells cut by the map's edges, cells of several
+blocks, capacities above the device-side count.  Pure copies: every result is exact."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2210_00129_b200 as sbp
+
+pytestmark = pytest.mark.gpu
+
+
+def _list(n_rows, n_keep, cap, seed):
+    gen = torch.Generator().manual_seed(seed)
+    rows = torch.zeros(max(cap, 1), dtype=torch.int32)
+    rows[:n_keep] = torch.randperm(n_rows, generator=gen)[:n_keep].sort().values.int()
+    return rows.cuda(), torch.tensor([n_keep], dtype=torch.int32, device="cuda")
+
+
+@pytest.mark.parametrize("M,C,keep,cap", [
+    (1, 4, 1, 1), (3000, 4, 1500, 1501), (700, 12, 699, 700), (50, 4 * 1023, 20, 25), (50, 4 * 1024, 20, 20), (50, 4 * 1025, 20, 21),
+    (9, 4 * 5000, 4, 9), (40000, 20, 20000, 20003), (64, 260, 0, 7),
+])
+def test_forward_cache_spans(M, C, keep, cap):
+    X = torch.randn(M, C, device="cuda")
+    rows, cnt = _list(M, keep, cap, M + C)
+    out = torch.full((cap, C), float("nan"), device="cuda")
+    sbp.sbp_forward_cache(sbp.SBP_F32, X, M, C, rows, cnt, cap, out)
+    torch.cuda.synchronize()
+    assert torch.equal(out[:keep], X[rows[:keep].long()])
+    assert not out[keep:].view(torch.int32).any()
+
+
+@pytest.mark.parametrize("B,H,W,C,k,s,ratio", [
+    (2, 8, 8, 4, 1, 1, 0.5), (3, 9, 7, 8, 2, 2, 0.5),          # the last row and column belong to no patch
+    (2, 14, 11, 4, 2, 5, 0.6), (4, 6, 7, 12, 3, 100, 1.0),      # strides beyond the kernel, beyond the map
+    (1, 64, 64, 4, 4, 4, 0.1), (70, 4, 4, 4, 2, 2, 0.5),        # many cells a block; samples inside a block
+    (2, 20, 20, 2000, 5, 10, 0.5),                              # a cell is written by many blocks
+    (1, 7, 300, 36, 3, 3, 0.0),                                 # nothing kept
+])
+def test_patch_cache_and_scatter(B, H, W, C, k, s, ratio):
+    Ho, Wo = (H - k) // s + 1, (W - k) // s + 1
+    Mo, Kc = B * Ho * Wo, k * k * C
+    keep = int(round(ratio * Mo))
+    cap = min(Mo, keep + 3)
+    rows, cnt = _list(Mo, keep, cap, H * W + C)
+    X = torch.randn(B, H, W, C, device="cuda")
+    Xk = torch.full((cap, Kc), float("nan"), device="cuda")
+    sbp.sbp_patch_cache(sbp.SBP_F32, X, B, H, W, C, k, s, rows, cnt, cap, Xk)
+    patches = X[:, :(Ho - 1) * s + k, :(Wo - 1) * s + k].unfold(1, k, s).unfold(2, k, s)          # [B, Ho, Wo, C, k, k]
+    patches = patches.permute(0, 1, 2, 4, 5, 3).reshape(Mo, Kc)
+    pick = rows[:keep].long()
+    dXp = torch.randn(cap, Kc, device="cuda")
+    nbytes = sbp.sbp_patch_scatter_workspace_bytes(B, H, W, k, s)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    dX = torch.full((B, H, W, C), float("nan"), device="cuda")
+    sbp.sbp_patch_scatter(sbp.SBP_F32, dXp, B, H, W, C, k, s, rows, cnt, cap, dX, ws, nbytes)
+    torch.cuda.synchronize()
+    assert torch.equal(Xk[:keep], patches[pick])
+    assert not Xk[keep:].view(torch.int32).any()
+    want = torch.zeros(B, H, W, C, device="cuda")
+    b, ho, wo = pick // (Ho * Wo), (pick // Wo) % Ho, pick % Wo
+    for dh in range(k):
+        for dw in range(k):
+            want[b, ho * s + dh, wo * s + dw] = dXp[:keep].view(keep, k, k, C)[:, dh, dw]
+    assert torch.equal(dX, want)
+    assert not (dX.view(torch.int32) == -2147483648).any()                                         # the zeros are +0.0
