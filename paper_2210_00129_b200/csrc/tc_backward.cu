@@ -20,9 +20,8 @@
 // copies signal the stage's barrier when they land (cp.async.mbarrier.arrive).  TMA tile::gather4
 // was measured at ~45 ns of issue time per instruction per SM whatever it fetches - far too slow
 // to feed a tile - and is not used.  Every wait is bounded and reports through the status word.
-// Four side warps work next to the pipeline: they write the zeros of the dropped rows of dX for the
-// block's dX tiles (ahead of the MMAs, so every row of dX is written exactly once and no memset pass
-// is needed), then sum the block's share of the kept rows of dY column-wise for the bias gradient
+// Four side warps work next to the pipeline: they write the zeros of the dropped rows in the block's
+// share of dX (so every row of dX is written exactly once and no memset pass is needed), then sum the block's share of the kept rows of dY column-wise for the bias gradient
 // and leave one partial row per block for a fixed-order reduce.  The row maps are compile-time
 // variants: keep_rows on both sides, or identity on either side for gradients kept packed between
 // chained layers (Sec. 3.3.1).
@@ -31,6 +30,7 @@
 #include <tuple>
 
 #include "tc_ptx.cuh"
+#include "zero_rows.cuh"
 
 namespace sbp {
 namespace {
@@ -234,11 +234,6 @@ __device__ __forceinline__ uint32_t swizzled(uint32_t row, uint32_t chunk) {
     return row * kRowBytes + ((chunk ^ (row & 7u)) << 4);
 }
 
-// Zero the dropped rows of dX that belong to quarter `wq` (32 kept rows) of a dX tile, in the tile's
-// column strip: from just after the kept row preceding the quarter's first one up to its last kept
-// row (to the end of dX if it holds the very last kept row).  The rows are walked in windows of 32; a
-// warp-wide OR marks the kept rows of a window, the rest get zeros.  One warp, no other data needed:
-// the side warps run this for every dX tile of the block while the tensor pipe works.
 // Row lookups of the kernel: with kPacked false both row maps are the keep_rows list (the usual, scattered
 // form) and the lookup is a plain load; the packed forms for chained layers allow a null map (row m itself).
 // Kept apart at compile time (and, in the usual form, read through one pointer): the extra test and the
@@ -249,46 +244,20 @@ __device__ __forceinline__ int32_t map_row(const int32_t* rows, int64_t m) {
     else return __ldg(rows + m);
 }
 
-template <int BNX, bool kPacked>
-__device__ __forceinline__ void zero_dropped_rows(const TcParams& p, const Tile& t, int64_t M_keep, int wq, int lane) {
-    const int C_in = p.C_in;
-    const int n0 = (int)(t.col_tile * BNX);
-    const int strip_cols = (C_in - n0 < BNX) ? C_in - n0 : BNX;   // multiple of 8
-    const int strip_vecs = strip_cols >> 3;
-    const int64_t m0 = (int64_t)t.row_tile * kBM;
-    const int64_t m = m0 + wq * 32 + lane;
-    const bool valid = m < M_keep;
-    const int64_t cur = valid ? (int64_t)map_row<kPacked>(kPacked ? p.dx_rows : p.dy_rows, m) : -1;
-    const int64_t prev = (valid && m > 0) ? (int64_t)map_row<kPacked>(kPacked ? p.dx_rows : p.dy_rows, m - 1) : -1;
-    const int nvalid = __popc(__ballot_sync(0xffffffffu, valid));
-    if (nvalid == 0) return;
-    const int64_t lo = __shfl_sync(0xffffffffu, prev, 0) + 1;
-    const int64_t last_cur = __shfl_sync(0xffffffffu, cur, nvalid - 1);
-    const int64_t hi = (m0 + wq * 32 + nvalid == M_keep) ? p.M : last_cur;
-    for (int64_t base = lo; base < hi; base += 32) {
-        const int64_t d = cur - base;
-        uint32_t todo = ~__reduce_or_sync(0xffffffffu, (valid && d >= 0 && d < 32) ? (1u << d) : 0u);
-        if (hi - base < 32) todo &= (1u << (hi - base)) - 1u;
-        if (strip_vecs <= 16) {                      // narrow strip: two rows per store instruction
-            while (todo) {
-                const int b0 = __ffs(todo) - 1;
-                todo &= todo - 1u;
-                const int b1 = todo ? __ffs(todo) - 1 : -1;
-                if (todo) todo &= todo - 1u;
-                const int b = (lane < 16) ? b0 : b1;
-                const int v = lane & 15;
-                if (b >= 0 && v < strip_vecs)
-                    ptx::st_global_v4(p.dX + (base + b) * C_in + n0 + v * 8, 0u, 0u, 0u, 0u);
-            }
-        } else {
-            while (todo) {
-                const int b = __ffs(todo) - 1;
-                todo &= todo - 1u;
-                if (lane < strip_vecs)
-                    ptx::st_global_v4(p.dX + (base + b) * C_in + n0 + lane * 8, 0u, 0u, 0u, 0u);
-            }
+// Zero the dropped rows of dX: an equal share of all its rows for each of the `workers` side warps of the grid, whatever the
+// mask (the warps of a tile that cleared the rows between its own kept rows had hundreds of rows more than others with whole
+// frames kept: dW + db + dX of a clip of 8 frames x 196
+// positions, 768 -> 768: 46 -> 16.5 us).
+template <bool kPacked>
+__device__ __forceinline__ void zero_dropped_rows(const TcParams& p, int64_t M_keep, int64_t worker, int64_t workers, int lane) {
+    const int64_t per = (p.M + workers - 1) / workers, lo = per * worker, hi = lo + per < p.M ? lo + per : p.M;
+    const int vecs = p.C_in >> 3;
+    warp_visit_dropped_rows(kPacked ? p.dx_rows : p.dy_rows, M_keep, lo, hi, lane, [&](int64_t base, uint32_t todo) {
+        for (; todo; todo &= todo - 1u) {
+            __nv_bfloat16* row = p.dX + (base + __ffs(todo) - 1) * p.C_in;
+            for (int v = lane; v < vecs; v += 32) ptx::st_global_v4(row + v * 8, 0u, 0u, 0u, 0u);
         }
-    }
+    });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -604,13 +573,8 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
         ptx::cp_async_wait_all();
     } else if (warp >= kGatherWarp0) {
         // ---------------- side warps: zeros for the dropped rows of dX, then the bias sums ----------------
-        if (p.dX != nullptr && M_keep > 0) {
-            for (uint32_t pass = 0;; ++pass) {
-                Tile t;
-                if (!fetch_tile(pass, t)) break;
-                if (!t.is_dw) zero_dropped_rows<BNX, kPacked>(p, t, M_keep, side_index<kNarrow>(warp), lane);
-            }
-        }
+        if (p.dX != nullptr)
+            zero_dropped_rows<kPacked>(p, M_keep, (int64_t)blockIdx.x * 4 + side_index<kNarrow>(warp), (int64_t)gridDim.x * 4, lane);
         // db partial of this CTA's share of the kept rows
         if (p.db_partial != nullptr && !p.db_from_mma) {
             float* red = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kRingBytes + 256);
@@ -675,11 +639,6 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
         }
     } else {
         // ---------------- epilogue warps ----------------
-        if (M_keep == 0 && p.dX != nullptr) {                        // nothing kept: dX is all zeros
-            const int64_t vecs = p.M * (int64_t)(C_in / 8);
-            for (int64_t v = (int64_t)blockIdx.x * 128 + threadIdx.x; v < vecs; v += (int64_t)gridDim.x * 128)
-                ptx::st_global_v4(p.dX + v * 8, 0u, 0u, 0u, 0u);
-        }
         uint32_t used = 0, staged = 0;                               // accumulator uses, staging-buffer uses
         bool ok = true;
         for (uint32_t pass = 0; ok; ++pass) {
