@@ -12,6 +12,10 @@
 // once.  Ring of four 48 KB stages behind full/empty mbarriers, two 256-column fp32 accumulators so
 // the epilogue of one tile overlaps the MMAs of the next.  Every wait is bounded and reports through
 // the status word.
+//
+// Pairs of blocks (256-wide tiles, see choose_pair): the two blocks of a cluster share a tile of 256 rows through the two-SM
+// instructions, as in the backward kernel: each block loads its own 128 rows of X and half of the W tile (32 KB a stage
+// instead of 48, six stages), the even block issues, both read out their own rows.
 #include "tc_ptx.cuh"
 
 namespace sbp {
@@ -33,11 +37,14 @@ constexpr uint32_t kStageBytes = kABytes + kBBytesMax;
 constexpr uint32_t kAccCols = 256;
 constexpr int kEpiBarrier = 2;
 constexpr uint32_t kEpiBytes = 4 * 4096 + 2 * 256 * 4;   // one 4 KB transpose buffer per epilogue warp + two bias strips
-constexpr uint32_t kSmemBytes = kStages * kStageBytes + 256 + kEpiBytes + 1024;
+constexpr int kStagesPair = 6;                          // ... of 32 KB: the same ring memory
+constexpr uint32_t kRingBytes = kStages * kStageBytes;
+static_assert(kRingBytes == kStagesPair * (kABytes + 128 * kRowBytes), "both ring shapes fill the same memory");
+constexpr uint32_t kSmemBytes = kRingBytes + 256 + kEpiBytes + 1024;
 
 struct FwdControl {
-    uint64_t full_bar[kStages];    // 1 arrival carrying the byte count of both TMA operands
-    uint64_t empty_bar[kStages];   // 1 arrival: tcgen05.commit of the MMAs that read the stage
+    uint64_t full_bar[kStagesPair];    // 1 arrival carrying the byte count of both TMA operands
+    uint64_t empty_bar[kStagesPair];   // 1 arrival: tcgen05.commit of the MMAs that read the stage
     uint64_t acc_full[2];
     uint64_t acc_empty[2];         // 4 arrivals: each epilogue warp has read the accumulator out
     uint32_t tmem_slot;
@@ -64,34 +71,43 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-template <int BN>
+template <int BN, bool kPair>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                   const FwdParams p) {
+    static_assert(!kPair || BN == 256, "pairs of blocks run the wide tiles only");
+    constexpr int kS = kPair ? kStagesPair : kStages;
+    constexpr uint32_t kSB = kABytes + (kPair ? 128u : 256u) * kRowBytes;
+    const uint32_t rank = kPair ? ptx::cluster_ctarank() : 0u;                // 0: the block that issues the MMAs
+    const uint32_t workers = kPair ? gridDim.x >> 1 : gridDim.x, worker = kPair ? blockIdx.x >> 1 : blockIdx.x;
     extern __shared__ uint8_t smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t raw_addr = ptx::smem_addr(smem_raw);
     const uint32_t ring = (raw_addr + 1023u) & ~1023u;
-    FwdControl* ctl = reinterpret_cast<FwdControl*>(smem_raw + (ring - raw_addr) + kStages * kStageBytes);
+    FwdControl* ctl = reinterpret_cast<FwdControl*>(smem_raw + (ring - raw_addr) + kRingBytes);
 
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < kS; ++s) {
             ptx::mbar_init(ptx::smem_addr(&ctl->full_bar[s]), 1);
             ptx::mbar_init(ptx::smem_addr(&ctl->empty_bar[s]), 1);
         }
         for (int a = 0; a < 2; ++a) {
             ptx::mbar_init(ptx::smem_addr(&ctl->acc_full[a]), 1);
-            ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[a]), 4);
+            ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[a]), kPair ? 8 : 4);
         }
         ctl->abort_flag = 0;
         ptx::fence_mbar_init();
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_w);
     }
-    if (warp == 5) ptx::tmem_alloc(ptx::smem_addr(&ctl->tmem_slot), 2 * kAccCols);
+    if (warp == 5) {
+        if constexpr (kPair) ptx::tmem_alloc_pair(ptx::smem_addr(&ctl->tmem_slot), 2 * kAccCols);
+        else ptx::tmem_alloc(ptx::smem_addr(&ctl->tmem_slot), 2 * kAccCols);
+    }
     ptx::tc_fence_before_sync();
     __syncthreads();
+    if constexpr (kPair) ptx::cluster_sync_all();                    // the peer's barriers exist before anything is sent to them
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&ctl->tmem_slot);
     volatile int* abort_flag = &ctl->abort_flag;
@@ -101,7 +117,8 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const bool skip_all = status_word != nullptr && *reinterpret_cast<volatile int32_t*>(status_word) != 0;
     const int C_in = p.C_in, C_out = p.C_out;
     const uint32_t ncol = (uint32_t)((C_out + BN - 1) / BN);
-    const uint32_t total = (uint32_t)((p.M + kBM - 1) / kBM) * ncol;
+    constexpr int kTM = kPair ? 2 * kBM : kBM;                       // rows of a worker's tile
+    const uint32_t total = (uint32_t)((p.M + kTM - 1) / kTM) * ncol;
     const uint32_t num_kb = (uint32_t)((C_in + kBK - 1) / kBK);
 
     if (skip_all) {
@@ -111,64 +128,87 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (uint32_t q = blockIdx.x; q < total && ok; q += gridDim.x) {
-                const int row0 = (int)((q / ncol) * kBM), n0 = (int)((q % ncol) * BN);
+            for (uint32_t q = worker; q < total && ok; q += workers) {
+                const int row0 = (int)((q / ncol) * kTM + rank * kBM), n0 = (int)((q % ncol) * BN);
                 for (uint32_t k = 0; k < num_kb; ++k, ++it) {
-                    const int s = it % kStages;
-                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->empty_bar[s]), ((it / kStages) & 1u) ^ 1u, abort_flag, status_word);
+                    const int s = it % kS;
+                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->empty_bar[s]), ((it / kS) & 1u) ^ 1u, abort_flag, status_word);
                     if (!ok) break;
                     const uint32_t full = ptx::smem_addr(&ctl->full_bar[s]);
-                    const uint32_t a_dst = ring + s * kStageBytes;
-                    ptx::mbar_arrive_expect_tx(full, kABytes + BN * kRowBytes);
-                    ptx::tma_load_2d(a_dst, &map_x, (int)(k * kBK), row0, full);                 // 128 rows x 64 columns of X
-                    if (p.w_out_in) {                                                           // BN rows (j) x 64 columns (i) of W
-                        ptx::tma_load_2d(a_dst + kABytes, &map_w, (int)(k * kBK), n0, full);
-                    } else {
+                    const uint32_t a_dst = ring + s * kSB;
+                    if constexpr (kPair) {
+                        // this block's rows of X and its 128 of the tile's columns of W; the bytes of both blocks are credited
+                        // to the even block's barrier, which expects them all
+                        const uint32_t full0 = ptx::map_to_cta(full, 0);
+                        const int j0 = n0 + (int)rank * 128;
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(full, 2u * kSB);
+                        ptx::tma_load_2d_pair(a_dst, &map_x, (int)(k * kBK), row0, full0);
+                        if (p.w_out_in) {
+                            ptx::tma_load_2d_pair(a_dst + kABytes, &map_w, (int)(k * kBK), j0, full0);
+                        } else {
 #pragma unroll
-                        for (int b = 0; b < BN / 64; ++b)                                       // 64 rows (i) x 64 columns (j) of W
-                            ptx::tma_load_2d(a_dst + kABytes + b * kBlock64Bytes, &map_w, n0 + b * 64, (int)(k * kBK), full);
+                            for (int b = 0; b < 2; ++b)
+                                ptx::tma_load_2d_pair(a_dst + kABytes + b * kBlock64Bytes, &map_w, j0 + b * 64, (int)(k * kBK), full0);
+                        }
+                    } else {
+                        ptx::mbar_arrive_expect_tx(full, kABytes + BN * kRowBytes);
+                        ptx::tma_load_2d(a_dst, &map_x, (int)(k * kBK), row0, full);             // 128 rows x 64 columns of X
+                        if (p.w_out_in) {                                                       // BN rows (j) x 64 columns (i) of W
+                            ptx::tma_load_2d(a_dst + kABytes, &map_w, (int)(k * kBK), n0, full);
+                        } else {
+#pragma unroll
+                            for (int b = 0; b < BN / 64; ++b)                                   // 64 rows (i) x 64 columns (j) of W
+                                ptx::tma_load_2d(a_dst + kABytes + b * kBlock64Bytes, &map_w, n0 + b * 64, (int)(k * kBK), full);
+                        }
                     }
                 }
             }
-            if (!ok) {   // let the copies already issued land before shared memory goes away
-                for (uint32_t j = (it > (uint32_t)kStages ? it - kStages : 0u); j < it; ++j) {
-                    const uint32_t bar = ptx::smem_addr(&ctl->full_bar[j % kStages]);
+            if (!ok && kPair) {   // (pairs: the barrier may be the peer's; a fixed pause, far longer than any copy takes)
+                for (int i = 0; i < 64; ++i) __nanosleep(1000);
+            } else if (!ok) {   // let the copies already issued land before shared memory goes away
+                for (uint32_t j = (it > (uint32_t)kS ? it - kS : 0u); j < it; ++j) {
+                    const uint32_t bar = ptx::smem_addr(&ctl->full_bar[j % kS]);
                     for (int spin = 0; spin < (1 << 14); ++spin)
-                        if (ptx::mbar_try_wait(bar, (j / kStages) & 1u)) break;
+                        if (ptx::mbar_try_wait(bar, (j / kS) & 1u)) break;
                 }
             }
         }
         __syncwarp();
     } else if (warp == 5) {
-        // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        // ---------------- MMA issuer (of the pair: the even block's) ----------------
+        if (lane == 0 && rank == 0) {
             uint32_t it = 0, used = 0;
             bool ok = true;
             // A K-major; B MN-major for W [C_in, C_out], K-major for W [C_out, C_in]
-            const uint32_t idesc = ptx::umma_idesc_bf16(kBM, BN, false, p.w_out_in == 0);
+            const uint32_t idesc = ptx::umma_idesc_bf16(kTM, BN, false, p.w_out_in == 0);
             const uint32_t b_step = p.w_out_in ? kUmmaK * 2 : kUmmaK * kRowBytes, b_lbo = p.w_out_in ? 16u : kBlock64Bytes;
-            for (uint32_t q = blockIdx.x; q < total && ok; q += gridDim.x, ++used) {
+            for (uint32_t q = worker; q < total && ok; q += workers, ++used) {
                 const uint32_t acc = used & 1u;
                 ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[acc]), ((used >> 1) & 1u) ^ 1u, abort_flag, status_word);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kAccCols;
                 for (uint32_t k = 0; k < num_kb; ++k, ++it) {
-                    const int s = it % kStages;
-                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->full_bar[s]), (it / kStages) & 1u, abort_flag, status_word);
+                    const int s = it % kS;
+                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->full_bar[s]), (it / kS) & 1u, abort_flag, status_word);
                     if (!ok) break;
                     ptx::tc_fence_after_sync();
-                    const uint32_t a_addr = ring + s * kStageBytes, b_addr = a_addr + kABytes;
+                    const uint32_t a_addr = ring + s * kSB, b_addr = a_addr + kABytes;
 #pragma unroll
                     for (uint32_t u = 0; u < kBK / kUmmaK; ++u) {
                         // A: a 16-deep slice is 32 bytes along the swizzled row; B: 16 rows, 64-wide blocks 8 KB apart
                         const uint64_t da = ptx::umma_desc_sw128(a_addr + u * kUmmaK * 2, 16, kAtomBytes);
                         const uint64_t db = ptx::umma_desc_sw128(b_addr + u * b_step, b_lbo, kAtomBytes);
-                        ptx::umma_bf16(d_tmem, da, db, idesc, (k | u) != 0u);
+                        if constexpr (kPair) ptx::umma_bf16_pair(d_tmem, da, db, idesc, (k | u) != 0u);
+                        else ptx::umma_bf16(d_tmem, da, db, idesc, (k | u) != 0u);
                     }
-                    ptx::umma_commit(ptx::smem_addr(&ctl->empty_bar[s]));
+                    if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->empty_bar[s]));
+                    else ptx::umma_commit(ptx::smem_addr(&ctl->empty_bar[s]));
                 }
-                if (ok) ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[acc]));
+                if (ok) {
+                    if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[acc]));
+                    else ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[acc]));
+                }
             }
         }
         __syncwarp();
@@ -206,18 +246,18 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         // ---------------- epilogue warps ----------------
         uint32_t used = 0;
         bool ok = true;
-        uint8_t* wbuf = smem_raw + (ring - raw_addr) + kStages * kStageBytes + 256 + warp * 4096;
+        uint8_t* wbuf = smem_raw + (ring - raw_addr) + kRingBytes + 256 + warp * 4096;
         const int sub = lane >> 3, ch = lane & 7;
         int staged_n0[2] = {-1, -1};
-        for (uint32_t q = blockIdx.x; q < total; q += gridDim.x, ++used) {
+        for (uint32_t q = worker; q < total; q += workers, ++used) {
             const uint32_t acc = used & 1u;
             const uint32_t taddr = tmem_base + acc * kAccCols + ((uint32_t)(warp * 32) << 16);
-            const int64_t m0 = (int64_t)(q / ncol) * kBM + warp * 32;
+            const int64_t m0 = (int64_t)(q / ncol) * kTM + rank * kBM + warp * 32;
             const int n0 = (int)((q % ncol) * BN);
             const int strip_cols = (C_out - n0 < BN) ? C_out - n0 : BN;     // multiple of 8
             // The tile's strip of the bias goes to shared memory first (two buffers, by tile parity): read from
             // global memory inside the loop below, its 64 dependent loads per tile doubled the kernel's time.
-            float* bias_s = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kStages * kStageBytes + 256 + 4 * 4096) +
+            float* bias_s = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kRingBytes + 256 + 4 * 4096) +
                             (used & 1u) * 256;
             if (p.bias != nullptr && staged_n0[used & 1u] != n0) {        // with one or two column tiles the strip never changes
                 for (int c = threadIdx.x; c < BN; c += 128) bias_s[c] = (n0 + c < C_out) ? __ldg(p.bias + n0 + c) : 0.f;
@@ -263,14 +303,19 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                 __syncwarp();
             }
             ptx::tc_fence_before_sync();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->acc_empty[acc]));
+            if (lane == 0) {
+                if constexpr (kPair) ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_addr(&ctl->acc_empty[acc]), 0));
+                else ptx::mbar_arrive(ptx::smem_addr(&ctl->acc_empty[acc]));
+            }
         }
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
+    if constexpr (kPair) ptx::cluster_sync_all();                    // neither block leaves while the other may still reach into it
     if (warp == 5) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, 2 * kAccCols);
+        if constexpr (kPair) ptx::tmem_dealloc_pair(tmem_base, 2 * kAccCols);
+        else ptx::tmem_dealloc(tmem_base, 2 * kAccCols);
     }
 }
 
@@ -303,12 +348,29 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, ui
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
+template <int BN, bool PAIR>
 cudaError_t launch_forward(dim3 grid, cudaStream_t stream, const CUtensorMap& map_x, const CUtensorMap& map_w,
                            const FwdParams& prm) {
-    const cudaError_t opt = opt_in_dynamic_smem<tc_forward_kernel<BN>>((int)kSmemBytes);
+    const cudaError_t opt = opt_in_dynamic_smem<tc_forward_kernel<BN, PAIR>>((int)kSmemBytes);
     if (opt != cudaSuccess) return opt;
-    return launch_pdl(tc_forward_kernel<BN>, grid, dim3(kFwdThreads), kSmemBytes, stream, map_x, map_w, prm);
+    if constexpr (PAIR)
+        return launch_pdl_cluster(tc_forward_kernel<BN, PAIR>, grid, dim3(kFwdThreads), kSmemBytes, 2u, stream, map_x, map_w, prm);
+    else
+        return launch_pdl(tc_forward_kernel<BN, PAIR>, grid, dim3(kFwdThreads), kSmemBytes, stream, map_x, map_w, prm);
+}
+
+// Pairs where the two-SM instructions save more than a cluster launch and the coarser tile list cost: from about 1800 k-blocks
+// of 128 x 256 tiles on, and where the pairs' last wave is not much emptier.  Single blocks -> pairs on B200: 12544 x 768 ->
+// 3072 52.9 -> 47.6 us (1.24 PFLOP/s), 12544 x 3072 -> 768 46.9 -> 44.1, 25088 x 768 -> 2304 79.1 -> 70.6, 3136 x 1024 -> 4096
+// 25.3 -> 23.6, 19072 x 768 -> 256 (1788 k-blocks) 15.7 -> 14.8; below the line 9472 x 768 -> 512 10.8 -> 11.0, 3136 x 768 ->
+// 768 (900) 8.9 -> 9.4, 512 x 768 -> 768 8.3 -> 8.6.
+bool choose_pair(int64_t M, int64_t C_in, int64_t C_out) {
+    if (C_out < 256) return false;
+    const int64_t ncol = (C_out + 255) / 256, tiles = (M + kBM - 1) / kBM * ncol;
+    if (tiles * ((C_in + kBK - 1) / kBK) < 1780) return false;
+    const int64_t single = (tiles + kNumSMs - 1) / kNumSMs;
+    const int64_t pairs = ((M + 2 * kBM - 1) / (2 * kBM) * ncol + kNumSMs / 2 - 1) / (kNumSMs / 2);
+    return 5 * pairs <= 6 * single;
 }
 
 }  // namespace
@@ -323,8 +385,9 @@ sbp_status launch_tc_forward(const void* X, const void* W, bool w_out_in, const 
                              void* X_keep, int32_t* status_word, cudaStream_t stream) {
     CUtensorMap map_x, map_w;
     const int bn = C_out >= 256 ? 256 : 128;
+    const bool pair = choose_pair(M, C_in, C_out);
     if (!make_map(&map_x, X, M, C_in, (uint32_t)kBM)) return SBP_ERR_CUDA;
-    if (w_out_in ? !make_map(&map_w, W, C_out, C_in, (uint32_t)bn) : !make_map(&map_w, W, C_in, C_out, 64u)) return SBP_ERR_CUDA;
+    if (w_out_in ? !make_map(&map_w, W, C_out, C_in, (uint32_t)(pair ? 128 : bn)) : !make_map(&map_w, W, C_in, C_out, 64u)) return SBP_ERR_CUDA;
     FwdParams prm;
     prm.w_out_in = w_out_in ? 1 : 0;
     prm.bias = bias;
@@ -338,10 +401,13 @@ sbp_status launch_tc_forward(const void* X, const void* W, bool w_out_in, const 
     prm.M_keep_dev = M_keep_dev;
     prm.M_keep_cap = M_keep_cap;
     prm.status_word = status_word;
-    const int64_t tiles = ((M + kBM - 1) / kBM) * ((C_out + bn - 1) / bn);
-    const dim3 grid((unsigned)(tiles < kNumSMs ? tiles : kNumSMs));
-    const cudaError_t e = bn == 256 ? launch_forward<256>(grid, stream, map_x, map_w, prm)
-                                    : launch_forward<128>(grid, stream, map_x, map_w, prm);
+    const int tile_rows = pair ? 2 * kBM : kBM;
+    const int64_t tiles = ((M + tile_rows - 1) / tile_rows) * ((C_out + bn - 1) / bn), most = pair ? kNumSMs / 2 : kNumSMs;
+    const int64_t used = tiles < most ? tiles : most;
+    const dim3 grid((unsigned)(pair ? 2 * used : used));
+    const cudaError_t e = pair ? launch_forward<256, true>(grid, stream, map_x, map_w, prm)
+                        : bn == 256 ? launch_forward<256, false>(grid, stream, map_x, map_w, prm)
+                                    : launch_forward<128, false>(grid, stream, map_x, map_w, prm);
     return e == cudaSuccess ? SBP_OK : SBP_ERR_CUDA;
 }
 
