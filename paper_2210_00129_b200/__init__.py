@@ -3,18 +3,23 @@
 The compute lives in a C-ABI CUDA library (``include/sbp.h``, built in-tree as
 ``libsbp_b200.so``); this module is its thin Python binding: the functions below carry the
 same names as the C entry points and only marshal arguments (torch tensors -> device
-pointers, the current torch stream -> ``cudaStream_t``).  Every step of the path runs in the
-library's kernels; there is no fallback - a missing library raises at the first call.
+pointers, the current torch stream -> ``cudaStream_t``).  The calls a training step makes go
+through a small CPython module (``csrc/python_calls.cpp``), the queries and diagnostics through
+ctypes.  Every step of the path runs in the library's kernels; there is no fallback - a missing
+library raises at the first call.
 
 ``synth`` (seeded input generators) is importable without the library.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsbp_b200.so")
+CALLS_PATH = os.path.join(_HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 # enums of include/sbp.h
 SBP_OK, SBP_ERR_INVALID_ARG, SBP_ERR_UNSUPPORTED, SBP_ERR_WORKSPACE = 0, 1, 2, 3
@@ -33,6 +38,7 @@ EXPORTS = ("sbp_status_string", "sbp_keep_count", "sbp_sample_keep", "sbp_forwar
            "sbp_selftest_bounded_wait", "sbp_probe_gather_ring", "sbp_probe_mma_rate", "sbp_probe_mma_pair_rate", "sbp_probe_operand_feed")
 
 _lib = None
+_call = None          # the CPython module of the step's calls
 
 
 class SbpError(RuntimeError):
@@ -102,6 +108,20 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+def _calls():
+    """The CPython module with the calls of a training step."""
+    global _call
+    if _call is None or _lib is None:
+        load_library()
+        if not os.path.exists(CALLS_PATH):
+            raise RuntimeError(f"{CALLS_PATH} is missing: run `python -m paper_2210_00129_b200.build` with this interpreter")
+        spec = importlib.util.spec_from_file_location(__name__ + "._calls", CALLS_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _call = module
+    return _call
+
+
 def _ptr(t):
     """Device (or host) address of a torch tensor / raw integer address / None."""
     if t is None:
@@ -111,10 +131,22 @@ def _ptr(t):
     return t.data_ptr()
 
 
+_torch_stream = None  # (raw stream of a device, current device), once torch has initialised CUDA
+
+
 def _stream(stream):
     if stream is None:
+        global _torch_stream
+        if _torch_stream is not None:
+            raw, device = _torch_stream
+            return raw(device())
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        handle = torch.cuda.current_stream().cuda_stream
+        # the same handle without the Stream object around it (3 us a call); absent from a torch build: asked for as above
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and device is not None and raw(device()) == handle:
+            _torch_stream = (raw, device)
+        return handle
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -136,16 +168,15 @@ def sbp_keep_count(mode: int, H: int, W: int, keep_ratio: float) -> int:
 def sbp_sample_keep(mode, B, H, W, keep_ratio, seed, step, sample_offset, flags, keep_rows, keep_offsets,
                     stream=None, check=True) -> int:
     """Fill ``keep_rows`` / ``keep_offsets`` (int32 CUDA tensors) on the current stream."""
-    s = load_library().sbp_sample_keep(mode, B, H, W, float(keep_ratio), seed, step, sample_offset, flags,
-                                       _ptr(keep_rows), _ptr(keep_offsets), _stream(stream))
+    s = _calls().sbp_sample_keep(mode, B, H, W, keep_ratio, seed, step, sample_offset, flags, keep_rows, keep_offsets,
+                                 _stream(stream))
     if check:
         _check(s, "sbp_sample_keep")
     return s
 
 
 def sbp_forward_cache(dt, X, M, C, keep_rows, M_keep_dev, M_keep_cap, X_keep, stream=None, check=True) -> int:
-    s = load_library().sbp_forward_cache(dt, _ptr(X), M, C, _ptr(keep_rows), _ptr(M_keep_dev), M_keep_cap,
-                                         _ptr(X_keep), _stream(stream))
+    s = _calls().sbp_forward_cache(dt, X, M, C, keep_rows, M_keep_dev, M_keep_cap, X_keep, _stream(stream))
     if check:
         _check(s, "sbp_forward_cache")
     return s
@@ -154,9 +185,8 @@ def sbp_forward_cache(dt, X, M, C, keep_rows, M_keep_dev, M_keep_cap, X_keep, st
 def sbp_linear_forward(dt, X, W, bias, M, C_in, C_out, Y, keep_rows=None, M_keep_dev=None, M_keep_cap=0, X_keep=None,
                        flags=0, status_word=None, stream=None, check=True) -> int:
     """Y = X W + bias; with X_keep given the same launch also writes the forward cache."""
-    s = load_library().sbp_linear_forward(dt, _ptr(X), _ptr(W), _ptr(bias), M, C_in, C_out, _ptr(Y), _ptr(keep_rows),
-                                          _ptr(M_keep_dev), M_keep_cap, _ptr(X_keep), flags, _ptr(status_word),
-                                          _stream(stream))
+    s = _calls().sbp_linear_forward(dt, X, W, bias, M, C_in, C_out, Y, keep_rows, M_keep_dev, M_keep_cap, X_keep, flags,
+                                    status_word, _stream(stream))
     if check:
         _check(s, "sbp_linear_forward")
     return s
@@ -168,9 +198,8 @@ def sbp_linear_backward_workspace_bytes(dt, M, M_keep_cap, C_in, C_out) -> int:
 
 def sbp_linear_backward(dt, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX,
                         flags, workspace, workspace_bytes, status_word=None, stream=None, check=True) -> int:
-    s = load_library().sbp_linear_backward(dt, _ptr(X_keep), _ptr(dY), _ptr(W), _ptr(keep_rows), _ptr(M_keep_dev),
-                                           M, M_keep_cap, C_in, C_out, _ptr(dW), _ptr(db), _ptr(dX), flags,
-                                           _ptr(workspace), workspace_bytes, _ptr(status_word), _stream(stream))
+    s = _calls().sbp_linear_backward(dt, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX,
+                                     flags, workspace, workspace_bytes, status_word, _stream(stream))
     if check:
         _check(s, "sbp_linear_backward")
     return s
@@ -185,10 +214,8 @@ def sbp_linear_backward_kernel_count(dt, M, M_keep_cap, C_in, C_out, want_dW=Tru
 def sbp_attention_backward(dt, Q, K, V, ld_qkv, dA, ld_da, q_rows, q_offsets, kv_rows, kv_offsets, B, N, heads, head_dim,
                            max_kept, dQ, dK, dV, ld_out, flags=0, status_word=None, stream=None, check=True) -> int:
     """dQ, dK, dV of attention restricted to the listed query and key / value tokens (Drop QKV / Drop Query only)."""
-    s = load_library().sbp_attention_backward(dt, _ptr(Q), _ptr(K), _ptr(V), ld_qkv, _ptr(dA), ld_da, _ptr(q_rows),
-                                              _ptr(q_offsets), _ptr(kv_rows), _ptr(kv_offsets), B, N, heads, head_dim,
-                                              max_kept, _ptr(dQ), _ptr(dK), _ptr(dV), ld_out, flags, _ptr(status_word),
-                                              _stream(stream))
+    s = _calls().sbp_attention_backward(dt, Q, K, V, ld_qkv, dA, ld_da, q_rows, q_offsets, kv_rows, kv_offsets, B, N,
+                                        heads, head_dim, max_kept, dQ, dK, dV, ld_out, flags, status_word, _stream(stream))
     if check:
         _check(s, "sbp_attention_backward")
     return s
@@ -196,8 +223,7 @@ def sbp_attention_backward(dt, Q, K, V, ld_qkv, dA, ld_da, q_rows, q_offsets, kv
 
 def sbp_patch_cache(dt, X, B, H, W, C, k, stride, keep_rows, M_keep_dev, M_keep_cap, X_keep, stream=None, check=True) -> int:
     """Forward cache of a stride >= kernel convolution: the kept output positions' k x k patches as rows of k*k*C values."""
-    s = load_library().sbp_patch_cache(dt, _ptr(X), B, H, W, C, k, stride, _ptr(keep_rows), _ptr(M_keep_dev), M_keep_cap,
-                                       _ptr(X_keep), _stream(stream))
+    s = _calls().sbp_patch_cache(dt, X, B, H, W, C, k, stride, keep_rows, M_keep_dev, M_keep_cap, X_keep, _stream(stream))
     if check:
         _check(s, "sbp_patch_cache")
     return s
@@ -210,9 +236,8 @@ def sbp_patch_scatter_workspace_bytes(B, H, W, k, stride) -> int:
 def sbp_patch_scatter(dt, dX_patches, B, H, W, C, k, stride, keep_rows, M_keep_dev, M_keep_cap, dX, workspace, workspace_bytes,
                       status_word=None, stream=None, check=True) -> int:
     """Packed patch gradients [M_keep_cap, k*k*C] back into dX [B, H, W, C], zeros everywhere else."""
-    s = load_library().sbp_patch_scatter(dt, _ptr(dX_patches), B, H, W, C, k, stride, _ptr(keep_rows), _ptr(M_keep_dev),
-                                         M_keep_cap, _ptr(dX), _ptr(workspace), workspace_bytes, _ptr(status_word),
-                                         _stream(stream))
+    s = _calls().sbp_patch_scatter(dt, dX_patches, B, H, W, C, k, stride, keep_rows, M_keep_dev, M_keep_cap, dX, workspace,
+                                   workspace_bytes, status_word, _stream(stream))
     if check:
         _check(s, "sbp_patch_scatter")
     return s
@@ -220,8 +245,7 @@ def sbp_patch_scatter(dt, dX_patches, B, H, W, C, k, stride, keep_rows, M_keep_d
 
 def sbp_act_backward(dt, act, Z_keep, dH, M_keep_dev, M_keep_cap, C, dZ, status_word=None, stream=None, check=True) -> int:
     """dZ = dH * act'(Z_keep) on packed kept rows (the activation between two layers of a packed block)."""
-    s = load_library().sbp_act_backward(dt, act, _ptr(Z_keep), _ptr(dH), _ptr(M_keep_dev), M_keep_cap, C, _ptr(dZ),
-                                        _ptr(status_word), _stream(stream))
+    s = _calls().sbp_act_backward(dt, act, Z_keep, dH, M_keep_dev, M_keep_cap, C, dZ, status_word, _stream(stream))
     if check:
         _check(s, "sbp_act_backward")
     return s
@@ -239,10 +263,9 @@ def sbp_step_host(dt, mode, B, H, W, C_in, C_out, keep_ratio, seed, step, sample
                   W_host, dW_host, db_host, dX_host, keep_rows_host, keep_offsets_host, status_host, arena,
                   arena_bytes, stream=None, check=True) -> int:
     """Whole step from host (ideally pinned) tensors; results land in the host outputs once the stream is synced."""
-    s = load_library().sbp_step_host(dt, mode, B, H, W, C_in, C_out, float(keep_ratio), seed, step, sample_offset,
-                                     flags, _ptr(X_host), _ptr(dY_host), _ptr(W_host), _ptr(dW_host), _ptr(db_host),
-                                     _ptr(dX_host), _ptr(keep_rows_host), _ptr(keep_offsets_host), _ptr(status_host),
-                                     _ptr(arena), arena_bytes, _stream(stream))
+    s = _calls().sbp_step_host(dt, mode, B, H, W, C_in, C_out, keep_ratio, seed, step, sample_offset, flags, X_host,
+                               dY_host, W_host, dW_host, db_host, dX_host, keep_rows_host, keep_offsets_host, status_host, arena,
+                               arena_bytes, _stream(stream))
     if check:
         _check(s, "sbp_step_host")
     return s
@@ -251,8 +274,7 @@ def sbp_step_host(dt, mode, B, H, W, C_in, C_out, keep_ratio, seed, step, sample
 def sbp_bias_grad_static(dt, dY, keep_rows, M_keep_dev, M, M_keep_cap, C_out, db, flags=0, stream=None,
                          check=True) -> int:
     """Bias gradient with the library's built-in scratch: for callers that cannot allocate a workspace."""
-    s = load_library().sbp_bias_grad_static(dt, _ptr(dY), _ptr(keep_rows), _ptr(M_keep_dev), M, M_keep_cap, C_out,
-                                            _ptr(db), flags, _stream(stream))
+    s = _calls().sbp_bias_grad_static(dt, dY, keep_rows, M_keep_dev, M, M_keep_cap, C_out, db, flags, _stream(stream))
     if check:
         _check(s, "sbp_bias_grad_static")
     return s

@@ -1,7 +1,7 @@
 """Build the CUDA library in-tree: ``python -m paper_2210_00129_b200.build``.
 
-Compiles every ``csrc/*.cu`` for sm_100a with nvcc into ``libsbp_b200.so`` next to this file.
-Cross-compiles without a GPU.
+Compiles every ``csrc/*.cu`` for sm_100a with nvcc into ``libsbp_b200.so`` next to this file, and
+``csrc/python_calls.cpp`` into the CPython module of the calls.  Cross-compiles without a GPU.
 """
 from __future__ import annotations
 
@@ -9,10 +9,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB_PATH = os.path.join(_HERE, "libsbp_b200.so")
+
+CALLS_SRC = os.path.join(CSRC, "python_calls.cpp")
+CALLS_PATH = os.path.join(_HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-Xcompiler", "-fPIC", "-shared"]
@@ -23,11 +27,11 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(CALLS_PATH):
         return True
-    t = os.path.getmtime(LIB_PATH)
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(CALLS_PATH))
     deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + \
-        [os.path.join(os.path.dirname(_HERE), "include", "sbp.h")]
+        [CALLS_SRC, os.path.join(os.path.dirname(_HERE), "include", "sbp.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -35,12 +39,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB_PATH] + sources()
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed building libsbp_b200.so")
+    lib = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB_PATH] + sources()
+    calls = [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-I", sysconfig.get_paths()["include"],
+             "-o", CALLS_PATH, CALLS_SRC, "-L", _HERE, "-Xlinker", "-l:" + os.path.basename(LIB_PATH), "-Xlinker", "-rpath,$ORIGIN"]
+    for cmd, out in ((lib, LIB_PATH), (calls, CALLS_PATH)):
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if verbose or res.returncode != 0:
+            sys.stderr.write(res.stdout + res.stderr)
+        if res.returncode != 0:
+            raise RuntimeError("nvcc failed building " + os.path.basename(out))
     return LIB_PATH
 
 
