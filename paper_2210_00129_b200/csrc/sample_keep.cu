@@ -1,10 +1,14 @@
 // Keep-index sampler (Sec. 3.2.1 index sets; Sec. 4 random and grid-wise masks).
 //
-// One thread block per sample.  Random mode finds the K-th smallest 64-bit score
-// (philox word << 32 | position) with a four-pass, 8-bit radix select over the philox words -
-// which are recomputed on every pass, never stored - and then emits the kept positions in
-// ascending order with a block-wide prefix sum.  Grid mode evaluates the lattice predicate and
-// uses the same ordered compaction; per-sample offsets come from closed-form counts.
+// Random mode: one thread block per sample, or a cluster of blocks for large maps.  It finds the K-th smallest 64-bit score
+// (philox word << 32 | position) and emits the kept positions in ascending order.  Bound by the chain of barriers, not by
+// work, so the chain is short: one histogram of the words' top eight bits names the bin that holds the K-th smallest; that
+// bin's words (about N / 256) are collected and each is ranked against the others, which gives the threshold word; each
+// thread then owns a contiguous stretch of positions, so one block scan of their counts places every kept position.  (Should
+// a bin ever hold more words than the list, the next eight bits are taken, as often as needed.)  Four passes of eight bits
+// and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.5 us
+// and 4.6 us (the words are drawn while the kernel before drains).
+// Grid mode evaluates the lattice predicate with an ordered compaction; per-sample offsets come from closed-form counts.
 #include "sbp_common.cuh"
 
 namespace sbp {
@@ -14,11 +18,7 @@ constexpr int kSampThreads = 512;
 constexpr int kSampWarps = kSampThreads / 32;
 
 struct SampShared {
-    uint32_t hist[256];
-    uint32_t warp_sums_a[kSampWarps];
     uint32_t warp_sums_b[kSampWarps];
-    uint32_t sel_digit;
-    uint32_t sel_below;
     uint64_t red64[kSampWarps];
 };
 
@@ -32,140 +32,21 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
 }
 
 // Exclusive prefix over the block of per-thread counts; returns (exclusive prefix, block total).
+template <int kThreads>
 __device__ __forceinline__ uint2 block_excl_scan(uint32_t v, uint32_t* warp_sums) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t incl = warp_incl_scan(v, lane);
     if (lane == 31) warp_sums[warp] = incl;
     __syncthreads();
-    uint32_t ws = (lane < kSampWarps) ? warp_sums[lane] : 0u;
+    uint32_t ws = (lane < kThreads / 32) ? warp_sums[lane] : 0u;
     const uint32_t ws_incl = warp_incl_scan(ws, lane);
-    const uint32_t total = __shfl_sync(0xffffffffu, ws_incl, kSampWarps - 1);
+    const uint32_t total = __shfl_sync(0xffffffffu, ws_incl, kThreads / 32 - 1);
     const uint32_t warp_base = __shfl_sync(0xffffffffu, ws_incl - ws, warp);
     __syncthreads();
     return make_uint2(warp_base + incl - v, total);
 }
 
-// words of the four positions 4q .. 4q+3 of sample gid
-__device__ __forceinline__ PhiloxWords position_words(uint32_t q, uint32_t gid, uint32_t step,
-                                                      uint32_t k0, uint32_t k1) {
-    return philox4x32_10(q, gid, step, 0u, k0, k1);
-}
-
-__global__ void __launch_bounds__(kSampThreads)
-sample_keep_random_kernel(uint32_t N, uint32_t K, uint32_t k0, uint32_t k1, uint32_t step,
-                          uint32_t first_sample, int share_mask,
-                          int32_t* __restrict__ keep_rows, int32_t* __restrict__ keep_offsets) {
-    __shared__ SampShared sh;
-    // the selection looks at every word five times: maps of up to 8192 positions keep their words here
-    constexpr uint32_t kCacheGroups = 2048;
-    __shared__ uint4 word_cache[kCacheGroups];
-    pdl_launch_dependents();
-    pdl_wait();                 // earlier kernels of the stream may still be reading the index buffers
-    const uint32_t b = blockIdx.x;
-    const uint32_t gid = share_mask ? 0u : first_sample + b;
-    const uint32_t groups = (N + 3u) >> 2;
-    const int64_t row_base = (int64_t)b * N;
-    int32_t* out = keep_rows + (int64_t)b * K;
-    if (threadIdx.x == 0) {
-        keep_offsets[b + 1] = (int32_t)((b + 1) * (int64_t)K);
-        if (b == 0) keep_offsets[0] = 0;
-    }
-
-    const bool cached = groups <= kCacheGroups && K < N;
-    if (cached) {
-        for (uint32_t q = threadIdx.x; q < groups; q += kSampThreads) {
-            const PhiloxWords pw = position_words(q, gid, step, k0, k1);
-            word_cache[q] = make_uint4(pw.w[0], pw.w[1], pw.w[2], pw.w[3]);
-        }
-        __syncthreads();
-    }
-    auto words_of = [&](uint32_t q) {
-        if (!cached) return position_words(q, gid, step, k0, k1);
-        const uint4 v = word_cache[q];
-        PhiloxWords pw;
-        pw.w[0] = v.x; pw.w[1] = v.y; pw.w[2] = v.z; pw.w[3] = v.w;
-        return pw;
-    };
-
-    // ---- radix select: threshold word `prefix` and how many positions equal to it are kept ----
-    uint32_t prefix = 0, known = 0, remaining = K;
-    if (K < N) {
-        for (int shift = 24; shift >= 0; shift -= 8) {
-            for (int i = threadIdx.x; i < 256; i += kSampThreads) sh.hist[i] = 0;
-            __syncthreads();
-            for (uint32_t q = threadIdx.x; q < groups; q += kSampThreads) {
-                const PhiloxWords pw = words_of(q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const uint32_t n = 4u * q + e;
-                    if (n < N && (pw.w[e] & known) == prefix) atomicAdd(&sh.hist[(pw.w[e] >> shift) & 0xffu], 1u);
-                }
-            }
-            __syncthreads();
-            // exclusive scan over the 256 bins; the bin where the running count crosses `remaining` wins
-            const uint32_t cnt = (threadIdx.x < 256) ? sh.hist[threadIdx.x] : 0u;
-            const uint2 sc = block_excl_scan(cnt, sh.warp_sums_a);
-            if (threadIdx.x < 256 && sc.x < remaining && remaining <= sc.x + cnt) {
-                sh.sel_digit = threadIdx.x;
-                sh.sel_below = sc.x;
-            }
-            __syncthreads();
-            prefix |= sh.sel_digit << shift;
-            known |= 0xffu << shift;
-            remaining -= sh.sel_below;
-            __syncthreads();
-        }
-    }
-    const bool keep_all = (K >= N);
-    const uint32_t threshold = prefix;       // kept: word < threshold, plus the first `remaining` equal to it
-
-    // ---- ordered compaction, kSampThreads*4 positions per sweep ----
-    uint32_t eq_seen = 0, written = 0;
-    for (uint32_t q0 = 0; q0 < groups; q0 += kSampThreads) {
-        const uint32_t q = q0 + threadIdx.x;
-        uint32_t lt_mask = 0, eq_mask = 0;
-        if (q < groups) {
-            if (keep_all) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) if (4u * q + e < N) lt_mask |= 1u << e;
-            } else {
-                const PhiloxWords pw = words_of(q);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (4u * q + e < N) {
-                        if (pw.w[e] < threshold) lt_mask |= 1u << e;
-                        else if (pw.w[e] == threshold) eq_mask |= 1u << e;
-                    }
-                }
-            }
-        }
-        uint32_t keep_mask = lt_mask;
-        if (!keep_all) {
-            const uint2 se = block_excl_scan(__popc(eq_mask), sh.warp_sums_a);
-            uint32_t rank = eq_seen + se.x;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (eq_mask & (1u << e)) {
-                    if (rank < remaining) keep_mask |= 1u << e;
-                    ++rank;
-                }
-            }
-            eq_seen += se.y;
-        }
-        const uint2 sk = block_excl_scan(__popc(keep_mask), sh.warp_sums_b);
-        uint32_t pos = written + sk.x;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (keep_mask & (1u << e)) out[pos++] = (int32_t)(row_base + 4u * q + e);
-        }
-        written += sk.y;
-    }
-}
-
-// ---- large maps: one sample spread over a cluster of C thread blocks ----
-// Each block owns a contiguous slice of the positions.  The per-pass digit histograms stay in the
-// blocks' shared memory and are summed through distributed shared memory, so every block derives
-// the same threshold; slice counts exchanged the same way give each block its output offset.
+// ---- clusters: one sample spread over C thread blocks, each with a contiguous slice of the positions ----
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -182,137 +63,215 @@ __device__ __forceinline__ uint32_t cluster_load(const uint32_t* local_ptr, uint
     return v;
 }
 
-template <int C>
-__global__ void __launch_bounds__(kSampThreads)
-sample_keep_random_cluster_kernel(uint32_t N, uint32_t K, uint32_t k0, uint32_t k1, uint32_t step,
-                                  uint32_t first_sample, int share_mask, int cache_words,
-                                  int32_t* __restrict__ keep_rows, int32_t* __restrict__ keep_offsets) {
-    // The selection looks at every word six times (four digit passes, the tie count, the compaction).  When the
-    // slice's words fit in shared memory they are generated once and kept there; otherwise each look recomputes them.
+constexpr uint32_t kMaxListed = 1024;      // words of the chosen bin that are ranked directly
+
+struct RandomShared {
+    // Two histograms used alternately: the one a pass clears was last read by other blocks of a cluster two passes earlier,
+    // before the barrier of the pass in between, so one barrier per pass is enough.
+    uint32_t hist[2][256];
+    uint32_t listed[kMaxListed];           // this block's words of the chosen bin
+    uint32_t all_listed[kMaxListed];       // a cluster's: those of all its blocks
+    uint32_t n_listed;
+    uint32_t warp_sums[kSampWarps];
+    uint32_t bin, below, in_bin;           // the chosen bin, words in lower bins, words in it
+    uint32_t threshold, less, equal;       // the K-th smallest word; listed words below it, equal to it
+    uint32_t slice_counts[2];              // positions of this slice below / equal to the threshold
+};
+
+// C blocks a sample.  kThreads: 128 for small maps (fewer warps to bring to each barrier), 512 otherwise.  cache_groups: how
+// many groups of four words the dynamic shared memory holds (0: every look at a word computes it again).
+template <int C, int kThreads>
+__global__ void __launch_bounds__(kThreads)
+sample_keep_random_kernel(uint32_t N, uint32_t K, uint32_t k0, uint32_t k1, uint32_t step,
+                          uint32_t first_sample, int share_mask, uint32_t cache_groups,
+                          int32_t* __restrict__ keep_rows, int32_t* __restrict__ keep_offsets) {
     extern __shared__ uint4 word_cache[];
-    __shared__ SampShared sh;
-    __shared__ uint32_t slice_counts[2];          // positions of this slice below / equal to the threshold
-    // Two histograms used alternately: the one a pass clears was last read by the other blocks two passes
-    // earlier, before the cluster barrier of the pass in between, so one barrier per pass is enough.
-    __shared__ uint32_t hist2[2][256];
+    __shared__ RandomShared sh;
     pdl_launch_dependents();
-    pdl_wait();
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = C > 1 ? cluster_rank() : 0u;
     const uint32_t b = blockIdx.x / C;
     const uint32_t gid = share_mask ? 0u : first_sample + b;
     const uint32_t groups = (N + 3u) >> 2;
     const uint32_t per = (groups + C - 1) / C;
-    const uint32_t g_begin = rank * per;
+    const uint32_t g_begin = rank * per < groups ? rank * per : groups;
     const uint32_t g_end = (g_begin + per < groups) ? g_begin + per : groups;
     const int64_t row_base = (int64_t)b * N;
+    const bool cached = cache_groups >= per;
     int32_t* out = keep_rows + (int64_t)b * K;
-    if (rank == 0 && threadIdx.x == 0) {
-        keep_offsets[b + 1] = (int32_t)((b + 1) * (int64_t)K);
-        if (b == 0) keep_offsets[0] = 0;
-    }
-
-    if (cache_words) {
-        for (uint32_t q = g_begin + threadIdx.x; q < g_end; q += kSampThreads) {
-            const PhiloxWords pw = position_words(q, gid, step, k0, k1);
-            word_cache[q - g_begin] = make_uint4(pw.w[0], pw.w[1], pw.w[2], pw.w[3]);
-        }
-        __syncthreads();
-    }
+    auto sync_all = [] {
+        if constexpr (C > 1) cluster_sync();
+        else __syncthreads();
+    };
     auto words_of = [&](uint32_t q) {
-        if (!cache_words) return position_words(q, gid, step, k0, k1);
+        if (!cached) return philox4x32_10(q, gid, step, 0u, k0, k1);
         const uint4 v = word_cache[q - g_begin];
         PhiloxWords pw;
         pw.w[0] = v.x; pw.w[1] = v.y; pw.w[2] = v.z; pw.w[3] = v.w;
         return pw;
     };
 
-    uint32_t prefix = 0, known = 0, remaining = K;
-    for (int shift = 24, pass = 0; shift >= 0; shift -= 8, ++pass) {
-        uint32_t* hist = hist2[pass & 1];
-        for (int i = threadIdx.x; i < 256; i += kSampThreads) hist[i] = 0;
-        __syncthreads();
-        for (uint32_t q = g_begin + threadIdx.x; q < g_end; q += kSampThreads) {
-            const PhiloxWords pw = words_of(q);
+    uint32_t threshold = 0xffffffffu, ties = 0xffffffffu;    // kept: word < threshold, and the first `ties` equal to it
+    bool all_ties = true;
+    if (K < N) {
+        uint32_t prefix = 0, known = 0, remaining = K;
+        for (int shift = 24, pass = 0;; shift -= 8, ++pass) {
+            uint32_t* hist = sh.hist[pass & 1];
+            for (int i = threadIdx.x; i < 256; i += kThreads) hist[i] = 0;
+            __syncthreads();
+            for (uint32_t q = g_begin + threadIdx.x; q < g_end; q += kThreads) {
+                PhiloxWords pw;
+                if (pass == 0) {
+                    pw = philox4x32_10(q, gid, step, 0u, k0, k1);
+                    if (cached) word_cache[q - g_begin] = make_uint4(pw.w[0], pw.w[1], pw.w[2], pw.w[3]);
+                } else {
+                    pw = words_of(q);
+                }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t n = 4u * q + e;
-                if (n < N && (pw.w[e] & known) == prefix) atomicAdd(&hist[(pw.w[e] >> shift) & 0xffu], 1u);
+                for (int e = 0; e < 4; ++e)
+                    if (4u * q + e < N && (pw.w[e] & known) == prefix) atomicAdd(&hist[(pw.w[e] >> shift) & 0xffu], 1u);
             }
+            sync_all();                                      // every slice's histogram is complete
+            // running count over the 256 bins; the bin where it crosses `remaining` is the one
+            constexpr int kBins = kThreads >= 256 ? 1 : 256 / kThreads;
+            uint32_t cnt[kBins], mine = 0;
+#pragma unroll
+            for (int i = 0; i < kBins; ++i) {
+                const int bin = threadIdx.x * kBins + i;
+                cnt[i] = 0;
+                if (bin < 256) {
+                    if constexpr (C > 1) {
+#pragma unroll
+                        for (uint32_t r = 0; r < (uint32_t)C; ++r) cnt[i] += cluster_load(&hist[bin], r);
+                    } else {
+                        cnt[i] = hist[bin];
+                    }
+                }
+                mine += cnt[i];
+            }
+            uint32_t before = block_excl_scan<kThreads>(mine, sh.warp_sums).x;
+#pragma unroll
+            for (int i = 0; i < kBins; ++i) {
+                if (before < remaining && remaining <= before + cnt[i]) {
+                    sh.bin = threadIdx.x * kBins + i;
+                    sh.below = before;
+                    sh.in_bin = cnt[i];
+                }
+                before += cnt[i];
+            }
+            if (threadIdx.x == 0) sh.n_listed = 0;
+            __syncthreads();
+            prefix |= sh.bin << shift;
+            known |= 0xffu << shift;
+            remaining -= sh.below;
+            const uint32_t in_bin = sh.in_bin;
+            if (in_bin > kMaxListed && shift > 0) {
+                __syncthreads();                             // the bin is read before the next pass rewrites it
+                continue;
+            }
+            if (in_bin > kMaxListed) {                       // more than 1024 equal words
+                threshold = prefix;
+                ties = remaining;
+                all_ties = in_bin == remaining;
+                break;
+            }
+            // the bin's words, ranked against each other: the remaining-th smallest is the threshold
+            for (uint32_t q = g_begin + threadIdx.x; q < g_end; q += kThreads) {
+                const PhiloxWords pw = words_of(q);          // (its own thread wrote it to the cache)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (4u * q + e < N && (pw.w[e] & known) == prefix) sh.listed[atomicAdd(&sh.n_listed, 1u)] = pw.w[e];
+            }
+            sync_all();
+            const uint32_t* list = sh.listed;
+            if constexpr (C > 1) {
+                uint32_t at = 0;
+                for (uint32_t r = 0; r < (uint32_t)C; ++r) {
+                    const uint32_t n = cluster_load(&sh.n_listed, r);
+                    for (uint32_t i = threadIdx.x; i < n; i += kThreads) sh.all_listed[at + i] = cluster_load(&sh.listed[i], r);
+                    at += n;
+                }
+                list = sh.all_listed;
+                __syncthreads();
+            }
+            for (uint32_t i = threadIdx.x; i < in_bin; i += kThreads) {
+                const uint32_t w = list[i];
+                uint32_t less = 0, leq = 0;
+                for (uint32_t j = 0; j < in_bin; ++j) {
+                    less += list[j] < w;
+                    leq += list[j] <= w;
+                }
+                if (less < remaining && remaining <= leq) {  // (equal words all write the same)
+                    sh.threshold = w;
+                    sh.less = less;
+                    sh.equal = leq - less;
+                }
+            }
+            __syncthreads();
+            threshold = sh.threshold;
+            ties = remaining - sh.less;
+            all_ties = sh.equal == ties;
+            break;
         }
-        cluster_sync();                                   // every slice's histogram is complete
-        uint32_t cnt = 0;
-        if (threadIdx.x < 256)
-            for (uint32_t r = 0; r < (uint32_t)C; ++r) cnt += cluster_load(&hist[threadIdx.x], r);
-        const uint2 sc = block_excl_scan(cnt, sh.warp_sums_a);
-        if (threadIdx.x < 256 && sc.x < remaining && remaining <= sc.x + cnt) {
-            sh.sel_digit = threadIdx.x;
-            sh.sel_below = sc.x;
-        }
-        __syncthreads();
-        prefix |= sh.sel_digit << shift;
-        known |= 0xffu << shift;
-        remaining -= sh.sel_below;
-        __syncthreads();                                  // sel_digit / sel_below are read before the next pass rewrites them
     }
-    const uint32_t threshold = prefix;
 
-    // slice counts -> rank of this slice's first tie and its first output slot
+    // ---- this thread's contiguous stretch of groups: counts, then the kept positions in order ----
+    const uint32_t mine_groups = (g_end - g_begin + kThreads - 1) / kThreads;
+    const uint32_t t_begin = g_begin + threadIdx.x * mine_groups < g_end ? g_begin + threadIdx.x * mine_groups : g_end;
+    const uint32_t t_end = t_begin + mine_groups < g_end ? t_begin + mine_groups : g_end;
     uint32_t lt = 0, eq = 0;
-    for (uint32_t q = g_begin + threadIdx.x; q < g_end; q += kSampThreads) {
-        const PhiloxWords pw = words_of(q);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (4u * q + e < N) {
-                lt += pw.w[e] < threshold;
-                eq += pw.w[e] == threshold;
-            }
-        }
-    }
-    const uint32_t lt_total = block_excl_scan(lt, sh.warp_sums_a).y;
-    const uint32_t eq_total = block_excl_scan(eq, sh.warp_sums_b).y;
-    if (threadIdx.x == 0) { slice_counts[0] = lt_total; slice_counts[1] = eq_total; }
-    cluster_sync();
-    uint32_t eq_seen = 0, written = 0;
-    for (uint32_t r = 0; r < rank; ++r) {
-        const uint32_t lt_r = cluster_load(&slice_counts[0], r), eq_r = cluster_load(&slice_counts[1], r);
-        const uint32_t room = remaining > eq_seen ? remaining - eq_seen : 0u;
-        written += lt_r + (eq_r < room ? eq_r : room);
-        eq_seen += eq_r;
-    }
-
-    // ordered compaction of this slice
-    for (uint32_t q0 = g_begin; q0 < g_end; q0 += kSampThreads) {
-        const uint32_t q = q0 + threadIdx.x;
-        uint32_t lt_mask = 0, eq_mask = 0;
-        if (q < g_end) {
+    for (uint32_t q = t_begin; q < t_end; ++q) {
+        if (K >= N) {
+            lt += N - 4u * q < 4u ? N - 4u * q : 4u;
+        } else {
             const PhiloxWords pw = words_of(q);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 if (4u * q + e < N) {
-                    if (pw.w[e] < threshold) lt_mask |= 1u << e;
-                    else if (pw.w[e] == threshold) eq_mask |= 1u << e;
+                    lt += pw.w[e] < threshold;
+                    eq += pw.w[e] == threshold;
                 }
             }
         }
-        uint32_t keep_mask = lt_mask;
-        const uint2 se = block_excl_scan(__popc(eq_mask), sh.warp_sums_a);
-        uint32_t tie_rank = eq_seen + se.x;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (eq_mask & (1u << e)) {
-                if (tie_rank < remaining) keep_mask |= 1u << e;
-                ++tie_rank;
+    }
+    uint32_t first, ties_before = 0;                          // kept positions and ties in front of this stretch
+    if (C == 1 && all_ties) {
+        first = block_excl_scan<kThreads>(lt + eq, sh.warp_sums).x;
+    } else {
+        const uint2 sl = block_excl_scan<kThreads>(lt, sh.warp_sums);
+        const uint2 se = block_excl_scan<kThreads>(eq, sh.warp_sums);
+        uint32_t lt_before = sl.x;
+        ties_before = se.x;
+        if constexpr (C > 1) {
+            if (threadIdx.x == 0) { sh.slice_counts[0] = sl.y; sh.slice_counts[1] = se.y; }
+            cluster_sync();
+            for (uint32_t r = 0; r < rank; ++r) {
+                lt_before += cluster_load(&sh.slice_counts[0], r);
+                ties_before += cluster_load(&sh.slice_counts[1], r);
             }
         }
-        eq_seen += se.y;
-        const uint2 sk = block_excl_scan(__popc(keep_mask), sh.warp_sums_b);
-        uint32_t pos = written + sk.x;
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (keep_mask & (1u << e)) out[pos++] = (int32_t)(row_base + 4u * q + e);
-        written += sk.y;
+        first = lt_before + (ties_before < ties ? ties_before : ties);
     }
-    cluster_sync();                                       // the slice counts stay readable until every block is done
+    pdl_wait();                 // earlier kernels of the stream may still be reading the index buffers
+    if (rank == 0 && threadIdx.x == 0) {
+        keep_offsets[b + 1] = (int32_t)((b + 1) * (int64_t)K);
+        if (b == 0) keep_offsets[0] = 0;
+    }
+    for (uint32_t q = t_begin; q < t_end; ++q) {
+        PhiloxWords pw;
+        if (K < N) pw = words_of(q);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (4u * q + e < N) {
+                bool keep = K >= N || pw.w[e] < threshold;
+                if (!keep && pw.w[e] == threshold) {
+                    keep = ties_before < ties;
+                    ++ties_before;
+                }
+                if (keep) out[first++] = (int32_t)(row_base + 4u * q + e);
+            }
+        }
+    }
+    if constexpr (C > 1) cluster_sync();                      // the slice counts stay readable until every block is done
 }
 
 // ---- grid-wise masks: 2x2-periodic lattice with a per-sample phase ----
@@ -389,7 +348,7 @@ sample_keep_grid_kernel(int family, uint32_t H, uint32_t W, uint32_t k0, uint32_
                 if (n < N && grid_keeps(family, p, n / W, n % W)) keep_mask |= 1u << e;
             }
         }
-        const uint2 sk = block_excl_scan(__popc(keep_mask), sh.warp_sums_b);
+        const uint2 sk = block_excl_scan<kSampThreads>(__popc(keep_mask), sh.warp_sums_b);
         uint32_t pos = written + sk.x;
 #pragma unroll
         for (int e = 0; e < 4; ++e)
@@ -498,17 +457,25 @@ sample_keep_temporal_kernel(int family, uint32_t T, uint32_t P, uint32_t KT, uin
 uint32_t sample_keep_max_frames() { return kMaxFrames; }
 
 namespace {
-constexpr size_t kClusterCacheMax = 160 * 1024;
+constexpr size_t kCacheMax = 160 * 1024;
 
-template <int C>
-cudaError_t launch_cluster_sampler(dim3 grid, dim3 block, size_t cache_bytes, cudaStream_t stream, int64_t N, int64_t K,
-                                   uint32_t k0, uint32_t k1, uint32_t step, uint32_t first_sample, bool share_mask,
-                                   int32_t* keep_rows, int32_t* keep_offsets) {
-    const cudaError_t opt = opt_in_dynamic_smem<sample_keep_random_cluster_kernel<C>>((int)kClusterCacheMax);
-    if (opt != cudaSuccess) return opt;
-    return launch_pdl_cluster(sample_keep_random_cluster_kernel<C>, grid, block, cache_bytes, C, stream, (uint32_t)N,
-                              (uint32_t)K, k0, k1, step, first_sample, share_mask ? 1 : 0, cache_bytes ? 1 : 0, keep_rows,
-                              keep_offsets);
+// shared-memory cache of a slice's words (16 bytes per group of four positions), when it fits
+template <int C, int kThreads>
+cudaError_t launch_random_sampler(int64_t B, cudaStream_t stream, int64_t N, int64_t K, uint32_t k0, uint32_t k1, uint32_t step,
+                                  uint32_t first_sample, bool share_mask, int32_t* keep_rows, int32_t* keep_offsets) {
+    const int64_t slice_groups = ((N + 3) / 4 + C - 1) / C;
+    const size_t cache_bytes = K < N && (size_t)slice_groups * 16 <= kCacheMax ? (size_t)slice_groups * 16 : 0;
+    if (cache_bytes > 32 * 1024) {                            // (the static part takes 10 KB of the default 48)
+        const cudaError_t opt = opt_in_dynamic_smem<sample_keep_random_kernel<C, kThreads>>((int)kCacheMax);
+        if (opt != cudaSuccess) return opt;
+    }
+    const dim3 grid((unsigned)(B * C)), block(kThreads);
+    const auto launch = [&](auto... args) {
+        if constexpr (C > 1) return launch_pdl_cluster(sample_keep_random_kernel<C, kThreads>, grid, block, cache_bytes, C, stream, args...);
+        else return launch_pdl(sample_keep_random_kernel<C, kThreads>, grid, block, cache_bytes, stream, args...);
+    };
+    return launch((uint32_t)N, (uint32_t)K, k0, k1, step, first_sample, share_mask ? 1 : 0, (uint32_t)(cache_bytes / 16), keep_rows,
+                  keep_offsets);
 }
 }  // namespace
 
@@ -520,20 +487,14 @@ cudaError_t launch_sample_keep(int mode, int grid_family, int64_t B, int64_t H, 
     if (mode == SBP_MASK_RANDOM) {
         const int64_t N = H * W;
         // large maps with few samples: spread each sample over a cluster so that more SMs take part
-        int cluster = 1;
-        if (K < N && N > 8192 && B * 8 <= 4 * kNumSMs) cluster = N > 32768 ? 8 : (N > 16384 ? 4 : 2);
-        const dim3 cgrid((unsigned)(B * cluster));
-        // shared-memory cache of the slice's words (16 bytes per group of four positions), when it fits
-        const int64_t slice_groups = (((N + 3) / 4) + cluster - 1) / cluster;
-        const size_t cache_bytes = (size_t)slice_groups * 16 <= kClusterCacheMax ? (size_t)slice_groups * 16 : 0;
-        switch (cluster) {
-            case 8: return launch_cluster_sampler<8>(cgrid, block, cache_bytes, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
-            case 4: return launch_cluster_sampler<4>(cgrid, block, cache_bytes, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
-            case 2: return launch_cluster_sampler<2>(cgrid, block, cache_bytes, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
-            default: break;
+        if (K < N && N > 8192 && B * 8 <= 4 * kNumSMs) {
+            if (N > 32768) return launch_random_sampler<8, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
+            if (N > 16384) return launch_random_sampler<4, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
+            return launch_random_sampler<2, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
         }
-        return launch_pdl(sample_keep_random_kernel, grid, block, 0, stream, (uint32_t)(H * W), (uint32_t)K, k0, k1,
-                          step, first_sample, share_mask ? 1 : 0, keep_rows, keep_offsets);
+        // four warps see up to 512 positions, one group of four a thread
+        if (N <= 512) return launch_random_sampler<1, 128>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
+        return launch_random_sampler<1, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
     }
     if (mode == SBP_MASK_TEMPORAL || mode == SBP_MASK_TEMPORAL_GRID)      // H frames of W positions; K = kept frames x W
         return launch_pdl(sample_keep_temporal_kernel, grid, block, 0, stream, mode == SBP_MASK_TEMPORAL ? 0 : grid_family,

@@ -1,0 +1,22 @@
+"""`sbp_sample_keep` with random masks where its block size, clusters, word cache and stretches change, bit for bit against
+the oracle: one position, one group more or less than the threads, every cluster size, maps beyond the cache, extreme ratios."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_harness import run_sample_keep
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,W,r", [
+    (3, 1, 1, 0.5), (2, 1, 3, 0.34), (2, 1, 5, 1.0), (300, 1, 196, 0.25), (2, 1, 511, 0.5), (2, 1, 512, 0.999), (2, 1, 513, 0.001),
+    (3, 1, 2047, 0.5), (3, 1, 2049, 0.5), (2, 1, 8192, 0.5), (2, 1, 8193, 0.5), (5, 1, 16385, 0.1), (3, 1, 32769, 0.9), (1, 1, 32773, 1e-5),
+    (2, 200, 334, 0.5), (80, 1, 8197, 0.5), (76, 1, 41003, 0.3), (1, 3, 100001, 0.5), (1, 1000, 1000, 0.25),
+])
+def test_random_masks_at_every_dispatch(B, H, W, r):
+    for share in (0, 1):
+        rows, offs, cap = run_sample_keep(0, B, H, W, r, seed=9 + share, step=3, offset=2, flags=share)
+        keep, want_offs = oracle.sample_keep(0, B, H, W, r, 9 + share, 3, 2, bool(share))
+        assert np.array_equal(offs.cpu().numpy(), want_offs)
+        assert np.array_equal(rows.cpu().numpy()[:len(keep)], keep)
