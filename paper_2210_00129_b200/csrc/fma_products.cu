@@ -4,28 +4,32 @@
 //   dW[i, j] = sum_m X_keep[m, i] dY[keep_rows[m], j],  db[j] = sum_m dY[keep_rows[m], j]       (Eq. 5)
 //   dX[keep_rows[m], i] = sum_j dY[keep_rows[m], j] W[i, j]; every other row of dX = +0.0
 //
-// Bound by the FMA pipes.  Blackwell issues two fp32 FMAs per lane with one packed instruction (fma.rn.f32x2, each half
-// rounded as its own fmaf); the scalar form reaches half of the peak at best.  A thread owns 8 x 8 outputs as 8 x 4 packed
-// pairs: per reduction step it reads 16 operands from shared memory (four 16-byte loads, each a broadcast or conflict-free
-// within the warp's 32 x 64 outputs) for 32 packed FMAs.  The 256 threads of a block form kG groups which make the same
-// 64 x BN outputs from different depths of each stage (2 groups for BN = 128, 4 for BN = 64) and add their accumulators up
-// through shared memory at the end: a tile takes 1 / kG of the time, each thread carries 1 / kG of the loads in flight, and
-// what a thread needs fits 128 registers, so sixteen warps per SM hide each other's shared-memory latency.  Operands go
-// global -> registers -> shared memory, two 16-deep stages, the next one's loads in flight during the current arithmetic.
+// Bound by the FMA pipes, with shared memory close behind.  Blackwell issues two fp32 FMAs per lane with one packed
+// instruction (fma.rn.f32x2, each half rounded as its own fmaf): alone they reach 71.5 TFLOP/s, but four 16-byte
+// shared-memory loads for 32 of them, an 8 x 8 tile a thread, already fill the load pipe as long as the FMA pipe (59
+// TFLOP/s in a loop of nothing else).  So a thread owns 8 x 16 outputs where tiles of 64 x 128 fill the GPU (six loads for
+// 64 packed FMAs) and 8 x 8 in tiles of 64 x 64 below that.  The threads of a block form 2 (wide) or 4 groups which make the
+// same outputs from different depths of each stage and add their accumulators up through shared memory at the end: a tile
+// takes a half or a quarter of the time.  Operands go global -> registers -> shared memory in two stages, the next one's loads
+// in flight during the current arithmetic.
 //
 // Measured on B200, fp32 768 -> 3072, 3136 rows with 1568 kept, against 64 x 64 tiles of scalar FMAs in a kernel per product
-// and two for db: forward 441 -> 338 us (43.7 TFLOP/s, FMA pipes busy 66 % of the time), dW + db + dX 612 -> 392 us.  One
-// group of 128 threads a block at 162 registers: forward 404 us.  Operand A stored as ready-made pairs {a, a}, which saves
-// the moves that double it: 450 us (the registers of eight more 64-bit operands cost more than the moves).
+// and two for db: forward 441 -> 304 us (48.7 TFLOP/s), dW + db + dX 612 -> 350 us.  8 x 8 outputs in the wide tiles: 321 and
+// 405 us, whether or not the next step's operands were fetched ahead.  Operand A stored as ready-made pairs {a, a}, which
+// saves the moves that double it: 450 us.
 #include "zero_rows.cuh"
 
 namespace sbp {
 namespace {
 
-constexpr int kBK = 16;                   // reduction depth of a stage
 constexpr int kBM = 64;                   // rows of a tile
-constexpr int kTM = 8, kTN = 8;           // outputs per thread
-constexpr int NT = 256;                   // threads of a block
+constexpr int kTM = 8;                    // rows of a thread's outputs
+
+// The two block shapes: columns of the tile, columns of a thread's outputs, threads, reduction depth of a stage.  (The small
+// tiles run where there are few of them, so that each stage's loads are waited for: deep stages.)
+template <int kBN> struct Shape;
+template <> struct Shape<128> { static constexpr int kTN = 16, kThreads = 128, kBK = 16; };
+template <> struct Shape<64> { static constexpr int kTN = 8, kThreads = 256, kBK = 32; };
 
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) {
@@ -75,7 +79,7 @@ struct Operand {
 };
 
 // Global -> register -> shared-memory path of one operand: a tile of B extent indices x kBK depth.
-template <typename T, int B, bool kDepthInner>
+template <typename T, int B, bool kDepthInner, int NT, int kBK>
 struct TileLoader {
     static constexpr int kVecs = B * kBK / 4 / NT;       // 4-element vectors per thread and stage
     static constexpr int kPitch = B + 4;                 // floats per depth row in shared memory
@@ -136,41 +140,45 @@ struct TileLoader {
 };
 
 template <int BN>
+using Accumulators = uint64_t[kTM][Shape<BN>::kTN / 2];
+
+template <int BN>
 union ProductShared {
     struct {
-        float a[2][kBK][kBM + 4];
-        float b[2][kBK][BN + 4];
+        float a[2][Shape<BN>::kBK][kBM + 4];
+        float b[2][Shape<BN>::kBK][BN + 4];
     } t;
-    ulonglong2 swap[8][NT];                // half a thread's accumulators, on their way to the partner group
+    ulonglong2 swap[kTM / 2 * Shape<BN>::kTN / 4][Shape<BN>::kThreads];     // half a thread's accumulators, on their way to the partner group
 };
 
-// Where a thread's outputs sit in the tile: before the groups add up, rows row0 + {0..3, 16..19}, columns col0 + {0..3,
-// 32..35} in every group; afterwards group g holds kRows of the eight rows, from number first on.
+// Where a thread's outputs sit in the tile: before the groups add up, rows row0 + {0..3, 16..19}, columns col0 + {0..3} +
+// 32 h (h < kQuads) in every group; afterwards group g holds kRows of the eight rows, from number first on.
 template <int BN>
 struct ThreadTile {
+    static constexpr int kTN = Shape<BN>::kTN, kQuads = kTN / 4, kWarpCols = 8 * kTN;
     static constexpr int kThreads = (kBM / kTM) * (BN / kTN);          // threads of a group
-    static constexpr int kG = NT / kThreads, kRows = kTM / kG;
+    static constexpr int kG = Shape<BN>::kThreads / kThreads, kRows = kTM / kG;
     int group, row0, col0, first;
     __device__ __forceinline__ ThreadTile() {
         group = threadIdx.x / kThreads;
         const int warp = (threadIdx.x % kThreads) >> 5, lane = threadIdx.x & 31;
-        row0 = (warp / (BN / 64)) * 32 + (lane >> 3) * 4;
-        col0 = (warp % (BN / 64)) * 64 + (lane & 7) * 4;
+        row0 = (warp / (BN / kWarpCols)) * 32 + (lane >> 3) * 4;
+        col0 = (warp % (BN / kWarpCols)) * kWarpCols + (lane & 7) * 4;
         first = group * kRows;
     }
     __device__ __forceinline__ int row(int q) const { return row0 + ((first + q) & 3) + ((first + q) >> 2) * 16; }
-    __device__ __forceinline__ int col(int half) const { return col0 + half * 32; }
+    __device__ __forceinline__ int col(int h) const { return col0 + h * 32; }
 };
 
 // One step of the sum over groups: partners exchange halves of kHave accumulator rows, `upper` keeps the upper half.
 template <int BN, int kHave>
-__device__ __forceinline__ void halve(ProductShared<BN>& sh, uint64_t (&acc)[kTM][kTN / 2], bool upper, int partner) {
-    constexpr int kKeep = kHave / 2;
+__device__ __forceinline__ void halve(ProductShared<BN>& sh, Accumulators<BN>& acc, bool upper, int partner) {
+    constexpr int kKeep = kHave / 2, kPairs = Shape<BN>::kTN / 2;
     if (upper) {
 #pragma unroll
         for (int r = 0; r < kKeep; ++r)
 #pragma unroll
-            for (int c = 0; c < kTN / 2; ++c) {
+            for (int c = 0; c < kPairs; ++c) {
                 const uint64_t t = acc[r][c];
                 acc[r][c] = acc[r + kKeep][c];
                 acc[r + kKeep][c] = t;
@@ -178,16 +186,19 @@ __device__ __forceinline__ void halve(ProductShared<BN>& sh, uint64_t (&acc)[kTM
     }
     __syncthreads();                       // the tiles (or the exchange before) have been read
 #pragma unroll
-    for (int r = 0; r < kKeep; ++r) {
-        sh.swap[2 * r][threadIdx.x] = make_ulonglong2(acc[kKeep + r][0], acc[kKeep + r][1]);
-        sh.swap[2 * r + 1][threadIdx.x] = make_ulonglong2(acc[kKeep + r][2], acc[kKeep + r][3]);
-    }
+    for (int r = 0; r < kKeep; ++r)
+#pragma unroll
+        for (int c = 0; c < kPairs; c += 2)
+            sh.swap[(r * kPairs + c) / 2][threadIdx.x] = make_ulonglong2(acc[kKeep + r][c], acc[kKeep + r][c + 1]);
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kKeep; ++r) {
-        const ulonglong2 u = sh.swap[2 * r][partner], w = sh.swap[2 * r + 1][partner];
-        add2(acc[r][0], u.x); add2(acc[r][1], u.y); add2(acc[r][2], w.x); add2(acc[r][3], w.y);
-    }
+    for (int r = 0; r < kKeep; ++r)
+#pragma unroll
+        for (int c = 0; c < kPairs; c += 2) {
+            const ulonglong2 u = sh.swap[(r * kPairs + c) / 2][partner];
+            add2(acc[r][c], u.x);
+            add2(acc[r][c + 1], u.y);
+        }
 }
 
 // acc = A[e_a0 .., d] * B[e_b0 .., d] over the depth range [d_begin, d_end), in the first kRows rows of `acc` (ThreadTile).
@@ -196,10 +207,12 @@ __device__ __forceinline__ void halve(ProductShared<BN>& sh, uint64_t (&acc)[kTM
 template <typename T, int BN, bool kAInner, bool kBInner, int kSum>
 __device__ __forceinline__ void product(ProductShared<BN>& sh, const ThreadTile<BN>& tt, const Operand<T>& A, const Operand<T>& B,
                                         int64_t e_a0, int64_t e_b0, int64_t d_begin, int64_t d_end, bool want_sum,
-                                        uint64_t (&acc)[kTM][kTN / 2], float& colsum) {
+                                        Accumulators<BN>& acc, float& colsum) {
+    constexpr int NT = Shape<BN>::kThreads, kTN = Shape<BN>::kTN, kBK = Shape<BN>::kBK;
     constexpr int kG = ThreadTile<BN>::kG, kMine = kBK / kG;           // depth steps of a stage for each group
-    TileLoader<T, kBM, kAInner> la;
-    TileLoader<T, BN, kBInner> lb;
+    static_assert(NT >= BN && NT >= kBM, "a thread for each column of the sums");
+    TileLoader<T, kBM, kAInner, NT, kBK> la;
+    TileLoader<T, BN, kBInner, NT, kBK> lb;
 #pragma unroll
     for (int r = 0; r < kTM; ++r)
 #pragma unroll
@@ -233,9 +246,14 @@ __device__ __forceinline__ void product(ProductShared<BN>& sh, const ThreadTile<
             const float* ak = &sh.t.a[buf][tt.group * kMine + k][tt.row0];
             const float* bk = &sh.t.b[buf][tt.group * kMine + k][tt.col0];
             const float4 a0 = *reinterpret_cast<const float4*>(ak), a1 = *reinterpret_cast<const float4*>(ak + 16);
-            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bk), b1 = *reinterpret_cast<const ulonglong2*>(bk + 32);
             const float a[kTM] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const uint64_t b[kTN / 2] = {b0.x, b0.y, b1.x, b1.y};
+            uint64_t b[kTN / 2];
+#pragma unroll
+            for (int h = 0; h < kTN / 4; ++h) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(bk + h * 32);
+                b[2 * h] = v.x;
+                b[2 * h + 1] = v.y;
+            }
 #pragma unroll
             for (int r = 0; r < kTM; ++r) {
                 const uint64_t a2 = twice(a[r]);
@@ -253,8 +271,9 @@ __device__ __forceinline__ void product(ProductShared<BN>& sh, const ThreadTile<
     }
 }
 
-__device__ __forceinline__ float4 quad(const uint64_t (&acc)[kTM][kTN / 2], int q, int half) {
-    const float2 lo = halves(acc[q][2 * half]), hi = halves(acc[q][2 * half + 1]);
+template <int kPairs>
+__device__ __forceinline__ float4 quad(const uint64_t (&acc)[kTM][kPairs], int q, int h) {
+    const float2 lo = halves(acc[q][2 * h]), hi = halves(acc[q][2 * h + 1]);
     return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
@@ -269,7 +288,7 @@ struct ForwardParams {
 };
 
 template <typename T, int BN, bool kOutIn>
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(Shape<BN>::kThreads, 2)
 fma_forward_kernel(const ForwardParams<T> p) {
     __shared__ __align__(16) ProductShared<BN> sh;
     pdl_launch_dependents();
@@ -278,11 +297,11 @@ fma_forward_kernel(const ForwardParams<T> p) {
     const int64_t m0 = (int64_t)blockIdx.x * kBM;
     const int j0 = blockIdx.y * BN;
     const ThreadTile<BN> tt;
-    uint64_t acc[kTM][kTN / 2];
+    Accumulators<BN> acc;
     float unused;
     product<T, BN, true, kOutIn, 0>(sh, tt, p.X, p.W, m0, j0, 0, p.C_in, false, acc, unused);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < tt.kQuads; ++h) {
         const int j = j0 + tt.col(h);
         if (j >= p.C_out) continue;
         float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -310,6 +329,7 @@ struct BackwardParams {
     T* dX;
     int w_tiles, w_col_tiles, splits, accumulate;
     int x_row_tiles, x_col_tiles;          // w_tiles / x_row_tiles 0: that product is not asked for
+    int zero_blocks;                       // blocks that clear the dropped rows of dX
     const int32_t* status_word;
 };
 
@@ -318,11 +338,11 @@ __device__ __forceinline__ void dw_tile(ProductShared<BN>& sh, const BackwardPar
     const int split = q % p.splits, tile = q / p.splits;
     const int row_tile = tile / p.w_col_tiles, col_tile = tile % p.w_col_tiles;
     int64_t per = (M_keep + p.splits - 1) / p.splits;
-    per = (per + kBK - 1) / kBK * kBK;
+    per = (per + Shape<BN>::kBK - 1) / Shape<BN>::kBK * Shape<BN>::kBK;
     const int64_t begin = per * split, end = begin + per < M_keep ? begin + per : M_keep;
     const Operand<T> X{p.X_keep, p.C_in, nullptr, p.C_in}, Y{p.dY, p.C_out, p.dy_rows, p.C_out};
     const ThreadTile<BN> tt;
-    uint64_t acc[kTM][kTN / 2];
+    Accumulators<BN> acc;
     float colsum;
     // rows of the output are C_in x columns C_out, or the other way round for weights stored [C_out, C_in]
     const bool want_sum = p.db != nullptr && (kOutIn ? col_tile : row_tile) == 0;
@@ -342,7 +362,7 @@ __device__ __forceinline__ void dw_tile(ProductShared<BN>& sh, const BackwardPar
         const int i = row_tile * kBM + tt.row(r);
         if (i >= rows) continue;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < tt.kQuads; ++h) {
             const int j = col_tile * BN + tt.col(h);
             if (j >= cols) continue;
             float4 v = quad(acc, r, h);
@@ -355,28 +375,13 @@ __device__ __forceinline__ void dw_tile(ProductShared<BN>& sh, const BackwardPar
 
 template <typename T, int BN, bool kOutIn>
 __device__ __forceinline__ void dx_tile(ProductShared<BN>& sh, const BackwardParams<T>& p, int q, int64_t M_keep) {
-    constexpr int kWarps = NT / 32;
     const int row_tile = q / p.x_col_tiles, i0 = (q % p.x_col_tiles) * BN;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int quads = ((p.C_in - i0 < BN) ? p.C_in - i0 : BN) / 4;
-    // zeros of the dropped rows: every block takes an equal share of the rows of dX, in its own column strip
-    {
-        const int64_t per = (p.M + p.x_row_tiles - 1) / p.x_row_tiles;
-        const int64_t begin = per * row_tile, end = begin + per < p.M ? begin + per : p.M;
-        const int64_t warp_per = ((per + kWarps - 1) / kWarps + 31) / 32 * 32;
-        const int64_t lo = begin + warp * warp_per, hi = lo + warp_per < end ? lo + warp_per : end;
-        const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        warp_visit_dropped_rows(p.dx_rows, M_keep, lo, hi, lane, [&](int64_t base, uint32_t todo) {
-            for (; todo; todo &= todo - 1u)
-                if (lane < quads) store4<T>(p.dX + (base + __ffs(todo) - 1) * p.C_in + i0 + lane * 4, zero4);
-        });
-    }
     const int64_t m0 = (int64_t)row_tile * kBM;
     if (m0 >= M_keep) return;
     const Operand<T> Y{p.dY, p.C_out, p.dy_rows, M_keep};
     const Operand<T> W{p.W, kOutIn ? p.C_in : p.C_out, nullptr, p.C_in};
     const ThreadTile<BN> tt;
-    uint64_t acc[kTM][kTN / 2];
+    Accumulators<BN> acc;
     float unused;
     product<T, BN, true, !kOutIn, 0>(sh, tt, Y, W, m0, i0, 0, p.C_out, false, acc, unused);
 #pragma unroll
@@ -385,25 +390,44 @@ __device__ __forceinline__ void dx_tile(ProductShared<BN>& sh, const BackwardPar
         if (m >= M_keep) continue;
         T* out = p.dX + (int64_t)mapped_row(p.dx_rows, m) * p.C_in;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < tt.kQuads; ++h) {
             const int i = i0 + tt.col(h);
             if (i < p.C_in) store4<T>(out + i, quad(acc, r, h));
         }
     }
 }
 
+// Zeros of the dropped rows: every warp of the blocks that do this takes an equal share of the rows of dX.  Blocks of their own:
+// in front of a dX tile the search and the stores delayed a small layer's only wave by 2 - 3 us.
+template <typename T, int kThreads>
+__device__ __forceinline__ void zero_rows(const BackwardParams<T>& p, int block, int64_t M_keep) {
+    constexpr int kWarps = kThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, quads = p.C_in / 4;
+    const int64_t workers = (int64_t)p.zero_blocks * kWarps, per = (p.M + workers - 1) / workers;
+    const int64_t lo = per * ((int64_t)block * kWarps + warp), hi = lo + per < p.M ? lo + per : p.M;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    warp_visit_dropped_rows(p.dx_rows, M_keep, lo, hi, lane, [&](int64_t base, uint32_t todo) {
+        for (; todo; todo &= todo - 1u) {
+            T* row = p.dX + (base + __ffs(todo) - 1) * p.C_in;
+            for (int v = lane; v < quads; v += 32) store4<T>(row + v * 4, zero4);
+        }
+    });
+}
+
 template <typename T, int BN, bool kOutIn>
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(Shape<BN>::kThreads, 2)
 fma_backward_kernel(const BackwardParams<T> p) {
     __shared__ __align__(16) ProductShared<BN> sh;
-    static_assert(BN / 4 <= 32, "a warp clears a strip of a row at once");
     pdl_launch_dependents();
     pdl_wait();
     if (p.status_word != nullptr && *p.status_word != 0) return;
     const int64_t M_keep = load_m_keep(p.M_keep_dev, p.M_keep_cap);
     const int x_blocks = p.x_row_tiles * p.x_col_tiles;
-    if ((int)blockIdx.x < x_blocks) dx_tile<T, BN, kOutIn>(sh, p, (int)blockIdx.x, M_keep);
-    else dw_tile<T, BN, kOutIn>(sh, p, (int)blockIdx.x - x_blocks, M_keep);
+    // the deepest reductions first, the zeros last
+    const int block = (int)blockIdx.x, w_blocks = p.w_tiles * p.splits;
+    if (block < x_blocks) dx_tile<T, BN, kOutIn>(sh, p, block, M_keep);
+    else if (block < x_blocks + w_blocks) dw_tile<T, BN, kOutIn>(sh, p, block - x_blocks, M_keep);
+    else zero_rows<T, Shape<BN>::kThreads>(p, block - x_blocks - w_blocks, M_keep);
 }
 
 // ---- host side: tile shape, splits of the dW reduction, launches ----
@@ -430,7 +454,7 @@ FmaPlan fma_plan(bool fp32, bool out_in, int64_t M_keep_cap, int64_t C_in, int64
     set(128);
     pl.wide = fp32 && pl.w_rows * pl.w_cols + pl.x_rows * pl.x_cols >= 2 * kNumSMs;
     if (!pl.wide) set(64);
-    const double w_depth = (double)ceil_div(M_keep_cap, kBK), x_depth = (double)ceil_div(C_out, kBK);
+    const double w_depth = (double)ceil_div(M_keep_cap, 16), x_depth = (double)ceil_div(C_out, 16);      // 16-deep steps
     const double per_sm = (pl.w_rows * pl.w_cols * w_depth + pl.x_rows * pl.x_cols * x_depth) / kNumSMs;
     const double limit = per_sm / 2 > 8.0 ? per_sm / 2 : 8.0;
     double s = want_w ? w_depth / limit : 1.0;
@@ -443,7 +467,7 @@ FmaPlan fma_plan(bool fp32, bool out_in, int64_t M_keep_cap, int64_t C_in, int64
 template <typename T, int BN, bool kOutIn>
 cudaError_t launch_forward(const ForwardParams<T>& p, cudaStream_t stream) {
     const dim3 grid((unsigned)ceil_div(p.M, kBM), (unsigned)ceil_div(p.C_out, BN));
-    return launch_pdl(fma_forward_kernel<T, BN, kOutIn>, grid, dim3(NT), 0, stream, p);
+    return launch_pdl(fma_forward_kernel<T, BN, kOutIn>, grid, dim3(Shape<BN>::kThreads), 0, stream, p);
 }
 
 template <typename T>
@@ -467,8 +491,8 @@ cudaError_t forward_typed(const void* X, const void* W, bool w_out_in, const flo
 
 template <typename T, int BN, bool kOutIn>
 cudaError_t launch_backward(const BackwardParams<T>& p, cudaStream_t stream) {
-    const int64_t blocks = (int64_t)p.x_row_tiles * p.x_col_tiles + (int64_t)p.w_tiles * p.splits;
-    return launch_pdl(fma_backward_kernel<T, BN, kOutIn>, dim3((unsigned)blocks), dim3(NT), 0, stream, p);
+    const int64_t blocks = (int64_t)p.x_row_tiles * p.x_col_tiles + (int64_t)p.w_tiles * p.splits + p.zero_blocks;
+    return launch_pdl(fma_backward_kernel<T, BN, kOutIn>, dim3((unsigned)blocks), dim3(Shape<BN>::kThreads), 0, stream, p);
 }
 
 template <typename T>
@@ -525,6 +549,9 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
         p.accumulate = (accumulate && !split) ? 1 : 0;
         p.x_row_tiles = (int)pl.x_rows;
         p.x_col_tiles = (int)pl.x_cols;
+        // 64 KB of rows or more a block, as many blocks as SMs at most
+        const int64_t zero_bytes = M * C_in * (dt == SBP_BF16 ? 2 : 4);
+        p.zero_blocks = dX == nullptr ? 0 : (int)(zero_bytes < (int64_t)kNumSMs << 16 ? ceil_div(zero_bytes, 1 << 16) : kNumSMs);
         p.status_word = status_word;
     };
     cudaError_t e;
