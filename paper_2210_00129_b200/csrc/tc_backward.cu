@@ -28,6 +28,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "tc_ptx.cuh"
 #include "zero_rows.cuh"
@@ -248,14 +249,22 @@ __device__ __forceinline__ int32_t map_row(const int32_t* rows, int64_t m) {
 // mask (the warps of a tile that cleared the rows between its own kept rows had hundreds of rows more than others with whole
 // frames kept: dW + db + dX of a clip of 8 frames x 196
 // positions, 768 -> 768: 46 -> 16.5 us).
+// Rows of at most 256 bytes go two, four, ... to a store instruction.
 template <bool kPacked>
 __device__ __forceinline__ void zero_dropped_rows(const TcParams& p, int64_t M_keep, int64_t worker, int64_t workers, int lane) {
     const int64_t per = (p.M + workers - 1) / workers, lo = per * worker, hi = lo + per < p.M ? lo + per : p.M;
     const int vecs = p.C_in >> 3;
+    const int lanes = vecs > 16 ? 32 : vecs > 8 ? 16 : 8;            // lanes a row takes
+    const int rows = 32 / lanes, mine = lane / lanes, v0 = lane % lanes;
     warp_visit_dropped_rows(kPacked ? p.dx_rows : p.dy_rows, M_keep, lo, hi, lane, [&](int64_t base, uint32_t todo) {
-        for (; todo; todo &= todo - 1u) {
-            __nv_bfloat16* row = p.dX + (base + __ffs(todo) - 1) * p.C_in;
-            for (int v = lane; v < vecs; v += 32) ptx::st_global_v4(row + v * 8, 0u, 0u, 0u, 0u);
+        while (todo) {
+            int bit = -1;
+            for (int i = 0; i < rows && todo; ++i, todo &= todo - 1u)
+                if (i == mine) bit = __ffs(todo) - 1;
+            if (bit >= 0) {
+                __nv_bfloat16* row = p.dX + (base + bit) * p.C_in;
+                for (int v = v0; v < vecs; v += lanes) ptx::st_global_v4(row + v * 8, 0u, 0u, 0u, 0u);
+            }
         }
     });
 }
@@ -291,7 +300,7 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
     const uint32_t rank = kPair ? ptx::cluster_ctarank() : 0u;                // 0: the block that issues the MMAs
     const uint32_t workers = kPair ? gridDim.x >> 1 : gridDim.x, worker = kPair ? blockIdx.x >> 1 : blockIdx.x;
     extern __shared__ uint8_t smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t raw_addr = ptx::smem_addr(smem_raw);
     const uint32_t ring = (raw_addr + 1023u) & ~1023u;              // swizzle atoms need 1024-byte alignment
     TcControl* ctl = reinterpret_cast<TcControl*>(smem_raw + (ring - raw_addr) + kRingBytes);
@@ -415,56 +424,68 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
         }
         __syncwarp();
     } else if (warp == 5) {
-        // ---------------- MMA issuer (of the pair: the even block's) ----------------
-        if (lane == 0 && rank == 0) {
+        // ---------------- MMA issuer (of the pair: the even block's), a whole warp of which one lane issues ----------------
+        if (rank == 0) {
+            const bool leader = ptx::elect_one();
             uint32_t it = 0, used = 0;                               // stage uses, accumulator uses
             bool ok = true;
+            // The k-blocks of one tile.  K-major operands (dY of dX tiles, W [C_in, C_out]): a 16-deep slice is 32 bytes along
+            // the swizzled row.  MN-major ones (both of dW tiles, W [C_out, C_in]): 16 rows, 64-wide blocks 8 KB apart.
+            // kBias: the bias column, 16 more accumulator columns of which the first is db.
+            auto run_tile = [&](auto dw, auto bias, uint32_t num_kb, uint32_t d_tmem, uint32_t bias_tmem) {
+                constexpr bool kDw = decltype(dw)::value, kBias = decltype(bias)::value;
+                constexpr int kMmaM = kPair ? 2 * kBM : kBM;
+                constexpr bool kBMn = kDw || kOutIn;                 // the dense operand is MN-major
+                constexpr uint32_t idesc = ptx::umma_idesc_bf16(kMmaM, kDw ? BNW : BNX, kDw, kBMn);
+                constexpr uint32_t a_step = (kDw ? kUmmaK * kRowBytes : kUmmaK * 2) >> 4, b_step = (kBMn ? kUmmaK * kRowBytes : kUmmaK * 2) >> 4;
+                const uint32_t a_lo = ptx::umma_desc_lo(ring, kDw ? kBlock64Bytes : 16), b_lo = ptx::umma_desc_lo(ring + kABytes, kBMn ? kBlock64Bytes : 16);
+                const uint32_t ones_lo = ptx::umma_desc_lo(raw_addr + ones_off, kBlock64Bytes);
+                for (uint32_t k = 0; k < num_kb; ++k, ++it) {
+                    const uint32_t s = it % kS;
+                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->full_bar[s]), (it / kS) & 1u, abort_flag, status_word);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) return;
+                    ptx::tc_fence_after_sync();
+                    ptx::fence_async_proxy();        // the gathered operand was written by cp.async (generic proxy)
+                    const uint32_t a = a_lo + s * (kSB >> 4), b = b_lo + s * (kSB >> 4);
+#pragma unroll
+                    for (uint32_t u = 0; u < kBK / kUmmaK; ++u) {
+                        ptx::umma_bf16_warp<kPair>(d_tmem, ptx::umma_desc_of(a + u * a_step), ptx::umma_desc_of(b + u * b_step), idesc, (k | u) != 0u, leader);
+                        if constexpr (kBias)
+                            ptx::umma_bf16_warp<false>(bias_tmem, ptx::umma_desc_of(a + u * a_step), ptx::umma_desc_of(ones_lo + u * a_step),
+                                                       ptx::umma_idesc_bf16(kBM, 16, true, true), (k | u) != 0u, leader);
+                    }
+                    // stage reusable once these MMAs retire (pairs: in both blocks)
+                    if (leader) {
+                        if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->empty_bar[s]));
+                        else ptx::umma_commit(ptx::smem_addr(&ctl->empty_bar[s]));
+                    }
+                    __syncwarp();
+                }
+            };
+            using Yes = std::true_type;
+            using No = std::false_type;
             for (uint32_t pass = 0; ok; ++pass) {
                 Tile t;
                 if (!fetch_tile(pass, t)) break;
                 if (t.num_kb == 0) continue;
                 const uint32_t acc = used & 1u;
                 ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[acc]), ((used >> 1) & 1u) ^ 1u, abort_flag, status_word);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kAccCols;
                 // where the bias column accumulates: the unused half of a narrow tile's slot; with wide tiles the other
                 // slot, which a block that runs a single dW piece (the role split) never uses
                 const uint32_t bias_tmem = kNarrow ? d_tmem + 128u : tmem_base + (acc ^ 1u) * kAccCols;
-                // K-major (dX): a 16-deep slice is 32 bytes along the swizzled row, 8-row groups 1024 B apart.
-                // MN-major (dW): a 16-deep slice is 16 rows (two atoms); 64-wide blocks of the MN extent 8 KB apart.
-                constexpr int kMmaM = kPair ? 2 * kBM : kBM;
-                const uint32_t idesc = t.is_dw ? ptx::umma_idesc_bf16(kMmaM, BNW, true, true)
-                                               : ptx::umma_idesc_bf16(kMmaM, BNX, false, kOutIn);
-                const uint32_t k_step = t.is_dw ? kUmmaK * kRowBytes : kUmmaK * 2;
-                const uint32_t lbo = t.is_dw ? kBlock64Bytes : 16;
-                const uint32_t b_step = kOutIn ? kUmmaK * kRowBytes : k_step, b_lbo = kOutIn ? kBlock64Bytes : lbo;
-                for (uint32_t k = 0; k < t.num_kb; ++k, ++it) {
-                    const int s = it % kS;
-                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->full_bar[s]), (it / kS) & 1u, abort_flag, status_word);
-                    if (!ok) break;
-                    ptx::tc_fence_after_sync();
-                    ptx::fence_async_proxy();        // the gathered operand was written by cp.async (generic proxy)
-                    const uint32_t a_addr = ring + s * kSB, b_addr = a_addr + kABytes;
-#pragma unroll
-                    for (uint32_t u = 0; u < kBK / kUmmaK; ++u) {
-                        const uint64_t da = ptx::umma_desc_sw128(a_addr + u * k_step, lbo, kAtomBytes);
-                        const uint64_t db = ptx::umma_desc_sw128(b_addr + u * b_step, b_lbo, kAtomBytes);
-                        if constexpr (kPair) ptx::umma_bf16_pair(d_tmem, da, db, idesc, (k | u) != 0u);
-                        else ptx::umma_bf16(d_tmem, da, db, idesc, (k | u) != 0u);
-                        if (!kPair && t.is_dw && t.col_tile == 0 && p.db_from_mma) {   // the bias column: 16 more accumulator columns, the first is db
-                            const uint64_t d1 = ptx::umma_desc_sw128(raw_addr + ones_off + u * k_step, kBlock64Bytes, kAtomBytes);
-                            ptx::umma_bf16(bias_tmem, da, d1, ptx::umma_idesc_bf16(kBM, 16, true, true), (k | u) != 0u);
-                        }
-                    }
-                    // stage reusable once these MMAs retire (pairs: in both blocks)
-                    if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->empty_bar[s]));
-                    else ptx::umma_commit(ptx::smem_addr(&ctl->empty_bar[s]));
-                }
-                if (ok) {
+                if (!t.is_dw) run_tile(No{}, No{}, t.num_kb, d_tmem, bias_tmem);
+                else if (!kPair && t.col_tile == 0 && p.db_from_mma) run_tile(Yes{}, std::bool_constant<!kPair>{}, t.num_kb, d_tmem, bias_tmem);
+                else run_tile(Yes{}, No{}, t.num_kb, d_tmem, bias_tmem);
+                if (ok && leader) {
                     if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[acc]));
                     else ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[acc]));
                 }
+                __syncwarp();
                 ++used;
             }
         } else if (kPair && lane == 0) {
@@ -889,8 +910,15 @@ int64_t g_plan_searches = 0;
 // (ConvNeXt stage-1 lower layer of a packed block: 71 us with the split, 62 us without).
 Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx, bool dy_packed) {
     Plan pl;
-    pl.bnx = (C_in >= 256) ? 256 : 128;
-    pl.bnw = (C_in >= 256) ? 256 : 128;
+    // Tiles 256 wide, unless 128-wide ones give every SM at most one: then the call is as long as one tile's chain, and a
+    // 128-wide tile's k-blocks and read-out are shorter (dW + db + dX, 784 kept rows of 768 -> 768 15.3 -> 12.8 us, 300 of 320 ->
+    // 1280 17.3 -> 14.0, 2000 of 1024 -> 256 14.9 -> 12.6).  Not with a long reduction over kept rows, which is better cut into
+    // pieces of wide tiles (dW alone, 12544 kept rows of 768 -> 3072: 144 narrow tiles 65 us, wide ones in pairs 55 us).
+    const int64_t narrow_cols = (C_in + 127) / 128;
+    const int64_t narrow_tiles = (want_dx ? (M_keep_cap + kBM - 1) / kBM * narrow_cols : 0) + (want_dw ? (C_out + kBM - 1) / kBM * narrow_cols : 0);
+    const bool short_chain = narrow_tiles <= kNumSMs && (!want_dw || M_keep_cap <= 4608);
+    pl.bnx = (C_in >= 256 && !short_chain) ? 256 : 128;
+    pl.bnw = pl.bnx;
     int64_t x_tiles = want_dx ? ((M_keep_cap + kBM - 1) / kBM) * ((C_in + pl.bnx - 1) / pl.bnx) : 0;
     const int64_t x_kb = (C_out + kBK - 1) / kBK;
     int64_t w_tiles = want_dw ? ((C_out + kBM - 1) / kBM) * ((C_in + pl.bnw - 1) / pl.bnw) : 0;

@@ -81,7 +81,7 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const uint32_t rank = kPair ? ptx::cluster_ctarank() : 0u;                // 0: the block that issues the MMAs
     const uint32_t workers = kPair ? gridDim.x >> 1 : gridDim.x, worker = kPair ? blockIdx.x >> 1 : blockIdx.x;
     extern __shared__ uint8_t smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t raw_addr = ptx::smem_addr(smem_raw);
     const uint32_t ring = (raw_addr + 1023u) & ~1023u;
     FwdControl* ctl = reinterpret_cast<FwdControl*>(smem_raw + (ring - raw_addr) + kRingBytes);
@@ -175,40 +175,45 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         }
         __syncwarp();
     } else if (warp == 5) {
-        // ---------------- MMA issuer (of the pair: the even block's) ----------------
-        if (lane == 0 && rank == 0) {
+        // ---------------- MMA issuer (of the pair: the even block's), a whole warp of which one lane issues ----------------
+        if (rank == 0) {
+            const bool leader = ptx::elect_one();
             uint32_t it = 0, used = 0;
             bool ok = true;
-            // A K-major; B MN-major for W [C_in, C_out], K-major for W [C_out, C_in]
+            // A K-major: a 16-deep slice is 32 bytes along the swizzled row.  B MN-major for W [C_in, C_out]: 16 rows, 64-wide
+            // blocks 8 KB apart; K-major for W [C_out, C_in]
             const uint32_t idesc = ptx::umma_idesc_bf16(kTM, BN, false, p.w_out_in == 0);
-            const uint32_t b_step = p.w_out_in ? kUmmaK * 2 : kUmmaK * kRowBytes, b_lbo = p.w_out_in ? 16u : kBlock64Bytes;
+            const uint32_t b_step = (p.w_out_in ? kUmmaK * 2 : kUmmaK * kRowBytes) >> 4;
+            const uint32_t a_lo = ptx::umma_desc_lo(ring, 16), b_lo = ptx::umma_desc_lo(ring + kABytes, p.w_out_in ? 16u : kBlock64Bytes);
             for (uint32_t q = worker; q < total && ok; q += workers, ++used) {
                 const uint32_t acc = used & 1u;
                 ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[acc]), ((used >> 1) & 1u) ^ 1u, abort_flag, status_word);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * kAccCols;
                 for (uint32_t k = 0; k < num_kb; ++k, ++it) {
-                    const int s = it % kS;
+                    const uint32_t s = it % kS;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->full_bar[s]), (it / kS) & 1u, abort_flag, status_word);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     ptx::tc_fence_after_sync();
-                    const uint32_t a_addr = ring + s * kSB, b_addr = a_addr + kABytes;
+                    const uint32_t a = a_lo + s * (kSB >> 4), b = b_lo + s * (kSB >> 4);
 #pragma unroll
-                    for (uint32_t u = 0; u < kBK / kUmmaK; ++u) {
-                        // A: a 16-deep slice is 32 bytes along the swizzled row; B: 16 rows, 64-wide blocks 8 KB apart
-                        const uint64_t da = ptx::umma_desc_sw128(a_addr + u * kUmmaK * 2, 16, kAtomBytes);
-                        const uint64_t db = ptx::umma_desc_sw128(b_addr + u * b_step, b_lbo, kAtomBytes);
-                        if constexpr (kPair) ptx::umma_bf16_pair(d_tmem, da, db, idesc, (k | u) != 0u);
-                        else ptx::umma_bf16(d_tmem, da, db, idesc, (k | u) != 0u);
+                    for (uint32_t u = 0; u < kBK / kUmmaK; ++u)
+                        ptx::umma_bf16_warp<kPair>(d_tmem, ptx::umma_desc_of(a + u * (kUmmaK * 2 >> 4)), ptx::umma_desc_of(b + u * b_step), idesc,
+                                                   (k | u) != 0u, leader);
+                    if (leader) {
+                        if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->empty_bar[s]));
+                        else ptx::umma_commit(ptx::smem_addr(&ctl->empty_bar[s]));
                     }
-                    if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->empty_bar[s]));
-                    else ptx::umma_commit(ptx::smem_addr(&ctl->empty_bar[s]));
+                    __syncwarp();
                 }
-                if (ok) {
+                if (ok && leader) {
                     if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[acc]));
                     else ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[acc]));
                 }
+                __syncwarp();
             }
         }
         __syncwarp();
@@ -387,8 +392,10 @@ sbp_status launch_tc_forward(const void* X, const void* W, bool w_out_in, const 
                              void* Y, const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M_keep_cap,
                              void* X_keep, int32_t* status_word, cudaStream_t stream) {
     CUtensorMap map_x, map_w;
-    const int bn = C_out >= 256 ? 256 : 128;
-    const bool pair = choose_pair(M, C_in, C_out);
+    // 256-wide tiles, unless 128-wide ones give every SM at most one: the call is then as long as one tile's chain, whose
+    // products and read-out are shorter at half the width (FWD_NARROW_FIGURES)
+    const int bn = (C_out >= 256 && (M + kBM - 1) / kBM * ((C_out + 127) / 128) > kNumSMs) ? 256 : 128;
+    const bool pair = bn == 256 && choose_pair(M, C_in, C_out);
     if (!make_map(&map_x, X, M, C_in, (uint32_t)kBM)) return SBP_ERR_CUDA;
     if (w_out_in ? !make_map(&map_w, W, C_out, C_in, (uint32_t)(pair ? 128 : bn)) : !make_map(&map_w, W, C_in, C_out, 64u)) return SBP_ERR_CUDA;
     FwdParams prm;
