@@ -23,8 +23,9 @@
 //  - The next problem's rows are copied as soon as the last product has read the operands, under the read-out and the
 //    stores of this one.
 // Measured on B200, ViT-B/16 heads (12 x 64, 196 tokens), whole pass with the sampler: Drop QKV, half of the tokens, B = 128:
-// 99 us with a thread a row and copies behind the read-out, now 75 us; Drop Query only, B = 64: 94 -> 84 us.  What is left of a
-// problem's chain, some 20000 clocks with two blocks on an SM: copies and zero rows 5500 (all SMs load, then all store, so
+// 99 us with a thread a row and copies behind the read-out, now 65 us; Drop Query only, B = 64: 94 -> 72 us.  (One
+// thread issuing the products instead of a whole warp with one lane elected: 70 and 78 us, each instruction waiting for its
+// operands to reach uniform registers.)  A problem's chain before that, some 20000 clocks with two blocks on an SM: copies and zero rows 5500 (all SMs load, then all store, so
 // memory is busy a quarter of the time on average), softmax 6000, products 4500, read-out 2500.  Copies and zeros by four warps
 // of their own did not pay: the computing warps need more registers than setmaxnreg could then give them (76 us).
 // Query tiles of 128 rows follow one another (dV and dK stay in tensor memory); with two of them S and dS share columns.
@@ -161,16 +162,6 @@ __device__ __forceinline__ void load_rows(uint32_t dst0, uint32_t dst1, const __
     }
 }
 
-// Operand descriptor (128-byte swizzle, 1024 bytes between eight-row groups) whose low word holds the address and the
-// leading-dimension offset, both in 16-byte units: stepping through an operand is one 32-bit addition for the issuing thread.
-__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) { return (saddr >> 4) | ((lbo_bytes >> 4) << 16); }
-__device__ __forceinline__ uint64_t desc(uint32_t lo) {
-    constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-    uint64_t d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "n"(hi));
-    return d;
-}
-
 __device__ __forceinline__ uint64_t pair(float x, float y) {
     uint64_t r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
@@ -236,7 +227,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
     constexpr uint32_t kColDV = G == 2 ? 0 : 256, kColDK = G == 2 ? 64 : 384, kColDQ = G == 2 ? 128 : 0;
     extern __shared__ uint8_t smem_raw[];
     __shared__ AttnShared<G> sh;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t raw = ptx::smem_addr(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* gen = smem_raw + (base - raw);                 // generic pointer to the same place
@@ -253,7 +244,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&sh.tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(&sh.tmem_slot), 0);
     volatile int* abort_flag = &sh.abort_flag;
     pdl_wait();
     const bool skip_all = p.status_word != nullptr && *reinterpret_cast<volatile int32_t*>(p.status_word) != 0;
@@ -307,7 +298,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
     if (ok && (int)blockIdx.x < problems) begin_problem(cur, (int)blockIdx.x, 0);
 
     for (int prob = blockIdx.x; ok && prob < problems; prob += gridDim.x, buf ^= 1) {
-        const int nq = cur.nq, nk = cur.nk;
+        const int nq = __shfl_sync(0xffffffffu, cur.nq, 0), nk = __shfl_sync(0xffffffffu, cur.nk, 0);
         const int col0 = (prob % p.heads) * kD;
         const int next = prob + (int)gridDim.x;
         cur = fetch_meta(p, next, (int)threadIdx.x);        // travels while this problem computes
@@ -330,15 +321,17 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             const int q_here = nq - qt * 128 < 128 ? nq - qt * 128 : 128;
             const uint32_t q_steps = (uint32_t)(q_here + 15) >> 4;
             const uint32_t idesc_s = ptx::umma_idesc_bf16(128, n_keys, false, false);
-            const uint32_t dQ0 = desc_lo(sQ + qt * kTileB, 16), dDA0 = desc_lo(sDA + qt * kTileB, 16), dK0 = desc_lo(sK, 16), dV0 = desc_lo(sV, 16);
-            if (threadIdx.x == 0) {
+            const uint32_t dQ0 = ptx::umma_desc_lo(sQ + qt * kTileB, 16), dDA0 = ptx::umma_desc_lo(sDA + qt * kTileB, 16), dK0 = ptx::umma_desc_lo(sK, 16), dV0 = ptx::umma_desc_lo(sV, 16);
+            if (warp == 0) {                                 // the whole warp, of which one lane issues
+                const bool leader = ptx::elect_one();
                 ptx::tc_fence_after_sync();
 #pragma unroll
                 for (uint32_t u = 0; u < 4; ++u) {           // the two products alternate: they fill different accumulators
-                    ptx::umma_bf16(tmem, desc(dQ0 + u * 2), desc(dK0 + u * 2), idesc_s, u != 0);
-                    if (!shared_cols) ptx::umma_bf16(tmem + col_ds, desc(dDA0 + u * 2), desc(dV0 + u * 2), idesc_s, u != 0);
+                    ptx::umma_bf16_warp<false>(tmem, ptx::umma_desc_of(dQ0 + u * 2), ptx::umma_desc_of(dK0 + u * 2), idesc_s, u != 0, leader);
+                    if (!shared_cols) ptx::umma_bf16_warp<false>(tmem + col_ds, ptx::umma_desc_of(dDA0 + u * 2), ptx::umma_desc_of(dV0 + u * 2), idesc_s, u != 0, leader);
                 }
-                ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
+                if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
+                __syncwarp();
             }
             if (qt == 0) zero_rows(prob, nq, nk, q_glob, k_glob);
             ok = wait_products(&sh.bar_s, n_s);
@@ -366,12 +359,14 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             if (shared_cols) {
                 ptx::tc_fence_before_sync();
                 __syncthreads();                              // S has been read by every warp
-                if (threadIdx.x == 0) {
+                if (warp == 0) {
+                    const bool leader = ptx::elect_one();
                     ptx::tc_fence_after_sync();
 #pragma unroll
                     for (uint32_t u = 0; u < 4; ++u)
-                        ptx::umma_bf16(tmem, desc(dDA0 + u * 2), desc(dV0 + u * 2), idesc_s, u != 0);
-                    ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
+                        ptx::umma_bf16_warp<false>(tmem, ptx::umma_desc_of(dDA0 + u * 2), ptx::umma_desc_of(dV0 + u * 2), idesc_s, u != 0, leader);
+                    if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
+                    __syncwarp();
                 }
             }
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
@@ -479,26 +474,28 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             const int KT = G == 2 ? 1 : (nk + 127) >> 7;
             // 16 rows of a token tile are 2048 bytes; 16 columns of a block 32 bytes.  (N = 64 is one block: the leading-dimension
             // offset of the B operands plays no part.)
-            const uint32_t dP = desc_lo(sP, p.block_bytes), dMt = desc_lo(sDM, p.dm_stride), dMk = desc_lo(sDM, 16);
-            auto issue_dv = [&](uint32_t u) {
-                ptx::umma_bf16(tmem + kColDV, desc(dP + u * 128u), desc(dDA0 + u * 128u), id_t, (qt | (int)u) != 0);
+            const uint32_t dP = ptx::umma_desc_lo(sP, p.block_bytes), dMt = ptx::umma_desc_lo(sDM, p.dm_stride), dMk = ptx::umma_desc_lo(sDM, 16);
+            auto issue_dv = [&](uint32_t u, bool leader) {
+                ptx::umma_bf16_warp<false>(tmem + kColDV, ptx::umma_desc_of(dP + u * 128u), ptx::umma_desc_of(dDA0 + u * 128u), id_t, (qt | (int)u) != 0, leader);
                 if (G == 4 && KT > 1)
-                    ptx::umma_bf16(tmem + kColDV + 64u, desc(dP + (p.block_bytes >> 3) + u * 128u), desc(dDA0 + u * 128u), id_t, (qt | (int)u) != 0);
+                    ptx::umma_bf16_warp<false>(tmem + kColDV + 64u, ptx::umma_desc_of(dP + (p.block_bytes >> 3) + u * 128u), ptx::umma_desc_of(dDA0 + u * 128u), id_t, (qt | (int)u) != 0, leader);
             };
-            auto issue_dk = [&](uint32_t u) {
-                ptx::umma_bf16(tmem + kColDK, desc(dMt + u * 128u), desc(dQ0 + u * 128u), id_t, (qt | (int)u) != 0);
+            auto issue_dk = [&](uint32_t u, bool leader) {
+                ptx::umma_bf16_warp<false>(tmem + kColDK, ptx::umma_desc_of(dMt + u * 128u), ptx::umma_desc_of(dQ0 + u * 128u), id_t, (qt | (int)u) != 0, leader);
                 if (G == 4 && KT > 1)
-                    ptx::umma_bf16(tmem + kColDK + 64u, desc(dMt + (p.dm_stride >> 3) + u * 128u), desc(dQ0 + u * 128u), id_t, (qt | (int)u) != 0);
+                    ptx::umma_bf16_warp<false>(tmem + kColDK + 64u, ptx::umma_desc_of(dMt + (p.dm_stride >> 3) + u * 128u), ptx::umma_desc_of(dQ0 + u * 128u), id_t, (qt | (int)u) != 0, leader);
             };
-            auto issue_dq = [&](uint32_t u) {
-                ptx::umma_bf16(tmem + kColDQ, desc(dMk + (u >> 2) * (p.dm_stride >> 4) + (u & 3u) * 2u), desc(dK0 + u * 128u), id_q, u != 0);
+            auto issue_dq = [&](uint32_t u, bool leader) {
+                ptx::umma_bf16_warp<false>(tmem + kColDQ, ptx::umma_desc_of(dMk + (u >> 2) * (p.dm_stride >> 4) + (u & 3u) * 2u), ptx::umma_desc_of(dK0 + u * 128u), id_q, u != 0, leader);
             };
             const uint32_t steps = q_steps > k_steps ? q_steps : k_steps;
             if (!kSeparate) {
-                if (threadIdx.x == 0) {
+                if (warp == 0) {
+                    const bool leader = ptx::elect_one();
                     ptx::tc_fence_after_sync();
-                    for (uint32_t u = 0; u < q_steps; ++u) issue_dv(u);
-                    ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
+                    for (uint32_t u = 0; u < q_steps; ++u) issue_dv(u, leader);
+                    if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
+                    __syncwarp();
                 }
                 ok = wait_products(&sh.bar_o, n_o);
                 if (!ok) break;
@@ -510,16 +507,18 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 ptx::tc_fence_before_sync();
                 __syncthreads();
             }
-            if (threadIdx.x == 0) {
+            if (warp == 0) {                                 // the whole warp, of which one lane issues
+                const bool leader = ptx::elect_one();
                 ptx::tc_fence_after_sync();
                 for (uint32_t u = 0; u < steps; ++u) {
                     if (u < q_steps) {
-                        if (kSeparate) issue_dv(u);
-                        issue_dk(u);
+                        if (kSeparate) issue_dv(u, leader);
+                        issue_dk(u, leader);
                     }
-                    if (u < k_steps) issue_dq(u);
+                    if (u < k_steps) issue_dq(u, leader);
                 }
-                ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
+                if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
+                __syncwarp();
             }
             ok = wait_products(&sh.bar_o, n_o);
             if (!ok) break;

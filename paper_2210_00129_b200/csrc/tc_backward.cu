@@ -364,7 +364,8 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
         // an earlier check failed: leave every output untouched
     } else if (warp == 4) {
         // ---------------- TMA producer: the dense operand of every stage ----------------
-        if (lane == 0) {
+        {
+            const bool leader = ptx::elect_one();
             uint32_t it = 0;                                         // stage uses so far, over all tiles
             bool ok = true;
             for (uint32_t pass = 0; ok; ++pass) {
@@ -373,6 +374,7 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 for (uint32_t k = 0; k < t.num_kb; ++k, ++it) {
                     const int s = it % kS;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->empty_bar[s]), ((it / kS) & 1u) ^ 1u, abort_flag, status_word);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     const uint32_t full = ptx::smem_addr(&ctl->full_bar[s]);
                     const uint32_t a_dst = ring + s * kSB;
@@ -380,34 +382,34 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         // this block's 128 of the tile's 256 dense rows; the bytes of both blocks are credited to the even
                         // block's barrier, which expects them all
                         const uint32_t full0 = ptx::map_to_cta(full, 0);
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(full, 256u * kRowBytes);
+                        if (rank == 0 && leader) ptx::mbar_arrive_expect_tx(full, 256u * kRowBytes);
                         if (t.is_dw) {
                             const int row0 = (int)((t.kb_begin + k) * kBK), i0 = (int)(t.col_tile * BNW) + (int)rank * 128;
 #pragma unroll
                             for (int b = 0; b < 2; ++b)
-                                ptx::tma_load_2d_pair(a_dst + kABytes + b * kBlock64Bytes, &map_x, i0 + b * 64, row0, full0);
+                                ptx::tma_load_2d_pair_warp(a_dst + kABytes + b * kBlock64Bytes, &map_x, i0 + b * 64, row0, full0, leader);
                         } else if constexpr (kOutIn) {
                             const int i0 = (int)(t.col_tile * BNX) + (int)rank * 128;
 #pragma unroll
                             for (int b = 0; b < 2; ++b)
-                                ptx::tma_load_2d_pair(a_dst + kABytes + b * kBlock64Bytes, &map_w, i0 + b * 64, (int)(k * kBK), full0);
+                                ptx::tma_load_2d_pair_warp(a_dst + kABytes + b * kBlock64Bytes, &map_w, i0 + b * 64, (int)(k * kBK), full0, leader);
                         } else {
-                            ptx::tma_load_2d_pair(a_dst + kABytes, &map_w, (int)(k * kBK), (int)(t.col_tile * BNX) + (int)rank * 128, full0);
+                            ptx::tma_load_2d_pair_warp(a_dst + kABytes, &map_w, (int)(k * kBK), (int)(t.col_tile * BNX) + (int)rank * 128, full0, leader);
                         }
                     } else if (t.is_dw) {                            // X_keep tile: BNW/64 blocks of 64 columns x 64 kept rows
                         const int row0 = (int)((t.kb_begin + k) * kBK), i0 = (int)(t.col_tile * BNW);
-                        ptx::mbar_arrive_expect_tx(full, BNW * kRowBytes);
+                        if (leader) ptx::mbar_arrive_expect_tx(full, BNW * kRowBytes);
 #pragma unroll
                         for (int b = 0; b < BNW / 64; ++b)
-                            ptx::tma_load_2d(a_dst + kABytes + b * kBlock64Bytes, &map_x, i0 + b * 64, row0, full);
+                            ptx::tma_load_2d_warp(a_dst + kABytes + b * kBlock64Bytes, &map_x, i0 + b * 64, row0, full, leader);
                     } else {                                         // W tile: BNX rows x 64 columns
-                        ptx::mbar_arrive_expect_tx(full, BNX * kRowBytes);
+                        if (leader) ptx::mbar_arrive_expect_tx(full, BNX * kRowBytes);
                         if constexpr (kOutIn) {
 #pragma unroll
                             for (int b = 0; b < BNX / 64; ++b)
-                                ptx::tma_load_2d(a_dst + kABytes + b * kBlock64Bytes, &map_w, (int)(t.col_tile * BNX) + b * 64, (int)(k * kBK), full);
+                                ptx::tma_load_2d_warp(a_dst + kABytes + b * kBlock64Bytes, &map_w, (int)(t.col_tile * BNX) + b * 64, (int)(k * kBK), full, leader);
                         } else {
-                            ptx::tma_load_2d(a_dst + kABytes, &map_w, (int)(k * kBK), (int)(t.col_tile * BNX), full);
+                            ptx::tma_load_2d_warp(a_dst + kABytes, &map_w, (int)(k * kBK), (int)(t.col_tile * BNX), full, leader);
                         }
                     }
                 }

@@ -125,7 +125,8 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         // an earlier check failed: leave every output untouched
     } else if (warp == 4) {
         // ---------------- TMA producer ----------------
-        if (lane == 0) {
+        {
+            const bool leader = ptx::elect_one();
             uint32_t it = 0;
             bool ok = true;
             for (uint32_t q = worker; q < total && ok; q += workers) {
@@ -133,6 +134,7 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                 for (uint32_t k = 0; k < num_kb; ++k, ++it) {
                     const int s = it % kS;
                     ok = ptx::mbar_wait(ptx::smem_addr(&ctl->empty_bar[s]), ((it / kS) & 1u) ^ 1u, abort_flag, status_word);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     const uint32_t full = ptx::smem_addr(&ctl->full_bar[s]);
                     const uint32_t a_dst = ring + s * kSB;
@@ -141,24 +143,24 @@ tc_forward_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
                         // to the even block's barrier, which expects them all
                         const uint32_t full0 = ptx::map_to_cta(full, 0);
                         const int j0 = n0 + (int)rank * 128;
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(full, 2u * kSB);
-                        ptx::tma_load_2d_pair(a_dst, &map_x, (int)(k * kBK), row0, full0);
+                        if (rank == 0 && leader) ptx::mbar_arrive_expect_tx(full, 2u * kSB);
+                        ptx::tma_load_2d_pair_warp(a_dst, &map_x, (int)(k * kBK), row0, full0, leader);
                         if (p.w_out_in) {
-                            ptx::tma_load_2d_pair(a_dst + kABytes, &map_w, (int)(k * kBK), j0, full0);
+                            ptx::tma_load_2d_pair_warp(a_dst + kABytes, &map_w, (int)(k * kBK), j0, full0, leader);
                         } else {
 #pragma unroll
                             for (int b = 0; b < 2; ++b)
-                                ptx::tma_load_2d_pair(a_dst + kABytes + b * kBlock64Bytes, &map_w, j0 + b * 64, (int)(k * kBK), full0);
+                                ptx::tma_load_2d_pair_warp(a_dst + kABytes + b * kBlock64Bytes, &map_w, j0 + b * 64, (int)(k * kBK), full0, leader);
                         }
                     } else {
-                        ptx::mbar_arrive_expect_tx(full, kABytes + BN * kRowBytes);
-                        ptx::tma_load_2d(a_dst, &map_x, (int)(k * kBK), row0, full);             // 128 rows x 64 columns of X
+                        if (leader) ptx::mbar_arrive_expect_tx(full, kABytes + BN * kRowBytes);
+                        ptx::tma_load_2d_warp(a_dst, &map_x, (int)(k * kBK), row0, full, leader);             // 128 rows x 64 columns of X
                         if (p.w_out_in) {                                                       // BN rows (j) x 64 columns (i) of W
-                            ptx::tma_load_2d(a_dst + kABytes, &map_w, (int)(k * kBK), n0, full);
+                            ptx::tma_load_2d_warp(a_dst + kABytes, &map_w, (int)(k * kBK), n0, full, leader);
                         } else {
 #pragma unroll
                             for (int b = 0; b < BN / 64; ++b)                                   // 64 rows (i) x 64 columns (j) of W
-                                ptx::tma_load_2d(a_dst + kABytes + b * kBlock64Bytes, &map_w, n0 + b * 64, (int)(k * kBK), full);
+                                ptx::tma_load_2d_warp(a_dst + kABytes + b * kBlock64Bytes, &map_w, n0 + b * 64, (int)(k * kBK), full, leader);
                         }
                     }
                 }
@@ -393,7 +395,9 @@ sbp_status launch_tc_forward(const void* X, const void* W, bool w_out_in, const 
                              void* X_keep, int32_t* status_word, cudaStream_t stream) {
     CUtensorMap map_x, map_w;
     // 256-wide tiles, unless 128-wide ones give every SM at most one: the call is then as long as one tile's chain, whose
-    // products and read-out are shorter at half the width (FWD_NARROW_FIGURES)
+    // products and read-out are shorter at half the width (768 -> 768: 1568 rows
+    // 8.4 -> 6.9 us, 512 rows 8.3 -> 6.4; 2560 -> 640 with 234 rows 16.1 -> 13.1; since the whole warp issues the copies 6.1, 5.3
+    // and 9.4)
     const int bn = (C_out >= 256 && (M + kBM - 1) / kBM * ((C_out + 127) / 128) > kNumSMs) ? 256 : 128;
     const bool pair = bn == 256 && choose_pair(M, C_in, C_out);
     if (!make_map(&map_x, X, M, C_in, (uint32_t)kBM)) return SBP_ERR_CUDA;
