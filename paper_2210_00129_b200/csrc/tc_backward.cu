@@ -116,6 +116,7 @@ struct TcParams {
     int dw_accumulate;             // add into dW_out (only with one split)
     int db_from_mma;               // narrow layers: db comes out of the dW tiles (a column of ones appended to X_keep);
                                    // db_partial is then [dw_splits, C_out]
+    int db_accumulate;             // one piece: db_partial is db itself, which is added to (1) or written (0)
     float* db_partial;             // nullptr: no bias sums; else [gridDim.x, C_out] per-CTA column sums of kept dY rows
     int dw_ctas;                   // 0: every block walks the one cost-sorted list of both tile kinds; > 0: the first
                                    // dw_ctas blocks take the dW pieces, the others the dX tiles, both sweeping the kept
@@ -727,7 +728,7 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 if (t.num_kb == 0) {                                 // a piece without kept rows contributes zero
                     if (!p.dw_accumulate && j < C_out)
                         for (int c0 = 0; c0 < BNW && i0 + c0 < C_in; ++c0) out_col[(int64_t)c0 * out_step] = 0.f;
-                    if (bias_col && j < C_out) p.db_partial[(int64_t)t.split * C_out + j] = 0.f;
+                    if (bias_col && j < C_out && !p.db_accumulate) p.db_partial[(int64_t)t.split * C_out + j] = 0.f;
                     continue;
                 }
                 if (lane == 0) ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_full[acc]), (used >> 1) & 1u, abort_flag, status_word);
@@ -777,7 +778,11 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                         float v[kEpiChunk];
                         ptx::tmem_ld_32x16(kNarrow ? taddr + 128u : tmem_base + (acc ^ 1u) * kAccCols + ((uint32_t)(warp * 32) << 16), v);
                         ptx::tmem_ld_wait();
-                        if (j < C_out) p.db_partial[(int64_t)t.split * C_out + j] = v[0];
+                        if (j < C_out) {
+                            float* out = p.db_partial + (int64_t)t.split * C_out + j;
+                            if (p.db_accumulate) v[0] += *out;
+                            *out = v[0];
+                        }
                     }
                 }
             }
@@ -1063,11 +1068,17 @@ size_t tc_dw_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
     return s > 1 ? (size_t)s * (size_t)C_in * (size_t)C_out * sizeof(float) : 0;
 }
 
+// Narrow layers (both tile kinds 128 wide), and wide ones under the role split (one dW piece per block, so the second
+// accumulator slot is free): db is one more output column of the dW tiles.  With one piece that column is db itself and no
+// reduce launch follows (dW + db + dX: 784 kept rows of 768 -> 768 11.5 -> 10.2 us, 117 of 2560 -> 640 7.9 -> 6.5).
+static bool db_in_dw_tiles(const Plan& pl, bool want_dw) { return want_dw && ((pl.bnx <= 128 && pl.bnw <= 128) || pl.dw_ctas > 0); }
+
 int tc_backward_kernel_count(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx,
                              bool want_db, bool dy_packed) {
     if (!want_dw && !want_dx) return 0;
-    const bool reduce_dw = want_dw && make_plan(M_keep_cap, C_in, C_out, want_dw, want_dx, dy_packed).splits > 1;
-    return 1 + ((reduce_dw || want_db) ? 1 : 0);       // the two reductions share one launch
+    const Plan pl = make_plan(M_keep_cap, C_in, C_out, want_dw, want_dx, dy_packed);
+    const bool reduce_dw = want_dw && pl.splits > 1, reduce_db = want_db && !(db_in_dw_tiles(pl, want_dw) && pl.splits == 1);
+    return 1 + ((reduce_dw || reduce_db) ? 1 : 0);     // the two reductions share one launch
 }
 
 sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W, const int32_t* dy_rows,
@@ -1105,11 +1116,10 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     } else {
         map_dw = map_x;                                              // never used
     }
-    prm.db_partial = (db != nullptr) ? db_workspace : nullptr;
-    // narrow layers (both tile kinds 128 wide), and wide ones under the role split (one dW piece per block, so the second
-    // accumulator slot is free): db is one more output column of the dW tiles, one partial row per split
-    const bool db_from_mma = db != nullptr && want_dw && ((pl.bnx <= 128 && pl.bnw <= 128) || pl.dw_ctas > 0);
+    const bool db_from_mma = db != nullptr && db_in_dw_tiles(pl, want_dw), db_direct = db_from_mma && pl.splits == 1;
     prm.db_from_mma = db_from_mma ? 1 : 0;
+    prm.db_partial = (db == nullptr) ? nullptr : db_direct ? db : db_workspace;
+    prm.db_accumulate = (db_direct && accumulate) ? 1 : 0;
     const int db_rows = db_from_mma ? pl.splits : 0;                 // 0: one row per block (set below)
     prm.status_word = status_word;
     prm.dw_ctas = pl.dw_ctas;
@@ -1138,7 +1148,7 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     else if (pl.bnx == 256) e = launch_fused<256, false>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in);
     else e = launch_fused<128, false>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in);
     if (e != cudaSuccess) return SBP_ERR_CUDA;
-    const bool reduce_dw = want_dw && pl.splits > 1, reduce_db = db != nullptr;
+    const bool reduce_dw = want_dw && pl.splits > 1, reduce_db = db != nullptr && !db_direct;
     cudaError_t r = cudaSuccess;
     if (reduce_dw && reduce_db)
         r = launch_reduce_partials_pair(workspace, pl.splits, C_in * C_out, dW, db_workspace, db_rows ? db_rows : (int)ctas, C_out, db,

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
     (130, 129, 64, 64, False, False), (512, 512, 256, 32, False, False), (513, 500, 256, 32, False, True), (512, 512, 264, 40, False, False),
     (700, 650, 120, 72, False, False), (3000, 2999, 64, 2048, True, True), (3000, 2000, 2056, 64, True, False),
     (5000, 4500, 8, 16384, True, False), (5000, 4500, 16384, 8, True, True), (6000, 5000, 96, 520, False, False), (5000, 5000, 512, 72, False, False),
+    (200, 0, 64, 136, False, False), (200, 0, 64, 136, False, True), (784, 700, 768, 768, False, True), (784, 784, 768, 768, True, False),
 ])
 def test_narrow_backward(cap, keep, C_in, C_out, w_out_in, accumulate):
     M = 2 * cap + 3
