@@ -74,13 +74,14 @@ constexpr uint32_t kABytes = kBM * kRowBytes;        // 16 KB
 constexpr uint32_t kBBytesMax = 256 * kRowBytes;     // 32 KB
 constexpr uint32_t kStageBytes = kABytes + kBBytesMax;
 constexpr uint32_t kAccCols = 256;       // TMEM columns per accumulator buffer (two buffers = all 512)
-constexpr int kBiasChunk = 64;           // kept rows whose ids the bias warps stage at a time
+constexpr int kBiasStrip = 32;            // 16-byte columns of dY a block sums: 512 bytes of each row
+constexpr int kBiasChunk = 128;           // kept rows whose ids the bias warps stage at a time, one a thread
 // 16-byte loads each side-warp thread keeps in flight for the bias sums: a template parameter of the kernel,
 // 8 or 16.  The deep queue finishes long row lists in time; with short lists it only takes memory
 // bandwidth from the operand copies (ViT-B fc1: 5 us per call), so the host picks per shape.
 // cross-row-group sums + staged row ids, padded so that the staging buffers after it start on a 1024-byte boundary
 // (one of them holds a swizzled tensor-core operand)
-constexpr uint32_t kBiasSmemBytes = kBiasThreads * 8 * sizeof(float) + kBiasChunk * sizeof(int) + 512;
+constexpr uint32_t kBiasSmemBytes = kBiasThreads * 8 * sizeof(float) + kBiasChunk * sizeof(int) + 256;
 constexpr int kEpiChunk = 16;            // accumulator columns (= rows of dW) per TMA store of the dW epilogue
 constexpr int kEpiBufs = 3;              // staging buffers the dW epilogue rotates through
 constexpr uint32_t kEpiBufBytes = kEpiChunk * kBM * sizeof(float);   // 8 KB: 16 rows of dW x 128 columns
@@ -117,7 +118,8 @@ struct TcParams {
     int db_from_mma;               // narrow layers: db comes out of the dW tiles (a column of ones appended to X_keep);
                                    // db_partial is then [dw_splits, C_out]
     int db_accumulate;             // one piece: db_partial is db itself, which is added to (1) or written (0)
-    float* db_partial;             // nullptr: no bias sums; else [gridDim.x, C_out] per-CTA column sums of kept dY rows
+    float* db_partial;             // nullptr: no bias sums; else [db_shares, C_out] column sums of shares of the kept dY rows
+    int db_shares;
     int dw_ctas;                   // 0: every block walks the one cost-sorted list of both tile kinds; > 0: the first
                                    // dw_ctas blocks take the dW pieces, the others the dX tiles, both sweeping the kept
                                    // rows in the same order (memory-bound layers: see next_tile)
@@ -604,25 +606,29 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
             float* red = reinterpret_cast<float*>(smem_raw + (ring - raw_addr) + kRingBytes + 256);
             const int t = side_index<kNarrow>(warp) * 32 + lane;
             const int V = C_out >> 3;                                  // 16-byte column vectors per row
-            int VT = 16;                                               // vectors covered per pass (power of two <= 128)
-            while (VT < V && VT < kBiasThreads) VT <<= 1;
+            const int VT = V > 16 ? kBiasStrip : 16;                   // vectors of a strip
             const int RG = kBiasThreads / VT;                          // row groups working on the same columns
             const int cvt = t % VT, rg = t / VT;
-            const int64_t rows_per = (M_keep + gridDim.x - 1) / gridDim.x;
-            const int64_t m_begin = rows_per * blockIdx.x;
-            const int64_t m_end = (m_begin + rows_per < M_keep) ? m_begin + rows_per : M_keep;
+            const int strips = (V + VT - 1) / VT, shares = p.db_shares;
+            const int64_t rows_per = (M_keep + shares - 1) / shares;
             const uint4* dY4 = reinterpret_cast<const uint4*>(p.dY);
-            float* out = p.db_partial + (int64_t)blockIdx.x * C_out;
             int* ids = reinterpret_cast<int*>(red + kBiasThreads * 8);  // row ids of the current chunk of kept rows
-            for (int cv0 = 0; cv0 < V; cv0 += VT) {
-                const int cv = cv0 + cvt;
+            for (int work = blockIdx.x; work < strips * shares; work += gridDim.x) {
+                const int share = work / strips, cv = (work - share * strips) * VT + cvt;
+                const int64_t m_begin = rows_per * share;
+                const int64_t m_end = (m_begin + rows_per < M_keep) ? m_begin + rows_per : M_keep;
+                float* out = p.db_partial + (int64_t)share * C_out;
                 float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                const auto row_id = [&](int64_t m) { return m < m_end ? map_row<kPacked>(p.dy_rows, m) : -1; };
+                int id = row_id(m_begin + t);
                 for (int64_t mc = m_begin; mc < m_end; mc += kBiasChunk) {
-                    // stage the chunk's row ids once, so that the dY loads below depend on no other load
-                    if (t < kBiasChunk) ids[t] = (mc + t < m_end) ? map_row<kPacked>(p.dy_rows, mc + t) : -1;
+                    // the chunk's row ids are staged once, so that the dY loads below depend on no other load; the next chunk's
+                    // are under way meanwhile
+                    ids[t] = id;
+                    id = row_id(mc + kBiasChunk + t);
                     asm volatile("bar.sync 1, %0;" ::"n"(kBiasThreads) : "memory");
                     if (cv < V) {
-                        for (int r0 = rg; r0 < kBiasChunk; r0 += RG * kBiasDepth) {
+                        for (int r0 = rg; r0 < kBiasChunk && mc + r0 < m_end; r0 += RG * kBiasDepth) {
                             uint4 v[kBiasDepth];
 #pragma unroll
                             for (int u = 0; u < kBiasDepth; ++u) {
@@ -1120,7 +1126,6 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     prm.db_from_mma = db_from_mma ? 1 : 0;
     prm.db_partial = (db == nullptr) ? nullptr : db_direct ? db : db_workspace;
     prm.db_accumulate = (db_direct && accumulate) ? 1 : 0;
-    const int db_rows = db_from_mma ? pl.splits : 0;                 // 0: one row per block (set below)
     prm.status_word = status_word;
     prm.dw_ctas = pl.dw_ctas;
     int64_t ctas = pl.tiles < kNumSMs ? pl.tiles : kNumSMs;
@@ -1130,6 +1135,14 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
         ctas = 2 * pairs;
     }
     const dim3 grid((unsigned)ctas);
+    // Bias sums on the side: a block sums a strip of columns over a share of the kept rows, as many shares as the strips leave
+    // blocks for.  A block's own share of all columns made 148 partial rows for the reduce launch to add, passes of 128 columns
+    // whose last one may be nearly empty, and a wait for row ids in each: dW + db + dX of 30000 kept rows of 320 -> 1280
+    // 79.4 -> 66.1 us, 12544 of 768 -> 2304 84.7 -> 80.8, 1570 of 1024 -> 4096 33.7 -> 31.6 (strips of 64 and 128 columns:
+    // 68.3 and 74.9, 81.0 and 81.9, 31.5 and 32.2).
+    const int64_t strips = (C_out / 8 + kBiasStrip - 1) / kBiasStrip;
+    prm.db_shares = (int)(ctas / strips < 1 ? 1 : ctas / strips);
+    const int db_rows = db_from_mma ? pl.splits : prm.db_shares;
     // Bias sums on the side: 16-byte loads per side-warp thread against the time the main loop leaves them
     // (about 1.3 us per batch of loads in flight, 0.45 us per k-block).  The shallow queue is enough when it
     // ends well within the main loop.
@@ -1151,12 +1164,12 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     const bool reduce_dw = want_dw && pl.splits > 1, reduce_db = db != nullptr && !db_direct;
     cudaError_t r = cudaSuccess;
     if (reduce_dw && reduce_db)
-        r = launch_reduce_partials_pair(workspace, pl.splits, C_in * C_out, dW, db_workspace, db_rows ? db_rows : (int)ctas, C_out, db,
+        r = launch_reduce_partials_pair(workspace, pl.splits, C_in * C_out, dW, db_workspace, db_rows, C_out, db,
                                         accumulate, status_word, stream);
     else if (reduce_dw)
         r = launch_reduce_partials(workspace, pl.splits, C_in * C_out, dW, accumulate, status_word, stream);
     else if (reduce_db)
-        r = launch_reduce_partials(db_workspace, db_rows ? db_rows : (int)ctas, C_out, db, accumulate, status_word, stream);
+        r = launch_reduce_partials(db_workspace, db_rows, C_out, db, accumulate, status_word, stream);
     if (r != cudaSuccess) return SBP_ERR_CUDA;
     return SBP_OK;
 }
