@@ -867,14 +867,23 @@ struct Plan {
     int64_t tiles;         // upper bound of the tile count (from the capacity); tiles of pairs when pair is set
 };
 
-// Estimated run time of the tile list for a given split count, in units of one dX k-block: the
-// longest per-block total under the kernel's own static assignment (block b takes list positions
-// b, 2G-1-b, 2G+b, ...), the epilogue of that block's last tile, and the reduce launch that
-// splitting costs.  The weights are measured ratios on ViT-B shapes; they only rank candidates.
-double estimate_cost(int64_t x_tiles, int64_t x_kb, int64_t w_tiles, int64_t w_kb, int64_t splits, int64_t dw_elems, int64_t workers) {
-    constexpr double kDwKb = 1.12;        // a dW k-block (two gathered MN-major operands) relative to a dX one
-    constexpr double kTileSwitch = 0.5;   // per tile: pipeline hand-over
-    constexpr double kTailDx = 9.0, kTailDw = 6.0;   // exposed epilogue of the last tile
+// Estimated run time (us) of the tile list for a given split count: the longest per-block total under the kernel's own static
+// assignment (block b takes list positions b, 2G-1-b, 2G+b, ...), a share of the mean one (blocks slow each other down) and
+// the reduce launch that splitting costs.  The rates come from a fit to some 800 timed (shape, split count) pairs on B200,
+// 49 layers of 784 to 50176 kept rows, that weighs the good split counts of each layer; its picks are within 1 % of the best
+// timed count on average, 7 % at worst.  Against the ratios before it, which an earlier build of the kernel had given, dW + db +
+// dX: 12544 kept rows of 768 -> 2304 79.4 -> 74.1 us (5 pieces -> 2), 512 -> 2048 52.6 -> 47.6 (7 -> 3), 3136 of 128 -> 1024
+// 12.2 -> 10.8 (3 -> 10).
+struct Rates {
+    double dx_kb, dw_kb;         // a k-block of either kind
+    double dx_min, dw_tile;      // a dX tile takes at least its read-out; the hand-over of a dW tile
+    double dx_tail, dw_tail;     // exposed read-out of a block's last tile
+    double fixed, reduce, reduce_mb, mean;
+};
+constexpr Rates kRatesSingle = {0.364, 0.308, 3.75, 5.30, 1.01, 0.00, 2.64, 2.91, 0.040, 0.254};
+constexpr Rates kRatesPair = {0.271, 0.239, 3.92, 2.95, 0.40, 0.80, 5.51, 0.00, 0.084, 0.600};
+constexpr Rates kRatesNarrow = {0.155, 0.306, 1.40, 2.26, 1.46, 0.03, 3.28, 2.28, 0.101, 0.103};
+double estimate_us(const Rates& r, int64_t x_tiles, int64_t x_kb, int64_t w_tiles, int64_t w_kb, int64_t splits, int64_t dw_elems, int64_t workers) {
     const int64_t kb_per = (w_kb + splits - 1) / splits;
     const int64_t w_pieces = w_tiles * splits;
     const int64_t total = x_tiles + w_pieces;
@@ -882,7 +891,7 @@ double estimate_cost(int64_t x_tiles, int64_t x_kb, int64_t w_tiles, int64_t w_k
     const int64_t G = total < workers ? total : workers;
     const bool w_first = kb_per >= x_kb;
     const int64_t first = w_first ? w_pieces : x_tiles;
-    double worst = 0.0;
+    double worst = 0.0, all = 0.0;
     for (int64_t b = 0; b < G; ++b) {
         double sum = 0.0, tail = 0.0;
         for (int64_t pass = 0;; ++pass) {
@@ -894,17 +903,18 @@ double estimate_cost(int64_t x_tiles, int64_t x_kb, int64_t w_tiles, int64_t w_k
                 int64_t n = w_kb - kb_per * split;
                 if (n > kb_per) n = kb_per;
                 if (n < 0) n = 0;
-                sum += kDwKb * (double)n + kTileSwitch;
-                tail = kTailDw;
+                sum += r.dw_kb * (double)n + r.dw_tile;
+                tail = r.dw_tail;
             } else {
-                sum += (double)x_kb + kTileSwitch;
-                tail = kTailDx;
+                sum += (double)x_kb * r.dx_kb > r.dx_min ? (double)x_kb * r.dx_kb : r.dx_min;
+                tail = r.dx_tail;
             }
         }
         if (sum + tail > worst) worst = sum + tail;
+        all += sum;
     }
-    if (splits > 1) worst += 7.0 + (double)(splits + 1) * (double)dw_elems * 4.0 / 1.7e6;   // launch + traffic of the reduce
-    return worst;
+    if (splits > 1) worst += r.reduce + r.reduce_mb * (double)(splits + 1) * (double)dw_elems * 4e-6;
+    return r.fixed + worst + r.mean * all / (double)workers;
 }
 
 struct PlanKey {
@@ -914,7 +924,7 @@ struct PlanKey {
     bool operator<(const PlanKey& o) const { return std::tie(cap, ci, co, dx, dy_packed) < std::tie(o.cap, o.ci, o.co, o.dx, o.dy_packed); }
 };
 std::mutex g_plan_mutex;
-struct PlanChoice { int splits, dw_ctas; };
+struct PlanChoice { int splits, dw_ctas; bool pair; };
 std::map<PlanKey, PlanChoice> g_plan_memo;
 int64_t g_plan_searches = 0;
 
@@ -932,30 +942,32 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
     const bool short_chain = narrow_tiles <= kNumSMs && (!want_dw || M_keep_cap <= 4608);
     pl.bnx = (C_in >= 256 && !short_chain) ? 256 : 128;
     pl.bnw = pl.bnx;
-    int64_t x_tiles = want_dx ? ((M_keep_cap + kBM - 1) / kBM) * ((C_in + pl.bnx - 1) / pl.bnx) : 0;
-    const int64_t x_kb = (C_out + kBK - 1) / kBK;
-    int64_t w_tiles = want_dw ? ((C_out + kBM - 1) / kBM) * ((C_in + pl.bnw - 1) / pl.bnw) : 0;
-    const int64_t w_kb = (M_keep_cap + kBK - 1) / kBK;
+    const int64_t x_kb = (C_out + kBK - 1) / kBK, w_kb = (M_keep_cap + kBK - 1) / kBK;
+    int64_t x_tiles = 0, w_tiles = 0;
+    const auto count_tiles = [&](bool pair) {
+        const int64_t rows = pair ? 2 * kBM : kBM;
+        x_tiles = want_dx ? ((M_keep_cap + rows - 1) / rows) * ((C_in + pl.bnx - 1) / pl.bnx) : 0;
+        w_tiles = want_dw ? ((C_out + rows - 1) / rows) * ((C_in + pl.bnw - 1) / pl.bnw) : 0;
+    };
+    count_tiles(false);
     pl.splits = 1;
     pl.dw_ctas = 0;
-    // Wide layers with enough work for every pair run as pairs of blocks unless the role split below takes them (the
-    // memory-bound layers gain nothing from the faster tensor-core form).  From some 4000 kept rows on the pairs win on
-    // every wide shape of the paper's models (ViT-B/16 at 6272 kept rows: backward 63 -> 55 us).  A call for dX alone has
-    // no dW pieces to even out its tile list, so there the pairs must fill their waves about as well as single blocks
-    // would (6272 kept rows x 768 columns: 75 tiles on 74 pairs, 43 us against 30 us).
+    // Wide layers run as pairs of blocks from some 4000 kept rows on, unless the role split below takes them (the
+    // memory-bound layers gain nothing from the faster tensor-core form): there the pairs win on every wide shape of the
+    // paper's models (ViT-B/16 at 6272 kept rows: backward 63 -> 55 us).  With fewer rows, where 74 pairs may fill their waves
+    // worse than 148 blocks, the tile lists decide (below).  A call for dX alone has no dW pieces to even out its tile list, so
+    // there the pairs must fill their waves about as well as single blocks would (6272 kept rows x 768 columns: 75 tiles on 74
+    // pairs, 43 us against 30 us).
     const bool memory_bound = 2.0 * (double)M_keep_cap * (double)(2 * C_in + C_out) / 6.5e12 >=
                               0.75 * 4.0 * (double)M_keep_cap * (double)C_in * (double)C_out / 1.4e15;
-    pl.pair = pl.bnx == 256 && pl.bnw == 256 && C_out >= 256 && M_keep_cap >= 4096 && !(want_dw && want_dx && !dy_packed && memory_bound);
+    const bool pair_ok = pl.bnx == 256 && pl.bnw == 256 && C_out >= 256 && !(want_dw && want_dx && !dy_packed && memory_bound);
+    pl.pair = pair_ok && M_keep_cap >= 4096;
     if (pl.pair && !want_dw) {
         const int64_t pair_tiles = ((M_keep_cap + 2 * kBM - 1) / (2 * kBM)) * ((C_in + pl.bnx - 1) / pl.bnx);
         const auto fill = [](int64_t tiles, int64_t workers) { return (double)tiles / (double)((tiles + workers - 1) / workers * workers); };
         pl.pair = fill(pair_tiles, kNumSMs / 2) + 0.1 >= fill(x_tiles, kNumSMs);
     }
-    if (pl.pair) {
-        x_tiles = want_dx ? ((M_keep_cap + 2 * kBM - 1) / (2 * kBM)) * ((C_in + pl.bnx - 1) / pl.bnx) : 0;
-        w_tiles = want_dw ? ((C_out + 2 * kBM - 1) / (2 * kBM)) * ((C_in + pl.bnw - 1) / pl.bnw) : 0;
-    }
-    const int64_t workers = pl.pair ? kNumSMs / 2 : kNumSMs;
+    count_tiles(pl.pair);
     if (want_dw) {
         // The same answer for the same shape: every shape a process has asked about is remembered (a few
         // dozen bytes per layer shape, never evicted), so a model's layers do not push each other out.
@@ -967,6 +979,8 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
             if (it != g_plan_memo.end()) {
                 pl.splits = it->second.splits;
                 pl.dw_ctas = it->second.dw_ctas;
+                pl.pair = it->second.pair;
+                count_tiles(pl.pair);
                 known = true;
             }
         }
@@ -997,18 +1011,33 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
                 }
             }
             if (!role_split) {
-                int64_t max_s = w_kb < 64 ? w_kb : 64;
-                if (max_s < 1) max_s = 1;
-                // the search walks every tile: with very many tiles any cut balances, so bound the work
-                while (max_s > 1 && (x_tiles + w_tiles * max_s) * max_s > (1 << 22)) max_s /= 2;
-                double best = 0.0;
-                for (int64_t sp = 1; sp <= max_s; ++sp) {
-                    const double c = estimate_cost(x_tiles, x_kb, w_tiles, w_kb, sp, C_in * C_out, workers);
-                    if (sp == 1 || c < best * 0.995) { best = c; pl.splits = (int)sp; }
+                const auto search = [&](const Rates& rates, bool pair, double* cost) {
+                    count_tiles(pair);
+                    int64_t max_s = w_kb < 64 ? w_kb : 64;
+                    if (max_s < 1) max_s = 1;
+                    // the search walks every tile: with very many tiles any cut balances, so bound the work
+                    while (max_s > 1 && (x_tiles + w_tiles * max_s) * max_s > (1 << 22)) max_s /= 2;
+                    int best = 1;
+                    for (int64_t sp = 1; sp <= max_s; ++sp) {
+                        const double c = estimate_us(rates, x_tiles, x_kb, w_tiles, w_kb, sp, C_in * C_out, pair ? kNumSMs / 2 : kNumSMs);
+                        if (sp == 1 || c < *cost * 0.995) { *cost = c; best = (int)sp; }
+                    }
+                    return best;
+                };
+                double cost = 0.0, alone = 0.0;
+                if (!pl.pair && pair_ok && want_dx) {
+                    // few rows: pairs unless their list fills the waves worse than that of single blocks would at the same rates
+                    // (1500 kept rows of 2048 -> 2048 30.9 us alone, 28.3 in pairs, 3000 of 3072 -> 768 34.9 and 32.0, 4000 of
+                    // 1024 -> 4096 59.6 and 55.4; the other way round 2600 of 1024 -> 1024 19.6 and 22.4, 1568 of 4096 -> 1024
+                    // 34.6 and 35.1; dW alone 1568 of 1024 -> 4096 19.7 and 20.5)
+                    search(kRatesPair, true, &cost);
+                    search(kRatesPair, false, &alone);
+                    pl.pair = cost <= 1.001 * alone;
                 }
+                pl.splits = search(pl.pair ? kRatesPair : pl.bnx == 256 ? kRatesSingle : kRatesNarrow, pl.pair, &cost);
             }
             std::lock_guard<std::mutex> lock(g_plan_mutex);
-            g_plan_memo[key] = PlanChoice{pl.splits, pl.dw_ctas};
+            g_plan_memo[key] = PlanChoice{pl.splits, pl.dw_ctas, pl.pair};
             ++g_plan_searches;
         }
     }
