@@ -1002,9 +1002,13 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
                 const double target = bytes_w / (bytes_w + bytes_x) * (double)kNumSMs;
                 int64_t sp = (int64_t)(target / (double)w_tiles + 0.5);
                 const int64_t x_rtiles = (M_keep_cap + kBM - 1) / kBM;
-                // worth it only with enough dX tiles per dX block to balance (a short list leaves the groups uneven)
+                // worth it only with enough dX tiles per dX block to balance (a short list leaves the groups uneven): 7/3 of them.
+                // dW + db + dX with one list -> split, by tiles per block: 6.9 (66800 kept rows of 128 -> 512) 39.1 -> 33.7 us,
+                // 4.3 (50176 of 256 -> 256) 38.7 -> 31.0, 3.3 (12544 of 768 -> 192) 26.1 -> 23.5, 2.8 (30000 of 128 -> 512) 23.0 ->
+                // 20.4, 2.4 (16000 of 512 -> 128) 22.4 -> 20.4; 2.3 (6272 of 1024 -> 256) 19.4 -> 19.8, 2.2 (12544 of 192 -> 768)
+                // 20.2 -> 22.2; out of line 3.4 (40000 of 64 -> 256) 15.5 -> 16.3.
                 if (sp >= 2 && w_kb / sp >= 8 && x_rtiles >= sp && w_tiles * sp <= kNumSMs - 16 &&
-                    x_tiles >= 8 * (kNumSMs - w_tiles * sp)) {
+                    3 * x_tiles >= 7 * (kNumSMs - w_tiles * sp)) {
                     pl.splits = (int)sp;
                     pl.dw_ctas = (int)(w_tiles * sp);
                     role_split = true;

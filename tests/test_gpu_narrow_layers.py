@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
     (5000, 4500, 8, 16384, True, False), (5000, 4500, 16384, 8, True, True), (6000, 5000, 96, 520, False, False), (5000, 5000, 512, 72, False, False),
     (200, 0, 64, 136, False, False), (200, 0, 64, 136, False, True), (784, 700, 768, 768, False, True), (784, 784, 768, 768, True, False),
     (1500, 1400, 2048, 2048, False, False), (1111, 1111, 2056, 1032, False, True), (3000, 2990, 3072, 768, True, False), (3001, 2875, 3080, 264, False, False),  # wide, few rows
+    (16000, 15873, 512, 128, False, False), (20000, 19990, 264, 264, False, True), (30000, 28000, 64, 64, True, False),         # dW and dX blocks apart
 ])
 def test_narrow_backward(cap, keep, C_in, C_out, w_out_in, accumulate):
     M = 2 * cap + 3
