@@ -8,7 +8,11 @@
 // a bin ever hold more words than the list, the next eight bits are taken, as often as needed.)  Four passes of eight bits
 // and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.5 us
 // and 4.6 us (the words are drawn while the kernel before drains).
-// Grid mode evaluates the lattice predicate with an ordered compaction; per-sample offsets come from closed-form counts.
+// Grid mode: everything has a closed form - a sample's offset from the counts of the samples before it, a kept position's place
+// from the kept positions in the rows above and to its left - so each block writes a stretch of one map without a scan, and a
+// large map is spread over as many blocks as the samples leave room for (a predicate and an ordered compaction by one block a
+// sample, back to back: 64 maps of 56 x 56 3.9 us, 2 of 200 x 334 31.5; now 2.2 and 2.1).
+#include "row_copy.cuh"
 #include "sbp_common.cuh"
 
 namespace sbp {
@@ -16,11 +20,6 @@ namespace {
 
 constexpr int kSampThreads = 512;
 constexpr int kSampWarps = kSampThreads / 32;
-
-struct SampShared {
-    uint32_t warp_sums_b[kSampWarps];
-    uint64_t red64[kSampWarps];
-};
 
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
 #pragma unroll
@@ -291,6 +290,17 @@ __device__ __forceinline__ uint32_t grid_count(int family, uint32_t p, uint32_t 
     }
 }
 
+// kept positions of row h in front of column w
+__device__ __forceinline__ uint32_t grid_before(int family, uint32_t p, uint32_t h, uint32_t w) {
+    const uint32_t on_lattice = (h & 1u) == (p >> 1) ? (w + 1u - (p & 1u)) >> 1 : 0u;
+    switch (family) {
+        case 1: return on_lattice;
+        case 2: return (w + 1u - ((p + h) & 1u)) >> 1;
+        case 3: return w - on_lattice;
+        default: return w;
+    }
+}
+
 __device__ __forceinline__ bool grid_keeps(int family, uint32_t p, uint32_t h, uint32_t w) {
     const bool on_lattice = ((h & 1u) == (p >> 1)) && ((w & 1u) == (p & 1u));
     switch (family) {
@@ -301,14 +311,14 @@ __device__ __forceinline__ bool grid_keeps(int family, uint32_t p, uint32_t h, u
     }
 }
 
+// `parts` blocks a sample, each with a contiguous stretch of the positions
 __global__ void __launch_bounds__(kSampThreads)
-sample_keep_grid_kernel(int family, uint32_t H, uint32_t W, uint32_t k0, uint32_t k1, uint32_t step,
+sample_keep_grid_kernel(int family, uint32_t H, uint32_t W, FastDiv by_width, uint32_t parts, uint32_t k0, uint32_t k1, uint32_t step,
                         uint32_t first_sample, int share_mask,
                         int32_t* __restrict__ keep_rows, int32_t* __restrict__ keep_offsets) {
-    __shared__ SampShared sh;
+    __shared__ uint64_t red[kSampWarps];
     pdl_launch_dependents();
-    pdl_wait();
-    const uint32_t b = blockIdx.x;
+    const uint32_t b = blockIdx.x / parts, part = blockIdx.x - b * parts;
     const uint32_t N = H * W;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
@@ -317,43 +327,28 @@ sample_keep_grid_kernel(int family, uint32_t H, uint32_t W, uint32_t k0, uint32_
     if (share_mask) {
         before = (uint64_t)b * grid_count(family, grid_phase(family, 0u, step, k0, k1), H, W);
     } else {
-        uint64_t part = 0;
+        uint64_t sum = 0;
         for (uint32_t s = threadIdx.x; s < b; s += kSampThreads)
-            part += grid_count(family, grid_phase(family, first_sample + s, step, k0, k1), H, W);
+            sum += grid_count(family, grid_phase(family, first_sample + s, step, k0, k1), H, W);
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(0xffffffffu, part, d);
-        if (lane == 0) sh.red64[warp] = part;
+        for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        if (lane == 0) red[warp] = sum;
         __syncthreads();
-        for (int i = 0; i < kSampWarps; ++i) before += sh.red64[i];
-        __syncthreads();
+        for (int i = 0; i < kSampWarps; ++i) before += red[i];
     }
-    const uint32_t gid = share_mask ? 0u : first_sample + b;
-    const uint32_t p = grid_phase(family, gid, step, k0, k1);
-    const uint32_t mine = grid_count(family, p, H, W);
-    if (threadIdx.x == 0) {
-        keep_offsets[b + 1] = (int32_t)(before + mine);
+    const uint32_t p = grid_phase(family, share_mask ? 0u : first_sample + b, step, k0, k1);
+    pdl_wait();                 // earlier kernels of the stream may still be reading the index buffers
+    if (part == 0 && threadIdx.x == 0) {
+        keep_offsets[b + 1] = (int32_t)(before + grid_count(family, p, H, W));
         if (b == 0) keep_offsets[0] = 0;
     }
     int32_t* out = keep_rows + before;
     const int64_t row_base = (int64_t)b * N;
-    const uint32_t groups = (N + 3u) >> 2;
-    uint32_t written = 0;
-    for (uint32_t q0 = 0; q0 < groups; q0 += kSampThreads) {
-        const uint32_t q = q0 + threadIdx.x;
-        uint32_t keep_mask = 0;
-        if (q < groups) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t n = 4u * q + e;
-                if (n < N && grid_keeps(family, p, n / W, n % W)) keep_mask |= 1u << e;
-            }
-        }
-        const uint2 sk = block_excl_scan<kSampThreads>(__popc(keep_mask), sh.warp_sums_b);
-        uint32_t pos = written + sk.x;
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (keep_mask & (1u << e)) out[pos++] = (int32_t)(row_base + 4u * q + e);
-        written += sk.y;
+    const uint32_t per = (N + parts - 1) / parts;
+    const uint32_t begin = part * per < N ? part * per : N, end = N - begin < per ? N : begin + per;
+    for (uint32_t n = begin + threadIdx.x; n < end; n += kSampThreads) {
+        const uint32_t h = by_width(n), w = n - h * W;
+        if (grid_keeps(family, p, h, w)) out[grid_count(family, p, h, W) + grid_before(family, p, h, w)] = (int32_t)(row_base + n);
     }
 }
 
@@ -500,7 +495,11 @@ cudaError_t launch_sample_keep(int mode, int grid_family, int64_t B, int64_t H, 
         return launch_pdl(sample_keep_temporal_kernel, grid, block, 0, stream, mode == SBP_MASK_TEMPORAL ? 0 : grid_family,
                           (uint32_t)H, (uint32_t)W, (uint32_t)(K / W),
                           k0, k1, step, first_sample, share_mask ? 1 : 0, keep_rows, keep_offsets);
-    return launch_pdl(sample_keep_grid_kernel, grid, block, 0, stream, grid_family, (uint32_t)H, (uint32_t)W, k0, k1,
+    // four positions a thread, on four blocks an SM at most
+    const int64_t by_size = (H * W + 4 * kSampThreads - 1) / (4 * kSampThreads), by_room = 4 * kNumSMs / B;
+    const int64_t parts = by_size < by_room ? by_size : by_room < 1 ? 1 : by_room;
+    return launch_pdl(sample_keep_grid_kernel, dim3((unsigned)(B * parts)), block, 0, stream, grid_family, (uint32_t)H, (uint32_t)W,
+                      FastDiv((uint32_t)W), (uint32_t)parts, k0, k1,
                       step, first_sample, share_mask ? 1 : 0, keep_rows, keep_offsets);
 }
 

@@ -1,5 +1,5 @@
-"""`sbp_sample_keep` with random masks where its block size, clusters, word cache and stretches change, bit for bit against
-the oracle: one position, one group more or less than the threads, every cluster size, maps beyond the cache, extreme ratios."""
+"""`sbp_sample_keep` where its block size, clusters, word cache and stretches (random masks) or its blocks per sample (grid masks)
+change, bit for bit against the oracle: one position, one group more or less than the threads, every cluster size, maps beyond the cache, extreme ratios."""
 import numpy as np
 import pytest
 
@@ -20,3 +20,13 @@ def test_random_masks_at_every_dispatch(B, H, W, r):
         keep, want_offs = oracle.sample_keep(0, B, H, W, r, 9 + share, 3, 2, bool(share))
         assert np.array_equal(offs.cpu().numpy(), want_offs)
         assert np.array_equal(rows.cpu().numpy()[:len(keep)], keep)
+
+
+@pytest.mark.parametrize("B,H,W", [(1, 1, 1), (3, 1, 7), (3, 7, 1), (2, 45, 46), (70, 7, 7), (600, 3, 5), (2, 200, 334), (3, 333, 201), (1, 1024, 1025)])
+def test_grid_masks_at_every_split(B, H, W):
+    for r in (0.25, 0.5, 0.75, 1.0):
+        for share in (0, 1):
+            rows, offs, cap = run_sample_keep(1, B, H, W, r, seed=9 + share, step=3, offset=2, flags=share)
+            keep, want_offs = oracle.sample_keep(1, B, H, W, r, 9 + share, 3, 2, bool(share))
+            assert np.array_equal(offs.cpu().numpy(), want_offs)
+            assert np.array_equal(rows.cpu().numpy()[:len(keep)], keep)
