@@ -30,3 +30,14 @@ def test_grid_masks_at_every_split(B, H, W):
             keep, want_offs = oracle.sample_keep(1, B, H, W, r, 9 + share, 3, 2, bool(share))
             assert np.array_equal(offs.cpu().numpy(), want_offs)
             assert np.array_equal(rows.cpu().numpy()[:len(keep)], keep)
+
+
+@pytest.mark.parametrize("B,T,P", [(1, 1, 1), (1, 8, 196), (3, 7, 1), (2, 33, 1000), (600, 5, 9), (1, 2048, 3), (2, 64, 3136)])
+@pytest.mark.parametrize("mode", [2, 3])
+def test_frame_masks_at_every_split(mode, B, T, P):
+    for r in (0.25, 0.5, 0.75):
+        for share in (0, 1):
+            rows, offs, cap = run_sample_keep(mode, B, T, P, r, seed=9 + share, step=3, offset=2, flags=share)
+            keep, want_offs = oracle.sample_keep(mode, B, T, P, r, 9 + share, 3, 2, bool(share))
+            assert np.array_equal(offs.cpu().numpy(), want_offs)
+            assert np.array_equal(rows.cpu().numpy()[:len(keep)], keep)
