@@ -7,7 +7,7 @@
 // thread then owns a contiguous stretch of positions, so one block scan of their counts places every kept position.  (Should
 // a bin ever hold more words than the list, the next eight bits are taken, as often as needed.)  Four passes of eight bits
 // and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.5 us
-// and 4.6 us (the words are drawn while the kernel before drains).
+// and 3.7 us (the words are drawn while the kernel before drains).
 // Grid mode: everything has a closed form - a sample's offset from the counts of the samples before it, a kept position's place
 // from the kept positions in the rows above and to its left - so each block writes a stretch of one map without a scan, and a
 // large map is spread over as many blocks as the samples leave room for (a predicate and an ordered compaction by one block a
@@ -71,13 +71,13 @@ struct RandomShared {
     uint32_t listed[kMaxListed];           // this block's words of the chosen bin
     uint32_t all_listed[kMaxListed];       // a cluster's: those of all its blocks
     uint32_t n_listed;
-    uint32_t warp_sums[kSampWarps];
+    uint32_t warp_sums[32];
     uint32_t bin, below, in_bin;           // the chosen bin, words in lower bins, words in it
     uint32_t threshold, less, equal;       // the K-th smallest word; listed words below it, equal to it
     uint32_t slice_counts[2];              // positions of this slice below / equal to the threshold
 };
 
-// C blocks a sample.  kThreads: 128 for small maps (fewer warps to bring to each barrier), 512 otherwise.  cache_groups: how
+// C blocks a sample.  kThreads: 128 for small maps (fewer warps to bring to each barrier), 512 otherwise, 1024 for a few large ones.  cache_groups: how
 // many groups of four words the dynamic shared memory holds (0: every look at a word computes it again).
 template <int C, int kThreads>
 __global__ void __launch_bounds__(kThreads)
@@ -485,6 +485,9 @@ cudaError_t launch_sample_keep(int mode, int grid_family, int64_t B, int64_t H, 
         const int64_t N = H * W;
         // large maps with few samples: spread each sample over a cluster so that more SMs take part
         if (K < N && N > 8192 && B * 8 <= 4 * kNumSMs) {
+            // 1024 threads for up to three samples, whose clusters find room beside the kernel before: 2 x 66800 positions 4.2 ->
+            // 3.7 us back to back, 3 x 4.3 -> 3.8, but 4 x 4.5 -> 5.4 and 8 x 5.5 -> 10.4
+            if (N > 32768 && B <= 3) return launch_random_sampler<8, 1024>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
             if (N > 32768) return launch_random_sampler<8, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
             if (N > 16384) return launch_random_sampler<4, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
             return launch_random_sampler<2, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);

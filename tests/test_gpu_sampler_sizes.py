@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,H,W,r", [
     (3, 1, 1, 0.5), (2, 1, 3, 0.34), (2, 1, 5, 1.0), (300, 1, 196, 0.25), (2, 1, 511, 0.5), (2, 1, 512, 0.999), (2, 1, 513, 0.001),
     (3, 1, 2047, 0.5), (3, 1, 2049, 0.5), (2, 1, 8192, 0.5), (2, 1, 8193, 0.5), (5, 1, 16385, 0.1), (3, 1, 32769, 0.9), (1, 1, 32773, 1e-5),
-    (2, 200, 334, 0.5), (80, 1, 8197, 0.5), (76, 1, 41003, 0.3), (1, 3, 100001, 0.5), (1, 1000, 1000, 0.25),
+    (2, 200, 334, 0.5), (4, 1, 32771, 0.5), (3, 1, 70001, 0.999), (80, 1, 8197, 0.5), (76, 1, 41003, 0.3), (1, 3, 100001, 0.5), (1, 1000, 1000, 0.25),
 ])
 def test_random_masks_at_every_dispatch(B, H, W, r):
     for share in (0, 1):
