@@ -305,6 +305,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         const int32_t *q_glob = sh.q_glob[buf], *k_glob = sh.k_glob[buf];
         if (nq <= 0 || nk <= 0) {                            // nothing to compute: only the zeros of the unlisted rows
             zero_rows(prob, nq, nk, q_glob, k_glob);
+            __syncthreads();                                 // the problem before this one may still be storing by the other half's rows
             if (next < problems) begin_problem(cur, next, buf ^ 1);
             continue;
         }
@@ -589,7 +590,8 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                     store_rows<kThreads>((i & 1) ? p.dK : p.dV, p.ld_out, col0, gen + (uint32_t)i * kTileB, k_glob + first, nk - first < 128 ? nk - first : 128);
             }
         }
-        // (the barrier at the next problem's start keeps its writers off stages still being stored)
+        // No barrier behind the last stores: the one in front of the next problem's products keeps its writers off the stages, and
+        // whoever writes this problem's half of q_glob / k_glob next does so behind a barrier of the next problem (of an empty one too).
         ptx::tc_fence_before_sync();
     }
     ptx::cp_async_wait_all();
