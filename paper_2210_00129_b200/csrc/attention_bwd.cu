@@ -303,8 +303,17 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         const int next = prob + (int)gridDim.x;
         cur = fetch_meta(p, next, (int)threadIdx.x);        // travels while this problem computes
         const int32_t *q_glob = sh.q_glob[buf], *k_glob = sh.k_glob[buf];
-        if (nq <= 0 || nk <= 0) {                            // nothing to compute: only the zeros of the unlisted rows
-            zero_rows(prob, nq, nk, q_glob, k_glob);
+        if (nq <= 0 || nk <= 0) {                            // nothing to compute: zeros for the unlisted rows, and for those of a side
+            zero_rows(prob, nq, nk, q_glob, k_glob);         // whose other side has no tokens (sums over nothing)
+            for (int r = (int)threadIdx.x >> 3; r < (nq > nk ? nq : nk); r += kThreads / 8) {
+                const int64_t at = (int64_t)((uint64_t)(uint32_t)(nk <= 0 ? q_glob : k_glob)[r] * p.ld_out * 8u) + col0 + (threadIdx.x & 7) * 8;
+                if (nk <= 0) {
+                    ptx::st_global_v4(p.dQ + at, 0u, 0u, 0u, 0u);
+                } else {
+                    ptx::st_global_v4(p.dK + at, 0u, 0u, 0u, 0u);
+                    ptx::st_global_v4(p.dV + at, 0u, 0u, 0u, 0u);
+                }
+            }
             __syncthreads();                                 // the problem before this one may still be storing by the other half's rows
             if (next < problems) begin_problem(cur, next, buf ^ 1);
             continue;

@@ -61,3 +61,39 @@ def test_empty_samples_between_others(B, N, heads, q_most, k_most, resident, emp
             assert np.linalg.norm(got - w) <= 5e-3 * np.linalg.norm(w) + 1e-12, name
             row_rms = np.sqrt(np.mean(w.reshape(len(rows), heads, D) ** 2, axis=2)).repeat(D, axis=1)
             assert (np.abs(got - w) <= 2.0 ** -8 * np.abs(w) + 3e-2 * row_rms + 1e-3 * np.sqrt(np.mean(w ** 2))).all(), name
+
+
+@pytest.mark.parametrize("kept_only", [False, True])
+@pytest.mark.parametrize("B,N,heads,q_most,k_most,all_keys,empty_side", [
+    (5, 40, 2, 33, 20, False, "q"), (5, 40, 2, 33, 20, False, "k"), (400, 20, 1, 9, 16, False, "q"), (400, 20, 1, 9, 16, False, "k"),
+    (4, 200, 2, 20, 190, False, "q"), (4, 200, 1, 190, 20, False, "k"), (3, 60, 2, 30, 60, True, "q"), (3, 150, 1, 30, 150, True, "q"),
+])
+def test_samples_with_one_side_empty(B, N, heads, q_most, k_most, all_keys, empty_side, kept_only):
+    """Queries without keys, keys without queries: the gradients of the listed tokens are sums over nothing, +0.0."""
+    rng = np.random.default_rng(B + N)
+    M, C = B * N, heads * D
+    Q, K, V, dA = (synth.gaussian_tensor((M, C), "bf16", 800 + N, i, 1.0 if i < 3 else 1e-2) for i in range(4))
+    odd = lambda b: b % 2 == 1
+    never = lambda b: False
+    qr, qo = _lists(rng, B, N, q_most, odd if empty_side == "q" else never)
+    kr, ko = _lists(rng, B, N, k_most, odd if empty_side == "k" else never)
+    if all_keys:
+        kr, ko = np.arange(M, dtype=np.int32), np.arange(0, M + 1, N, dtype=np.int32)
+    t = lambda a: torch.from_numpy(a).cuda()
+    out = [torch.full((M, C), -7.0, dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+    flags = (sbp.SBP_FLAG_ATTN_KEPT_ROWS_ONLY if kept_only else 0) | (sbp.SBP_FLAG_ATTN_ALL_KEYS if all_keys else 0)
+    k_args = (None, None) if all_keys else (t(kr), t(ko))
+    sbp.sbp_attention_backward(sbp.SBP_BF16, *(dev(a, "bf16") for a in (Q, K, V)), C, dev(dA, "bf16"), C, t(qr), t(qo), *k_args, B, N,
+                               heads, D, max(q_most, 0 if all_keys else k_most), *out, C, flags)
+    torch.cuda.synchronize()
+    listed_q, listed_k = np.zeros(M, dtype=bool), np.zeros(M, dtype=bool)
+    listed_q[qr], listed_k[kr] = True, True
+    one_sided = (np.arange(M) // N) % 2 == 1
+    for name, g, listed in zip(("dQ", "dK", "dV"), out, (listed_q, listed_k, listed_k)):
+        bits = host(g)
+        assert not bits[listed & one_sided].any(), name
+        assert bits[listed & ~one_sided].any(), name
+        if kept_only:
+            assert (synth.bf16_bits_to_f64(bits[~listed]) == -7.0).all(), name
+        else:
+            assert not bits[~listed].any(), name
