@@ -239,6 +239,7 @@ __device__ __forceinline__ void product(ProductShared<BN>& sh, const ThreadTile<
             for (int k = 0; k < kBK; ++k) part[k & 3] += kSum == 1 ? sh.t.a[buf][k][threadIdx.x % kBM] : sh.t.b[buf][k][threadIdx.x % BN];
             const float y = ((part[0] + part[1]) + (part[2] + part[3])) - lost, t = colsum + y;     // Kahan's sum: one chain
             lost = (t - colsum) - y;                                                                // of up to thousands of stages
+            if (!(fabsf(lost) < INFINITY)) lost = 0.f;       // an infinite sum has lost nothing (infinity - infinity would make it a NaN)
             colsum = t;
         }
 #pragma unroll
