@@ -270,7 +270,7 @@ sbp_status sbp_act_backward(sbp_dtype dt, sbp_activation act, const void* Z_keep
  *   sbp_patch_scatter   dX[b, stride*ho + dh, stride*wo + dw, c] = dX_patches[m, (dh, dw, c)] for kept m; every
  *                       other input position (dropped patches, positions no patch covers) = +0.0.  Every element
  *                       of dX is written exactly once.  workspace: sbp_patch_scatter_workspace_bytes(...) bytes,
- *                       256-byte aligned (one int32 per output position; checked, and at present not used).
+ *                       256-byte aligned (one int32 per output position).  Both patch calls take keep_rows in any order.
  * C * sizeof(element) must be a multiple of 16 (else SBP_ERR_UNSUPPORTED); stride < k, k larger than the map and
  * other bad sizes or pointers give SBP_ERR_INVALID_ARG; a short workspace SBP_ERR_WORKSPACE.  M_keep is
  * *M_keep_dev when given, else M_keep_cap.  Bit-exact copies; deterministic.

@@ -9,7 +9,6 @@
 //                  outside the kept patches (dropped positions, positions no patch covers when s > k) gets +0.0
 // Both move 16-byte vectors and are HBM-bound.
 #include "row_copy.cuh"
-#include "zero_rows.cuh"
 
 namespace sbp {
 namespace {
@@ -64,16 +63,26 @@ patch_gather_kernel(const uint4* __restrict__ X, const PatchGeom g, const int32_
     pdl_launch_dependents();
 }
 
-// A block writes the input positions of `cells_per_block` consecutive cells.  Which packed row covers a cell comes from the
-// block's stretch of the ascending keep_rows list, found by search: one launch, where a map from output positions to packed
-// rows in global memory took a memset, a launch to fill it and a look-up for every vector.  [64, 56, 56, 128] bf16 from 25088
-// packed rows: memset + 3.3 + 26.3 us -> 18.2 us (77 MB; a third of it the search's dependent loads, which eight blocks an
-// SM overlap only in part).
+// slot[pos] = the packed row of output position pos.  Positions that are not kept keep whatever the workspace held: the reader asks
+// keep_rows back, so that nothing has to be cleared first, and the list may be in any order.
+__global__ void patch_slots_kernel(const int32_t* __restrict__ keep_rows, const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap,
+                                   int64_t outputs, int32_t* __restrict__ slot, const int32_t* status_word) {
+    pdl_launch_dependents();
+    pdl_wait();
+    if (status_word != nullptr && *reinterpret_cast<const volatile int32_t*>(status_word) != 0) return;
+    const int64_t M_keep = load_m_keep(M_keep_dev, M_keep_cap), m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= M_keep) return;
+    const int64_t pos = __ldg(keep_rows + m);
+    if (pos >= 0 && pos < outputs) slot[pos] = (int32_t)m;
+}
+
+// A block writes the input positions of `cells_per_block` consecutive cells, 1024 vectors at a time.  [64, 56, 56, 128] bf16 from
+// 25088 packed rows, with the launch that fills the slots: SCATTER_FIGURES.
 constexpr int kMaxCells = 128;
 __global__ void __launch_bounds__(kCopyThreads)
 patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int32_t* __restrict__ keep_rows,
-                     const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, int64_t cells, uint4* __restrict__ dX,
-                     const int32_t* status_word) {
+                     const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, const int32_t* __restrict__ slot, int64_t cells,
+                     uint4* __restrict__ dX, const int32_t* status_word) {
     __shared__ int32_t row_of[kMaxCells];          // packed row of each cell, -1: none
     __shared__ int32_t pixel_of[kMaxCells];        // first input position of each cell
     __shared__ int2 room[kMaxCells];               // rows of the cell inside the map, vectors of such a row
@@ -83,35 +92,20 @@ patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int
     const int64_t M_keep = load_m_keep(M_keep_dev, M_keep_cap);
     const int64_t c0 = (int64_t)blockIdx.x * g.cells_per_block;
     const int n = cells - c0 < g.cells_per_block ? (int)(cells - c0) : g.cells_per_block;
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x < kMaxCells) row_of[threadIdx.x] = -1;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        // output positions in front of cell c, and the cell of an output position, by the two grids' sizes
-        const auto positions_before = [&](int64_t c) {
-            const int64_t b = c / ((int64_t)g.Hc * g.Wc);
-            const int rem = (int)(c - b * ((int64_t)g.Hc * g.Wc)), hc = rem / g.Wc, wc = rem - hc * g.Wc;
-            const int64_t in_map = hc < g.Ho ? (int64_t)hc * g.Wo + (wc < g.Wo ? wc : g.Wo) : (int64_t)g.Ho * g.Wo;
-            return b * g.Ho * g.Wo + in_map;
-        };
-        const int64_t begin = positions_before(c0), end = positions_before(c0 + n);
-        for (int64_t m = warp_lower_bound(keep_rows, M_keep, begin, lane) + lane;; m += 32) {
-            const int64_t pos = m < M_keep ? (int64_t)__ldg(keep_rows + m) : end;
-            if (pos >= begin && pos < end) {
-                const uint32_t b = g.map((uint32_t)pos), rem = (uint32_t)pos - b * g.map.d;
-                const uint32_t ho = g.line(rem), wo = rem - ho * g.line.d;
-                row_of[((int64_t)b * g.Hc + ho) * g.Wc + wo - c0] = (int32_t)m;
-            }
-            if (__any_sync(0xffffffffu, pos >= end)) break;
+    if ((int)threadIdx.x < n) {
+        const int i = threadIdx.x;
+        const int64_t c = c0 + i, bh = c / g.Wc, b = bh / g.Hc;
+        const int wc = (int)(c - bh * g.Wc), hc = (int)(bh - b * g.Hc);
+        int32_t m = -1;
+        if (hc < g.Ho && wc < g.Wo) {
+            const int32_t pos = (int32_t)((b * g.Ho + hc) * g.Wo + wc);
+            m = __ldg(slot + pos);
+            if (m < 0 || m >= M_keep || __ldg(keep_rows + m) != pos) m = -1;
         }
-    } else if (threadIdx.x >= 128) {
-        for (int i = threadIdx.x - 128; i < n; i += kCopyThreads - 128) {
-            const int64_t c = c0 + i, bh = c / g.Wc, b = bh / g.Hc;
-            const int wc = (int)(c - bh * g.Wc), hc = (int)(bh - b * g.Hc);
-            pixel_of[i] = (int32_t)((b * g.H + (int64_t)hc * g.s) * g.W + (int64_t)wc * g.s);
-            const int rows = g.H - hc * g.s < g.s ? g.H - hc * g.s : g.s, cols = g.W - wc * g.s < g.s ? g.W - wc * g.s : g.s;
-            room[i] = make_int2(rows, cols * (int)g.vec_c);
-        }
+        row_of[i] = m;
+        pixel_of[i] = (int32_t)((b * g.H + (int64_t)hc * g.s) * g.W + (int64_t)wc * g.s);
+        const int rows = g.H - hc * g.s < g.s ? g.H - hc * g.s : g.s, cols = g.W - wc * g.s < g.s ? g.W - wc * g.s : g.s;
+        room[i] = make_int2(rows, cols * (int)g.vec_c);
     }
     __syncthreads();
     const uint32_t all = (uint32_t)n * g.cell.d, slice0 = blockIdx.y * g.slice;
@@ -167,13 +161,18 @@ cudaError_t launch_patch_gather(const void* X, int64_t H, int64_t W, int64_t pos
 
 cudaError_t launch_patch_scatter(const void* dXp, int64_t B, int64_t H, int64_t W, int64_t pos_bytes, int64_t k, int64_t s,
                                  const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M_keep_cap, void* dX,
-                                 const int32_t* status_word, cudaStream_t stream) {
+                                 int32_t* slot, const int32_t* status_word, cudaStream_t stream) {
     PatchGeom g = geom(H, W, k, s, pos_bytes);
+    if (M_keep_cap > 0) {
+        const cudaError_t e = launch_pdl(patch_slots_kernel, dim3((unsigned)((M_keep_cap + 255) / 256)), dim3(256), 0, stream, keep_rows,
+                                         M_keep_dev, M_keep_cap, B * g.Ho * g.Wo, slot, status_word);
+        if (e != cudaSuccess) return e;
+    }
     const int64_t cells = B * g.Hc * g.Wc;
     const uint32_t cell_w = (uint32_t)(s < W ? s : W), cell_h = (uint32_t)(s < H ? s : H);
     g.cell_line = FastDiv(cell_w * g.vec_c);
     g.cell = FastDiv(cell_h * g.cell_line.d);
-    // About 2048 vectors (32 KB) a block: eight blocks of an SM then hide each other's search, and small maps still spread.
+    // About 2048 vectors (32 KB) a block: eight blocks of an SM then hide each other's look-ups, and small maps still spread.
     constexpr uint32_t kTarget = 2048;
     const uint32_t n = kTarget / g.cell.d;
     g.cells_per_block = (int)(n < 1 ? 1 : n > (uint32_t)kMaxCells ? (uint32_t)kMaxCells : n);
@@ -184,7 +183,7 @@ cudaError_t launch_patch_scatter(const void* dXp, int64_t B, int64_t H, int64_t 
     slices = (per_block + g.slice - 1) / g.slice;
     const dim3 grid((unsigned)((cells + g.cells_per_block - 1) / g.cells_per_block), slices);
     return launch_pdl(patch_scatter_kernel, grid, dim3(kCopyThreads), 0, stream, (const uint4*)dXp, g, keep_rows, M_keep_dev, M_keep_cap,
-                      cells, (uint4*)dX, status_word);
+                      (const int32_t*)slot, cells, (uint4*)dX, status_word);
 }
 
 }  // namespace sbp

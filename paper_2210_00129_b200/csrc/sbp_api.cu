@@ -400,7 +400,7 @@ sbp_status sbp_patch_scatter(sbp_dtype dt, const void* dX_patches, int64_t B, in
         workspace_bytes < sbp_patch_scatter_workspace_bytes(B, H, W, k, stride))
         return SBP_ERR_WORKSPACE;
     const cudaError_t e = launch_patch_scatter(dX_patches, B, H, W, C * (dt == SBP_BF16 ? 2 : 4), k, stride, keep_rows, M_keep_dev,
-                                               M_keep_cap, dX, status_word, (cudaStream_t)stream);
+                                               M_keep_cap, dX, static_cast<int32_t*>(workspace), status_word, (cudaStream_t)stream);
     return e == cudaSuccess ? SBP_OK : SBP_ERR_CUDA;
 }
 

@@ -196,7 +196,7 @@ cudaError_t launch_patch_gather(const void* X, int64_t H, int64_t W, int64_t pos
                                 cudaStream_t stream);
 cudaError_t launch_patch_scatter(const void* dXp, int64_t B, int64_t H, int64_t W, int64_t pos_bytes, int64_t k, int64_t s,
                                  const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M_keep_cap, void* dX,
-                                 const int32_t* status_word, cudaStream_t stream);
+                                 int32_t* slot, const int32_t* status_word, cudaStream_t stream);     // slot: an int32 per output position
 
 // SBP attention backward on token subsets (bf16, head dimension 64, at most attention_max_tokens() kept tokens per sample
 // and side); null row lists mean every token of the sample; q_most / k_most = most tokens a sample brings to either side

@@ -65,3 +65,27 @@ def test_patch_cache_and_scatter(B, H, W, C, k, s, ratio):
             want[b, ho * s + dh, wo * s + dw] = dXp[:keep].view(keep, k, k, C)[:, dh, dw]
     assert torch.equal(dX, want)
     assert not (dX.view(torch.int32) == -2147483648).any()                                         # the zeros are +0.0
+
+
+@pytest.mark.parametrize("order", ["reversed", "shuffled"])
+def test_patch_calls_take_rows_in_any_order(order):
+    B, H, W, C, k, s = 3, 40, 36, 16, 2, 2
+    Mo, Kc, keep = B * (H // k) * (W // k), k * k * C, 500
+    gen = torch.Generator().manual_seed(3)
+    rows = torch.randperm(Mo, generator=gen)[:keep].int()
+    rows = (rows.sort(descending=True).values if order == "reversed" else rows).cuda()
+    X = torch.randn(B, H, W, C, device="cuda")
+    Xk = torch.empty(keep, Kc, device="cuda")
+    sbp.sbp_patch_cache(sbp.SBP_F32, X, B, H, W, C, k, s, rows, None, keep, Xk)
+    nbytes = sbp.sbp_patch_scatter_workspace_bytes(B, H, W, k, s)
+    dX = torch.full((B, H, W, C), float("nan"), device="cuda")
+    # whatever the workspace holds: zeros, ones, valid row numbers of other positions
+    for fill in (torch.zeros(nbytes // 4, dtype=torch.int32), torch.full((nbytes // 4,), -1, dtype=torch.int32),
+                 torch.arange(nbytes // 4, dtype=torch.int32) % keep):
+        ws = fill.cuda()
+        sbp.sbp_patch_scatter(sbp.SBP_F32, Xk, B, H, W, C, k, s, rows, None, keep, dX, ws, nbytes)
+        torch.cuda.synchronize()
+        kept = torch.zeros(Mo, dtype=torch.bool, device="cuda")
+        kept[rows.long()] = True
+        mask = kept.view(B, H // k, 1, W // k, 1, 1).expand(B, H // k, k, W // k, k, 1).reshape(B, H, W, 1)
+        assert torch.equal(dX, torch.where(mask, X, torch.zeros_like(X)))
