@@ -4,9 +4,9 @@ The compute lives in a C-ABI CUDA library (``include/sbp.h``, built in-tree as
 ``libsbp_b200.so``); this module is its thin Python binding: the functions below carry the
 same names as the C entry points and only marshal arguments (torch tensors -> device
 pointers, the current torch stream -> ``cudaStream_t``).  The calls a training step makes go
-through a small CPython module (``csrc/python_calls.cpp``), the queries and diagnostics through
-ctypes.  Every step of the path runs in the library's kernels; there is no fallback - a missing
-library raises at the first call.
+through a small CPython module (``csrc/python_calls.cpp``), or through ctypes where that module was
+not built for this interpreter, the queries and diagnostics through ctypes.  Every step of the path
+runs in the library's kernels; there is no fallback - a missing library raises at the first call.
 
 ``synth`` (seeded input generators) is importable without the library.
 """
@@ -38,7 +38,7 @@ EXPORTS = ("sbp_status_string", "sbp_keep_count", "sbp_sample_keep", "sbp_forwar
            "sbp_selftest_bounded_wait", "sbp_probe_gather_ring", "sbp_probe_mma_rate", "sbp_probe_mma_pair_rate", "sbp_probe_operand_feed")
 
 _lib = None
-_call = None          # the CPython module of the step's calls
+_call = None          # the step's calls
 
 
 class SbpError(RuntimeError):
@@ -108,17 +108,35 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+class _CtypesCalls:
+    """The calls of a training step through ctypes, for interpreters the CPython module was not built for."""
+
+    def __init__(self, lib):
+        self._lib = lib
+
+    def __getattr__(self, name):
+        f = getattr(self._lib, name)
+        as_c = [_ptr if t is ctypes.c_void_p else float if t is ctypes.c_double else None for t in f.argtypes]
+
+        def call(*args):
+            return f(*(c(a) if c is not None else a for c, a in zip(as_c, args, strict=True)))
+
+        setattr(self, name, call)
+        return call
+
+
 def _calls():
-    """The CPython module with the calls of a training step."""
+    """The calls of a training step."""
     global _call
     if _call is None or _lib is None:
-        load_library()
-        if not os.path.exists(CALLS_PATH):
-            raise RuntimeError(f"{CALLS_PATH} is missing: run `python -m paper_2210_00129_b200.build` with this interpreter")
-        spec = importlib.util.spec_from_file_location(__name__ + "._calls", CALLS_PATH)
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
-        _call = module
+        lib = load_library()
+        if os.path.exists(CALLS_PATH):
+            spec = importlib.util.spec_from_file_location(__name__ + "._calls", CALLS_PATH)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+            _call = module
+        else:
+            _call = _CtypesCalls(lib)
     return _call
 
 

@@ -1,7 +1,8 @@
 """Build the CUDA library in-tree: ``python -m paper_2210_00129_b200.build``.
 
 Compiles every ``csrc/*.cu`` for sm_100a with nvcc into ``libsbp_b200.so`` next to this file, and
-``csrc/python_calls.cpp`` into the CPython module of the calls.  Cross-compiles without a GPU.
+``csrc/python_calls.cpp`` into the CPython module of the calls where Python's headers are installed
+(the binding goes through ctypes otherwise).  Cross-compiles without a GPU.
 """
 from __future__ import annotations
 
@@ -26,23 +27,26 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB_PATH) or not os.path.exists(CALLS_PATH):
-        return True
-    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(CALLS_PATH))
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + \
-        [CALLS_SRC, os.path.join(os.path.dirname(_HERE), "include", "sbp.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+def _has_python_headers() -> bool:
+    return os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h"))
+
+
+def _stale(out: str, deps) -> bool:
+    return not os.path.exists(out) or any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
-        return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    lib = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB_PATH] + sources()
-    calls = [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-I", sysconfig.get_paths()["include"],
-             "-o", CALLS_PATH, CALLS_SRC, "-L", _HERE, "-Xlinker", "-l:" + os.path.basename(LIB_PATH), "-Xlinker", "-rpath,$ORIGIN"]
-    for cmd, out in ((lib, LIB_PATH), (calls, CALLS_PATH)):
+    header = os.path.join(os.path.dirname(_HERE), "include", "sbp.h")
+    jobs = [(LIB_PATH, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + [header],
+             [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB_PATH] + sources())]
+    if _has_python_headers():
+        jobs.append((CALLS_PATH, [CALLS_SRC, header],
+                     [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-I", sysconfig.get_paths()["include"],
+                      "-o", CALLS_PATH, CALLS_SRC, "-L", _HERE, "-Xlinker", "-l:" + os.path.basename(LIB_PATH), "-Xlinker", "-rpath,$ORIGIN"]))
+    for out, deps, cmd in jobs:
+        if not force and not _stale(out, deps):
+            continue
         res = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or res.returncode != 0:
             sys.stderr.write(res.stdout + res.stderr)

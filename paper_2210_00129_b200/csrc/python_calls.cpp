@@ -1,5 +1,6 @@
-// Python side of the C ABI: each entry point as a function of positional arguments.  Integers and floats convert by value;
-// a pointer is None, an address, or an object with data_ptr() (a torch tensor).  The GIL is released during the call.
+// Python side of the C ABI: each entry point as a function of positional arguments.  They convert as through ctypes: a whole number is
+// an int or an object with __index__ (anything else is ctypes.ArgumentError), a float is what float() takes; a pointer is None, an
+// address, or an object with data_ptr() (a torch tensor).  The GIL is released during the call.
 //
 // Why not ctypes: a step of the smallest layer is three calls whose kernels take 12 us together, and the host needed 30 us to
 // issue them - 2 us and more a call to convert 9 to 22 arguments and 3 us for torch.cuda.current_stream().  With this module
@@ -18,10 +19,13 @@
 namespace {
 
 PyObject* g_data_ptr = nullptr;            // the interned name "data_ptr"
+PyObject* g_argument_error = nullptr;      // ctypes.ArgumentError
 
 bool to_integer(PyObject* o, unsigned long long& v) {
     v = PyLong_AsUnsignedLongLongMask(o);
-    return v != (unsigned long long)-1 || !PyErr_Occurred();
+    if (v != (unsigned long long)-1 || !PyErr_Occurred()) return true;
+    PyErr_Format(g_argument_error, "'%s' object cannot be interpreted as an integer", Py_TYPE(o)->tp_name);
+    return false;
 }
 
 bool to_address(PyObject* o, unsigned long long& v) {
@@ -37,11 +41,21 @@ bool to_address(PyObject* o, unsigned long long& v) {
     return ok;
 }
 
+bool to_float(PyObject* o, double& v) {
+    PyObject* f = PyNumber_Float(o);
+    if (f == nullptr) return false;
+    v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
+    return true;
+}
+
 template <typename T>
 bool convert(PyObject* o, T& out) {
     if constexpr (std::is_floating_point_v<T>) {
-        out = PyFloat_AsDouble(o);
-        return out != -1.0 || !PyErr_Occurred();
+        double v = 0.0;
+        if (!to_float(o, v)) return false;
+        out = v;
+        return true;
     } else {
         unsigned long long v = 0;
         if constexpr (std::is_pointer_v<T>) {
@@ -99,5 +113,9 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, g_methods,
 
 PyMODINIT_FUNC PyInit__calls(void) {
     g_data_ptr = PyUnicode_InternFromString("data_ptr");
-    return g_data_ptr == nullptr ? nullptr : PyModule_Create(&g_module);
+    PyObject* ctypes = PyImport_ImportModule("ctypes");
+    if (g_data_ptr == nullptr || ctypes == nullptr) return nullptr;
+    g_argument_error = PyObject_GetAttrString(ctypes, "ArgumentError");
+    Py_DECREF(ctypes);
+    return g_argument_error == nullptr ? nullptr : PyModule_Create(&g_module);
 }
