@@ -11,20 +11,20 @@ namespace {
 // A block writes 1024 consecutive vectors (16 KB); without a 64-bit division for each of them 12544 rows of 768 bf16 take
 // 7.7 us instead of 9.1 us (5.0 TB/s with launch and drain inside), 100352 rows of 512 28 us instead of 32 us (7.4 TB/s).
 __global__ void __launch_bounds__(kCopyThreads)
-gather_rows_kernel(const uint4* __restrict__ X, const FastDiv row, const int32_t* __restrict__ keep_rows,
+gather_rows_kernel(const uint4* __restrict__ X, const RowLength row, const int32_t* __restrict__ keep_rows,
                    const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, uint4* __restrict__ X_keep) {
     pdl_wait();
     const int64_t M_keep = load_m_keep(M_keep_dev, M_keep_cap);
-    const int64_t begin = (int64_t)blockIdx.x * kCopySpan, total = M_keep_cap * (int64_t)row.d;
-    const SpanRows span(begin, row.d);
+    const int64_t begin = (int64_t)blockIdx.x * kCopySpan, total = M_keep_cap * row.n;
+    const SpanRows span(begin, row);
     uint4 v[kCopyUnroll];
     int64_t src[kCopyUnroll];
 #pragma unroll
     for (int u = 0; u < kCopyUnroll; ++u) {
         uint32_t q;
-        const uint32_t c = span.place(threadIdx.x + u * kCopyThreads, row, &q);
+        const int64_t c = span.place(threadIdx.x + u * kCopyThreads, row, &q);
         const int64_t m = span.first + q;
-        src[u] = m < M_keep ? (int64_t)__ldg(keep_rows + m) * row.d + c : -1;
+        src[u] = m < M_keep ? (int64_t)__ldg(keep_rows + m) * row.n + c : -1;
     }
 #pragma unroll
     for (int u = 0; u < kCopyUnroll; ++u) v[u] = (src[u] >= 0) ? ld_stream(X + src[u]) : make_uint4(0u, 0u, 0u, 0u);
@@ -65,7 +65,7 @@ cudaError_t launch_gather_rows(const void* X, int64_t row_bytes, const int32_t* 
     const int64_t total = M_keep_cap * vec_per_row;
     if (total == 0) return cudaSuccess;
     return launch_pdl(gather_rows_kernel, dim3((unsigned)copy_blocks(total)), dim3(kCopyThreads), 0, stream, (const uint4*)X,
-                      FastDiv((uint32_t)vec_per_row), keep_rows, M_keep_dev, M_keep_cap, (uint4*)X_keep);
+                      RowLength(vec_per_row), keep_rows, M_keep_dev, M_keep_cap, (uint4*)X_keep);
 }
 
 cudaError_t launch_validate_keep_rows(const int32_t* keep_rows, const int32_t* M_keep_dev,

@@ -15,14 +15,15 @@ namespace {
 
 struct PatchGeom {
     int H, W, Ho, Wo, k, s;
-    int Hc, Wc;                     // cells of s x s input positions (cut short at the map's edges): output position
-                                    // (ho, wo) owns cell (ho, wo), cells past the output grid belong to none
-    uint32_t vec_c;                 // 16-byte vectors per input position (C * element size / 16)
-    FastDiv row;                    // vectors of a patch row (k * k positions)
-    FastDiv seg;                    // ... of one of its k pieces
+    int64_t vec_c;                  // 16-byte vectors per input position (C * element size / 16), below 2^22
+    RowLength piece;                // vectors of one of the k pieces of a patch row
+    FastDiv pieces;                 // k
     FastDiv map, line;              // output positions of a sample, of a row of the output map
+    // Scatter: the input map in cells of side x side positions (cut short at the map's edges).  side = s: output position
+    // (ho, wo) owns cell (ho, wo), cells past the output grid belong to none.  side = 1: every position by itself.
+    int side, Hc, Wc;
     FastDiv cell;                   // vectors of a whole cell
-    FastDiv cell_line;              // ... of one of its s rows
+    FastDiv cell_line;              // ... of one of its rows
     int cells_per_block;
     uint32_t slice;                 // vectors of its cells that a block writes (large cells: several blocks per cell)
 };
@@ -34,18 +35,17 @@ patch_gather_kernel(const uint4* __restrict__ X, const PatchGeom g, const int32_
                     const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, uint4* __restrict__ X_keep) {
     pdl_wait();
     const int64_t M_keep = load_m_keep(M_keep_dev, M_keep_cap);
-    const int64_t begin = (int64_t)blockIdx.x * kCopySpan, total = M_keep_cap * (int64_t)g.row.d;
-    const SpanRows span(begin, g.row.d);
+    const int64_t begin = (int64_t)blockIdx.x * kCopySpan, total = M_keep_cap * g.k * g.piece.n;
+    const SpanRows span(begin, g.piece);
     int64_t src[kCopyUnroll];
     uint4 v[kCopyUnroll];
 #pragma unroll
     for (int u = 0; u < kCopyUnroll; ++u) {
         uint32_t q;
-        const uint32_t in_row = span.place(threadIdx.x + u * kCopyThreads, g.row, &q);
-        const int64_t m = span.first + q;
+        const int64_t off = span.place(threadIdx.x + u * kCopyThreads, g.piece, &q);
+        const uint32_t i = (uint32_t)span.first + q, m = g.pieces(i), dh = i - m * g.pieces.d;
         src[u] = -1;                                                   // rows past M_keep are cleared
         if (m < M_keep) {
-            const uint32_t dh = g.seg(in_row), off = in_row - dh * g.seg.d;
             const uint32_t pos = (uint32_t)__ldg(keep_rows + m);
             const uint32_t b = g.map(pos), rem = pos - b * g.map.d;
             const uint32_t ho = g.line(rem), wo = rem - ho * g.line.d;
@@ -77,13 +77,14 @@ __global__ void patch_slots_kernel(const int32_t* __restrict__ keep_rows, const 
 }
 
 // A block writes the input positions of `cells_per_block` consecutive cells, 1024 vectors at a time.  [64, 56, 56, 128] bf16 from
-// 25088 packed rows, with the launch that fills the slots: SCATTER_FIGURES.
+// 25088 packed rows, with the launch that fills the slots: 18.2 us (77 MB; with the list searched by every block instead, which
+// needs it ascending: the same).
 constexpr int kMaxCells = 128;
 __global__ void __launch_bounds__(kCopyThreads)
 patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int32_t* __restrict__ keep_rows,
                      const int32_t* __restrict__ M_keep_dev, int64_t M_keep_cap, const int32_t* __restrict__ slot, int64_t cells,
                      uint4* __restrict__ dX, const int32_t* status_word) {
-    __shared__ int32_t row_of[kMaxCells];          // packed row of each cell, -1: none
+    __shared__ int64_t from_of[kMaxCells];         // first vector of each cell's packed patch, -1: none
     __shared__ int32_t pixel_of[kMaxCells];        // first input position of each cell
     __shared__ int2 room[kMaxCells];               // rows of the cell inside the map, vectors of such a row
     pdl_launch_dependents();
@@ -96,15 +97,16 @@ patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int
         const int i = threadIdx.x;
         const int64_t c = c0 + i, bh = c / g.Wc, b = bh / g.Hc;
         const int wc = (int)(c - bh * g.Wc), hc = (int)(bh - b * g.Hc);
-        int32_t m = -1;
-        if (hc < g.Ho && wc < g.Wo) {
-            const int32_t pos = (int32_t)((b * g.Ho + hc) * g.Wo + wc);
-            m = __ldg(slot + pos);
-            if (m < 0 || m >= M_keep || __ldg(keep_rows + m) != pos) m = -1;
+        const int h0 = hc * g.side, w0 = wc * g.side;
+        const int ho = g.side == g.s ? hc : h0 / g.s, wo = g.side == g.s ? wc : w0 / g.s, dh0 = h0 - ho * g.s, dw0 = w0 - wo * g.s;
+        int64_t from = -1;
+        if (ho < g.Ho && wo < g.Wo && dh0 < g.k && dw0 < g.k) {
+            const int32_t pos = (int32_t)((b * g.Ho + ho) * g.Wo + wo), m = __ldg(slot + pos);
+            if (m >= 0 && m < M_keep && __ldg(keep_rows + m) == pos) from = ((int64_t)m * g.k + dh0) * g.piece.n + dw0 * g.vec_c;
         }
-        row_of[i] = m;
-        pixel_of[i] = (int32_t)((b * g.H + (int64_t)hc * g.s) * g.W + (int64_t)wc * g.s);
-        const int rows = g.H - hc * g.s < g.s ? g.H - hc * g.s : g.s, cols = g.W - wc * g.s < g.s ? g.W - wc * g.s : g.s;
+        from_of[i] = from;
+        pixel_of[i] = (int32_t)((b * g.H + h0) * g.W + w0);
+        const int rows = g.H - h0 < g.side ? g.H - h0 : g.side, cols = g.W - w0 < g.side ? g.W - w0 : g.side;
         room[i] = make_int2(rows, cols * (int)g.vec_c);
     }
     __syncthreads();
@@ -123,8 +125,8 @@ patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int
                 const uint32_t dh = g.cell_line(in_cell), off = in_cell - dh * g.cell_line.d;
                 if ((int)dh < room[c].x && (int)off < room[c].y) {
                     dst[u] = ((int64_t)pixel_of[c] + (int64_t)dh * g.W) * g.vec_c + off;
-                    const int32_t m = row_of[c];
-                    if (m >= 0 && (int)dh < g.k && off < g.seg.d) v[u] = ld_stream(dXp + (int64_t)m * g.row.d + dh * g.seg.d + off);
+                    const int64_t from = from_of[c];
+                    if (from >= 0 && (int)dh < g.k && off < g.piece.n) v[u] = ld_stream(dXp + from + dh * g.piece.n + off);
                 }
             }
         }
@@ -135,13 +137,14 @@ patch_scatter_kernel(const uint4* __restrict__ dXp, const PatchGeom g, const int
 }
 
 PatchGeom geom(int64_t H, int64_t W, int64_t k, int64_t s, int64_t pos_bytes) {
+    const int64_t most = H > W ? H : W;
+    if (s > most) s = most;                        // (one output row or column either way)
     PatchGeom g;
     g.H = (int)H; g.W = (int)W; g.k = (int)k; g.s = (int)s;
     g.Ho = (int)((H - k) / s + 1); g.Wo = (int)((W - k) / s + 1);
-    g.Hc = (int)((H + s - 1) / s); g.Wc = (int)((W + s - 1) / s);
-    g.vec_c = (uint32_t)(pos_bytes / 16);
-    g.seg = FastDiv((uint32_t)k * g.vec_c);
-    g.row = FastDiv((uint32_t)k * g.seg.d);
+    g.vec_c = pos_bytes / 16;
+    g.piece = RowLength(k * g.vec_c);
+    g.pieces = FastDiv((uint32_t)k);               // (pieces in all: at most the input positions / k, so they fit 31 bits)
     g.map = FastDiv((uint32_t)((int64_t)g.Ho * g.Wo));
     g.line = FastDiv((uint32_t)g.Wo);
     return g;
@@ -153,7 +156,7 @@ cudaError_t launch_patch_gather(const void* X, int64_t H, int64_t W, int64_t pos
                                 const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M_keep_cap, void* X_keep,
                                 cudaStream_t stream) {
     const PatchGeom g = geom(H, W, k, s, pos_bytes);
-    const int64_t total = M_keep_cap * (int64_t)g.row.d;
+    const int64_t total = M_keep_cap * k * g.piece.n;
     if (total == 0) return cudaSuccess;
     return launch_pdl(patch_gather_kernel, dim3((unsigned)copy_blocks(total)), dim3(kCopyThreads), 0, stream, (const uint4*)X, g,
                       keep_rows, M_keep_dev, M_keep_cap, (uint4*)X_keep);
@@ -168,10 +171,16 @@ cudaError_t launch_patch_scatter(const void* dXp, int64_t B, int64_t H, int64_t 
                                          M_keep_dev, M_keep_cap, B * g.Ho * g.Wo, slot, status_word);
         if (e != cudaSuccess) return e;
     }
+    // Cells of more than a gigabyte (strides far beyond the kernel) are taken apart into positions, so that vectors are counted in
+    // 32 bits everywhere.
+    const auto cell_side = [&](int64_t extent) { return g.s < extent ? (int64_t)g.s : extent; };
+    g.side = cell_side(H) * cell_side(W) * g.vec_c <= (1ll << 26) ? g.s : 1;
+    g.Hc = (int)((H + g.side - 1) / g.side);
+    g.Wc = (int)((W + g.side - 1) / g.side);
     const int64_t cells = B * g.Hc * g.Wc;
-    const uint32_t cell_w = (uint32_t)(s < W ? s : W), cell_h = (uint32_t)(s < H ? s : H);
-    g.cell_line = FastDiv(cell_w * g.vec_c);
-    g.cell = FastDiv(cell_h * g.cell_line.d);
+    const int64_t cell_w = g.side < W ? g.side : W, cell_h = g.side < H ? g.side : H;
+    g.cell_line = FastDiv((uint32_t)(cell_w * g.vec_c));
+    g.cell = FastDiv((uint32_t)(cell_h * cell_w * g.vec_c));
     // About 2048 vectors (32 KB) a block: eight blocks of an SM then hide each other's look-ups, and small maps still spread.
     constexpr uint32_t kTarget = 2048;
     const uint32_t n = kTarget / g.cell.d;

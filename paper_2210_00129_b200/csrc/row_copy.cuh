@@ -22,19 +22,31 @@ constexpr int kCopyThreads = 256;
 constexpr int kCopyUnroll = 4;             // vectors a thread has in flight
 constexpr uint32_t kCopySpan = kCopyThreads * kCopyUnroll;
 
-// Position of a span in rows of `row.d` vectors: vector `i` of the span (i < kCopySpan) lies in row first + (*q), at the
+// Length of a row in vectors: any length, but only rows shorter than a span are divided by.
+struct RowLength {
+    int64_t n;
+    FastDiv by;
+    RowLength() = default;
+    explicit RowLength(int64_t vectors) : n(vectors), by(vectors < kCopySpan ? (uint32_t)vectors : 1u) {}
+};
+
+// Position of a span in rows of `row.n` vectors: vector `i` of the span (i < kCopySpan) lies in row first + (*q), at the
 // returned place in it.
 struct SpanRows {
-    int64_t first;
-    uint32_t rem;
-    __device__ __forceinline__ SpanRows(int64_t span_begin, uint32_t vec_per_row) {
-        first = span_begin / vec_per_row;
-        rem = (uint32_t)(span_begin - first * vec_per_row);
+    int64_t first, rem;
+    __device__ __forceinline__ SpanRows(int64_t span_begin, const RowLength& row) {
+        first = span_begin / row.n;
+        rem = span_begin - first * row.n;
     }
-    __device__ __forceinline__ uint32_t place(uint32_t i, const FastDiv& row, uint32_t* q) const {
-        const uint32_t o = rem + i;
-        *q = row.d >= kCopySpan ? (o >= row.d ? 1u : 0u) : row(o);       // long rows: a span touches two at most
-        return o - *q * row.d;
+    __device__ __forceinline__ int64_t place(uint32_t i, const RowLength& row, uint32_t* q) const {
+        if (row.n >= kCopySpan) {                                        // long rows: a span touches two at most
+            const int64_t o = rem + i;
+            *q = o >= row.n ? 1u : 0u;
+            return o >= row.n ? o - row.n : o;
+        }
+        const uint32_t o = (uint32_t)rem + i;
+        *q = row.by(o);
+        return o - *q * row.by.d;
     }
 };
 

@@ -89,3 +89,25 @@ def test_patch_calls_take_rows_in_any_order(order):
         kept[rows.long()] = True
         mask = kept.view(B, H // k, 1, W // k, 1, 1).expand(B, H // k, k, W // k, k, 1).reshape(B, H, W, 1)
         assert torch.equal(dX, torch.where(mask, X, torch.zeros_like(X)))
+
+
+@pytest.mark.parametrize("H,W,C,k,s,keep", [(72, 72, 2 ** 17, 5, 72, 1), (72, 73, 2 ** 17, 2, 2 ** 31 + 5, 1), (16, 17, 2 ** 23 + 8, 3, 8, 3)])
+def test_patch_scatter_with_cells_beyond_a_gigabyte(H, W, C, k, s, keep):
+    """Strides far beyond the kernel: every position is a cell of its own (the largest map here takes 4.6 GB)."""
+    Ho, Wo = (H - k) // s + 1, (W - k) // s + 1
+    assert min(s, H) * min(s, W) * C // 8 > 2 ** 26
+    gen = torch.Generator().manual_seed(k)
+    rows = torch.randperm(Ho * Wo, generator=gen)[:keep].sort().values.int().cuda()
+    dXp = torch.randint(-1000, 1000, (keep, k, k, C), device="cuda", dtype=torch.int16).view(torch.bfloat16)
+    dX = torch.full((H, W, C), 3.0, dtype=torch.bfloat16, device="cuda")
+    nbytes = sbp.sbp_patch_scatter_workspace_bytes(1, H, W, k, s)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    sbp.sbp_patch_scatter(sbp.SBP_BF16, dXp, 1, H, W, C, k, s, rows, None, keep, dX, ws, nbytes)
+    torch.cuda.synchronize()
+    bits = dX.view(torch.int16)
+    for m, pos in enumerate(rows.tolist()):
+        h, w = pos // Wo * s, pos % Wo * s
+        patch = bits[h:h + k, w:w + k]
+        assert torch.equal(patch, dXp[m].view(torch.int16))
+        patch.zero_()
+    assert not any(bool(line.any()) for line in bits)              # a row of the map at a time
