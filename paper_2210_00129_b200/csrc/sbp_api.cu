@@ -228,7 +228,7 @@ sbp_status backward_direct(sbp_dtype dt, bool w_out_in, const void* X_keep, cons
     if ((flags & SBP_FLAG_VALIDATE) && status_word == nullptr) return SBP_ERR_INVALID_ARG;
     const int64_t mult = (dt == SBP_BF16) ? 8 : 4;
     if (C_in % mult != 0 || C_out % mult != 0) return SBP_ERR_UNSUPPORTED;
-    const bool need_ws = (dW != nullptr) || (db != nullptr);
+    const bool need_ws = dW != nullptr || db != nullptr || w_out_in;      // (w_out_in: at every weight size, whether copies are made or not)
     if (need_ws) {
         if (workspace == nullptr || (reinterpret_cast<uintptr_t>(workspace) & 255u) ||
             workspace_bytes < workspace_required)
