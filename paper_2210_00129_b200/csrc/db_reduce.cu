@@ -230,10 +230,10 @@ cudaError_t launch_reduce_partials(const float* partials, int splits, int64_t n,
 }
 
 cudaError_t launch_reduce_partials_pair(const float* partials_a, int splits_a, int64_t n_a, float* out_a,
-                                        const float* partials_b, int splits_b, int64_t n_b, float* out_b,
-                                        bool accumulate, const int32_t* status_word, cudaStream_t stream) {
-    const ReduceJob a = make_reduce_job(partials_a, splits_a, n_a, out_a, accumulate);
-    const ReduceJob b = make_reduce_job(partials_b, splits_b, n_b, out_b, accumulate);
+                                        bool accumulate_a, const float* partials_b, int splits_b, int64_t n_b, float* out_b,
+                                        bool accumulate_b, const int32_t* status_word, cudaStream_t stream) {
+    const ReduceJob a = make_reduce_job(partials_a, splits_a, n_a, out_a, accumulate_a);
+    const ReduceJob b = make_reduce_job(partials_b, splits_b, n_b, out_b, accumulate_b);
     return launch_pdl(reduce_partials_kernel, dim3((unsigned)(a.blocks + b.blocks)), dim3(256), 0, stream, a, b,
                       status_word);
 }

@@ -328,7 +328,8 @@ struct BackwardParams {
     float* dW;                             // dW itself, or the partials [splits, C_in * C_out]
     float* db;                             // nullptr: not asked for; db itself, or the partials [splits, C_out]
     T* dX;
-    int w_tiles, w_col_tiles, splits, accumulate;
+    int w_tiles, w_col_tiles, splits;
+    int dw_accumulate, db_accumulate;      // add into dW, into db (only with one split)
     int x_row_tiles, x_col_tiles;          // w_tiles / x_row_tiles 0: that product is not asked for
     int zero_blocks;                       // blocks that clear the dropped rows of dX
     const int32_t* status_word;
@@ -353,7 +354,7 @@ __device__ __forceinline__ void dw_tile(ProductShared<BN>& sh, const BackwardPar
         const int t = threadIdx.x, j = (kOutIn ? row_tile * kBM : col_tile * BN) + t;
         if (t < (kOutIn ? kBM : BN) && j < p.C_out) {
             float* o = p.db + (int64_t)split * p.C_out + j;
-            *o = p.accumulate ? *o + colsum : colsum;
+            *o = p.db_accumulate ? *o + colsum : colsum;
         }
     }
     const int rows = kOutIn ? p.C_out : p.C_in, cols = kOutIn ? p.C_in : p.C_out;
@@ -368,7 +369,7 @@ __device__ __forceinline__ void dw_tile(ProductShared<BN>& sh, const BackwardPar
             if (j >= cols) continue;
             float4 v = quad(acc, r, h);
             float4* o = reinterpret_cast<float4*>(out + (int64_t)i * cols + j);
-            if (p.accumulate) { const float4 w = *o; v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w; }
+            if (p.dw_accumulate) { const float4 w = *o; v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w; }
             *o = v;
         }
     }
@@ -528,8 +529,8 @@ int fma_backward_kernel_count(sbp_dtype dt, bool w_out_in, int64_t M_keep_cap, i
 
 cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY, const void* W, bool w_out_in, const int32_t* dy_rows,
                                 const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
-                                int64_t C_out, float* dW, float* db, bool accumulate, void* dX, float* workspace,
-                                const int32_t* status_word, cudaStream_t stream) {
+                                int64_t C_out, float* dW, float* db, bool dw_accumulate, bool db_accumulate, void* dX,
+                                float* workspace, const int32_t* status_word, cudaStream_t stream) {
     const FmaPlan pl = fma_plan(dt == SBP_F32, w_out_in, M_keep_cap, C_in, C_out, dW != nullptr, dX != nullptr);
     const bool split = dW != nullptr && pl.splits > 1;
     float* ws_db = workspace;                                          // [splits, C_out], then [splits, C_in * C_out]
@@ -547,7 +548,8 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
         p.w_tiles = (int)(pl.w_rows * pl.w_cols);
         p.w_col_tiles = (int)pl.w_cols;
         p.splits = pl.splits;
-        p.accumulate = (accumulate && !split) ? 1 : 0;
+        p.dw_accumulate = (dw_accumulate && !split) ? 1 : 0;
+        p.db_accumulate = (db_accumulate && !split) ? 1 : 0;
         p.x_row_tiles = (int)pl.x_rows;
         p.x_col_tiles = (int)pl.x_cols;
         // 64 KB of rows or more a block, as many blocks as SMs at most
@@ -569,8 +571,9 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
     }
     if (e != cudaSuccess || !split) return e;
     if (db != nullptr)
-        return launch_reduce_partials_pair(ws_dw, pl.splits, C_in * C_out, dW, ws_db, pl.splits, C_out, db, accumulate, status_word, stream);
-    return launch_reduce_partials(ws_dw, pl.splits, C_in * C_out, dW, accumulate, status_word, stream);
+        return launch_reduce_partials_pair(ws_dw, pl.splits, C_in * C_out, dW, dw_accumulate, ws_db, pl.splits, C_out, db, db_accumulate,
+                                           status_word, stream);
+    return launch_reduce_partials(ws_dw, pl.splits, C_in * C_out, dW, dw_accumulate, status_word, stream);
 }
 
 }  // namespace sbp

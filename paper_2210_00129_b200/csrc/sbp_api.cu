@@ -206,8 +206,9 @@ size_t base_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_keep_cap, int64_t
 }  // namespace
 
 namespace {
-// the backward with W and dW in the paper's [C_in, C_out] layout, or (w_out_in) in the other one where the kernels take it
-sbp_status backward_direct(sbp_dtype dt, bool w_out_in, const void* X_keep, const void* dY, const void* W,
+// the backward with W and dW in the paper's [C_in, C_out] layout, or (w_out_in) in the other one where the kernels take it; fresh_dw:
+// dW is written, whatever the flags say about accumulation (db follows them)
+sbp_status backward_direct(sbp_dtype dt, bool w_out_in, bool fresh_dw, const void* X_keep, const void* dY, const void* W,
                            const int32_t* keep_rows, const int32_t* M_keep_dev, int64_t M,
                            int64_t M_keep_cap, int64_t C_in, int64_t C_out, float* dW, float* db, void* dX,
                            uint32_t flags, void* workspace, size_t workspace_bytes, size_t workspace_required,
@@ -234,7 +235,7 @@ sbp_status backward_direct(sbp_dtype dt, bool w_out_in, const void* X_keep, cons
             workspace_bytes < workspace_required)
             return SBP_ERR_WORKSPACE;
     }
-    const bool accumulate = (flags & SBP_FLAG_ACCUMULATE) != 0;
+    const bool accumulate = (flags & SBP_FLAG_ACCUMULATE) != 0, dw_accumulate = accumulate && !fresh_dw;
     float* ws_db = static_cast<float*>(workspace);
     float* ws_dw = need_ws ? reinterpret_cast<float*>(static_cast<char*>(workspace) +
                                                       db_scratch_bytes(dt, M_keep_cap, C_out))
@@ -259,12 +260,12 @@ sbp_status backward_direct(sbp_dtype dt, bool w_out_in, const void* X_keep, cons
     if (tc) {
         // both products (and the bias sums) in one persistent tensor-core kernel
         const sbp_status s = launch_tc_backward(X_keep, dY, W, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap, C_in, C_out, dW,
-                                                accumulate, dX, db_rides ? db : nullptr, w_out_in, ws_dw, ws_db, status_word,
-                                                stream);
+                                                dw_accumulate, dX, db_rides ? db : nullptr, accumulate, w_out_in, ws_dw, ws_db,
+                                                status_word, stream);
         if (s != SBP_OK) return s;
     } else if (dW != nullptr || dX != nullptr) {
         if (launch_fma_backward(dt, X_keep, dY, W, w_out_in, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap, C_in, C_out, dW,
-                                db_rides ? db : nullptr, accumulate, dX, ws_dw, status_word, stream) != cudaSuccess)
+                                db_rides ? db : nullptr, dw_accumulate, accumulate, dX, ws_dw, status_word, stream) != cudaSuccess)
             return SBP_ERR_CUDA;
     }
     return SBP_OK;
@@ -279,13 +280,13 @@ sbp_status sbp_linear_backward(sbp_dtype dt, const void* X_keep, const void* dY,
                                void* stream_v) {
     cudaStream_t stream = (cudaStream_t)stream_v;
     if (!(flags & SBP_FLAG_W_OUT_IN) || (dW == nullptr && dX == nullptr))
-        return backward_direct(dt, false, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX, flags,
+        return backward_direct(dt, false, false, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX, flags,
                                workspace, workspace_bytes,
                                (M > 0 && M_keep_cap >= 0 && C_in > 0 && C_out > 0)
                                    ? sbp_linear_backward_workspace_bytes(dt, M, M_keep_cap, C_in, C_out) : 0,
                                status_word, stream);
     if (out_in_direct(C_in, C_out))
-        return backward_direct(dt, true, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX, flags,
+        return backward_direct(dt, true, false, X_keep, dY, W, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, dW, db, dX, flags,
                                workspace, workspace_bytes,
                                (M > 0 && M_keep_cap >= 0 && C_in > 0 && C_out > 0)
                                    ? sbp_linear_backward_workspace_bytes(dt, M, M_keep_cap, C_in, C_out) : 0,
@@ -306,19 +307,10 @@ sbp_status sbp_linear_backward(sbp_dtype dt, const void* X_keep, const void* dY,
         launch_transpose(dt == SBP_BF16 ? 2 : 4, W, w_copy, C_out, C_in, status_word, stream) != cudaSuccess)
         return SBP_ERR_CUDA;
     const bool accumulate = (flags & SBP_FLAG_ACCUMULATE) != 0;
-    sbp_status s;
-    if (accumulate && dW != nullptr) {
-        // dW is produced fresh in the copy and added in by the transpose; db accumulates in place on its own
-        s = backward_direct(dt, false, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in,
-                            C_out, dw_copy, nullptr, dX, inner & ~(uint32_t)SBP_FLAG_ACCUMULATE, workspace, base, base,
-                            status_word, stream);
-        if (s == SBP_OK && db != nullptr)
-            s = backward_direct(dt, false, nullptr, dY, nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in, C_out, nullptr, db,
-                                nullptr, inner & ~(uint32_t)SBP_FLAG_VALIDATE, workspace, base, base, status_word, stream);
-    } else {
-        s = backward_direct(dt, false, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap, C_in,
-                            C_out, dW != nullptr ? dw_copy : nullptr, db, dX, inner, workspace, base, base, status_word, stream);
-    }
+    // dW is produced fresh in the copy, and added in by the transpose where the call accumulates
+    const sbp_status s = backward_direct(dt, false, true, X_keep, dY, dX != nullptr ? w_copy : nullptr, keep_rows, M_keep_dev, M, M_keep_cap,
+                                         C_in, C_out, dW != nullptr ? dw_copy : nullptr, db, dX, inner, workspace, base, base, status_word,
+                                         stream);
     if (s != SBP_OK) return s;
     if (dW != nullptr &&
         launch_transpose_add_f32(dw_copy, dW, C_in, C_out, accumulate, status_word, stream) != cudaSuccess)

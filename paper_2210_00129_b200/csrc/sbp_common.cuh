@@ -153,10 +153,10 @@ cudaError_t launch_db(sbp_dtype dt, const void* dY, const int32_t* keep_rows, co
 cudaError_t launch_reduce_partials(const float* partials, int splits, int64_t n, float* out,
                                    bool accumulate, const int32_t* status_word, cudaStream_t stream);
 
-// two such reductions in one launch (both with the same accumulate setting)
+// two such reductions in one launch
 cudaError_t launch_reduce_partials_pair(const float* partials_a, int splits_a, int64_t n_a, float* out_a,
-                                        const float* partials_b, int splits_b, int64_t n_b, float* out_b,
-                                        bool accumulate, const int32_t* status_word, cudaStream_t stream);
+                                        bool accumulate_a, const float* partials_b, int splits_b, int64_t n_b, float* out_b,
+                                        bool accumulate_b, const int32_t* status_word, cudaStream_t stream);
 
 // CUDA-core products (fp32 FMAs) for fp32 and for bf16 shapes the tensor-core kernels do not take: dW (nullable), db
 // (nullable, made on the way to dW and only with it) and dX (nullable) in one launch, plus one reduce when the dW
@@ -167,8 +167,8 @@ size_t fma_dw_workspace_bytes(sbp_dtype dt, int64_t M_keep_cap, int64_t C_in, in
 int    fma_backward_kernel_count(sbp_dtype dt, bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY, const void* W, bool w_out_in, const int32_t* dy_rows,
                                 const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
-                                int64_t C_out, float* dW, float* db, bool accumulate, void* dX, float* workspace,
-                                const int32_t* status_word, cudaStream_t stream);
+                                int64_t C_out, float* dW, float* db, bool dw_accumulate, bool db_accumulate, void* dX,
+                                float* workspace, const int32_t* status_word, cudaStream_t stream);
 
 // transposes for weights in the [C_out, C_in] layout
 cudaError_t launch_transpose(int elem_bytes, const void* in, void* out, int64_t rows, int64_t cols,
@@ -218,7 +218,7 @@ int    tc_backward_kernel_count(int64_t M_keep_cap, int64_t C_in, int64_t C_out,
 // (dy_rows / dx_rows as for launch_fma_backward; w_out_in: W and dW are [C_out, C_in])
 sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W, const int32_t* dy_rows,
                               const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
-                              int64_t C_out, float* dW, bool accumulate, void* dX, float* db, bool w_out_in, float* workspace,
-                              float* db_workspace, int32_t* status_word, cudaStream_t stream);
+                              int64_t C_out, float* dW, bool dw_accumulate, void* dX, float* db, bool db_accumulate, bool w_out_in,
+                              float* workspace, float* db_workspace, int32_t* status_word, cudaStream_t stream);
 
 }  // namespace sbp

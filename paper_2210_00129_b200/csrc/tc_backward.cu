@@ -1122,8 +1122,8 @@ int tc_backward_kernel_count(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bo
 
 sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W, const int32_t* dy_rows,
                               const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in, int64_t C_out,
-                              float* dW, bool accumulate, void* dX, float* db, bool w_out_in, float* workspace, float* db_workspace,
-                              int32_t* status_word, cudaStream_t stream) {
+                              float* dW, bool dw_accumulate, void* dX, float* db, bool db_accumulate, bool w_out_in, float* workspace,
+                              float* db_workspace, int32_t* status_word, cudaStream_t stream) {
     const bool want_dw = dW != nullptr, want_dx = dX != nullptr;
     if (!want_dw && !want_dx) return SBP_OK;
     const Plan pl = make_plan(M_keep_cap, C_in, C_out, want_dw, want_dx, dy_rows == nullptr);
@@ -1148,7 +1148,7 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     prm.dW_out = want_dw ? (pl.splits > 1 ? workspace : dW) : nullptr;
     prm.dw_split_stride = C_in * C_out;
     prm.dw_splits = pl.splits;
-    prm.dw_accumulate = (pl.splits == 1 && accumulate) ? 1 : 0;
+    prm.dw_accumulate = (pl.splits == 1 && dw_accumulate) ? 1 : 0;
     // the dW tiles leave through TMA stores: dW and the workspace are 16-byte aligned (checked at the entry point)
     if (want_dw) {
         if (!make_map_dw(&map_dw, prm.dW_out, pl.splits, C_in, C_out, w_out_in)) return SBP_ERR_CUDA;
@@ -1158,7 +1158,7 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     const bool db_from_mma = db != nullptr && db_in_dw_tiles(pl, want_dw), db_direct = db_from_mma && pl.splits == 1;
     prm.db_from_mma = db_from_mma ? 1 : 0;
     prm.db_partial = (db == nullptr) ? nullptr : db_direct ? db : db_workspace;
-    prm.db_accumulate = (db_direct && accumulate) ? 1 : 0;
+    prm.db_accumulate = (db_direct && db_accumulate) ? 1 : 0;
     prm.status_word = status_word;
     prm.dw_ctas = pl.dw_ctas;
     int64_t ctas = pl.tiles < kNumSMs ? pl.tiles : kNumSMs;
@@ -1197,12 +1197,12 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
     const bool reduce_dw = want_dw && pl.splits > 1, reduce_db = db != nullptr && !db_direct;
     cudaError_t r = cudaSuccess;
     if (reduce_dw && reduce_db)
-        r = launch_reduce_partials_pair(workspace, pl.splits, C_in * C_out, dW, db_workspace, db_rows, C_out, db,
-                                        accumulate, status_word, stream);
+        r = launch_reduce_partials_pair(workspace, pl.splits, C_in * C_out, dW, dw_accumulate, db_workspace, db_rows, C_out, db,
+                                        db_accumulate, status_word, stream);
     else if (reduce_dw)
-        r = launch_reduce_partials(workspace, pl.splits, C_in * C_out, dW, accumulate, status_word, stream);
+        r = launch_reduce_partials(workspace, pl.splits, C_in * C_out, dW, dw_accumulate, status_word, stream);
     else if (reduce_db)
-        r = launch_reduce_partials(db_workspace, db_rows, C_out, db, accumulate, status_word, stream);
+        r = launch_reduce_partials(db_workspace, db_rows, C_out, db, db_accumulate, status_word, stream);
     if (r != cudaSuccess) return SBP_ERR_CUDA;
     return SBP_OK;
 }
