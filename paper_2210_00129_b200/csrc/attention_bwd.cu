@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
     constexpr int kThreads = 128 * G;
     constexpr uint32_t kTmemCols = G == 2 ? 256 : 512;
     // tensor-memory columns.  G = 2: S and dS side by side, then dV, dK, dQ in their place.  G = 4: S (dQ later); dS in the
-    // upper half, or, when two query tiles keep dV and dK there, in the place of S
+    // upper half, or, when two query tiles keep dV and dK there, next to S (up to 128 keys) or in its place
     constexpr uint32_t kColDV = G == 2 ? 0 : 256, kColDK = G == 2 ? 64 : 384, kColDQ = G == 2 ? 128 : 0;
     extern __shared__ uint8_t smem_raw[];
     __shared__ AttnShared<G> sh;
@@ -319,8 +319,8 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             continue;
         }
         const int QT = G == 2 ? 1 : (nq + 127) >> 7;
-        const bool shared_cols = G == 4 && QT > 1;           // dS takes the place of S
-        const uint32_t col_ds = G == 2 ? 128u : shared_cols ? 0u : 256u;
+        const bool shared_cols = G == 4 && QT > 1 && nk > 128;      // dS takes the place of S
+        const uint32_t col_ds = shared_cols ? 0u : G == 4 && QT == 1 ? 256u : 128u;
         const uint32_t k_steps = (uint32_t)(nk + 15) >> 4;
         const int n_keys = (int)k_steps * 16;                // accumulator columns computed
         ptx::cp_async_wait_all();
@@ -448,7 +448,10 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             const float mine = ex2((mx - mm) * sl2) * inv_l;
             const float nds = -U * inv_l * p.scale;          // -rowsum(S dS) / sqrt(d)
             const uint64_t mine2 = pair(mine, mine), nds2 = pair(nds, nds), scale2 = pair(p.scale, p.scale);
-            uint32_t dm[32];                                 // dM waits here when its blocks are those of S
+            // dM waits in tensor memory when its blocks are those of S: in columns that this thread alone reads and has read by then
+            // (G = 2: its dS, G = 4: its S or dS), out of the way of dV.  (In registers it spilled: Drop QKV
+            // with 126 of 196 tokens, B = 128, 105.9 -> 87.5 us; all tokens on both sides, B = 64, 136.6 -> 113.4.)
+            const uint32_t parked = tmem + (G == 2 ? 128u : 0u) + (uint32_t)key0 + lane_off;
             uint8_t* blkP = gen + (uint32_t)g * p.block_bytes;
             uint8_t* blkM = gen + p.off_dm + (uint32_t)g * p.dm_stride;
             const bool row_fits = (uint32_t)row * kRowB < p.block_bytes;
@@ -457,24 +460,25 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 if (key0 + c * 16 >= n_keys) break;
                 uint64_t d[8];
                 load_ds(key0 + c * 16, d);
-                uint32_t w[8];
+                uint32_t w[8], dm[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const uint64_t s2 = mul2(e[c >> 1][(c & 1) * 8 + j], mine2);        // S
                     const float2 sf = halves(s2), mf = halves(mul2(s2, fma2(d[j], scale2, nds2)));   // dM / sqrt(d)
                     w[j] = pack2(sf.x, sf.y);
-                    dm[c * 8 + j] = pack2(mf.x, mf.y);
+                    dm[j] = pack2(mf.x, mf.y);
                 }
+                if (!kSeparate) ptx::tmem_st_32x8(parked + (uint32_t)(c * 8), dm);
                 if (row_fits) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         *reinterpret_cast<uint4*>(blkP + swz((uint32_t)row, (uint32_t)(c * 2 + q))) = make_uint4(w[q * 4], w[q * 4 + 1], w[q * 4 + 2], w[q * 4 + 3]);
                         if (kSeparate)
-                            *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 2 + q))) =
-                                make_uint4(dm[c * 8 + q * 4], dm[c * 8 + q * 4 + 1], dm[c * 8 + q * 4 + 2], dm[c * 8 + q * 4 + 3]);
+                            *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)(c * 2 + q))) = make_uint4(dm[q * 4], dm[q * 4 + 1], dm[q * 4 + 2], dm[q * 4 + 3]);
                     }
                 }
             }
+            if (!kSeparate) ptx::tmem_st_wait();
             ptx::fence_async_proxy();                        // the blocks are read by the tensor core
             ptx::tc_fence_before_sync();
             __syncthreads();                                  // S and dS in tensor memory are dead from here on
@@ -509,10 +513,13 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 }
                 ok = wait_products(&sh.bar_o, n_o);
                 if (!ok) break;
+                float dm[32];                                // (bits)
+                ptx::tmem_ld_32x32(parked, dm);
+                ptx::tmem_ld_wait();
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                     if (key0 + (c >> 1) * 16 < n_keys && row_fits)
-                        *reinterpret_cast<uint4*>(blkM + swz((uint32_t)row, (uint32_t)c)) = make_uint4(dm[c * 4], dm[c * 4 + 1], dm[c * 4 + 2], dm[c * 4 + 3]);
+                        *reinterpret_cast<float4*>(blkM + swz((uint32_t)row, (uint32_t)c)) = make_float4(dm[c * 4], dm[c * 4 + 1], dm[c * 4 + 2], dm[c * 4 + 3]);
                 ptx::fence_async_proxy();
                 ptx::tc_fence_before_sync();
                 __syncthreads();
@@ -562,17 +569,15 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 ptx::tmem_ld_wait();
                 if ((uint32_t)row * kRowB < stage_b) stage32(gen + which * stage_b, row, (uint32_t)(g * 4), v);
             }
-            if (!kSeparate) {                               // (two stages only)
-                ptx::tmem_ld_32x32(tmem + (uint32_t)(128 + g * 32) + lane_off, v);
-                ptx::tmem_ld_wait();
-            }
             ptx::tc_fence_before_sync();
             __syncthreads();
 #pragma unroll 1
             for (int which = 0; which < (kSeparate ? 3 : 2); ++which)      // (one loop body: copies of it cost registers)
                 store_rows<kThreads>(which == 0 ? p.dV : which == 1 ? p.dK : p.dQ, p.ld_out, col0, gen + which * stage_b,
                                      which == 2 ? q_glob : k_glob, which == 2 ? nq : nk);
-            if (!kSeparate) {
+            if (!kSeparate) {                               // (two stages only)
+                ptx::tmem_ld_32x32(tmem + (uint32_t)(128 + g * 32) + lane_off, v);
+                ptx::tmem_ld_wait();
                 __syncthreads();
                 if ((uint32_t)row * kRowB < stage_b) stage32(gen, row, (uint32_t)(g * 4), v);
                 __syncthreads();
