@@ -4,7 +4,7 @@
 // (philox word << 32 | position) and emits the kept positions in ascending order.  Bound by the chain of barriers, not by
 // work, so the chain is short: one histogram of the words' top eight bits names the bin that holds the K-th smallest; that
 // bin's words (about N / 256) are collected and each is ranked against the others, which gives the threshold word; each
-// thread then owns a contiguous stretch of positions, so one block scan of their counts places every kept position.  (Should
+// warp then owns a contiguous stretch of positions, so one scan of the warps' counts places every kept position.  (Should
 // a bin ever hold more words than the list, the next eight bits are taken, as often as needed.)  Four passes of eight bits
 // and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.5 us
 // and 3.7 us (the words are drawn while the kernel before drains).
@@ -62,7 +62,9 @@ __device__ __forceinline__ uint32_t cluster_load(const uint32_t* local_ptr, uint
     return v;
 }
 
-constexpr uint32_t kMaxListed = 1024;      // words of the chosen bin that are ranked directly
+// Words of the chosen bin that are ranked directly.  Every block of a cluster ranks them all, n x n comparisons; from some 400 on eight
+// more bits of the words are the cheaper way (32 samples of 200000 positions, 781 words in a bin: 88 us, now 31).
+constexpr uint32_t kMaxListed = 384;
 
 struct RandomShared {
     // Two histograms used alternately: the one a pass clears was last read by other blocks of a cluster two passes earlier,
@@ -71,7 +73,7 @@ struct RandomShared {
     uint32_t listed[kMaxListed];           // this block's words of the chosen bin
     uint32_t all_listed[kMaxListed];       // a cluster's: those of all its blocks
     uint32_t n_listed;
-    uint32_t warp_sums[32];
+    uint32_t warp_sums[32], warp_ties[32];
     uint32_t bin, below, in_bin;           // the chosen bin, words in lower bins, words in it
     uint32_t threshold, less, equal;       // the K-th smallest word; listed words below it, equal to it
     uint32_t slice_counts[2];              // positions of this slice below / equal to the threshold
@@ -109,9 +111,18 @@ sample_keep_random_kernel(uint32_t N, uint32_t K, uint32_t k0, uint32_t k1, uint
         return pw;
     };
 
-    uint32_t threshold = 0xffffffffu, ties = 0xffffffffu;    // kept: word < threshold, and the first `ties` equal to it
-    bool all_ties = true;
-    if (K < N) {
+    if (C == 1 && K >= N) {                                  // nothing to choose (small maps; larger ones do not come here)
+        pdl_wait();
+        if (threadIdx.x == 0) {
+            keep_offsets[b + 1] = (int32_t)((b + 1) * (int64_t)N);
+            if (b == 0) keep_offsets[0] = 0;
+        }
+        for (uint32_t n = threadIdx.x; n < N; n += kThreads) out[n] = (int32_t)(row_base + n);
+        return;
+    }
+    uint32_t threshold, ties;                                // kept: word < threshold, and the first `ties` equal to it
+    bool all_ties;
+    {
         uint32_t prefix = 0, known = 0, remaining = K;
         for (int shift = 24, pass = 0;; shift -= 8, ++pass) {
             uint32_t* hist = sh.hist[pass & 1];
@@ -167,7 +178,7 @@ sample_keep_random_kernel(uint32_t N, uint32_t K, uint32_t k0, uint32_t k1, uint
                 __syncthreads();                             // the bin is read before the next pass rewrites it
                 continue;
             }
-            if (in_bin > kMaxListed) {                       // more than 1024 equal words
+            if (in_bin > kMaxListed) {                       // more equal words than that
                 threshold = prefix;
                 ties = remaining;
                 all_ties = in_bin == remaining;
@@ -213,62 +224,85 @@ sample_keep_random_kernel(uint32_t N, uint32_t K, uint32_t k0, uint32_t k1, uint
         }
     }
 
-    // ---- this thread's contiguous stretch of groups: counts, then the kept positions in order ----
-    const uint32_t mine_groups = (g_end - g_begin + kThreads - 1) / kThreads;
-    const uint32_t t_begin = g_begin + threadIdx.x * mine_groups < g_end ? g_begin + threadIdx.x * mine_groups : g_end;
-    const uint32_t t_end = t_begin + mine_groups < g_end ? t_begin + mine_groups : g_end;
+    // ---- each warp's contiguous stretch of groups, a group a lane at a time: counts, then the kept positions in order.  (With a
+    //      stretch a thread every store is a transaction of its own.) ----
+    constexpr int kWarps = kThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t slice = g_end - g_begin, per_warp = ((slice + kWarps - 1) / kWarps + 31u) & ~31u;
+    const uint32_t w_begin = g_begin + ((uint32_t)warp * per_warp < slice ? (uint32_t)warp * per_warp : slice);
+    const uint32_t w_end = g_end - w_begin < per_warp ? g_end : w_begin + per_warp;
     uint32_t lt = 0, eq = 0;
-    for (uint32_t q = t_begin; q < t_end; ++q) {
-        if (K >= N) {
-            lt += N - 4u * q < 4u ? N - 4u * q : 4u;
-        } else {
-            const PhiloxWords pw = words_of(q);
+    for (uint32_t q = w_begin + lane; q < w_end; q += 32) {
+        const PhiloxWords pw = words_of(q);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (4u * q + e < N) {
-                    lt += pw.w[e] < threshold;
-                    eq += pw.w[e] == threshold;
-                }
+        for (int e = 0; e < 4; ++e) {
+            if (4u * q + e < N) {
+                lt += pw.w[e] < threshold;
+                eq += pw.w[e] == threshold;
             }
         }
     }
-    uint32_t first, ties_before = 0;                          // kept positions and ties in front of this stretch
-    if (C == 1 && all_ties) {
-        first = block_excl_scan<kThreads>(lt + eq, sh.warp_sums).x;
-    } else {
-        const uint2 sl = block_excl_scan<kThreads>(lt, sh.warp_sums);
-        const uint2 se = block_excl_scan<kThreads>(eq, sh.warp_sums);
-        uint32_t lt_before = sl.x;
-        ties_before = se.x;
-        if constexpr (C > 1) {
-            if (threadIdx.x == 0) { sh.slice_counts[0] = sl.y; sh.slice_counts[1] = se.y; }
-            cluster_sync();
-            for (uint32_t r = 0; r < rank; ++r) {
-                lt_before += cluster_load(&sh.slice_counts[0], r);
-                ties_before += cluster_load(&sh.slice_counts[1], r);
-            }
-        }
-        first = lt_before + (ties_before < ties ? ties_before : ties);
+    lt = __reduce_add_sync(0xffffffffu, lt);
+    eq = __reduce_add_sync(0xffffffffu, eq);
+    if (lane == 0) {
+        sh.warp_sums[warp] = lt;
+        sh.warp_ties[warp] = eq;
     }
+    __syncthreads();
+    const uint32_t all_lt = lane < kWarps ? sh.warp_sums[lane] : 0u, all_eq = lane < kWarps ? sh.warp_ties[lane] : 0u;
+    uint32_t kept_before = __reduce_add_sync(0xffffffffu, lane < warp ? all_lt : 0u);      // below the threshold in front of this warp's stretch
+    uint32_t ties_before = __reduce_add_sync(0xffffffffu, lane < warp ? all_eq : 0u);
+    if constexpr (C > 1) {
+        const uint32_t slice_lt = __reduce_add_sync(0xffffffffu, all_lt), slice_eq = __reduce_add_sync(0xffffffffu, all_eq);
+        if (threadIdx.x == 0) { sh.slice_counts[0] = slice_lt; sh.slice_counts[1] = slice_eq; }
+        cluster_sync();
+        for (uint32_t r = 0; r < rank; ++r) {
+            kept_before += cluster_load(&sh.slice_counts[0], r);
+            ties_before += cluster_load(&sh.slice_counts[1], r);
+        }
+    }
+    uint32_t first = kept_before + (ties_before < ties ? ties_before : ties);
     pdl_wait();                 // earlier kernels of the stream may still be reading the index buffers
     if (rank == 0 && threadIdx.x == 0) {
         keep_offsets[b + 1] = (int32_t)((b + 1) * (int64_t)K);
         if (b == 0) keep_offsets[0] = 0;
     }
-    for (uint32_t q = t_begin; q < t_end; ++q) {
+    const uint32_t lanes_before = (1u << lane) - 1u;
+    for (uint32_t q0 = w_begin; q0 < w_end; q0 += 32) {
+        const uint32_t q = q0 + lane;
+        const bool live = q < w_end;
         PhiloxWords pw;
-        if (K < N) pw = words_of(q);
+        if (live) pw = words_of(q);
+        bool keep[4];
+        if (all_ties) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (4u * q + e < N) {
-                bool keep = K >= N || pw.w[e] < threshold;
-                if (!keep && pw.w[e] == threshold) {
-                    keep = ties_before < ties;
-                    ++ties_before;
-                }
-                if (keep) out[first++] = (int32_t)(row_base + 4u * q + e);
+            for (int e = 0; e < 4; ++e) keep[e] = live && 4u * q + e < N && pw.w[e] <= threshold;
+        } else {                                                   // ties are kept in order of position until there are enough
+            bool tie[4];
+            uint32_t mine = ties_before;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                tie[e] = live && 4u * q + e < N && pw.w[e] == threshold;
+                const uint32_t all = __ballot_sync(0xffffffffu, tie[e]);
+                mine += __popc(all & lanes_before);
+                ties_before += __popc(all);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                keep[e] = (live && 4u * q + e < N && pw.w[e] < threshold) || (tie[e] && mine < ties);
+                mine += tie[e];
             }
         }
+        uint32_t at = first;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t all = __ballot_sync(0xffffffffu, keep[e]);
+            at += __popc(all & lanes_before);
+            first += __popc(all);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (keep[e]) out[at++] = (int32_t)(row_base + 4u * q + e);
     }
     if constexpr (C > 1) cluster_sync();                      // the slice counts stay readable until every block is done
 }
@@ -324,7 +358,7 @@ sample_keep_grid_kernel(int family, uint32_t H, uint32_t W, FastDiv by_width, ui
 
     // offset of this sample = sum of the closed-form counts of the samples before it
     uint64_t before = 0;
-    if (share_mask) {
+    if (share_mask || family == 4) {                         // every sample keeps as many as the first
         before = (uint64_t)b * grid_count(family, grid_phase(family, 0u, step, k0, k1), H, W);
     } else {
         uint64_t sum = 0;
@@ -462,7 +496,9 @@ template <int C, int kThreads>
 cudaError_t launch_random_sampler(int64_t B, cudaStream_t stream, int64_t N, int64_t K, uint32_t k0, uint32_t k1, uint32_t step,
                                   uint32_t first_sample, bool share_mask, int32_t* keep_rows, int32_t* keep_offsets) {
     const int64_t slice_groups = ((N + 3) / 4 + C - 1) / C;
-    const size_t cache_bytes = K < N && (size_t)slice_groups * 16 <= kCacheMax ? (size_t)slice_groups * 16 : 0;
+    size_t cache_bytes = (size_t)slice_groups * 16 <= kCacheMax ? (size_t)slice_groups * 16 : 0;
+    // the large blocks one to an SM: two of a cluster side by side on one made the detection step (2 x 66800) 4 us longer
+    if (kThreads == 1024 && cache_bytes < 116 * 1024) cache_bytes = 116 * 1024;
     if (cache_bytes > 32 * 1024) {                            // (the static part takes 10 KB of the default 48)
         const cudaError_t opt = opt_in_dynamic_smem<sample_keep_random_kernel<C, kThreads>>((int)kCacheMax);
         if (opt != cudaSuccess) return opt;
@@ -481,10 +517,14 @@ cudaError_t launch_sample_keep(int mode, int grid_family, int64_t B, int64_t H, 
                                uint64_t seed, uint32_t step, uint32_t first_sample, bool share_mask,
                                int32_t* keep_rows, int32_t* keep_offsets, cudaStream_t stream) {
     const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
+    const int64_t N = H * W;
+    if (mode == SBP_MASK_RANDOM && K >= N && N > 8192) {     // nothing to choose: the grid mask that keeps everything
+        mode = SBP_MASK_GRID;
+        grid_family = 4;
+    }
     if (mode == SBP_MASK_RANDOM) {
-        const int64_t N = H * W;
         // large maps with few samples: spread each sample over a cluster so that more SMs take part
-        if (K < N && N > 8192 && B * 8 <= 4 * kNumSMs) {
+        if (N > 8192 && B * 8 <= 4 * kNumSMs) {
             // 1024 threads for up to three samples, whose clusters find room beside the kernel before: 2 x 66800 positions 4.2 ->
             // 3.7 us back to back, 3 x 4.3 -> 3.8, but 4 x 4.5 -> 5.4 and 8 x 5.5 -> 10.4
             if (N > 32768 && B <= 3) return launch_random_sampler<8, 1024>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
@@ -501,7 +541,7 @@ cudaError_t launch_sample_keep(int mode, int grid_family, int64_t B, int64_t H, 
         const int64_t by_size = (positions + 4 * kSampThreads - 1) / (4 * kSampThreads), by_room = 4 * kNumSMs / B;
         return by_size < by_room ? by_size : by_room < 1 ? 1 : by_room;
     };
-    const int64_t parts = blocks_for(mode == SBP_MASK_GRID ? H * W : K);
+    const int64_t parts = blocks_for(mode == SBP_MASK_GRID ? N : K);
     const dim3 grid((unsigned)(B * parts)), block(kSampThreads);
     if (mode == SBP_MASK_TEMPORAL || mode == SBP_MASK_TEMPORAL_GRID)      // H frames of W positions; K = kept frames x W
         return launch_pdl(sample_keep_temporal_kernel, grid, block, 0, stream, mode == SBP_MASK_TEMPORAL ? 0 : grid_family,
