@@ -385,9 +385,13 @@ bool choose_pair(int64_t M, int64_t C_in, int64_t C_out) {
 bool tc_forward_supported(int64_t M, int64_t C_in, int64_t C_out) {
     if (M >= (1ll << 31) || C_in % 8 != 0 || C_out % 8 != 0) return false;
     // Ragged and narrow shapes included: 64 -> 2048 with 65536 rows 657 us on the CUDA cores, 93 us here, 512 -> 32 with 64 rows
-    // 24.0 and 5.0.  One or two reduction steps over few rows are quicker there: 16 -> 2048 with 64 rows 3.3 us and 4.8 us, with
-    // 320 4.4 and 5.2, with 1024 7.4 and 5.6.
-    return !(C_in <= 32 && M <= 512);
+    // 24.0 and 5.0.  One to three reduction steps are quicker there where the tiles are few or hardly filled: 16 -> 64 with 784 rows
+    // 2.2 and 3.0 us, 16 -> 192 with 12544 4.1 and 5.8, 8 -> 4096 with 196 4.0 and 4.7, 32 -> 256 with 196 3.0 and 3.5, 32 -> 8 with
+    // 100352 14.3 and 18.4; not 16 -> 256 with 12544 5.6 and 5.4, 32 -> 1024 with 784 6.1 and 3.7, 48 -> 16 with 100352 19.3 and 17.1.
+    const int64_t tiles = (M + 63) / 64 * ((C_out + 63) / 64);
+    if (C_in <= 16 && (C_out <= 64 || tiles <= (M <= 256 ? 256 : kNumSMs) || (C_out < 256 && M <= 32768))) return false;
+    if (C_in <= 32 && tiles <= 32) return false;
+    return !(M > 16384 && ((C_in <= 32 && C_out <= 16) || (C_in <= 48 && C_out <= 8)));
 }
 
 sbp_status launch_tc_forward(const void* X, const void* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,
