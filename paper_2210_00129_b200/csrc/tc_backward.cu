@@ -526,8 +526,10 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 const __nv_bfloat16* src[kInstr];
 #pragma unroll
                 for (int i = 0; i < kInstr; ++i) {
+                    // padding rows of the last tile, never stored: the list from its start again (a hundred reads of one and the same
+                    // row hold up a k-block: dX of 1000 -> 1000 with 392 kept rows 19.7 -> 10.6 us)
                     int64_t m = m0 + (gw * kInstr + i) * 4 + sub;
-                    if (m >= M_keep) m = M_keep - 1;                  // padding rows of the last tile: never stored
+                    if (m >= M_keep) m = M_keep >= kBM ? m - M_keep : M_keep - 1;
                     src[i] = p.dY + (int64_t)map_row<kPacked>(p.dy_rows, m) * C_out + chunk * 8;
                 }
                 for (uint32_t k = 0; k < t.num_kb; ++k, ++it) {
