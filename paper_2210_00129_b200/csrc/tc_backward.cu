@@ -228,6 +228,20 @@ __device__ __forceinline__ bool next_tile(const Schedule& s, uint32_t pass, Tile
     return true;
 }
 
+// The tensor core cuts its running fp32 sum short (towards zero) instead of rounding it, so the relative error of a dW sum grows with
+// the length of its chain: 7e-8 a k-block of 64 rows on B200, whatever the tile.  A long piece is therefore summed in two or three
+// equal parts, each read out under the products of the next one and added to the ones before by the TMA store, which rounds.
+// Uncut, 768 -> 2304 and 768 -> 3072 with 12544 kept rows are off by 6.9e-6 and with 50176 the latter by 2.9e-5; now 3.3e-6 and 9.3e-6,
+// for 1 to 2.5 % of the call (94.1 -> 96.3 us, 361 -> 368; 512 -> 128 with 100352 rows 70.8 -> 72.5).  More parts cost more than that
+// (28 k-blocks each: 768 -> 3072 4 %; 128 -> 512 6 to 15 %), and shorter pieces than these, whose parts end with the call, 10 %.
+__host__ __device__ constexpr uint32_t whole_piece(bool pair, bool apart) { return pair ? 56u : apart ? 20u : 32u; }     // apart: the role split
+template <bool kPair, bool kParts>
+__device__ __forceinline__ uint32_t chain_part(const Schedule& s, const Tile& t) {
+    if (!kParts || !t.is_dw || t.num_kb <= whole_piece(kPair, s.dw_ctas != 0u)) return t.num_kb;
+    const uint32_t parts = kPair && t.num_kb > 128 ? 3 : 2;
+    return (t.num_kb + parts - 1) / parts;
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -287,9 +301,11 @@ __device__ __forceinline__ void zero_dropped_rows(const TcParams& p, int64_t M_k
 // kOutIn: W and dW are stored [C_out, C_in].  The W tile of a dX stage is then 64 rows (j) x BNX columns (i), an MN-major
 // operand which arrives in 64 x 64 boxes like the X_keep tile of a dW stage; a dW tile leaves by 128 rows x 16 columns, each
 // lane's sixteen numbers side by side (64 bytes, swizzled so that neither the lanes' writes nor the copy meet bank conflicts).
+// kParts: some dW piece may be long enough to be summed in parts (a variant of its own: the loop over parts cost every call of a
+// narrow layer 0.2 - 0.3 us).
 // The kernel takes the same time in both layouts; transposing W before it and dW after it took 17 us of a ConvNeXt stage-4
 // block's forward and backward (183 -> 158 us), 12 us of a ViT-B/16 MLP's at B = 64.
-template <int BNX, int BNW, int kBiasDepth, bool kPacked, bool kPair, bool kOutIn>
+template <int BNX, int BNW, int kBiasDepth, bool kPacked, bool kPair, bool kOutIn, bool kParts>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                    const __grid_constant__ CUtensorMap map_dw, const TcParams p) {
@@ -474,24 +490,33 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                 Tile t;
                 if (!fetch_tile(pass, t)) break;
                 if (t.num_kb == 0) continue;
-                const uint32_t acc = used & 1u;
-                ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[acc]), ((used >> 1) & 1u) ^ 1u, abort_flag, status_word);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + acc * kAccCols;
-                // where the bias column accumulates: the unused half of a narrow tile's slot; with wide tiles the other
-                // slot, which a block that runs a single dW piece (the role split) never uses
-                const uint32_t bias_tmem = kNarrow ? d_tmem + 128u : tmem_base + (acc ^ 1u) * kAccCols;
-                if (!t.is_dw) run_tile(No{}, No{}, t.num_kb, d_tmem, bias_tmem);
-                else if (!kPair && t.col_tile == 0 && p.db_from_mma) run_tile(Yes{}, std::bool_constant<!kPair>{}, t.num_kb, d_tmem, bias_tmem);
-                else run_tile(Yes{}, No{}, t.num_kb, d_tmem, bias_tmem);
-                if (ok && leader) {
-                    if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[acc]));
-                    else ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[acc]));
-                }
-                __syncwarp();
-                ++used;
+                const uint32_t part = chain_part<kPair, kParts>(sched, t);
+                uint32_t done = 0;
+                do {
+                    const uint32_t n = kParts && t.num_kb - done < part ? t.num_kb - done : part, acc = used & 1u;
+                    const bool bias = !kPair && t.is_dw && t.col_tile == 0 && p.db_from_mma;
+                    // where the bias column accumulates: the unused half of a narrow tile's slot; with wide tiles the other
+                    // slot's first columns.  Such a block runs a single dW piece (the role split), whose next part then waits for the
+                    // read-out of this part's bias column and of the sums that its own bias column overwrites.
+                    uint32_t phase = ((used >> 1) & 1u) ^ 1u;
+                    if (kParts && !kNarrow && bias) phase = done != 0 ? ((used - 1u) >> 1) & 1u : 1u;
+                    ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_empty[acc]), phase, abort_flag, status_word);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+                    const uint32_t d_tmem = tmem_base + acc * kAccCols;
+                    const uint32_t bias_tmem = kNarrow ? d_tmem + 128u : tmem_base + (acc ^ 1u) * kAccCols;
+                    if (!t.is_dw) run_tile(No{}, No{}, n, d_tmem, bias_tmem);
+                    else if (bias) run_tile(Yes{}, std::bool_constant<!kPair>{}, n, d_tmem, bias_tmem);
+                    else run_tile(Yes{}, No{}, n, d_tmem, bias_tmem);
+                    if (ok && leader) {
+                        if constexpr (kPair) ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[acc]));
+                        else ptx::umma_commit(ptx::smem_addr(&ctl->acc_full[acc]));
+                    }
+                    __syncwarp();
+                    ++used;
+                    done += part;
+                } while (kParts && ok && done < t.num_kb);
             }
         } else if (kPair && lane == 0) {
             // ---------------- odd block of a pair: tell the issuer when this block's gathered rows have landed ----------------
@@ -676,8 +701,20 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
         for (uint32_t pass = 0; ok; ++pass) {
             Tile t;
             if (!fetch_tile(pass, t)) break;
-            const uint32_t acc = used & 1u;
-            const uint32_t taddr = tmem_base + acc * kAccCols + ((uint32_t)(warp * 32) << 16);
+            uint32_t acc = used & 1u, taddr = tmem_base + acc * kAccCols + ((uint32_t)(warp * 32) << 16);
+            // this warp is done with accumulator `slot`: hand it back to the MMA issuer
+            const auto release = [&](uint32_t slot) {
+                ptx::tc_fence_before_sync();
+                if (lane == 0) {
+                    if constexpr (kPair) ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_addr(&ctl->acc_empty[slot]), 0));
+                    else ptx::mbar_arrive(ptx::smem_addr(&ctl->acc_empty[slot]));
+                }
+            };
+            const auto next_accumulator = [&] {
+                ++used;
+                acc = used & 1u;
+                taddr = tmem_base + acc * kAccCols + ((uint32_t)(warp * 32) << 16);
+            };
             if (!t.is_dw) {
                 // ---- dX tile: scatter the kept rows (the dropped rows are zeroed by the side warps) ----
                 const int n0 = (int)(t.col_tile * BNX);
@@ -726,25 +763,43 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                     }
                     __syncwarp();
                 }
+                release(acc);
+                next_accumulator();
             } else {
                 // ---- dW tile: accumulator row = output column j, accumulator column = output row i ----
                 const int j = (int)(t.row_tile * kBM) + warp * 32 + lane;
                 const int i0 = (int)(t.col_tile * BNW);
                 const int64_t out_step = kOutIn ? 1 : C_out;                 // from one row i of dW to the next
                 float* out_col = p.dW_out + (int64_t)t.split * p.dw_split_stride + (kOutIn ? (int64_t)j * C_in + i0 : (int64_t)i0 * C_out + j);
-                const bool bias_col = p.db_from_mma && t.col_tile == 0;
+                const bool bias_col = p.db_from_mma && t.col_tile == 0, bias_wide = kParts && !kNarrow && bias_col;
                 if (t.num_kb == 0) {                                 // a piece without kept rows contributes zero
                     if (!p.dw_accumulate && j < C_out)
                         for (int c0 = 0; c0 < BNW && i0 + c0 < C_in; ++c0) out_col[(int64_t)c0 * out_step] = 0.f;
                     if (bias_col && j < C_out && !p.db_accumulate) p.db_partial[(int64_t)t.split * C_out + j] = 0.f;
                     continue;
                 }
-                if (lane == 0) ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_full[acc]), (used >> 1) & 1u, abort_flag, status_word);
-                ok = !ptx::bar_or<kEpiBarrier, 128>(!ok);            // the four epilogue warps go on, or give up, together
-                if (!ok) break;
-                ptx::tc_fence_after_sync();
-                const bool add_in = p.dw_accumulate != 0;
-                {
+                const uint32_t part = chain_part<kPair, kParts>(sched, t);
+                uint32_t done = 0;
+                do {
+                    if (lane == 0) ok = ptx::mbar_wait(ptx::smem_addr(&ctl->acc_full[acc]), (used >> 1) & 1u, abort_flag, status_word);
+                    // the parts of a tile are added in order: the stores of the one before have landed
+                    if (kParts && done != 0 && threadIdx.x == 0) ptx::bulk_wait_all();
+                    ok = !ptx::bar_or<kEpiBarrier, 128>(!ok);            // the four epilogue warps go on, or give up, together
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+                    const bool add_in = (kParts && done != 0) || p.dw_accumulate != 0;
+                    // this part's share of db: accumulator column 128, or with wide tiles the other slot's first
+                    const auto take_bias = [&] {
+                        float v[kEpiChunk];
+                        ptx::tmem_ld_32x16(kNarrow ? taddr + 128u : tmem_base + (acc ^ 1u) * kAccCols + ((uint32_t)(warp * 32) << 16), v);
+                        ptx::tmem_ld_wait();
+                        if (j < C_out) {
+                            float* out = p.db_partial + (int64_t)t.split * C_out + j;
+                            if ((kParts && done != 0) || p.db_accumulate) v[0] += *out;
+                            *out = v[0];
+                        }
+                    };
+                    const bool bias_early = kParts && !kNarrow && !kPair && bias_col && done + part < t.num_kb;
                     // 16 rows of dW x 128 columns at a time: registers -> staging buffer -> one TMA store (or
                     // reduce-add), which clips at the edges of dW.  A buffer is rewritten three chunks later;
                     // the issuing thread has by then waited for all but the newest store to have read theirs.
@@ -781,26 +836,20 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
                             else ptx::tma_store_3d(&map_dw, raw_addr + buf_off, x, y, (int)t.split);
                             ptx::bulk_commit();
                         }
-                    }
-                    if (bias_col) {                                  // accumulator column 128: this piece's share of db
-                        float v[kEpiChunk];
-                        ptx::tmem_ld_32x16(kNarrow ? taddr + 128u : tmem_base + (acc ^ 1u) * kAccCols + ((uint32_t)(warp * 32) << 16), v);
-                        ptx::tmem_ld_wait();
-                        if (j < C_out) {
-                            float* out = p.db_partial + (int64_t)t.split * C_out + j;
-                            if (p.db_accumulate) v[0] += *out;
-                            *out = v[0];
+                        // the next part may start: its sums take the other slot, its bias column the first columns of this one, which
+                        // have been read
+                        if (bias_early && c == 0) {
+                            take_bias();
+                            release(acc ^ 1u);
                         }
                     }
-                }
+                    if (bias_col && !bias_early) take_bias();
+                    if (!bias_wide) release(acc);
+                    next_accumulator();
+                    done += part;
+                } while (kParts && done < t.num_kb);
+                if (!ok) break;
             }
-            // this warp is done with the accumulator: hand it back to the MMA issuer
-            ptx::tc_fence_before_sync();
-            if (lane == 0) {
-                if constexpr (kPair) ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_addr(&ctl->acc_empty[acc]), 0));
-                else ptx::mbar_arrive(ptx::smem_addr(&ctl->acc_empty[acc]));
-            }
-            ++used;
         }
     }
     if (threadIdx.x == 0) ptx::bulk_wait_all();                      // the TMA stores of the dW epilogue have landed
@@ -919,6 +968,17 @@ double estimate_us(const Rates& r, int64_t x_tiles, int64_t x_kb, int64_t w_tile
     return r.fixed + worst + r.mean * all / (double)workers;
 }
 
+// Layers with a side below 128 channels, whose dW is small, are cut into pieces of at most 14 k-blocks, which the reduce launch adds
+// with rounding: within 1e-6 of 64-bit sums (see chain_part; the CUDA cores, which these layers ran on once, stay within 7e-7), as long
+// as a piece for each SM suffices: 132000 rows.  48 -> 2048 with 50176 kept rows is off by 1.4e-5 in the pieces that are fastest, by
+// 8.7e-7 so (71 -> 88 us; 64 -> 256 21 -> 22, 96 -> 384 26 -> 30, 256 -> 64 21 -> 27).
+int64_t fewest_pieces(int64_t w_kb, int64_t C_in, int64_t C_out) {
+    constexpr int64_t kChain = 14;
+    if (C_in >= 128 && C_out >= 128) return 1;
+    const int64_t n = (w_kb + kChain - 1) / kChain;
+    return n < 1 ? 1 : n > kNumSMs ? kNumSMs : n;
+}
+
 struct PlanKey {
     int64_t cap, ci, co;
     bool dx;
@@ -992,6 +1052,7 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
             // each kept row of dY once.  The groups are sized by the bytes each has to pull into its SMs: the
             // gathered rows of dY and the dense operand once per tile, plus the dX rows written (the row count of
             // dX is not known here; twice the kept rows is assumed, the paper's usual keep ratio).
+            const int64_t fewest = fewest_pieces(w_kb, C_in, C_out);
             const double t_flop = 4.0 * (double)M_keep_cap * (double)C_in * (double)C_out / 1.4e15;
             const double t_mem = 2.0 * (double)M_keep_cap * (double)(2 * C_in + C_out) / 6.5e12;
             bool role_split = false;
@@ -1009,7 +1070,7 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
                 // 4.3 (50176 of 256 -> 256) 38.7 -> 31.0, 3.3 (12544 of 768 -> 192) 26.1 -> 23.5, 2.8 (30000 of 128 -> 512) 23.0 ->
                 // 20.4, 2.4 (16000 of 512 -> 128) 22.4 -> 20.4; 2.3 (6272 of 1024 -> 256) 19.4 -> 19.8, 2.2 (12544 of 192 -> 768)
                 // 20.2 -> 22.2; out of line 3.4 (40000 of 64 -> 256) 15.5 -> 16.3.
-                if (sp >= 2 && w_kb / sp >= 8 && x_rtiles >= sp && w_tiles * sp <= kNumSMs - 16 &&
+                if (sp >= 2 && sp >= fewest && w_kb / sp >= 8 && x_rtiles >= sp && w_tiles * sp <= kNumSMs - 16 &&
                     3 * x_tiles >= 7 * (kNumSMs - w_tiles * sp)) {
                     pl.splits = (int)sp;
                     pl.dw_ctas = (int)(w_tiles * sp);
@@ -1023,10 +1084,11 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
                     if (max_s < 1) max_s = 1;
                     // the search walks every tile: with very many tiles any cut balances, so bound the work
                     while (max_s > 1 && (x_tiles + w_tiles * max_s) * max_s > (1 << 22)) max_s /= 2;
-                    int best = 1;
-                    for (int64_t sp = 1; sp <= max_s; ++sp) {
+                    if (max_s < fewest) max_s = fewest;
+                    int best = (int)fewest;
+                    for (int64_t sp = fewest; sp <= max_s; ++sp) {
                         const double c = estimate_us(rates, x_tiles, x_kb, w_tiles, w_kb, sp, C_in * C_out, pair ? kNumSMs / 2 : kNumSMs);
-                        if (sp == 1 || c < *cost * 0.995) { *cost = c; best = (int)sp; }
+                        if (sp == fewest || c < *cost * 0.995) { *cost = c; best = (int)sp; }
                     }
                     return best;
                 };
@@ -1051,35 +1113,30 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
     return pl;
 }
 
-template <int BN, int DEPTH, bool PACKED, bool PAIR, bool OUT_IN>
+template <int BN, int DEPTH, bool PACKED, bool PAIR, bool OUT_IN, bool PARTS>
 cudaError_t launch_fused_variant(dim3 grid, cudaStream_t stream, const CUtensorMap& map_w, const CUtensorMap& map_x,
                                  const CUtensorMap& map_dw, const TcParams& prm) {
-    const cudaError_t opt = opt_in_dynamic_smem<tc_backward_kernel<BN, BN, DEPTH, PACKED, PAIR, OUT_IN>>((int)kSmemBytes);
+    constexpr auto kernel = tc_backward_kernel<BN, BN, DEPTH, PACKED, PAIR, OUT_IN, PARTS>;
+    const cudaError_t opt = opt_in_dynamic_smem<kernel>((int)kSmemBytes);
     if (opt != cudaSuccess) return opt;
-    if constexpr (PAIR)
-        return launch_pdl_cluster(tc_backward_kernel<BN, BN, DEPTH, PACKED, PAIR, OUT_IN>, grid, dim3(kTcThreads), kSmemBytes, 2u, stream,
-                                  map_w, map_x, map_dw, prm);
-    else
-        return launch_pdl(tc_backward_kernel<BN, BN, DEPTH, PACKED, PAIR, OUT_IN>, grid, dim3(kTcThreads), kSmemBytes, stream, map_w,
-                          map_x, map_dw, prm);
-}
-
-template <int BN, int DEPTH, bool PAIR, bool OUT_IN>
-cudaError_t launch_fused_depth(dim3 grid, cudaStream_t stream, const CUtensorMap& map_w, const CUtensorMap& map_x,
-                               const CUtensorMap& map_dw, const TcParams& prm) {
-    const bool packed = prm.dy_rows == nullptr || prm.dx_rows == nullptr;
-    return packed ? launch_fused_variant<BN, DEPTH, true, PAIR, OUT_IN>(grid, stream, map_w, map_x, map_dw, prm)
-                  : launch_fused_variant<BN, DEPTH, false, PAIR, OUT_IN>(grid, stream, map_w, map_x, map_dw, prm);
+    if constexpr (PAIR) return launch_pdl_cluster(kernel, grid, dim3(kTcThreads), kSmemBytes, 2u, stream, map_w, map_x, map_dw, prm);
+    else return launch_pdl(kernel, grid, dim3(kTcThreads), kSmemBytes, stream, map_w, map_x, map_dw, prm);
 }
 
 template <int BN, bool PAIR>
 cudaError_t launch_fused(dim3 grid, cudaStream_t stream, const CUtensorMap& map_w, const CUtensorMap& map_x,
-                         const CUtensorMap& map_dw, const TcParams& prm, bool deep_side_queue, bool out_in) {
-    if (out_in)
-        return deep_side_queue ? launch_fused_depth<BN, 16, PAIR, true>(grid, stream, map_w, map_x, map_dw, prm)
-                               : launch_fused_depth<BN, 8, PAIR, true>(grid, stream, map_w, map_x, map_dw, prm);
-    return deep_side_queue ? launch_fused_depth<BN, 16, PAIR, false>(grid, stream, map_w, map_x, map_dw, prm)
-                           : launch_fused_depth<BN, 8, PAIR, false>(grid, stream, map_w, map_x, map_dw, prm);
+                         const CUtensorMap& map_dw, const TcParams& prm, bool deep_side_queue, bool out_in, bool parts) {
+    const bool packed = prm.dy_rows == nullptr || prm.dx_rows == nullptr;
+    const auto go = [&](auto deep, auto is_packed, auto is_out_in, auto has_parts) {
+        return launch_fused_variant<BN, decltype(deep)::value ? 16 : 8, decltype(is_packed)::value, PAIR, decltype(is_out_in)::value,
+                                    decltype(has_parts)::value>(grid, stream, map_w, map_x, map_dw, prm);
+    };
+    const auto pick = [](bool v, auto f) { return v ? f(std::true_type{}) : f(std::false_type{}); };
+    return pick(deep_side_queue, [&](auto deep) {
+        return pick(packed, [&](auto pk) {
+            return pick(out_in, [&](auto oi) { return pick(parts, [&](auto pt) { return go(deep, pk, oi, pt); }); });
+        });
+    });
 }
 
 }  // namespace
@@ -1200,9 +1257,11 @@ sbp_status launch_tc_backward(const void* X_keep, const void* dY, const void* W,
         deep_side = loads / 8.0 * 1.3 > 0.6 * loop_us;
     }
     cudaError_t e;
-    if (pl.pair) e = launch_fused<256, true>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in);
-    else if (pl.bnx == 256) e = launch_fused<256, false>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in);
-    else e = launch_fused<128, false>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in);
+    const int64_t piece = want_dw ? ((M_keep_cap + kBK - 1) / kBK + pl.splits - 1) / pl.splits : 0;
+    const bool parts = piece > whole_piece(pl.pair, pl.dw_ctas > 0);
+    if (pl.pair) e = launch_fused<256, true>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in, parts);
+    else if (pl.bnx == 256) e = launch_fused<256, false>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in, parts);
+    else e = launch_fused<128, false>(grid, stream, map_w, map_x, map_dw, prm, deep_side, w_out_in, parts);
     if (e != cudaSuccess) return SBP_ERR_CUDA;
     const bool reduce_dw = want_dw && pl.splits > 1, reduce_db = db != nullptr && !db_direct;
     cudaError_t r = cudaSuccess;
