@@ -66,7 +66,6 @@ constexpr int kBM = 128;                 // accumulator rows per tile (= TMEM la
 constexpr int kBK = 64;                  // reduction depth per stage: 64 bf16 = one 128-byte swizzle row
 constexpr uint32_t kUmmaK = 16;          // reduction depth of one tcgen05.mma for 16-bit operands
 constexpr uint32_t kRowBytes = 128;      // bytes per swizzled smem row
-constexpr uint32_t kAtomBytes = 1024;    // 8 rows x 128 B: one swizzle atom
 constexpr uint32_t kBlock64Bytes = 64 * kRowBytes;   // a 64-row slab (MN-major operands: one 64-wide block)
 constexpr int kStages = 4;               // ring depth with 256-wide tiles (48 KB stages)
 constexpr int kStagesNarrow = 6;         // ... when both tile kinds are 128 wide (32 KB stages): same 192 KB, half as many again in flight

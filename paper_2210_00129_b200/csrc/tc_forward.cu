@@ -28,7 +28,6 @@ constexpr int kBM = 128;                 // accumulator rows per tile (= TMEM la
 constexpr int kBK = 64;                  // reduction depth per stage: 64 bf16 = one 128-byte swizzle row
 constexpr uint32_t kUmmaK = 16;
 constexpr uint32_t kRowBytes = 128;
-constexpr uint32_t kAtomBytes = 1024;
 constexpr uint32_t kBlock64Bytes = 64 * kRowBytes;
 constexpr int kStages = 4;
 constexpr uint32_t kABytes = kBM * kRowBytes;        // 16 KB
