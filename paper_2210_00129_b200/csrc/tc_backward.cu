@@ -933,7 +933,8 @@ struct Rates {
 constexpr Rates kRatesSingle = {0.364, 0.308, 3.75, 5.30, 1.01, 0.00, 2.64, 2.91, 0.040, 0.254};
 constexpr Rates kRatesPair = {0.271, 0.239, 3.92, 2.95, 0.40, 0.80, 5.51, 0.00, 0.084, 0.600};
 constexpr Rates kRatesNarrow = {0.155, 0.306, 1.40, 2.26, 1.46, 0.03, 3.28, 2.28, 0.101, 0.103};
-double estimate_us(const Rates& r, int64_t x_tiles, int64_t x_kb, int64_t w_tiles, int64_t w_kb, int64_t splits, int64_t dw_elems, int64_t workers) {
+double estimate_us(const Rates& r, int64_t x_tiles, int64_t x_kb, int64_t w_tiles, int64_t w_kb, int64_t splits, int64_t dw_elems, int64_t workers,
+                   double limit = -1.0) {
     const int64_t kb_per = (w_kb + splits - 1) / splits;
     const int64_t w_pieces = w_tiles * splits;
     const int64_t total = x_tiles + w_pieces;
@@ -941,6 +942,13 @@ double estimate_us(const Rates& r, int64_t x_tiles, int64_t x_kb, int64_t w_tile
     const int64_t G = total < workers ? total : workers;
     const bool w_first = kb_per >= x_kb;
     const int64_t first = w_first ? w_pieces : x_tiles;
+    const double x_tile = (double)x_kb * r.dx_kb > r.dx_min ? (double)x_kb * r.dx_kb : r.dx_min;
+    const double added = splits > 1 ? r.reduce + r.reduce_mb * (double)(splits + 1) * (double)dw_elems * 4e-6 : 0.0;
+    if (limit >= 0.0) {                                     // the longest block is no shorter than the mean one
+        const double work = (double)x_tiles * x_tile + (double)w_pieces * r.dw_tile + (double)(w_tiles * w_kb) * r.dw_kb;
+        const double least = r.fixed + work / (double)G + added + r.mean * work / (double)workers;
+        if (least > limit * (1.0 + 1e-9)) return least;
+    }
     double worst = 0.0, all = 0.0;
     for (int64_t b = 0; b < G; ++b) {
         double sum = 0.0, tail = 0.0;
@@ -956,15 +964,14 @@ double estimate_us(const Rates& r, int64_t x_tiles, int64_t x_kb, int64_t w_tile
                 sum += r.dw_kb * (double)n + r.dw_tile;
                 tail = r.dw_tail;
             } else {
-                sum += (double)x_kb * r.dx_kb > r.dx_min ? (double)x_kb * r.dx_kb : r.dx_min;
+                sum += x_tile;
                 tail = r.dx_tail;
             }
         }
         if (sum + tail > worst) worst = sum + tail;
         all += sum;
     }
-    if (splits > 1) worst += r.reduce + r.reduce_mb * (double)(splits + 1) * (double)dw_elems * 4e-6;
-    return r.fixed + worst + r.mean * all / (double)workers;
+    return r.fixed + (worst + added) + r.mean * all / (double)workers;
 }
 
 // Layers with a side below 128 channels, whose dW is small, are cut into pieces of at most 14 k-blocks, which the reduce launch adds
@@ -1086,7 +1093,8 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
                     if (max_s < fewest) max_s = fewest;
                     int best = (int)fewest;
                     for (int64_t sp = fewest; sp <= max_s; ++sp) {
-                        const double c = estimate_us(rates, x_tiles, x_kb, w_tiles, w_kb, sp, C_in * C_out, pair ? kNumSMs / 2 : kNumSMs);
+                        const double c = estimate_us(rates, x_tiles, x_kb, w_tiles, w_kb, sp, C_in * C_out, pair ? kNumSMs / 2 : kNumSMs,
+                                                     sp == fewest ? -1.0 : *cost * 0.995);
                         if (sp == fewest || c < *cost * 0.995) { *cost = c; best = (int)sp; }
                     }
                     return best;
