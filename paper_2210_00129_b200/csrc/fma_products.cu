@@ -454,7 +454,7 @@ __device__ __forceinline__ void dx_tile(ProductShared<BN>& sh, const BackwardPar
 
 // Zeros of the dropped rows: every warp of the blocks that do this takes an equal share of the rows of dX.  Blocks of their own:
 // in front of a dX tile the search and the stores delayed a small layer's only wave by 2 - 3 us.  Rows of at most four vectors go 8,
-// 16 or 32 to a store instruction (fp32 4 -> 4 channels, 157 of 3136 rows kept: a row an instruction 57 us, now 7.2).
+// 16 or 32 to a store instruction (fp32 4 -> 4 channels, 157 of 3136 rows kept: a row an instruction 57 us, now 9.1).
 template <typename T, int kThreads>
 __device__ __forceinline__ void zero_rows(const BackwardParams<T>& p, int block, int64_t M_keep) {
     constexpr int kWarps = kThreads / 32;

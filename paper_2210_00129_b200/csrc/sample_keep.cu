@@ -7,7 +7,7 @@
 // warp then owns a contiguous stretch of positions, so one scan of the warps' counts places every kept position.  (Should
 // a bin ever hold more words than the list, the next eight bits are taken, as often as needed.)  Four passes of eight bits
 // and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.5 us
-// and 3.7 us (the words are drawn while the kernel before drains).
+// and 3.1 us (the words are drawn while the kernel before drains).
 // Grid mode: everything has a closed form - a sample's offset from the counts of the samples before it, a kept position's place
 // from the kept positions in the rows above and to its left - so each block writes a stretch of one map without a scan, and a
 // large map is spread over as many blocks as the samples leave room for (a predicate and an ordered compaction by one block a

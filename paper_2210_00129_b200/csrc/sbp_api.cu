@@ -21,8 +21,8 @@ inline bool ratio_ok(double r) { return r > 0.0 && r <= 1.0; }   // false for Na
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// scratch for the bias sums: the stand-alone kernel's row splits, or one partial row per SM when the
-// sums ride along in the tensor-core kernel
+// scratch for the bias sums: the stand-alone kernel's row splits, or, when the sums ride along in the tensor-core kernel, one
+// partial row per share of the kept rows or per piece of a dW tile (as many as SMs at most)
 inline size_t db_scratch_bytes(sbp_dtype dt, int64_t M_keep_cap, int64_t C_out) {
     const size_t a = db_workspace_bytes(dt, M_keep_cap, C_out, kDbMaxSplits);
     const size_t b = (size_t)kNumSMs * (size_t)C_out * sizeof(float);
@@ -36,7 +36,8 @@ inline bool use_tensor_cores(sbp_dtype dt, uint32_t flags, int64_t M, int64_t M_
 // Weights stored [C_out, C_in]: whether the products read W and write dW in place, or work on transposed copies in the
 // workspace.  In place saves two launches and 12 bytes a weight at any size (2000 rows, half of them kept, 368 x 368 bf16:
 // 12.7 us against 16.5 us with copies; 360 x 360 with copies: 16.6 us).  The line is not drawn for speed: the number of
-// kernels that sbp_linear_backward_kernel_count gives for small weights, two transposes among them, is a fixed answer.
+// kernels that sbp_linear_backward_kernel_count gives for small weights, two transposes among them, is a fixed answer.  (Both
+// sides give the same numbers; moving the line needs that answer to change first.)
 inline bool out_in_direct(int64_t C_in, int64_t C_out) { return C_in * C_out >= (1 << 17); }
 
 }  // namespace

@@ -21,8 +21,9 @@
 // was measured at ~45 ns of issue time per instruction per SM whatever it fetches - far too slow
 // to feed a tile - and is not used.  Every wait is bounded and reports through the status word.
 // Four side warps work next to the pipeline: they write the zeros of the dropped rows in the block's
-// share of dX (so every row of dX is written exactly once and no memset pass is needed), then sum the block's share of the kept rows of dY column-wise for the bias gradient
-// and leave one partial row per block for a fixed-order reduce.  The row maps are compile-time
+// share of dX (so every row of dX is written exactly once and no memset pass is needed), then, where db is
+// not a column of the dW tiles, sum a strip of columns of dY over a share of the kept rows, which leaves one
+// partial row per share for a fixed-order reduce.  The row maps are compile-time
 // variants: keep_rows on both sides, or identity on either side for gradients kept packed between
 // chained layers (Sec. 3.3.1).
 #include <map>
@@ -344,7 +345,7 @@ tc_backward_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_const
     // output column of the dW tiles: db[j] = sum_m dY[m, j] * 1.  The "column of ones" is a constant 64 x 64 operand
     // block (MN-major, only its first column set) kept in the third staging buffer; a second, 16-wide MMA per k-step
     // multiplies it with the same gathered rows of dY.  Wide layers have no spare columns in a slot, but under the role
-    // split a dW block runs a single piece and never touches the second slot, so the column goes there.
+    // split a dW block runs a single piece, in one part or two, and the column goes to the slot that the part does not use.
     const uint32_t dw_bufs = p.db_from_mma ? kEpiBufs - 1 : kEpiBufs;   // staging buffers left to the dW epilogue
     const uint32_t ones_off = (ring - raw_addr) + kRingBytes + 256 + kBiasSmemBytes + (kEpiBufs - 1) * kEpiBufBytes;
     if (p.db_from_mma) {
@@ -1071,7 +1072,8 @@ Plan make_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bo
                 const double target = bytes_w / (bytes_w + bytes_x) * (double)kNumSMs;
                 int64_t sp = (int64_t)(target / (double)w_tiles + 0.5);
                 const int64_t x_rtiles = (M_keep_cap + kBM - 1) / kBM;
-                // worth it only with enough dX tiles per dX block to balance (a short list leaves the groups uneven): 7/3 of them.
+                // worth it only with enough dX tiles per dX block to balance (a short list leaves the groups uneven): 7/3 of them, a fit to
+                // the timings below and not a rule that they prove - the two sides lie close together around it, and one is out of line.
                 // dW + db + dX with one list -> split, by tiles per block: 6.9 (66800 kept rows of 128 -> 512) 39.1 -> 33.7 us,
                 // 4.3 (50176 of 256 -> 256) 38.7 -> 31.0, 3.3 (12544 of 768 -> 192) 26.1 -> 23.5, 2.8 (30000 of 128 -> 512) 23.0 ->
                 // 20.4, 2.4 (16000 of 512 -> 128) 22.4 -> 20.4; 2.3 (6272 of 1024 -> 256) 19.4 -> 19.8, 2.2 (12544 of 192 -> 768)

@@ -366,7 +366,8 @@ cudaError_t launch_forward(dim3 grid, cudaStream_t stream, const CUtensorMap& ma
 }
 
 // Pairs where the two-SM instructions save more than a cluster launch and the coarser tile list cost: from about 1800 k-blocks
-// of 128 x 256 tiles on, and where the pairs' last wave is not much emptier.  Single blocks -> pairs on B200: 12544 x 768 ->
+// of 128 x 256 tiles on (a fit: 1776 of one shape lose 2 %, 1788 of another gain 6 %), and where the pairs' last wave is not much
+// emptier.  Single blocks -> pairs on B200: 12544 x 768 ->
 // 3072 52.9 -> 47.6 us (1.24 PFLOP/s), 12544 x 3072 -> 768 46.9 -> 44.1, 25088 x 768 -> 2304 79.1 -> 70.6, 3136 x 1024 -> 4096
 // 25.3 -> 23.6, 19072 x 768 -> 256 (1788 k-blocks) 15.7 -> 14.8; below the line 9472 x 768 -> 512 10.8 -> 11.0, 3136 x 768 ->
 // 768 (900) 8.9 -> 9.4, 512 x 768 -> 768 8.3 -> 8.6.
