@@ -6,8 +6,8 @@
 // bin's words (about N / 256) are collected and each is ranked against the others, which gives the threshold word; each
 // warp then owns a contiguous stretch of positions, so one scan of the warps' counts places every kept position.  (Should
 // a bin ever hold more words than the list, the next eight bits are taken, as often as needed.)  Four passes of eight bits
-// and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.5 us
-// and 3.1 us (the words are drawn while the kernel before drains).
+// and a scan for every 2048 positions took 6.1 us for 128 x 196 positions and 16.6 us for 2 x 66800 back to back; now 1.1 us
+// and 2.7 us (the words are drawn while the kernel before drains).
 // Grid mode: everything has a closed form - a sample's offset from the counts of the samples before it, a kept position's place
 // from the kept positions in the rows above and to its left - so each block writes a stretch of one map without a scan, and a
 // large map is spread over as many blocks as the samples leave room for (a predicate and an ordered compaction by one block a
@@ -525,8 +525,8 @@ cudaError_t launch_sample_keep(int mode, int grid_family, int64_t B, int64_t H, 
     if (mode == SBP_MASK_RANDOM) {
         // large maps with few samples: spread each sample over a cluster so that more SMs take part
         if (N > 8192 && B * 8 <= 4 * kNumSMs) {
-            // 1024 threads for up to three samples, whose clusters find room beside the kernel before: 2 x 66800 positions 4.2 ->
-            // 3.7 us back to back, 3 x 4.3 -> 3.8, but 4 x 4.5 -> 5.4 and 8 x 5.5 -> 10.4
+            // 1024 threads for up to three samples, whose clusters find room beside the kernel before: 1, 2 and 3 x 66800 positions
+            // 2.95 -> 2.63, 3.06 -> 2.70 and 3.19 -> 3.32 us back to back, 3 x 200000 6.2 -> 5.1, but 8 x 66800 4.1 -> 9.0
             if (N > 32768 && B <= 3) return launch_random_sampler<8, 1024>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
             if (N > 32768) return launch_random_sampler<8, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
             if (N > 16384) return launch_random_sampler<4, 512>(B, stream, N, K, k0, k1, step, first_sample, share_mask, keep_rows, keep_offsets);
