@@ -65,7 +65,7 @@ enum {
     SBP_FLAG_SHARE_MASK = 1,  /* every sample of the call uses sample 0's mask (one mask per iteration, Supp. A.4) */
     SBP_FLAG_ACCUMULATE = 2,  /* dW += and db += instead of overwrite (gradient accumulation) */
     SBP_FLAG_VALIDATE = 4,    /* check keep_rows on the device before use; result in the status word */
-    SBP_FLAG_PLAIN_FMA = 8,   /* bf16 only: use the CUDA-core FMA kernels instead of the tensor-core ones */
+    SBP_FLAG_PLAIN_FMA = 8,   /* use the CUDA-core FMA kernels instead of the tensor-core ones */
     SBP_FLAG_DY_COMPACT = 16, /* dY holds only the kept rows, packed: [M_keep_cap, C_out] (chained layers, Sec. 3.3.1) */
     SBP_FLAG_DX_COMPACT = 32, /* dX receives only the kept rows, packed: [M_keep_cap, C_in]; no zero rows are written */
     SBP_FLAG_W_OUT_IN = 64,   /* W, and dW, are stored [C_out, C_in] (the usual layout of framework linear layers) */
@@ -158,7 +158,8 @@ sbp_status sbp_forward_cache(sbp_dtype dt, const void* X /* dev */, int64_t M, i
  * cache: keep_rows and M_keep_dev are then ignored); otherwise it is what
  * sbp_forward_cache would produce, written by the same launch so that X is read
  * from memory once.  SBP_BF16: bf16 inputs and output, fp32 accumulation on the
- * tensor cores, one rounding of (sum + bias) to bf16.  SBP_F32: fp32 FMA arithmetic.
+ * tensor cores, one rounding of (sum + bias) to bf16.  SBP_F32: fp32 precision (see
+ * sbp_linear_backward).
  * C_in and C_out must be multiples of 8 (bf16) / 4 (fp32), else SBP_ERR_UNSUPPORTED.
  * flags: SBP_FLAG_PLAIN_FMA, SBP_FLAG_W_OUT_IN (W is [C_out, C_in]; read in place, no
  * copy) or 0.  status_word as for sbp_linear_backward.
@@ -208,7 +209,10 @@ size_t sbp_linear_backward_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_ke
  *
  * SBP_BF16: inputs bf16, products accumulated in fp32 on the tensor cores (relative
  * error of dW against 64-bit sums: 1e-7 to 1e-5, growing with the number of kept
- * rows), dX rounded to bf16 (nearest even).  SBP_F32: plain fp32 FMA arithmetic.
+ * rows), dX rounded to bf16 (nearest even).  SBP_F32: fp32 FMA arithmetic, or, for
+ * products large enough, six tensor-core products of operands in three bf16 parts each,
+ * summed in fp32: no further from 64-bit sums than the FMAs (1e-7 against 2e-7 to 7e-7),
+ * infinities and NaNs as the FMAs have them; SBP_FLAG_PLAIN_FMA keeps to the FMAs.
  * C_in and C_out must be multiples of 8 (bf16) / 4 (fp32), else SBP_ERR_UNSUPPORTED.
  *
  * flags: SBP_FLAG_ACCUMULATE adds into dW and db; SBP_FLAG_VALIDATE first checks

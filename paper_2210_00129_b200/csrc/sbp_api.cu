@@ -33,6 +33,11 @@ inline bool use_tensor_cores(sbp_dtype dt, uint32_t flags, int64_t M, int64_t M_
     return dt == SBP_BF16 && !(flags & SBP_FLAG_PLAIN_FMA) && tc_shapes_supported(M, M_keep_cap, C_in, C_out);
 }
 
+// fp32 layers: the tensor cores take the products in three bf16 parts each where that is quicker than the CUDA cores
+inline bool use_split(sbp_dtype dt, uint32_t flags, int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
+    return dt == SBP_F32 && !(flags & SBP_FLAG_PLAIN_FMA) && split_backward_supported(M_keep_cap, C_in, C_out);
+}
+
 // Weights stored [C_out, C_in]: whether the products read W and write dW in place, or work on transposed copies in the
 // workspace.  In place saves two launches and 12 bytes a weight at any size (2000 rows, half of them kept, 368 x 368 bf16:
 // 12.7 us against 16.5 us with copies; 360 x 360 with copies: 16.6 us).  The line is not drawn for speed: the number of
@@ -168,8 +173,10 @@ sbp_status sbp_linear_forward(sbp_dtype dt, const void* X, const void* W, const 
             return SBP_ERR_CUDA;
         return SBP_OK;
     }
-    if (launch_fma_forward(dt, X, W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, Y, status_word, stream) !=
-        cudaSuccess)
+    const bool split = dt == SBP_F32 && !(flags & SBP_FLAG_PLAIN_FMA) && split_forward_supported(M, C_in, C_out);
+    if ((split ? launch_split_forward((const float*)X, (const float*)W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, (float*)Y,
+                                      status_word, stream)
+               : launch_fma_forward(dt, X, W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, Y, status_word, stream)) != cudaSuccess)
         return SBP_ERR_CUDA;
     if (X_keep != nullptr &&
         launch_gather_rows(X, C_in * (dt == SBP_BF16 ? 2 : 4), keep_rows, M_keep_dev, M_keep_cap, X_keep, stream) !=
@@ -200,6 +207,10 @@ size_t base_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_keep_cap, int64_t
     size_t dw_part = fma_dw_workspace_bytes(dt, M_keep_cap, C_in, C_out);
     if (dt == SBP_BF16 && tc_shapes_supported(M, M_keep_cap, C_in, C_out)) {
         const size_t t = tc_dw_workspace_bytes(M_keep_cap, C_in, C_out);
+        if (t > dw_part) dw_part = t;
+    }
+    if (dt == SBP_F32 && split_backward_supported(M_keep_cap, C_in, C_out)) {
+        const size_t t = split_workspace_bytes(M_keep_cap, C_in, C_out);
         if (t > dw_part) dw_part = t;
     }
     return db_part + align_up(dw_part, 256) + 256;
@@ -264,6 +275,11 @@ sbp_status backward_direct(sbp_dtype dt, bool w_out_in, bool fresh_dw, const voi
                                                 dw_accumulate, dX, db_rides ? db : nullptr, accumulate, w_out_in, ws_dw, ws_db,
                                                 status_word, stream);
         if (s != SBP_OK) return s;
+    } else if ((dW != nullptr || dX != nullptr) && use_split(dt, flags, M_keep_cap, C_in, C_out)) {
+        if (launch_split_backward((const float*)X_keep, (const float*)dY, (const float*)W, w_out_in, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap,
+                                  C_in, C_out, dW, db_rides ? db : nullptr, dw_accumulate, accumulate, (float*)dX, ws_dw, status_word,
+                                  stream) != cudaSuccess)
+            return SBP_ERR_CUDA;
     } else if (dW != nullptr || dX != nullptr) {
         if (launch_fma_backward(dt, X_keep, dY, W, w_out_in, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap, C_in, C_out, dW,
                                 db_rides ? db : nullptr, dw_accumulate, accumulate, dX, ws_dw, status_word, stream) != cudaSuccess)
@@ -329,6 +345,8 @@ int sbp_linear_backward_kernel_count(sbp_dtype dt, int64_t M, int64_t M_keep_cap
     if (want_db && !db_rides) n += 2;                      // strip partials + fixed-order reduce
     if (tc) return n + tc_backward_kernel_count(M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0, db_rides,
                                                 (flags & SBP_FLAG_DY_COMPACT) != 0);
+    if (use_split(dt, flags, M_keep_cap, C_in, C_out))
+        return n + split_backward_kernel_count(direct, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0);
     return n + fma_backward_kernel_count(dt, direct, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0);
 }
 

@@ -170,6 +170,18 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
                                 int64_t C_out, float* dW, float* db, bool dw_accumulate, bool db_accumulate, void* dX,
                                 float* workspace, const int32_t* status_word, cudaStream_t stream);
 
+// the same products of fp32 layers on the tensor cores, each operand as a sum of three bf16 numbers
+bool   split_forward_supported(int64_t M, int64_t C_in, int64_t C_out);
+bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
+size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
+int    split_backward_kernel_count(bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
+cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,
+                                 float* Y, int32_t* status_word, cudaStream_t stream);
+cudaError_t launch_split_backward(const float* X_keep, const float* dY, const float* W, bool w_out_in, const int32_t* dy_rows,
+                                  const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
+                                  int64_t C_out, float* dW, float* db, bool dw_accumulate, bool db_accumulate, float* dX, float* workspace,
+                                  int32_t* status_word, cudaStream_t stream);
+
 // transposes for weights in the [C_out, C_in] layout
 cudaError_t launch_transpose(int elem_bytes, const void* in, void* out, int64_t rows, int64_t cols,
                              const int32_t* status_word, cudaStream_t stream);

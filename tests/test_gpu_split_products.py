@@ -1,0 +1,111 @@
+"""fp32 products on the tensor cores (operands in three bf16 parts) at the edges of their tiles, stages and pieces: against the oracle, and
+no further from it than fp32 sums are; infinities and NaNs as the plain products have them."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2210_00129_b200 as sbp
+from paper_2210_00129_b200 import synth
+from gpu_harness import dev, host, run_forward_cache
+
+pytestmark = pytest.mark.gpu
+
+# A stage of 64 is off by at most 4 cuts of 2^-23 of its running sum (a quarter of that on average, and in proportion), the stages add up
+# with roundings of 2^-24: sqrt(n / 128) * 2.4e-8 for a depth of n.  1e-7 + 2e-7 up to 8000.
+REL = 3e-7
+
+
+def _rel(got, want):
+    return float(np.linalg.norm(host(got).astype(np.float64) - want) / np.linalg.norm(want))
+
+
+def _elements(got, want):
+    scale = float(np.sqrt(np.mean(want * want)))
+    return float((np.abs(host(got).astype(np.float64) - want) / np.maximum(np.abs(want), scale)).max())
+
+
+def _backward(X_keep, dY, W, rows, count, M, cap, C_in, C_out, flags, fill):
+    nb = sbp.sbp_linear_backward_workspace_bytes(sbp.SBP_F32, M, cap, C_in, C_out)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    dW = torch.full_like(W, fill)
+    db = torch.full((C_out,), fill, device="cuda")
+    dX = torch.full((M, C_in), float("nan"), device="cuda")
+    sbp.sbp_linear_backward(sbp.SBP_F32, X_keep, dY, W, rows, count, M, cap, C_in, C_out, dW, db, dX, flags, ws, nb, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    return dW, db, dX
+
+
+@pytest.mark.parametrize("M,kept,padding,C_in,C_out,out_in,accumulate", [
+    (1027, 513, 0, 260, 388, False, False),          # one row beyond two row tiles; 4 columns beyond two tiles; depth 4 beyond 6 stages
+    (900, 512, 0, 256, 384, False, True),            # full tiles; sums into dW and db
+    (1500, 700, 57, 508, 516, True, True),           # rows past the count known on the device; weights [C_out, C_in]
+    (6000, 5000, 0, 132, 640, False, False),         # dW cut into pieces
+    (4000, 4000, 3000, 384, 132, False, False),      # pieces without rows
+    (2000, 1100, 0, 1028, 128, True, False),
+])
+def test_backward(M, kept, padding, C_in, C_out, out_in, accumulate):
+    X, Wt, dY = synth.layer_inputs("f32", M, C_in, C_out, 91)
+    keep = np.sort(np.random.default_rng(5).permutation(M)[:kept]).astype(np.int32)
+    valid = keep[:kept - padding]
+    rows = torch.from_numpy(keep).cuda()
+    count = torch.tensor([len(valid)], dtype=torch.int32, device="cuda") if padding else None
+    Xk = run_forward_cache("f32", dev(X, "f32"), rows, kept, count)
+    want = oracle.linear_backward(synth.to_f64(X[valid], "f32"), synth.to_f64(dY, "f32"), synth.to_f64(Wt, "f32"), valid)
+    fill = 0.25 if accumulate else float("nan")
+    W = dev(np.ascontiguousarray(Wt.T) if out_in else Wt, "f32")
+    flags = (sbp.SBP_FLAG_W_OUT_IN if out_in else 0) | (sbp.SBP_FLAG_ACCUMULATE if accumulate else 0)
+    dW, db, dX = _backward(Xk, dev(dY, "f32"), W, rows, count, M, kept, C_in, C_out, flags, fill)
+    add = fill if accumulate else 0.0
+    for got, exact in ((dW.t() if out_in else dW, want["dW"] + add), (db, want["db"] + add), (dX, want["dX"])):
+        assert _rel(got.contiguous(), exact) <= REL and _elements(got.contiguous(), exact) <= 1e-5
+    dropped = np.setdiff1d(np.arange(M), valid)
+    assert not host(dX)[dropped].view(np.uint8).any()
+
+
+@pytest.mark.parametrize("M,C_in,C_out,out_in", [(3000, 260, 388, False), (3000, 260, 388, True), (2561, 1028, 900, False), (8192, 512, 128, True)])
+def test_forward(M, C_in, C_out, out_in):
+    X, Wt, _ = synth.layer_inputs("f32", M, C_in, C_out, 92)
+    bias = np.linspace(-1, 1, C_out, dtype=np.float32)
+    want = oracle.linear_forward(synth.to_f64(X, "f32"), synth.to_f64(Wt, "f32"), bias)
+    Y = torch.full((M, C_out), float("nan"), device="cuda")
+    W = dev(np.ascontiguousarray(Wt.T) if out_in else Wt, "f32")
+    sbp.sbp_linear_forward(sbp.SBP_F32, dev(X, "f32"), W, torch.from_numpy(bias).cuda(), M, C_in, C_out, Y, flags=sbp.SBP_FLAG_W_OUT_IN if out_in else 0)
+    torch.cuda.synchronize()
+    assert _rel(Y, want) <= REL and _elements(Y, want) <= 1e-5
+
+
+@pytest.mark.parametrize("out_in", [False, True])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_not_finite(out_in, accumulate):
+    """Infinite, NaN and nearly infinite inputs (3.4e38 rounds to infinity in bf16) give what the CUDA-core products give."""
+    M, kept, C_in, C_out = 1500, 1100, 512, 384
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    X, dY, W = (torch.randn(*s, device="cuda", generator=g) for s in ((kept, C_in), (M, C_out), (C_out, C_in) if out_in else (C_in, C_out)))
+    inf, big = float("inf"), 3.4e38
+    rows = torch.arange(0, kept, dtype=torch.int32, device="cuda")
+    X[5, 3], X[7, 100], dY[11, 2], dY[12, 5], dY[500, 200] = inf, 1.0, -inf, float("nan"), big
+    dY[40] = 0.0
+    dY[40, 1] = inf
+    W[4, 5], W[8, 9], W[300, 17] = big, inf, -inf
+    W[2] = 0.0
+    X[:, 20] = 0.0
+    X[600, 20] = big
+    flags = (sbp.SBP_FLAG_W_OUT_IN if out_in else 0) | (sbp.SBP_FLAG_ACCUMULATE if accumulate else 0)
+    run = lambda extra: _backward(X, dY, W, rows, None, M, kept, C_in, C_out, flags | extra, 0.25)
+    pairs = list(zip(run(0), run(sbp.SBP_FLAG_PLAIN_FMA)))
+    Y = [torch.empty(kept, C_out, device="cuda") for _ in range(2)]
+    for y, extra in zip(Y, (0, sbp.SBP_FLAG_PLAIN_FMA)):
+        sbp.sbp_linear_forward(sbp.SBP_F32, X, W, None, kept, C_in, C_out, y, flags=(flags & sbp.SBP_FLAG_W_OUT_IN) | extra)
+    torch.cuda.synchronize()
+    for got, plain in pairs + [tuple(Y)]:
+        got, plain = host(got).astype(np.float64), host(plain).astype(np.float64)
+        assert np.array_equal(np.isnan(got), np.isnan(plain))
+        infinite = np.isinf(plain)
+        assert np.array_equal(np.isinf(got), infinite) and np.array_equal(got[infinite], plain[infinite])
+        ok = np.isfinite(plain)
+        # sums that hold 3.4e38 are compared by themselves: nothing else in them is visible
+        assert (np.abs(got[ok] - plain[ok]) <= 1e-5 * np.maximum(np.abs(plain[ok]), 30.0)).all()
