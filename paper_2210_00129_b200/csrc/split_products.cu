@@ -25,7 +25,7 @@ constexpr uint32_t kBlock64B = 64 * kRowB;
 constexpr int kEpiWarps = 8, kProducerWarps = 8, kMmaWarp = kEpiWarps + kProducerWarps;
 constexpr int kProducers = 32 * kProducerWarps;
 constexpr int kThreads = 32 * (kMmaWarp + 4);   // (three of the last four warps only hand their registers on)
-constexpr int kLaunchRegs = 96, kEpiRegs = 104, kProducerRegs = 104, kMmaRegs = 48;
+constexpr int kLaunchRegs = 96, kEpiRegs = 104, kProducerRegs = 112, kMmaRegs = 40;
 static_assert(kEpiWarps * kEpiRegs + kProducerWarps * kProducerRegs + 4 * kMmaRegs <= (kMmaWarp + 4) * kLaunchRegs,
               "registers that the block is launched with");
 constexpr int kProducerBarrier = 1;
@@ -74,7 +74,7 @@ struct Control {
     uint32_t tmem_slot;
     int abort_flag;
 };
-constexpr uint32_t kSumBytes = 1024 * sizeof(float);
+constexpr uint32_t kSumBytes = 1024 * sizeof(double);
 constexpr uint32_t kSmemBytes = kStages * kStageBytes + kSlotBytes + 256 + kSumBytes + 1024;
 static_assert(sizeof(Control) <= 256 && kSmemBytes <= 227 * 1024, "shared memory of a block");
 
@@ -256,7 +256,7 @@ __device__ __noinline__ void repair(const Product& p, int64_t m, int64_t n0, uin
 
 // A producer thread's part of one item: its vectors of both operands, stage after stage.  False when a wait gave up.
 template <bool kAOuter, bool kBOuter>
-__device__ __forceinline__ bool produce(const Product& p, const Item& item, uint32_t ring, Control* ctl, float* sums_s, uint32_t rank, uint32_t& it,
+__device__ __forceinline__ bool produce(const Product& p, const Item& item, uint32_t ring, Control* ctl, double* sums_s, uint32_t rank, uint32_t& it,
                                         int32_t* status_word) {
     using FA = Feed<kTile / 16, kAOuter>;
     using FB = Feed<kBCols / 16, kBOuter>;
@@ -319,7 +319,9 @@ __device__ __forceinline__ bool produce(const Product& p, const Item& item, uint
     if (kAOuter && kBOuter && side != 0) {
         // thread t holds extent indices 4 (t % kPerRow) + {0..3} over its share of the depth
         const int extent = side == 1 ? kTile : kBCols, per_row = extent / 4;
-        *reinterpret_cast<float4*>(sums_s + (t / per_row) * extent + (t % per_row) * 4) = cs.sum;
+        double* to = sums_s + (t / per_row) * extent + (t % per_row) * 4;
+        to[0] = (double)cs.sum.x - (double)cs.lost.x; to[1] = (double)cs.sum.y - (double)cs.lost.y;
+        to[2] = (double)cs.sum.z - (double)cs.lost.z; to[3] = (double)cs.sum.w - (double)cs.lost.w;
     }
     ok = !ptx::bar_or<kProducerBarrier, kProducers>(!ok);                   // the producers go on, or give up, together
     if (kAOuter && kBOuter && side != 0 && ok) {
@@ -327,7 +329,7 @@ __device__ __forceinline__ bool produce(const Product& p, const Item& item, uint
         const int e = (side == 1 ? e_a0 : e_b0) + t, all = side == 1 ? p.rows : p.cols;
         if (t < extent && e < all) {
             double total = 0.0;
-            for (int g = 0; g < 1024 / extent; ++g) total += (double)sums_s[g * extent + t];
+            for (int g = 0; g < 1024 / extent; ++g) total += sums_s[g * extent + t];
             float* o = p.sums + (int64_t)item.split * all + e;
             *o = p.sums_accumulate ? *o + (float)total : (float)total;
         }
@@ -345,7 +347,7 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
     const uint32_t raw = ptx::smem_addr(smem_raw), ring = (raw + 1023u) & ~1023u;
     uint8_t* tail = smem_raw + (ring - raw) + kStages * kStageBytes + kSlotBytes;
     Control* ctl = reinterpret_cast<Control*>(tail);
-    float* sums_s = reinterpret_cast<float*>(tail + 256);
+    double* sums_s = reinterpret_cast<double*>(tail + 256);
 
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
@@ -571,7 +573,7 @@ double list_time(int64_t nx, double cx, int64_t nw, double cw, int64_t g) {
 }
 
 // Pieces of the dW reduction.
-constexpr double kKbUs = 1.3, kItemUs = 2.5;                               // us of a k-block, of an item's start and read-out
+constexpr double kKbUs = 1.4, kItemUs = 2.5;                               // us of a k-block, of an item's start and read-out
 
 int64_t tiles_of(int64_t rows, int64_t cols) { return ceil_div(rows, 2 * kTile) * ceil_div(cols, kTile); }
 
@@ -592,11 +594,21 @@ int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, boo
 
 }  // namespace
 
+// The lines against the CUDA cores, which start in 3 us where this kernel takes 8 (a cluster of whole SMs, one deep stage), but whose
+// blocks take 4 us for every 100 of depth.  Forward, CUDA cores and here: depth 128 with 491 rows and 376 columns 6.9, 9.2 us, 104 with
+// 1839 and 184 10.4, 9.4, 152 with 2597 and 104 11.8, 10.6; 88 with 3193 and 264 9.4, 10.2, 64 with 3339 and 1232 20.6, 13.7, 32 with
+// 21611 and 168 11.1, 15.2; 232 with 164 and 128 10.8, 11.4, 296 with 162 and 72 13.7, 12.4, 304 with 103 and 32 13.3, 11.3.
+// dW + db + dX: 104 kept rows of 128 -> 144 11.5, 12.7 us, 649 of 152 -> 104 13.7, 12.1, 942 of 472 -> 48 15.9, 13.7; 6770 of 32 -> 72
+// 13.1, 13.7; few rows behind deep sums 95 of 80 -> 376 16.2, 12.0, 72 of 32 -> 720 30.5, 21.9.
 bool split_forward_supported(int64_t M, int64_t C_in, int64_t C_out) {
-    return C_in >= 64 && C_out >= 64 && M >= 256 && M * C_in * C_out >= 150000000;
+    if (M < 32 || C_in < 32 || C_out < 32) return false;
+    const int64_t work = M * C_in * C_out;
+    return C_in >= 288 || (C_in >= 96 && work >= 36000000) || (C_in >= 56 && work >= 100000000) || (C_in >= 40 && work >= 400000000);
 }
 bool split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
-    return C_in >= 64 && C_out >= 64 && M_keep_cap >= 256 && M_keep_cap * C_in * C_out >= 80000000;
+    if (M_keep_cap < 16 || C_in < 32 || C_out < 32) return false;
+    const int64_t work = M_keep_cap * C_in * C_out;
+    return C_out >= 256 || (C_in >= 40 && C_out >= 40 && work >= 10000000) || work >= 80000000;
 }
 
 cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,
