@@ -32,6 +32,7 @@
 // Rows outside the token sets are zeroed here too, while the first products run.  Every wait is bounded and reports through
 // the status word.
 #include "tc_ptx.cuh"
+#include "zero_rows.cuh"
 
 namespace sbp {
 namespace {
@@ -48,7 +49,8 @@ struct AttnParams {
     int B, N, heads;
     __nv_bfloat16 *dQ, *dK, *dV;
     float scale;
-    int zero_fill;                // 1: the rows of a sample that its list leaves out are written as zeros
+    int zero_fill;                // 1: the rows that the lists leave out are written as zeros
+    int zero_blocks, zero_first, zero_rest;    // rows of the outputs that each of the first zero_blocks blocks looks after, each of the others
     int rq, rk;                   // rows of the query-side and key-side buffers: the token bounds rounded up to 16
     uint32_t block_bytes;         // one 64-key block of S: 128 bytes for each query row of a tile
     uint32_t off_dm, dm_stride;   // dM blocks (separate: next to S; otherwise the S blocks themselves)
@@ -70,39 +72,73 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// Zeros for one head's 64 columns in the rows of sample b that an ascending token list leaves out.  `glob` holds the
-// global row of every listed token of the sample (shared memory).  The z-th unlisted row lies behind g listed ones, with g
-// the first list position whose token has more than z unlisted rows in front of it: a search of at most eight steps.  Every
-// lane of a warp searches for a row of its own; then eight lanes at a time clear one 128-byte line, 16 bytes each, so that a
-// warp's store covers four whole lines.  (Walking the gaps between listed tokens, a group of eight lanes each, gave the warps
-// very different amounts of work: 3000 - 4700 clocks a problem.)  Rows are clamped to the sample, so that a list that breaks the
-// ascending order cannot send a store anywhere else.
-__device__ __forceinline__ void zero_unlisted_rows(__nv_bfloat16* out0, __nv_bfloat16* out1, __nv_bfloat16* out2, uint32_t ld, int col0,
-                                                   const int32_t* glob, int count, int base_row, int N, int warp, int warps, int lane) {
-    const int unlisted = N - count;
-    int per = ((unlisted + warps - 1) / warps + 3) & ~3;     // rows of a warp's turn: an equal share, at most one for each lane
-    per = per < 32 ? per : 32;
-    for (int z0 = warp * per; z0 < unlisted; z0 += warps * per) {
-        const int want = z0 + lane + base_row;
-        int g = 0;                                           // tokens with glob[i] - i <= want are in front of the row
-#pragma unroll
-        for (int step = 128; step > 0; step >>= 1)
-            if (g + step <= count && glob[g + step - 1] - (g + step - 1) <= want) g += step;
-        if (g < count && glob[g] - g <= want) ++g;           // (lists of 256 tokens)
-        int r = z0 + lane + g;
-        r = base_row + (r < N ? r : N - 1);
-        const int here = unlisted - z0 < per ? unlisted - z0 : per;
-#pragma unroll 2
-        for (int i = 0; i < here; i += 4) {
-            const int row = __shfl_sync(0xffffffffu, r, i + (lane >> 3));
-            if (i + (lane >> 3) < here) {
-                const int64_t at = (int64_t)((uint64_t)(uint32_t)row * ld * 8u) + col0 + (lane & 7) * 8;
-                if (out0 != nullptr) ptx::st_global_v4(out0 + at, 0u, 0u, 0u, 0u);
-                if (out1 != nullptr) ptx::st_global_v4(out1 + at, 0u, 0u, 0u, 0u);
-                if (out2 != nullptr) ptx::st_global_v4(out2 + at, 0u, 0u, 0u, 0u);
+// Zeros for the rows that an ascending list of token rows leaves out, whole rows (all heads) of the outputs.  A warp walks a range of
+// rows of its own, a few unlisted ones at a time: the stores go out while the block waits for products, so that memory works then too.
+// (In front of the first products, an equal share of the problem's own rows a warp and 128 bytes of each, they took 3500 of a problem's
+// 17500 clocks with the products' 1000 underneath.)
+struct ZeroWalk {                 // kept in shared memory between a warp's turns: it would cost the computing threads registers
+    int pass;                     // 0: the rows that the query list leaves out, 1: the key list; 2: done
+    int budget;                   // rows to clear in a turn
+    int p, n;                     // position in the list, its end
+    int base, next, end;          // first row of the window of 32 at hand, of the next one; end of the range
+    uint32_t todo;                // unlisted rows of the window that are still to be cleared
+};
+
+// A warp's range of the rows that are cleared where the lists leave them out: first those of dQ (or of all outputs, with one list for
+// both sides), then, with a list of their own, those of dK and dV.
+__device__ __forceinline__ void start_walk(const AttnParams& p, ZeroWalk& z, int warp, int warps, int lane) {
+    const int32_t* offs = z.pass == 0 ? p.q_offs : p.k_offs;
+    const int first = __ldg(offs), blk = (int)blockIdx.x, share = blk < p.zero_blocks ? p.zero_first : p.zero_rest;
+    z.n = __ldg(offs + p.B);
+    const int64_t all = (int64_t)p.B * p.N, before = blk < p.zero_blocks ? blk : p.zero_blocks;
+    const int64_t at = before * p.zero_first + (blk - before) * p.zero_rest;
+    const int per = (share + warps - 1) / warps;
+    int64_t lo = at + (int64_t)per * warp, hi = lo + per < at + share ? lo + per : at + share;
+    if (hi > all) hi = all;
+    if (lo > hi) lo = hi;
+    z.next = (int)lo;
+    z.end = (int)hi;
+    z.todo = 0u;
+    z.p = lo < hi ? first + (int)warp_lower_bound((z.pass == 0 ? p.q_rows : p.k_rows) + first, z.n - first, lo, lane) : z.n;
+    // two turns a problem: an even part of the rows that this warp can expect to clear, rounded up
+    const int turns = 2 * ((p.B * p.heads - blk + (int)gridDim.x - 1) / (int)gridDim.x);
+    const int expect = (int)((float)(hi - lo) * (1.f - (float)(z.n - first) / (float)all)) + 1;
+    z.budget = (expect + turns - 1) / turns;
+}
+
+// A turn of a warp, or all that is left.
+__device__ __forceinline__ void zero_rows(const AttnParams& p, ZeroWalk* walk, int warp, int warps, int lane, bool rest) {
+    ZeroWalk z = *walk;
+    const bool same = p.q_rows == p.k_rows && p.q_offs == p.k_offs;
+    int most = rest ? 0x7fffffff : z.budget;
+    while (most > 0 && z.pass < 2) {
+        if (z.todo != 0u) {
+            const int64_t at = (int64_t)((uint64_t)(uint32_t)(z.base + __ffs(z.todo) - 1) * p.ld_out * 8u);
+            for (int c = lane * 8; c < p.heads * kD; c += 256) {
+                if (z.pass == 0) ptx::st_global_v4(p.dQ + at + c, 0u, 0u, 0u, 0u);
+                if (z.pass == 1 || same) {
+                    ptx::st_global_v4(p.dK + at + c, 0u, 0u, 0u, 0u);
+                    ptx::st_global_v4(p.dV + at + c, 0u, 0u, 0u, 0u);
+                }
             }
+            z.todo &= z.todo - 1u;
+            --most;
+        } else if (z.next < z.end) {                        // the next window of 32 rows
+            const int d = z.p + lane < z.n ? __ldg((z.pass == 0 ? p.q_rows : p.k_rows) + z.p + lane) - z.next : 32;
+            const uint32_t listed = __reduce_or_sync(0xffffffffu, (d >= 0 && d < 32) ? 1u << d : 0u);
+            const int here = z.end - z.next < 32 ? z.end - z.next : 32;
+            z.p += __popc(listed);
+            z.base = z.next;
+            z.next += here;
+            z.todo = ~listed & (here < 32 ? (1u << here) - 1u : 0xffffffffu);
+        } else {
+            z.pass = z.pass == 0 && !same && p.k_rows != nullptr ? 1 : 2;
+            if (z.pass == 1) start_walk(p, z, warp, warps, lane);
         }
     }
+    __syncwarp();
+    if (lane == 0) *walk = z;
+    __syncwarp();
 }
 
 __device__ __forceinline__ void prefetch_row(const __nv_bfloat16* p, int32_t row, uint32_t ld) {
@@ -115,6 +151,7 @@ struct AttnShared {
     uint64_t bar_s, bar_o;        // products of S and dS; gradient products
     uint32_t tmem_slot;
     int abort_flag;
+    ZeroWalk walk[4 * G];         // of each warp
     float part[G][128][3];        // per 64 columns of a row: maximum, sum of e = 2^((s - maximum) log2 e / sqrt(d)), sum of e dS
     int32_t q_glob[2][kTok], k_glob[2][kTok];   // global rows of the listed tokens (0 past the last): this problem's, the next one's
 };
@@ -219,7 +256,7 @@ __device__ __forceinline__ void store_rows(__nv_bfloat16* out, uint32_t ld, int 
 
 // kSeparate: dM has blocks of its own
 template <int G, bool kSeparate>
-__global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(const AttnParams p) {
+__global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(const __grid_constant__ AttnParams p) {
     constexpr int kThreads = 128 * G;
     constexpr uint32_t kTmemCols = G == 2 ? 256 : 512;
     // tensor-memory columns.  G = 2: S and dS side by side, then dV, dK, dQ in their place.  G = 4: S (dQ later); dS in the
@@ -274,16 +311,6 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             load_rows<kThreads>(side ? sK : sQ, side ? sV : sDA, (side ? p.K : p.Q) + col0, p.ld_qkv, (side ? p.V : p.dA) + col0,
                                 side ? p.ld_qkv : p.ld_da, side ? sh.k_glob[b] : sh.q_glob[b], side ? m.nk : m.nq, t);
     };
-    // zeros for the rows of problem `prob` outside its lists
-    auto zero_rows = [&](int prob, int nq, int nk, const int32_t* q_glob, const int32_t* k_glob) {
-        if (!p.zero_fill) return;
-        const int b = prob / p.heads, col0 = (prob % p.heads) * kD;
-        const bool same = p.q_rows == p.k_rows && p.q_offs == p.k_offs;
-        if (p.q_rows != nullptr)
-            zero_unlisted_rows(p.dQ, same ? p.dK : nullptr, same ? p.dV : nullptr, p.ld_out, col0, q_glob, nq, b * p.N, p.N, warp, kThreads / 32, lane);
-        if (p.k_rows != nullptr && !same)
-            zero_unlisted_rows(nullptr, p.dK, p.dV, p.ld_out, col0, k_glob, nk, b * p.N, p.N, warp, kThreads / 32, lane);
-    };
     // every thread of the block waits for a commit (one polls); false for all of them when the wait gave up
     auto wait_products = [&](uint64_t* bar, uint32_t& n) {
         bool good = true;
@@ -296,6 +323,13 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
 
     Meta cur = fetch_meta(p, ok ? (int)blockIdx.x : problems, (int)threadIdx.x);
     if (ok && (int)blockIdx.x < problems) begin_problem(cur, (int)blockIdx.x, 0);
+    {
+        ZeroWalk z{};
+        z.pass = !ok || !p.zero_fill ? 2 : p.q_rows != nullptr ? 0 : 1;
+        if (z.pass < 2) start_walk(p, z, warp, kThreads / 32, lane);
+        if (lane == 0) sh.walk[warp] = z;
+        __syncwarp();
+    }
 
     for (int prob = blockIdx.x; ok && prob < problems; prob += gridDim.x, buf ^= 1) {
         const int nq = __shfl_sync(0xffffffffu, cur.nq, 0), nk = __shfl_sync(0xffffffffu, cur.nk, 0);
@@ -303,8 +337,8 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         const int next = prob + (int)gridDim.x;
         cur = fetch_meta(p, next, (int)threadIdx.x);        // travels while this problem computes
         const int32_t *q_glob = sh.q_glob[buf], *k_glob = sh.k_glob[buf];
-        if (nq <= 0 || nk <= 0) {                            // nothing to compute: zeros for the unlisted rows, and for those of a side
-            zero_rows(prob, nq, nk, q_glob, k_glob);         // whose other side has no tokens (sums over nothing)
+        if (nq <= 0 || nk <= 0) {                            // nothing to compute: zeros for the listed rows of a side whose other side has
+                                                             // no tokens (sums over nothing)
             for (int r = (int)threadIdx.x >> 3; r < (nq > nk ? nq : nk); r += kThreads / 8) {
                 const int64_t at = (int64_t)((uint64_t)(uint32_t)(nk <= 0 ? q_glob : k_glob)[r] * p.ld_out * 8u) + col0 + (threadIdx.x & 7) * 8;
                 if (nk <= 0) {
@@ -343,7 +377,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
                 __syncwarp();
             }
-            if (qt == 0) zero_rows(prob, nq, nk, q_glob, k_glob);
+            if (qt == 0) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, false);
             ok = wait_products(&sh.bar_s, n_s);
             if (!ok) break;
             // ---- this thread's 64 columns of its row, in two chunks of 32 which are skipped past n_keys.  Columns from nk on
@@ -537,6 +571,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
                 __syncwarp();
             }
+            if (qt + 1 == QT) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, false);
             ok = wait_products(&sh.bar_o, n_o);
             if (!ok) break;
             // the operands have been read: the next problem's rows may come in (the read-out stages in the S and dM blocks,
@@ -608,6 +643,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         // whoever writes this problem's half of q_glob / k_glob next does so behind a barrier of the next problem (of an empty one too).
         ptx::tc_fence_before_sync();
     }
+    if (ok) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, true);                            // what the turns have left
     ptx::cp_async_wait_all();
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -625,8 +661,17 @@ cudaError_t launch_attention_kernel(const AttnParams& prm, uint32_t bytes, int m
     const cudaError_t opt = opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate>>(most_bytes);
     if (opt != cudaSuccess) return opt;
     const int64_t problems = (int64_t)prm.B * prm.heads, resident = G == 2 ? 2 * kNumSMs : kNumSMs;
-    return launch_pdl(attention_bwd_kernel<G, kSeparate>, dim3((unsigned)(problems < resident ? problems : resident)), dim3(128 * G), bytes,
-                      stream, prm);
+    const int64_t grid = problems < resident ? problems : resident;
+    // Zeros: equal shares of the rows, less for the first blocks where these have a problem more than the others, by the rows that can be
+    // visited in a problem's time: some 3600 / (heads x outputs), half of them unlisted.
+    AttnParams q = prm;
+    const int64_t rows = (int64_t)prm.B * prm.N, outs = prm.q_rows == nullptr ? 2 : prm.k_rows == prm.q_rows ? 3 : 1;
+    const int64_t more = problems % grid, worth = 3600 / (prm.heads * outs) + 1;
+    const int64_t spare = rows - (grid - more) * worth;
+    q.zero_blocks = (int)more;
+    q.zero_first = more == 0 || spare <= 0 ? 0 : (int)((spare + grid - 1) / grid);
+    q.zero_rest = (int)((rows - more * q.zero_first + (grid - more) - 1) / (grid - more));
+    return launch_pdl(attention_bwd_kernel<G, kSeparate>, dim3((unsigned)grid), dim3(128 * G), bytes, stream, q);
 }
 
 template <int G>
