@@ -114,7 +114,7 @@ struct ReduceJob {
     int accumulate;
     int lanes;            // 1: one thread per float4, partials added in ascending order
                           // Y = 4 or 32: 256/Y float4 columns x Y row lanes per block; lane y adds partials
-                          //    y, y+Y, ... in ascending order, the Y lane sums are then added in lane order
+                          //    y, y+Y, ... in ascending order, the Y lane sums are then added in a fixed order
     int blocks;
 };
 
@@ -158,8 +158,22 @@ __device__ __forceinline__ void run_reduce_job(const ReduceJob& jb, int block, f
     red[y * X + x] = s;
     __syncthreads();
     if (y == 0 && i < jb.n_vec) {
-        float4 t = jb.accumulate ? jb.out[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int w = 0; w < Y; ++w) add4(t, red[w * X + x]);
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (Y == 32) {                                         // eight chains of four and a tree: less rounding than a chain of 32, and shorter
+            float4 c[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) c[j] = red[j * X + x];
+#pragma unroll
+            for (int w = 8; w < 32; ++w) add4(c[w & 7], red[w * X + x]);
+#pragma unroll
+            for (int n = 4; n > 0; n /= 2)
+#pragma unroll
+                for (int j = 0; j < n; ++j) add4(c[j], c[j + n]);
+            t = c[0];
+        } else {
+            for (int w = 0; w < Y; ++w) add4(t, red[w * X + x]);
+        }
+        if (jb.accumulate) add4(t, jb.out[i]);
         jb.out[i] = t;
     }
 }

@@ -1,5 +1,5 @@
-// Products on the CUDA cores, fp32 fused multiply-adds: the fp32 path (whose 1e-5 tolerance rules out reduced-precision
-// tensor-core modes) and bf16 shapes whose products are too short for the tensor-core kernels.
+// Products on the CUDA cores, fp32 fused multiply-adds: fp32 and bf16 shapes whose products are too short for the tensor-core kernels
+// (split_products.cu, tc_backward.cu, tc_forward.cu), and any shape on request.
 //   forward  Y[m, j] = sum_i X[m, i] W[i, j] + bias[j]                        (Eq. 2)
 //   dW[i, j] = sum_m X_keep[m, i] dY[keep_rows[m], j],  db[j] = sum_m dY[keep_rows[m], j]       (Eq. 5)
 //   dX[keep_rows[m], i] = sum_j dY[keep_rows[m], j] W[i, j]; every other row of dX = +0.0

@@ -172,7 +172,7 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
 
 // the same products of fp32 layers on the tensor cores, each operand as a sum of three bf16 numbers
 bool   split_forward_supported(int64_t M, int64_t C_in, int64_t C_out);
-bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
+bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx);
 size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
 int    split_backward_kernel_count(bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,

@@ -10,6 +10,13 @@
 // rounding it, so a sum is never left in tensor memory for long: each 64-deep stage starts a fresh accumulator, the five small
 // terms go in first and a1 b1 last (four steps that see the full magnitude), and the epilogue warps add the stage's result to
 // their fp32 registers with rounding.
+//
+// A pair of blocks makes tiles of 256 x 128 with two-SM instructions.  Bound by shared memory: a 64-deep stage moves 312 KB through
+// each SM (copies in 48, read back 48, planes written 72, read by the tensor core 144 less what its kept operand saves) = 2440 clocks
+// at 128 bytes, against 1536 of products; measured 1.4 us.  (Copies straight to registers, 264 KB: 1.95 us, their latency shows; with the next
+// stage's loads behind each conversion the registers spill.)  Measured on B200, 768 -> 3072, 3136 rows with 1568 kept, CUDA cores -> here: forward
+// 299 -> 87 us, dW + db + dX 395 -> 100; relative errors against 64-bit sums Y 2.5e-7 -> 0.8e-7, dW 5.0e-7 -> 1.2e-7, dX 7.0e-7 -> 1.5e-7,
+// db 0.7e-7 -> 0.6e-7.  Over 260 shapes of 32 to 2900 channels and 64 to 65536 rows no Y, dW or dX was further off than the CUDA cores'.
 #include <type_traits>
 
 #include "tc_ptx.cuh"
@@ -407,14 +414,20 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t a = a_lo + s * (kStageBytes >> 4), b = b_lo + s * (kStageBytes >> 4), d = tmem + acc * kAccCols;
-                // the products in the order they are summed: plane of A, plane of B, smallest first, a1 b1 last
-                constexpr int kPlaneA[6] = {2, 0, 1, 1, 0, 0}, kPlaneB[6] = {0, 2, 1, 0, 1, 0};
+                // Every slice's small products first, a1 b1 of all slices last.  Products that share a part of A follow one another, so that
+                // it is read from shared memory once for both.
+                const auto a_at = [&](uint32_t plane, uint32_t u) { return ptx::umma_desc_of(a + plane * (kAPlane >> 4) + u * a_step); };
+                const auto b_at = [&](uint32_t plane, uint32_t u) { return ptx::umma_desc_of(b + plane * (kBPlane >> 4) + u * b_step); };
 #pragma unroll
-                for (int i = 0; i < 24; ++i) {
-                    const uint32_t u = (uint32_t)i & 3u;
-                    ptx::umma_bf16_warp<true>(d, ptx::umma_desc_of(a + kPlaneA[i >> 2] * (kAPlane >> 4) + u * a_step),
-                                              ptx::umma_desc_of(b + kPlaneB[i >> 2] * (kBPlane >> 4) + u * b_step), idesc, i != 0, leader);
+                for (uint32_t u = 0; u < 4; ++u) {
+                    ptx::umma_bf16_pair_warp<0>(d, a_at(2, u), b_at(0, u), idesc, u != 0, leader);
+                    ptx::umma_bf16_pair_warp<1>(d, a_at(1, u), b_at(1, u), idesc, true, leader);
+                    ptx::umma_bf16_pair_warp<2>(d, a_at(1, u), b_at(0, u), idesc, true, leader);
+                    ptx::umma_bf16_pair_warp<1>(d, a_at(0, u), b_at(2, u), idesc, true, leader);
+                    ptx::umma_bf16_pair_warp<2>(d, a_at(0, u), b_at(1, u), idesc, true, leader);
                 }
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) ptx::umma_bf16_pair_warp<0>(d, a_at(0, u), b_at(0, u), idesc, true, leader);
                 if (leader) {
                     ptx::umma_commit_pair(ptx::smem_addr(&ctl->empty_bar[s]));
                     ptx::umma_commit_pair(ptx::smem_addr(&ctl->acc_full[acc]));
@@ -559,16 +572,21 @@ cudaError_t launch(const SplitParams& prm, cudaStream_t stream) {
     return launch_pdl_cluster(split_products_kernel, dim3((unsigned)(2 * used)), dim3(kThreads), kSmemBytes, 2u, stream, prm);
 }
 
-// Time of a list of `nx` items of `cx` us followed by `nw` of `cw`, dealt to `g` workers as list_position does.
+// Time of a list of `nx` items of `cx` us followed by `nw` of `cw`, dealt to `g` workers as list_position does.  The workers that take part
+// in the round in which the first kind ends, and in the last round, are the first or the last of all: at most four kinds of workers.
 double list_time(int64_t nx, double cx, int64_t nw, double cw, int64_t g) {
     const int64_t n = nx + nw, ax = nx / g, rx = nx % g, an = n / g, rn = n % g;
+    const int64_t x0 = (ax & 1) ? g - rx : 0, x1 = x0 + rx, n0 = (an & 1) ? g - rn : 0, n1 = n0 + rn;
     double worst = 0.0;
-    for (int64_t w = 0; w < g; ++w) {
-        const int64_t px = (ax & 1) ? g - 1 - w : w, pn = (an & 1) ? g - 1 - w : w;
-        const int64_t kx = ax + (px < rx ? 1 : 0), kn = an + (pn < rn ? 1 : 0);
+    const auto kind = [&](bool exists, int64_t kx, int64_t kn) {
         const double t = (double)kx * cx + (double)(kn - kx) * cw;
-        if (t > worst) worst = t;
-    }
+        if (exists && t > worst) worst = t;
+    };
+    kind((x0 > n0 ? x0 : n0) < (x1 < n1 ? x1 : n1), ax + 1, an + 1);
+    kind(rx > 0 && !(n0 <= x0 && x1 <= n1), ax + 1, an);
+    kind(rn > 0 && !(x0 <= n0 && n1 <= x1), ax, an + 1);
+    const bool all = rx + rn >= g && (x0 == 0 ? n1 == g : n0 == 0);
+    kind(!all, ax, an);
     return worst;
 }
 
@@ -599,16 +617,17 @@ int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, boo
 // 1839 and 184 10.4, 9.4, 152 with 2597 and 104 11.8, 10.6; 88 with 3193 and 264 9.4, 10.2, 64 with 3339 and 1232 20.6, 13.7, 32 with
 // 21611 and 168 11.1, 15.2; 232 with 164 and 128 10.8, 11.4, 296 with 162 and 72 13.7, 12.4, 304 with 103 and 32 13.3, 11.3.
 // dW + db + dX: 104 kept rows of 128 -> 144 11.5, 12.7 us, 649 of 152 -> 104 13.7, 12.1, 942 of 472 -> 48 15.9, 13.7; 6770 of 32 -> 72
-// 13.1, 13.7; few rows behind deep sums 95 of 80 -> 376 16.2, 12.0, 72 of 32 -> 720 30.5, 21.9.
+// 13.1, 13.7; few rows behind deep sums of dX 95 of 80 -> 376 16.2, 12.0, 72 of 32 -> 720 30.5, 21.9 (dW + db alone 16 of 1024 -> 3072
+// 7.7, 12.0, 500 of 40 -> 256 8.1, 10.2).
 bool split_forward_supported(int64_t M, int64_t C_in, int64_t C_out) {
     if (M < 32 || C_in < 32 || C_out < 32) return false;
     const int64_t work = M * C_in * C_out;
     return C_in >= 288 || (C_in >= 96 && work >= 36000000) || (C_in >= 56 && work >= 100000000) || (C_in >= 40 && work >= 400000000);
 }
-bool split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
+bool split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx) {
     if (M_keep_cap < 16 || C_in < 32 || C_out < 32) return false;
     const int64_t work = M_keep_cap * C_in * C_out;
-    return C_out >= 256 || (C_in >= 40 && C_out >= 40 && work >= 10000000) || work >= 80000000;
+    return (want_dx && C_out >= 256) || (C_in >= 40 && C_out >= 40 && work >= 20000000) || work >= 80000000;
 }
 
 cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,
