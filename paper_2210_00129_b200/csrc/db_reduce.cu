@@ -159,20 +159,16 @@ __device__ __forceinline__ void run_reduce_job(const ReduceJob& jb, int block, f
     __syncthreads();
     if (y == 0 && i < jb.n_vec) {
         float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (Y == 32) {                                         // eight chains of four and a tree: less rounding than a chain of 32, and shorter
-            float4 c[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) c[j] = red[j * X + x];
-#pragma unroll
-            for (int w = 8; w < 32; ++w) add4(c[w & 7], red[w * X + x]);
-#pragma unroll
-            for (int n = 4; n > 0; n /= 2)
-#pragma unroll
-                for (int j = 0; j < n; ++j) add4(c[j], c[j + n]);
-            t = c[0];
-        } else {
-            for (int w = 0; w < Y; ++w) add4(t, red[w * X + x]);
+        float4 u = t;                                          // two chains: less rounding than one, and shorter (eight cost the kernel registers)
+#pragma unroll 1
+        for (int w = 0; w < Y; w += 4) {
+            float4 a = red[w * X + x], b = red[(w + 2) * X + x];
+            add4(a, red[(w + 1) * X + x]);
+            add4(b, red[(w + 3) * X + x]);
+            add4(t, a);
+            add4(u, b);
         }
+        add4(t, u);
         if (jb.accumulate) add4(t, jb.out[i]);
         jb.out[i] = t;
     }
