@@ -23,13 +23,15 @@
 //  - The next problem's rows are copied as soon as the last product has read the operands, under the read-out and the
 //    stores of this one.
 // Measured on B200, ViT-B/16 heads (12 x 64, 196 tokens), whole pass with the sampler: Drop QKV, half of the tokens, B = 128:
-// 99 us with a thread a row and copies behind the read-out, now 65 us; Drop Query only, B = 64: 94 -> 72 us.  (One
-// thread issuing the products instead of a whole warp with one lane elected: 70 and 78 us, each instruction waiting for its
-// operands to reach uniform registers.)  A problem's chain before that, some 20000 clocks with two blocks on an SM: copies and zero rows 5500 (all SMs load, then all store, so
-// memory is busy a quarter of the time on average), softmax 6000, products 4500, read-out 2500.  Copies and zeros by four warps
-// of their own did not pay: the computing warps need more registers than setmaxnreg could then give them (76 us).
+// 99 us with a thread a row and copies behind the read-out, 64 with the zeros of a problem's own rows in front of its first wait, now 58;
+// Drop Query only, B = 64: 94 -> 71 -> 61.  (One thread issuing the products instead of a whole warp with one lane elected: 70 and 78 us,
+// each instruction waiting for its operands to reach uniform registers.)  A problem's chain, some 17000 clocks with two blocks on an SM: wait
+// for the copies 900, first products and zeros 2300, softmax 5300, gradient products and zeros 3200, next copies 2900, read-out and stores 2400.
+// Not kept: copies and zeros by four warps of their own (the computing warps need more registers than setmaxnreg could then give
+// them, 76 us); dV made first so that the next problem's rows of dA come in under dK and dQ (62 and 63.5 us: products that do not take turns
+// between accumulators are slower); a problem's stores under the next one's first products (64 us: they then hold up the softmax).
 // Query tiles of 128 rows follow one another (dV and dK stay in tensor memory); with two of them S and dS share columns.
-// Rows outside the token sets are zeroed here too, while the first products run.  Every wait is bounded and reports through
+// Rows outside the token sets are zeroed here too, while products run.  Every wait is bounded and reports through
 // the status word.
 #include "tc_ptx.cuh"
 #include "zero_rows.cuh"
@@ -72,7 +74,49 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// Zeros for the rows that an ascending list of token rows leaves out, whole rows (all heads) of the outputs.  A warp walks a range of
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// Calls of one problem a block: zeros for the problem's own 64 columns in the rows of sample b that an ascending token list leaves out, with
+// no look at memory (the walk's dependent loads are longer than the first products: 7.7 us here, 8.5 with it).  `glob` holds the
+// global row of every listed token of the sample (shared memory).  The z-th unlisted row lies behind g listed ones, with g
+// the first list position whose token has more than z unlisted rows in front of it: a search of at most eight steps.  Every
+// lane of a warp searches for a row of its own; then eight lanes at a time clear one 128-byte line, 16 bytes each, so that a
+// warp's store covers four whole lines.  (Walking the gaps between listed tokens, a group of eight lanes each, gave the warps
+// very different amounts of work: 3000 - 4700 clocks a problem.)  Rows are clamped to the sample, so that a list that breaks the
+// ascending order cannot send a store anywhere else.
+__device__ __forceinline__ void zero_unlisted_rows(__nv_bfloat16* out0, __nv_bfloat16* out1, __nv_bfloat16* out2, uint32_t ld, int col0,
+                                                   const int32_t* glob, int count, int base_row, int N, int warp, int warps, int lane) {
+    const int unlisted = N - count;
+    int per = ((unlisted + warps - 1) / warps + 3) & ~3;     // rows of a warp's turn: an equal share, at most one for each lane
+    per = per < 32 ? per : 32;
+    for (int z0 = warp * per; z0 < unlisted; z0 += warps * per) {
+        const int want = z0 + lane + base_row;
+        int g = 0;                                           // tokens with glob[i] - i <= want are in front of the row
+#pragma unroll
+        for (int step = 128; step > 0; step >>= 1)
+            if (g + step <= count && glob[g + step - 1] - (g + step - 1) <= want) g += step;
+        if (g < count && glob[g] - g <= want) ++g;           // (lists of 256 tokens)
+        int r = z0 + lane + g;
+        r = base_row + (r < N ? r : N - 1);
+        const int here = unlisted - z0 < per ? unlisted - z0 : per;
+#pragma unroll 2
+        for (int i = 0; i < here; i += 4) {
+            const int row = __shfl_sync(0xffffffffu, r, i + (lane >> 3));
+            if (i + (lane >> 3) < here) {
+                const int64_t at = (int64_t)((uint64_t)(uint32_t)row * ld * 8u) + col0 + (lane & 7) * 8;
+                if (out0 != nullptr) ptx::st_global_v4(out0 + at, 0u, 0u, 0u, 0u);
+                if (out1 != nullptr) ptx::st_global_v4(out1 + at, 0u, 0u, 0u, 0u);
+                if (out2 != nullptr) ptx::st_global_v4(out2 + at, 0u, 0u, 0u, 0u);
+            }
+        }
+    }
+}
+
+// Calls of several: zeros for the rows that an ascending list of token rows leaves out, whole rows (all heads) of the outputs.  A warp walks a range of
 // rows of its own, a few unlisted ones at a time: the stores go out while the block waits for products, so that memory works then too.
 // (In front of the first products, an equal share of the problem's own rows a warp and 128 bytes of each, they took 3500 of a problem's
 // 17500 clocks with the products' 1000 underneath.)
@@ -254,8 +298,8 @@ __device__ __forceinline__ void store_rows(__nv_bfloat16* out, uint32_t ld, int 
     }
 }
 
-// kSeparate: dM has blocks of its own
-template <int G, bool kSeparate>
+// kSeparate: dM has blocks of its own; kOwn: one problem a block at most, which clears its own unlisted rows
+template <int G, bool kSeparate, bool kOwn>
 __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(const __grid_constant__ AttnParams p) {
     constexpr int kThreads = 128 * G;
     constexpr uint32_t kTmemCols = G == 2 ? 256 : 512;
@@ -311,6 +355,16 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
             load_rows<kThreads>(side ? sK : sQ, side ? sV : sDA, (side ? p.K : p.Q) + col0, p.ld_qkv, (side ? p.V : p.dA) + col0,
                                 side ? p.ld_qkv : p.ld_da, side ? sh.k_glob[b] : sh.q_glob[b], side ? m.nk : m.nq, t);
     };
+    // zeros for the rows of problem `prob` outside its lists
+    auto zero_own_rows = [&](int prob, int nq, int nk, const int32_t* q_glob, const int32_t* k_glob) {
+        if (!p.zero_fill) return;
+        const int b = prob / p.heads, col0 = (prob % p.heads) * kD;
+        const bool same = p.q_rows == p.k_rows && p.q_offs == p.k_offs;
+        if (p.q_rows != nullptr)
+            zero_unlisted_rows(p.dQ, same ? p.dK : nullptr, same ? p.dV : nullptr, p.ld_out, col0, q_glob, nq, b * p.N, p.N, warp, kThreads / 32, lane);
+        if (p.k_rows != nullptr && !same)
+            zero_unlisted_rows(nullptr, p.dK, p.dV, p.ld_out, col0, k_glob, nk, b * p.N, p.N, warp, kThreads / 32, lane);
+    };
     // every thread of the block waits for a commit (one polls); false for all of them when the wait gave up
     auto wait_products = [&](uint64_t* bar, uint32_t& n) {
         bool good = true;
@@ -323,7 +377,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
 
     Meta cur = fetch_meta(p, ok ? (int)blockIdx.x : problems, (int)threadIdx.x);
     if (ok && (int)blockIdx.x < problems) begin_problem(cur, (int)blockIdx.x, 0);
-    {
+    if constexpr (!kOwn) {
         ZeroWalk z{};
         z.pass = !ok || !p.zero_fill ? 2 : p.q_rows != nullptr ? 0 : 1;
         if (z.pass < 2) start_walk(p, z, warp, kThreads / 32, lane);
@@ -339,6 +393,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         const int32_t *q_glob = sh.q_glob[buf], *k_glob = sh.k_glob[buf];
         if (nq <= 0 || nk <= 0) {                            // nothing to compute: zeros for the listed rows of a side whose other side has
                                                              // no tokens (sums over nothing)
+            if constexpr (kOwn) zero_own_rows(prob, nq, nk, q_glob, k_glob);
             for (int r = (int)threadIdx.x >> 3; r < (nq > nk ? nq : nk); r += kThreads / 8) {
                 const int64_t at = (int64_t)((uint64_t)(uint32_t)(nk <= 0 ? q_glob : k_glob)[r] * p.ld_out * 8u) + col0 + (threadIdx.x & 7) * 8;
                 if (nk <= 0) {
@@ -377,7 +432,10 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_s));
                 __syncwarp();
             }
-            if (qt == 0) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, false);
+            if (qt == 0) {
+                if constexpr (kOwn) zero_own_rows(prob, nq, nk, q_glob, k_glob);
+                else zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, false);
+            }
             ok = wait_products(&sh.bar_s, n_s);
             if (!ok) break;
             // ---- this thread's 64 columns of its row, in two chunks of 32 which are skipped past n_keys.  Columns from nk on
@@ -396,7 +454,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                     for (int j = 0; j < 32; ++j) v[j] = first + j < nk ? v[j] : -INFINITY;
                 }
 #pragma unroll
-                for (int j = 0; j < 32; ++j) mx4[j & 3] = fmaxf(mx4[j & 3], v[j]);
+                for (int j = 0; j < 32; j += 2) mx4[(j >> 1) & 3] = max3(mx4[(j >> 1) & 3], v[j], v[j + 1]);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) e[c][j] = pair(v[2 * j], v[2 * j + 1]);
             }
@@ -571,7 +629,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
                 if (leader) ptx::umma_commit(ptx::smem_addr(&sh.bar_o));
                 __syncwarp();
             }
-            if (qt + 1 == QT) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, false);
+            if (!kOwn && qt + 1 == QT) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, false);
             ok = wait_products(&sh.bar_o, n_o);
             if (!ok) break;
             // the operands have been read: the next problem's rows may come in (the read-out stages in the S and dM blocks,
@@ -643,7 +701,7 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
         // whoever writes this problem's half of q_glob / k_glob next does so behind a barrier of the next problem (of an empty one too).
         ptx::tc_fence_before_sync();
     }
-    if (ok) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, true);                            // what the turns have left
+    if (!kOwn && ok) zero_rows(p, &sh.walk[warp], warp, kThreads / 32, lane, true);                            // what the turns have left
     ptx::cp_async_wait_all();
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -658,20 +716,23 @@ int round16(int64_t v) { return (int)((v + 15) / 16 * 16); }
 
 template <int G, bool kSeparate>
 cudaError_t launch_attention_kernel(const AttnParams& prm, uint32_t bytes, int most_bytes, cudaStream_t stream) {
-    const cudaError_t opt = opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate>>(most_bytes);
-    if (opt != cudaSuccess) return opt;
     const int64_t problems = (int64_t)prm.B * prm.heads, resident = G == 2 ? 2 * kNumSMs : kNumSMs;
     const int64_t grid = problems < resident ? problems : resident;
+    const auto go = [&](auto kernel, cudaError_t opt, const AttnParams& q) {
+        return opt != cudaSuccess ? opt : launch_pdl(kernel, dim3((unsigned)grid), dim3(128 * G), bytes, stream, q);
+    };
+    if (problems <= resident)
+        return go(attention_bwd_kernel<G, kSeparate, true>, opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate, true>>(most_bytes), prm);
     // Zeros: equal shares of the rows, less for the first blocks where these have a problem more than the others, by the rows that can be
-    // visited in a problem's time: some 3600 / (heads x outputs), half of them unlisted.
+    // visited in a problem's time: some 7200 / (heads x outputs), half of them unlisted (Drop QKV, B = 128: 2400 60.0 us, 3600 58.9, 7200 58.5).
     AttnParams q = prm;
     const int64_t rows = (int64_t)prm.B * prm.N, outs = prm.q_rows == nullptr ? 2 : prm.k_rows == prm.q_rows ? 3 : 1;
-    const int64_t more = problems % grid, worth = 3600 / (prm.heads * outs) + 1;
+    const int64_t more = problems % grid, worth = 7200 / (prm.heads * outs) + 1;
     const int64_t spare = rows - (grid - more) * worth;
     q.zero_blocks = (int)more;
     q.zero_first = more == 0 || spare <= 0 ? 0 : (int)((spare + grid - 1) / grid);
     q.zero_rest = (int)((rows - more * q.zero_first + (grid - more) - 1) / (grid - more));
-    return launch_pdl(attention_bwd_kernel<G, kSeparate>, dim3((unsigned)grid), dim3(128 * G), bytes, stream, q);
+    return go(attention_bwd_kernel<G, kSeparate, false>, opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate, false>>(most_bytes), q);
 }
 
 template <int G>
