@@ -45,6 +45,7 @@ def _backward(X_keep, dY, W, rows, count, M, cap, C_in, C_out, flags, fill):
     (6000, 5000, 0, 132, 640, False, False),         # dW cut into pieces
     (4000, 4000, 3000, 384, 132, False, False),      # pieces without rows
     (2000, 1100, 0, 1028, 128, True, False),
+    (900, 600, 0, 256, 260, True, True),             # weights [C_out, C_in] small enough to go through transposed copies
 ])
 def test_backward(M, kept, padding, C_in, C_out, out_in, accumulate):
     X, Wt, dY = synth.layer_inputs("f32", M, C_in, C_out, 91)
@@ -63,6 +64,24 @@ def test_backward(M, kept, padding, C_in, C_out, out_in, accumulate):
         assert _rel(got.contiguous(), exact) <= REL and _elements(got.contiguous(), exact) <= 1e-5
     dropped = np.setdiff1d(np.arange(M), valid)
     assert not host(dX)[dropped].view(np.uint8).any()
+
+
+def test_packed_forms_are_the_scattered_ones():
+    """The same numbers, bit for bit, with dY read packed and dX written packed; rows past the count become zeros."""
+    M, kept, valid, C_in, C_out = 2000, 1100, 1037, 260, 388
+    X, Wt, dY = synth.layer_inputs("f32", M, C_in, C_out, 93)
+    rows = torch.from_numpy(np.sort(np.random.default_rng(6).permutation(M)[:kept]).astype(np.int32)).cuda()
+    count = torch.tensor([valid], dtype=torch.int32, device="cuda")
+    W, dY_d = dev(Wt, "f32"), dev(dY, "f32")
+    Xk = run_forward_cache("f32", dev(X, "f32"), rows, kept, count)
+    plain = _backward(Xk, dY_d, W, rows, count, M, kept, C_in, C_out, 0, float("nan"))
+    packed_dY = dY_d[rows.long()].contiguous()
+    from_packed = _backward(Xk, packed_dY, W, rows, count, M, kept, C_in, C_out, sbp.SBP_FLAG_DY_COMPACT, float("nan"))
+    both = _backward(Xk, packed_dY, W, rows, count, M, kept, C_in, C_out, sbp.SBP_FLAG_DY_COMPACT | sbp.SBP_FLAG_DX_COMPACT, float("nan"))
+    for a, b in zip(plain, from_packed):
+        assert torch.equal(a, b)
+    assert torch.equal(both[0], plain[0]) and torch.equal(both[1], plain[1])
+    assert torch.equal(both[2][:valid], plain[2][rows[:valid].long()]) and not both[2][valid:kept].any()
 
 
 @pytest.mark.parametrize("M,C_in,C_out,out_in", [(3000, 260, 388, False), (3000, 260, 388, True), (2561, 1028, 900, False), (8192, 512, 128, True)])
