@@ -160,7 +160,7 @@ __device__ __forceinline__ void run_reduce_job(const ReduceJob& jb, int block, f
     if (y == 0 && i < jb.n_vec) {
         float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
         float4 u = t;                                          // two chains: less rounding than one, and shorter (eight cost the kernel registers)
-#pragma unroll 1
+#pragma unroll 2
         for (int w = 0; w < Y; w += 4) {
             float4 a = red[w * X + x], b = red[(w + 2) * X + x];
             add4(a, red[(w + 1) * X + x]);
