@@ -212,7 +212,8 @@ size_t sbp_linear_backward_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_ke
  * rows), dX rounded to bf16 (nearest even).  SBP_F32: fp32 FMA arithmetic, or, for
  * products large enough, six tensor-core products of operands in three bf16 parts each,
  * summed in fp32: no further from 64-bit sums than the FMAs (1e-7 against 2e-7 to 7e-7),
- * infinities and NaNs as the FMAs have them; SBP_FLAG_PLAIN_FMA keeps to the FMAs.
+ * subnormal operands and sums included, infinities and NaNs as the FMAs have them;
+ * SBP_FLAG_PLAIN_FMA keeps to the FMAs.
  * C_in and C_out must be multiples of 8 (bf16) / 4 (fp32), else SBP_ERR_UNSUPPORTED.
  *
  * flags: SBP_FLAG_ACCUMULATE adds into dW and db; SBP_FLAG_VALIDATE first checks

@@ -6,7 +6,11 @@
 // Every operand x is written as a sum of three bf16 numbers, x = x1 + x2 + x3, each the rounded rest of the one before (8
 // significant bits each, so what is left is below 2^-26 x), and a product of two of them as
 //   a b = a1 b1 + (a1 b2 + a2 b1) + (a2 b2 + a1 b3 + a3 b1),
-// dropping terms below 2^-26: six bf16 products with fp32 accumulation.  The tensor core cuts its running sum short instead of
+// dropping terms below 2^-26: six bf16 products with fp32 accumulation.  The parts are those of 2^16 x: bf16 numbers end at 2^-133, so that
+// the third part of an x below 2^-109 would lose bits, while the last bit of any fp32 number is 2^-149 or more.  The sums are brought back by
+// 2^-32.  (Sums beyond 2^96 come out infinite that way, and are made again like other sums that are not finite.)  The tensor core also
+// drops sums that are subnormal: sums of 1e-39 came out as zeros.  The scaling costs 1 us of a layer's 200.
+// The tensor core cuts its running sum short instead of
 // rounding it, so a sum is never left in tensor memory for long: each 64-deep stage starts a fresh accumulator, the five small
 // terms go in first and a1 b1 last (four steps that see the full magnitude), and the epilogue warps add the stage's result to
 // their fp32 registers with rounding.
@@ -100,7 +104,18 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ float4 plus(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+constexpr float kScale = 65536.f, kUnscale = 1.f / (kScale * kScale);     // of the operands before they are split, of the sums
+__device__ __forceinline__ float4 scaled(float4 v) {
+    const float2 a = halves(mul2(pack2(v.x, v.y), pack2(kScale, kScale))), b = halves(mul2(pack2(v.z, v.w), pack2(kScale, kScale)));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
 
 // two numbers to their leading bf16 parts (packed, the first in the low half); the rests replace them
 __device__ __forceinline__ uint32_t take_bf16(float& x, float& y) {
@@ -173,6 +188,8 @@ struct Feed {
     static __device__ __forceinline__ void put(float4 (&x)[kHalf], uint32_t planes, uint32_t plane, int t) {
         const uint32_t q = t % kPerRow, r = t / kPerRow;
         const uint32_t to = planes + (kOuter ? q / 16 : 0u) * kBlock64B + (r + H * kHalf * kStep) * kRowB + ((((q % 16) >> 1) ^ (r & 7u)) << 4) + (q & 1u) * 8;
+#pragma unroll
+        for (int i = 0; i < kHalf; ++i) x[i] = scaled(x[i]);
 #pragma unroll
         for (int s = 0; s < 3; ++s)
 #pragma unroll
@@ -515,8 +532,8 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float2 f = halves(tot[4 * j + i]);
-                    v[2 * i] = f.x;
-                    v[2 * i + 1] = f.y;
+                    v[2 * i] = f.x * kUnscale;
+                    v[2 * i + 1] = f.y * kUnscale;
                     z += f.x * 0.f + f.y * 0.f;
                 }
                 if (z != 0.f) {

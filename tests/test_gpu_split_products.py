@@ -128,3 +128,27 @@ def test_not_finite(out_in, accumulate):
         ok = np.isfinite(plain)
         # sums that hold 3.4e38 are compared by themselves: nothing else in them is visible
         assert (np.abs(got[ok] - plain[ok]) <= 1e-5 * np.maximum(np.abs(plain[ok]), 30.0)).all()
+
+
+@pytest.mark.parametrize("out_in", [False, True])
+@pytest.mark.parametrize("x_exp,dy_exp,w_exp", [(0, -118, 0), (-122, 0, 0), (0, 0, -126), (-70, -70, -70), (0, -140, 0), (-140, 12, -140)])
+def test_smallest_numbers(x_exp, dy_exp, w_exp, out_in):
+    """Operands down to the subnormal numbers keep the bits that an fp32 number has there (parts in bf16 would end at 2^-133)."""
+    M, kept, C_in, C_out = 1300, 700, 388, 516
+    scale = lambda a, e: (a * np.float32(2.0 ** (e // 2)) * np.float32(2.0 ** (e - e // 2))).astype(np.float32)
+    X, Wt, dY = (scale(a, e) for a, e in zip(synth.layer_inputs("f32", M, C_in, C_out, 94), (x_exp, w_exp, dy_exp)))
+    keep = np.sort(np.random.default_rng(7).permutation(M)[:kept]).astype(np.int32)
+    rows = torch.from_numpy(keep).cuda()
+    want = oracle.linear_backward(synth.to_f64(X[keep], "f32"), synth.to_f64(dY, "f32"), synth.to_f64(Wt, "f32"), keep)
+    want["Y"] = oracle.linear_forward(synth.to_f64(X, "f32"), synth.to_f64(Wt, "f32"), np.zeros(C_out, dtype=np.float32))
+    W = dev(np.ascontiguousarray(Wt.T) if out_in else Wt, "f32")
+    flags = sbp.SBP_FLAG_W_OUT_IN if out_in else 0
+    dW, db, dX = _backward(dev(X[keep], "f32"), dev(dY, "f32"), W, rows, None, M, kept, C_in, C_out, flags, float("nan"))
+    Y = torch.empty(M, C_out, device="cuda")
+    sbp.sbp_linear_forward(sbp.SBP_F32, dev(X, "f32"), W, None, M, C_in, C_out, Y, flags=flags)
+    torch.cuda.synchronize()
+    for name, got in dict(Y=Y, dW=dW.t() if out_in else dW, db=db, dX=dX).items():
+        w = want[name]
+        off = host(got.contiguous()).astype(np.float64) - w
+        # beside the error of any sum one rounding to a multiple of 2^-149
+        assert np.linalg.norm(off) <= REL * np.linalg.norm(w) + 2.0 ** -150 * np.sqrt(w.size), name
