@@ -39,7 +39,7 @@ constexpr int kThreads = 32 * (kMmaWarp + 4);   // (three of the last four warps
 constexpr int kLaunchRegs = 96, kEpiRegs = 104, kProducerRegs = 112, kMmaRegs = 40;
 static_assert(kEpiWarps * kEpiRegs + kProducerWarps * kProducerRegs + 4 * kMmaRegs <= (kMmaWarp + 4) * kLaunchRegs,
               "registers that the block is launched with");
-constexpr int kProducerBarrier = 1;
+constexpr int kProducerBarrier = 1, kEpiBarrier = 2;
 
 constexpr int kBCols = 64;                                                // columns of B that a block stages: half of the tile's
 constexpr uint32_t kAPlane = kTile * kRowB, kBPlane = kBCols * kRowB;
@@ -71,6 +71,7 @@ struct Product {
 struct SplitParams {
     Product p[2];                          // p[0] first: the deeper tiles
     uint32_t items[2];
+    uint32_t first, count;                 // the part of the list that this launch works through
     const int32_t* M_keep_dev;
     int64_t M_keep_cap;
     float* dX;                             // dropped rows to clear (nullptr: none)
@@ -80,13 +81,16 @@ struct SplitParams {
     int32_t* status_word;
 };
 
+// Behind it: room for the bias sums, then a byte for every item of the worker: which epilogue warps found sums that are not finite.
 struct Control {
     uint64_t full_bar[kStages], empty_bar[kStages], acc_full[kAccs], acc_empty[kAccs];
     uint32_t tmem_slot;
     int abort_flag;
 };
 constexpr uint32_t kSumBytes = 1024 * sizeof(double);
-constexpr uint32_t kSmemBytes = kStages * kStageBytes + kSlotBytes + 256 + kSumBytes + 1024;
+constexpr uint32_t kFlagsAt = kStages * kStageBytes + kSlotBytes + 256 + kSumBytes;
+constexpr uint32_t kMaxRounds = 1024;                                     // items of a worker in a launch: a byte each, see Control
+constexpr uint32_t kSmemBytes = kFlagsAt + kMaxRounds + 1024;
 static_assert(sizeof(Control) <= 256 && kSmemBytes <= 227 * 1024, "shared memory of a block");
 
 __device__ __forceinline__ uint64_t pack2(float x, float y) {
@@ -107,6 +111,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
 __device__ __forceinline__ float4 plus(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
@@ -254,27 +263,155 @@ __device__ __forceinline__ uint32_t list_position(uint32_t n, uint32_t worker, u
     return n * workers + ((n & 1u) ? workers - 1u - worker : worker);
 }
 
-// One output element the plain way, for sums that did not come out finite: with an infinite (or all but infinite) operand the parts
-// are infinity and NaN, whatever the product itself is.
-__device__ __noinline__ float plain_sum(const Product& p, int64_t m, int64_t n, int64_t d_begin, int64_t d_end) {
-    const float* a = p.a_outer ? p.A + m : p.A + (int64_t)mapped_row(p.a_map, m) * p.lda;
-    const float* b = p.b_outer ? p.B + n : p.B + (int64_t)mapped_row(p.b_map, n) * p.ldb;
-    float s = 0.f;
-#pragma unroll 4
-    for (int64_t d = d_begin; d < d_end; ++d) {
-        const float x = p.a_outer ? __ldg(a + (int64_t)mapped_row(p.a_map, d) * p.lda) : __ldg(a + d);
-        const float y = p.b_outer ? __ldg(b + (int64_t)mapped_row(p.b_map, d) * p.ldb) : __ldg(b + d);
-        s = fmaf(x, y, s);
-    }
-    return s;
+// position in the whole list of the n-th item of a worker; past its part: none
+__device__ __forceinline__ bool next_item(const SplitParams& prm, uint32_t n, uint32_t worker, uint32_t workers, uint32_t& q) {
+    const uint32_t at = list_position(n, worker, workers);
+    q = prm.first + at;
+    return at < prm.count;
 }
-__device__ __noinline__ void repair(const Product& p, int64_t m, int64_t n0, uint64_t bad, int64_t d_begin, int64_t d_end, float* dst) {
-    for (; bad != 0; bad &= bad - 1) {
-        const int c = __ffsll((long long)bad) - 1;
-        if (n0 + c >= p.cols) break;
-        float s = plain_sum(p, m, n0 + c, d_begin, d_end);
-        if (p.bias != nullptr) s += __ldg(p.bias + n0 + c);
-        dst[c] = p.accumulate ? dst[c] + s : s;
+
+// ---- sums that did not come out finite ----
+// With an infinite (or all but infinite) operand the parts are infinity and NaN, whatever the product itself is.  Such sums are made again
+// with FMAs once the block's list is done: the products then wait for nobody (their waits are bounded, and this work is as deep as the reduction).
+// The eight epilogue warps take 64 rows x 128 columns at a time, 16 columns a warp and 8 x 4 sums a thread (4 x 4: twice the time, shared
+// memory reads), over stages of 64 that they copy into the ring; each stage's sums are added to totals in shared memory, which leaves the registers
+// to the FMAs.  768 -> 3072, 3136 rows with 1568 kept, forward and dW + db + dX, finite 110 and 114 us: one infinite row of X and dY 204 and 642,
+// all NaN 227 and 167, all sums (operands of 2^114) 987 and 1121; 25000 kept rows, dW + db + dX, finite 1.15 ms: one infinite row 6.5, all NaN 1.3.
+// (One thread a sum, to the end whatever it had become, took 13 and 69 ms for the infinite row at 1568, 92 and 89 for the NaNs.)
+constexpr int kStripRows = 64, kPlainStages = 3, kPlainLd = kBK + 4;     // a row of an operand stored by extent: 16 bytes more, other banks
+constexpr uint32_t kPlainA = kStripRows * kPlainLd * 4, kPlainB = kTile * kPlainLd * 4, kPlainStage = kPlainA + kPlainB;
+constexpr uint32_t kTotalsAt = kPlainStages * kPlainStage;
+static_assert(kTotalsAt + kStripRows * kTile * 4 <= kStages * kStageBytes + kSlotBytes, "the ring holds the stages and the totals");
+
+template <bool kOuter, int kExtent>
+__device__ __forceinline__ void copy_plain(uint32_t to, const float* base, uint32_t ld, const int32_t* map, int e0, int extent, int d0, int d_end, int t) {
+    constexpr int kPerRow = kOuter ? kExtent / 4 : kBK / 4, kRows = kOuter ? kBK : kExtent;
+#pragma unroll 2
+    for (int i = 0; i < kRows * kPerRow / (32 * kEpiWarps); ++i) {
+        const int v = t + i * 32 * kEpiWarps, r = v / kPerRow, c = v % kPerRow * 4;
+        const int row = (kOuter ? d0 : e0) + r, col = (kOuter ? e0 : d0) + c;
+        const bool in = row < (kOuter ? d_end : extent) && col < (kOuter ? extent : d_end);
+        ptx::cp_async_16(to + (r * (kOuter ? kExtent : kPlainLd) + c) * 4, in ? base + (int64_t)mapped_row(map, row) * ld + col : base, in ? 16u : 0u);
+    }
+}
+// rows [m0, m0 + 64) of an item; want: the warps' regions (32 rows x 64 columns) among them that are written
+template <bool kAOuter, bool kBOuter>
+__device__ __forceinline__ void plain_strip(const Product& p, const Item& item, int m0, uint32_t want, uint32_t ring) {
+    int t;                                                                 // read anew: what follows from it would else be kept from the kernel's start
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    const int warp = t >> 5, lane = t & 31;                                // the epilogue warps are the block's first
+    const uint32_t a_at = (kAOuter ? (lane >> 2) * 4 : (lane >> 2) * kPlainLd) * 4;
+    const uint32_t b_at = kPlainA + (kBOuter ? warp * 16 + (lane & 3) * 4 : (warp * 16 + (lane & 3)) * kPlainLd) * 4;
+    const uint32_t totals = ring + kTotalsAt + t * 8;
+    const auto row_of = [&](int i) { return kAOuter ? (lane >> 2) * 4 + i % 4 + i / 4 * 32 : (lane >> 2) + 8 * i; };
+    const auto col_of = [&](int i) { return item.e_b0 + warp * 16 + (kBOuter ? (lane & 3) * 4 + i : (lane & 3) + 4 * i); };
+    // whether the sum of row i and column c is one to write: regions in `want` are (row / 32) + 2 (column / 64)
+    const auto mine = [&](int i, int c) { return ((want >> (row_of(i) / 32 + warp / 4 * 2)) & 1u) != 0 && m0 + row_of(i) < item.rows && col_of(c) < p.cols; };
+    const auto copy = [&](uint32_t k) {
+        if (k < item.num_kb) {
+            const uint32_t to = ring + k % kPlainStages * kPlainStage;
+            const int d0 = item.d_begin + (int)k * kBK;
+            copy_plain<kAOuter, kStripRows>(to, p.A, p.lda, p.a_map, m0, item.rows, d0, item.d_end, t);
+            copy_plain<kBOuter, kTile>(to + kPlainA, p.B, p.ldb, p.b_map, item.e_b0, p.cols, d0, item.d_end, t);
+        }
+        ptx::cp_async_commit();
+    };
+    const auto read2 = [](uint32_t from) {
+        float2 v;
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(from));
+        return v;
+    };
+    const auto read4 = [](uint32_t from) {
+        float4 v;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(from));
+        return v;
+    };
+#pragma unroll 1
+    for (uint32_t ahead = 0; ahead < item.num_kb + kPlainStages - 1; ++ahead) {
+        copy(ahead);
+        if (ahead < kPlainStages - 1) continue;
+        const uint32_t k = ahead - (kPlainStages - 1);
+        ptx::cp_async_wait<kPlainStages - 1>();
+        ptx::bar_named<kEpiBarrier, 32 * kEpiWarps>();
+        const uint32_t stage = ring + k % kPlainStages * kPlainStage;
+        uint64_t s[4][4] = {};                                             // rows in pairs
+#pragma unroll 2
+        for (int d = 0; d < kBK; d += 2) {
+            float2 a2[8], b2[4];                                           // inner: two depths of each row; outer: four rows of each depth
+#pragma unroll
+            for (int i = 0; i < (kAOuter ? 0 : 8); ++i) a2[i] = read2(stage + a_at + (i * 8 * kPlainLd + d) * 4);
+#pragma unroll
+            for (int i = 0; i < (kBOuter ? 0 : 4); ++i) b2[i] = read2(stage + b_at + (i * 4 * kPlainLd + d) * 4);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float4 a4[2], b4;
+#pragma unroll
+                for (int i = 0; i < (kAOuter ? 2 : 0); ++i) a4[i] = read4(stage + a_at + ((d + j) * kStripRows + i * 32) * 4);
+                if (kBOuter) b4 = read4(stage + b_at + (d + j) * kTile * 4);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint64_t rows = kAOuter ? (r % 2 ? pack2(a4[r / 2].z, a4[r / 2].w) : pack2(a4[r / 2].x, a4[r / 2].y))
+                                                  : (j ? pack2(a2[2 * r].y, a2[2 * r + 1].y) : pack2(a2[2 * r].x, a2[2 * r + 1].x));
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float col = kBOuter ? (c == 0 ? b4.x : c == 1 ? b4.y : c == 2 ? b4.z : b4.w) : (j ? b2[c].y : b2[c].x);
+                        s[r][c] = fma2(rows, pack2(col, col), s[r][c]);
+                    }
+                }
+            }
+        }
+        bool open = false;                                                 // a NaN stays one: nothing is left to do once all sums are
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t at = totals + (r * 4 + c) * (32 * kEpiWarps * 8);
+                uint64_t sum = 0ull;
+                if (k != 0) asm volatile("ld.shared.b64 %0, [%1];" : "=l"(sum) : "r"(at));
+                sum = add2(sum, s[r][c]);
+                asm volatile("st.shared.b64 [%0], %1;" ::"r"(at), "l"(sum) : "memory");
+                const float2 f = halves(sum);
+                open = open || (f.x == f.x && mine(2 * r, c)) || (f.y == f.y && mine(2 * r + 1, c));
+            }
+        if (!ptx::bar_or<kEpiBarrier, 32 * kEpiWarps>(open)) break;        // (and the stage has been read)
+    }
+    ptx::cp_async_wait<0>();
+    ptx::bar_named<kEpiBarrier, 32 * kEpiWarps>();                         // before the next strip's copies
+#pragma unroll 1
+    for (int i = 0; i < 8; ++i) {
+        if (m0 + row_of(i) >= item.rows) continue;
+        float* dst = p.out + (int64_t)item.split * p.split_stride + (int64_t)mapped_row(p.out_map, m0 + row_of(i)) * p.ld_out;
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+            if (!mine(i, c)) continue;
+            float v;
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(totals + (i / 2 * 4 + c) * (32 * kEpiWarps * 8) + i % 2 * 4));
+            if (p.bias != nullptr) v += __ldg(p.bias + col_of(c));
+            dst[col_of(c)] = p.accumulate ? dst[col_of(c)] + v : v;
+        }
+    }
+}
+
+// every strip that the epilogue warps have noted
+__device__ __forceinline__ void make_plain_sums(const SplitParams& prm, int M_keep) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = ptx::smem_addr(smem_raw), ring = (raw + 1023u) & ~1023u, rank = ptx::cluster_ctarank();
+    const uint32_t workers = gridDim.x >> 1, worker = blockIdx.x >> 1;
+    for (uint32_t n = 0; n * workers < prm.count; ++n) {
+        uint32_t warps;
+        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(warps) : "r"(ring + kFlagsAt + n));
+        uint32_t q;
+        if (warps == 0 || !next_item(prm, n, worker, workers, q)) continue;
+        const Product& p = prm.p[q < prm.items[0] ? 0 : 1];
+        const Item item = item_of(p, q < prm.items[0] ? q : q - prm.items[0], M_keep);
+        for (int s = 0; s < kTile / kStripRows; ++s) {                     // warp w has rows 32 (w % 4) + {0..31}, half w / 4 of the columns
+            const uint32_t want = ((warps >> (2 * s)) & 3u) | ((warps >> (2 * s + 4)) & 3u) << 2;
+            if (want == 0) continue;
+            const int m0 = item.e_a0 + (int)rank * kTile + s * kStripRows;
+            if (p.a_outer) plain_strip<true, true>(p, item, m0, want, ring);
+            else if (p.b_outer) plain_strip<false, true>(p, item, m0, want, ring);
+            else plain_strip<false, false>(p, item, m0, want, ring);
+        }
     }
 }
 
@@ -386,6 +523,7 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
         ctl->abort_flag = 0;
         ptx::fence_mbar_init();
     }
+    for (uint32_t i = threadIdx.x; i < kMaxRounds / 4; i += kThreads) reinterpret_cast<uint32_t*>(tail + 256 + kSumBytes)[i] = 0u;
     if (warp == kMmaWarp) ptx::tmem_alloc_pair(ptx::smem_addr(&ctl->tmem_slot), 512);
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -396,7 +534,6 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
     pdl_wait();
     const bool skip_all = status_word != nullptr && *reinterpret_cast<volatile int32_t*>(status_word) != 0;
     const int M_keep = (int)load_m_keep(prm.M_keep_dev, prm.M_keep_cap);
-    const uint32_t items = prm.items[0] + prm.items[1];
 
     if (warp >= kMmaWarp) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMmaRegs));
     if (skip_all || warp > kMmaWarp) {
@@ -405,9 +542,9 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
         const bool leader = ptx::elect_one();
         uint32_t it = 0;
         bool ok = true;
-        for (uint32_t n = 0; ok && n * workers < items; ++n) {
-            const uint32_t q = list_position(n, worker, workers);
-            if (q >= items) continue;
+        for (uint32_t n = 0; ok && n * workers < prm.count; ++n) {
+            uint32_t q;
+            if (!next_item(prm, n, worker, workers, q)) continue;
             const Product& p = prm.p[q < prm.items[0] ? 0 : 1];
             const Item item = item_of(p, q < prm.items[0] ? q : q - prm.items[0], M_keep);
             // depth inner: a 16-deep slice is 32 bytes along the swizzled rows; outer: 16 rows, 64-wide blocks 8 KB apart
@@ -456,9 +593,9 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kProducerRegs));
         uint32_t it = 0;
         bool ok = true;
-        for (uint32_t n = 0; ok && n * workers < items; ++n) {
-            const uint32_t q = list_position(n, worker, workers);
-            if (q >= items) continue;
+        for (uint32_t n = 0; ok && n * workers < prm.count; ++n) {
+            uint32_t q;
+            if (!next_item(prm, n, worker, workers, q)) continue;
             const Product& p = prm.p[q < prm.items[0] ? 0 : 1];
             const Item item = item_of(p, q < prm.items[0] ? q : q - prm.items[0], M_keep);
             if (p.a_outer) ok = produce<true, true>(p, item, ring, ctl, sums_s, rank, it, status_word);
@@ -489,9 +626,9 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
         const uint32_t lane_off = (quad * 32u) << 16;
         uint32_t it = 0;
         bool ok = true;
-        for (uint32_t n = 0; ok && n * workers < items; ++n) {
-            const uint32_t q = list_position(n, worker, workers);
-            if (q >= items) continue;
+        for (uint32_t n = 0; ok && n * workers < prm.count; ++n) {
+            uint32_t q;
+            if (!next_item(prm, n, worker, workers, q)) continue;
             const Product& p = prm.p[q < prm.items[0] ? 0 : 1];
             const Item item = item_of(p, q < prm.items[0] ? q : q - prm.items[0], M_keep);
             if (item.none) continue;
@@ -519,27 +656,27 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
             }
             if (!ok) break;
             const int m = item.e_a0 + (int)rank * kTile + (int)quad * 32 + lane, n0 = item.e_b0 + (int)half * 64;
-            if (m >= item.rows || n0 >= p.cols) continue;
+            uint64_t z2 = 0ull;                                            // zeros times the sums
+#pragma unroll
+            for (int j = 0; j < 32; ++j) z2 = fma2(tot[j], 0ull, z2);
+            const float2 z = halves(z2);
+            // Not finite: all sums of this warp are made again below, and nothing is written here.  (A branch for the note costs spilled registers.)
+            const bool again = __any_sync(0xffffffffu, m < item.rows && n0 < p.cols && !(z.x + z.y == 0.f));
+            asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q red.shared.or.b32 [%0], %1;\n\t}"
+                         ::"r"(ring + kFlagsAt + n / 4 * 4), "r"(1u << (8 * (n % 4) + warp)), "r"((uint32_t)(again && lane == 0)) : "memory");
+            if (again || m >= item.rows || n0 >= p.cols) continue;
             float* dst = p.out + (int64_t)item.split * p.split_stride + (int64_t)mapped_row(p.out_map, m) * p.ld_out + n0;
             const int cols = p.cols - n0 < 64 ? p.cols - n0 : 64;
             const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31u) == 0;
-            uint64_t bad = 0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {                                  // a row's sums leave eight, a whole sector, at a time
                 if (j * 8 >= cols) break;
-                float v[8], z = 0.f;
-                uint32_t not_finite = 0;
+                float v[8];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float2 f = halves(tot[4 * j + i]);
                     v[2 * i] = f.x * kUnscale;
                     v[2 * i + 1] = f.y * kUnscale;
-                    z += f.x * 0.f + f.y * 0.f;
-                }
-                if (z != 0.f) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) not_finite |= fabsf(v[i]) < INFINITY ? 0u : 1u << i;
-                    bad |= (uint64_t)not_finite << (8 * j);
                 }
                 const int n8 = cols - j * 8 < 8 ? 4 : 8;
                 if (p.bias != nullptr) {
@@ -547,10 +684,10 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
                     for (int i = 0; i < 8; ++i) v[i] += i < n8 ? __ldg(p.bias + n0 + j * 8 + i) : 0.f;
                 }
                 float* o = dst + j * 8;
-                if (p.accumulate) {                                        // sums that are made again below leave what is there
+                if (p.accumulate) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        if (i < n8) v[i] = (not_finite >> i) & 1u ? o[i] : o[i] + v[i];
+                        if (i < n8) v[i] = o[i] + v[i];
                 }
                 if (wide && n8 == 8) {
                     asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
@@ -560,8 +697,9 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
                     if (n8 == 8) *reinterpret_cast<float4*>(o + 4) = make_float4(v[4], v[5], v[6], v[7]);
                 }
             }
-            if (bad != 0) repair(p, m, n0, bad, item.d_begin, item.d_end, dst);
         }
+        // The last products have been read out, so nothing of the ring is in use any more.
+        if (!ptx::bar_or<kEpiBarrier, 32 * kEpiWarps>(!ok)) make_plain_sums(prm, M_keep);
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -576,7 +714,10 @@ split_products_kernel(const __grid_constant__ SplitParams prm) {
 constexpr int64_t kPairs = kNumSMs / 2;
 constexpr int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-cudaError_t launch(const SplitParams& prm, cudaStream_t stream) {
+// A launch holds at most kMaxRounds items of a worker: 2.5e9 sums.
+int64_t launches_of(int64_t items) { return ceil_div(items, kMaxRounds * kPairs); }
+
+cudaError_t launch(SplitParams prm, cudaStream_t stream) {
     const cudaError_t opt = opt_in_dynamic_smem<split_products_kernel>((int)kSmemBytes);
     if (opt != cudaSuccess) return opt;
     // the roles' registers come out of those that the block is launched with: a build that gives it fewer must not run
@@ -585,8 +726,17 @@ cudaError_t launch(const SplitParams& prm, cudaStream_t stream) {
         return cudaFuncGetAttributes(&a, split_products_kernel) == cudaSuccess && a.numRegs >= kLaunchRegs;
     }();
     if (!enough) return cudaErrorLaunchOutOfResources;
-    const int64_t items = (int64_t)prm.items[0] + prm.items[1], used = prm.dX != nullptr || items > kPairs ? kPairs : items;    // the zeros take every SM
-    return launch_pdl_cluster(split_products_kernel, dim3((unsigned)(2 * used)), dim3(kThreads), kSmemBytes, 2u, stream, prm);
+    const int64_t items = (int64_t)prm.items[0] + prm.items[1];
+    for (int64_t first = 0; first < items; first += kMaxRounds * kPairs) {
+        const int64_t count = items - first < kMaxRounds * kPairs ? items - first : kMaxRounds * kPairs;
+        prm.first = (uint32_t)first;
+        prm.count = (uint32_t)count;
+        const int64_t used = prm.dX != nullptr || count > kPairs ? kPairs : count;                 // the zeros take every SM
+        const cudaError_t e = launch_pdl_cluster(split_products_kernel, dim3((unsigned)(2 * used)), dim3(kThreads), kSmemBytes, 2u, stream, prm);
+        if (e != cudaSuccess) return e;
+        prm.dX = nullptr;                                                                          // the first launch has written them
+    }
+    return cudaSuccess;
 }
 
 // Time of a list of `nx` items of `cx` us followed by `nw` of `cw`, dealt to `g` workers as list_position does.  The workers that take part
@@ -675,7 +825,9 @@ size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
 
 int split_backward_kernel_count(bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
     if (!want_dw && !want_dx) return 0;
-    return 1 + (want_dw && split_plan(M_keep_cap, C_in, C_out, w_out_in, want_dx) > 1 ? 1 : 0);
+    const int splits = want_dw ? split_plan(M_keep_cap, C_in, C_out, w_out_in, want_dx) : 1;
+    const int64_t nx = want_dx ? tiles_of(M_keep_cap, C_in) : 0, nw = want_dw ? (w_out_in ? tiles_of(C_out, C_in) : tiles_of(C_in, C_out)) * splits : 0;
+    return (int)launches_of(nx + nw) + (splits > 1 ? 1 : 0);
 }
 
 cudaError_t launch_split_backward(const float* X_keep, const float* dY, const float* W, bool w_out_in, const int32_t* dy_rows,

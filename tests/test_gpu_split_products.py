@@ -152,3 +152,87 @@ def test_smallest_numbers(x_exp, dy_exp, w_exp, out_in):
         off = host(got.contiguous()).astype(np.float64) - w
         # beside the error of any sum one rounding to a multiple of 2^-149
         assert np.linalg.norm(off) <= REL * np.linalg.norm(w) + 2.0 ** -150 * np.sqrt(w.size), name
+
+
+def _poisoned(what, X, dY, rows, g):
+    """rows: the kept rows; X, dY as wide as the layer's output and input"""
+    inf, nan = float("inf"), float("nan")
+    r = int(rows[5])
+    if what == "one infinite row":
+        X[r], dY[r] = inf, -inf
+    elif what == "one NaN row":
+        X[r], dY[r] = nan, nan
+    elif what == "one infinite element":
+        X[r, 3], dY[r, 7] = inf, inf
+    elif what == "NaN":
+        X.fill_(nan)
+        dY.fill_(nan)
+    elif what == "infinite":
+        X.mul_(inf)
+        dY.mul_(inf)
+    else:                                            # finite, but beyond what the parts hold
+        X.mul_(2.0 ** 114)
+        dY.mul_(2.0 ** -20)
+
+
+@pytest.mark.parametrize("what", ["one infinite row", "one NaN row", "one infinite element", "NaN", "infinite", "huge"])
+@pytest.mark.parametrize("M,kept,C_in,C_out,out_in", [(3136, 1568, 768, 3072, False), (30000, 25001, 772, 260, True)])
+def test_sums_that_are_made_again(M, kept, C_in, C_out, out_in, what):
+    """Any share of sums that are not finite, at any depth: what the CUDA-core products give, for a bounded multiple of the finite call's time."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    X, dY = torch.randn(M, C_in, device="cuda", generator=g), torch.randn(M, C_out, device="cuda", generator=g)
+    W = torch.randn(*((C_out, C_in) if out_in else (C_in, C_out)), device="cuda", generator=g) * C_in ** -0.5
+    rows = torch.randperm(M, device="cuda", generator=g)[:kept].sort().values.int()
+    flags = sbp.SBP_FLAG_W_OUT_IN if out_in else 0
+    nb = sbp.sbp_linear_backward_workspace_bytes(sbp.SBP_F32, M, kept, C_in, C_out)
+    ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Y, dW, db, dX = torch.empty(M, C_out, device="cuda"), torch.empty_like(W), torch.empty(C_out, device="cuda"), torch.empty_like(X)
+
+    def call(extra=0):
+        Xk = X[rows.long()]
+        marks = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+        marks[0].record()
+        sbp.sbp_linear_forward(sbp.SBP_F32, X, W, None, M, C_in, C_out, Y, flags=flags | extra, status_word=status)
+        marks[1].record()
+        sbp.sbp_linear_backward(sbp.SBP_F32, Xk, dY, W, rows, None, M, kept, C_in, C_out, dW, db, dX, flags | extra, ws, nb, status)
+        marks[2].record()
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        return np.array([marks[0].elapsed_time(marks[1]), marks[1].elapsed_time(marks[2])]), [t.clone() for t in (Y, dW, db, dX)]
+
+    finite = np.min([call()[0] for _ in range(4)], axis=0)
+    _poisoned(what, X, dY, rows, g)
+    times, outs = zip(*[call() for _ in range(4)])
+    # Measured: up to 9 times (all sums made again, none of them a NaN).  One thread a sum, without an early end, took 100 to 800 times.
+    assert (np.min(times, axis=0) <= 25.0 * finite + 0.1).all(), (np.min(times, axis=0), finite)
+    plain = call(sbp.SBP_FLAG_PLAIN_FMA)[1]
+    for name, got, want in zip(("Y", "dW", "db", "dX"), outs[0], plain):
+        assert torch.equal(got.isnan(), want.isnan()) and torch.equal(got.isinf(), want.isinf()), name
+        assert torch.equal(got[want.isinf()], want[want.isinf()]), name
+        a, b = (torch.where(want.isfinite(), t, torch.zeros_like(t)).double() for t in (got, want))
+        # two fp32 sums of the same terms: 2.5e-7 to 2e-6 (chains of FMAs) and below 3e-7 off
+        assert float((a - b).norm()) <= 4e-6 * float(b.norm()), name
+
+
+def test_more_items_than_a_launch_holds():
+    """A worker notes sums to be made again for 1024 items; longer lists go in several launches.  Rows of either side of the cut, the first
+    launch's last tile and the last, ragged one with a NaN in them."""
+    M, C_in, C_out = 1024 * 74 * 256 + 300, 40, 32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(12)
+    X, W = torch.randn(M, C_in, device="cuda", generator=g), torch.randn(C_in, C_out, device="cuda", generator=g)
+    X[M - 400, 3] = X[M - 7, 5] = float("nan")
+    Y = torch.full((M, C_out), 7.0, device="cuda")
+    sbp.sbp_linear_forward(sbp.SBP_F32, X, W, None, M, C_in, C_out, Y)
+    plain = torch.full((M, C_out), -7.0, device="cuda")
+    sbp.sbp_linear_forward(sbp.SBP_F32, X, W, None, M, C_in, C_out, plain, flags=sbp.SBP_FLAG_PLAIN_FMA)
+    torch.cuda.synchronize()
+    bad = torch.zeros(M, dtype=torch.bool, device="cuda")
+    bad[[M - 400, M - 7]] = True
+    assert bool(Y[bad].isnan().all()) and not bool(Y[~bad].isnan().any())
+    # sums of 40 terms of size 1 in two orders: below 40 * 2^-24 of the terms' sum of squares' root each
+    Y[bad], plain[bad] = 0.0, 0.0
+    assert float((Y - plain).abs().max()) <= 2 * 40 * 2.0 ** -24 * 40 ** 0.5
+    assert float((Y - plain).norm() / plain.norm()) <= 3e-7
