@@ -236,3 +236,20 @@ def test_more_items_than_a_launch_holds():
     Y[bad], plain[bad] = 0.0, 0.0
     assert float((Y - plain).abs().max()) <= 2 * 40 * 2.0 ** -24 * 40 ** 0.5
     assert float((Y - plain).norm() / plain.norm()) <= 3e-7
+
+
+@pytest.mark.parametrize("kept,padding,C_in,C_out,out_in", [(1500, 0, 768, 3072, True), (1501, 77, 772, 3076, False)])
+def test_bias_sums_of_one_piece_are_rounded_once(kept, padding, C_in, C_out, out_in):
+    assert sbp.sbp_linear_backward_kernel_count(sbp.SBP_F32, 2 * kept, kept, C_in, C_out, 1, 1, 1, sbp.SBP_FLAG_W_OUT_IN if out_in else 0) == 1
+    g = torch.Generator(device="cuda")
+    g.manual_seed(13)
+    M, valid = 2 * kept, kept - padding
+    dY, X, W = (torch.randn(*s, device="cuda", generator=g) for s in ((M, C_out), (kept, C_in), (C_out, C_in) if out_in else (C_in, C_out)))
+    rows = torch.randperm(M, device="cuda", generator=g)[:kept].sort().values.int()
+    count = torch.tensor([valid], dtype=torch.int32, device="cuda") if padding else None
+    _, db, _ = _backward(X, dY, W, rows, count, M, kept, C_in, C_out, sbp.SBP_FLAG_W_OUT_IN if out_in else 0, float("nan"))
+    kept_dY = dY[rows[:valid].long()].double()
+    want = kept_dY.sum(0)
+    # half a unit in the last place, and what the sums of the rounding errors lose: each below 2^-24 of an error of 2^-24 of a partial sum
+    bound = 2.0 ** -24 * want.abs() + valid * 2.0 ** -48 * kept_dY.abs().sum(0)
+    assert bool(((db.double() - want).abs() <= bound).all())
