@@ -601,6 +601,16 @@ size_t fma_dw_workspace_bytes(sbp_dtype dt, int64_t M_keep_cap, int64_t C_in, in
     return most > 1 ? (size_t)most * (size_t)(C_in + 1) * (size_t)C_out * sizeof(float) : 0;
 }
 
+// a 16-deep step of a 64 x 64 (64 x 128) tile as part of the longest chain and of an SM's share, us; the start; the reduce launch
+double fma_backward_us(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
+    const FmaPlan pl = fma_plan(true, out_in, M_keep_cap, C_in, C_out, want_dw, want_dx);
+    const double x_steps = (double)ceil_div(C_out, 16), w_steps = (double)ceil_div(ceil_div(M_keep_cap, 16), pl.splits);
+    const double share = ((double)(pl.x_rows * pl.x_cols) * x_steps + (double)(pl.w_rows * pl.w_cols * pl.splits) * w_steps) / kNumSMs;
+    const double chain = want_dx && (!want_dw || x_steps > w_steps) ? x_steps : w_steps;
+    const double reduce = pl.splits > 1 ? 2.2 + 0.5 * (double)pl.splits * (double)C_in * (double)C_out * 8.0 / 4e6 : 0.0;
+    return 3.6 + (pl.wide ? 0.8 * (chain + share) : 0.48 * chain + 0.36 * share) + reduce;
+}
+
 int fma_backward_kernel_count(sbp_dtype dt, bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
     if (!want_dw && !want_dx) return 0;
     return 1 + (want_dw && fma_plan(dt == SBP_F32, w_out_in, M_keep_cap, C_in, C_out, want_dw, want_dx).splits > 1 ? 1 : 0);

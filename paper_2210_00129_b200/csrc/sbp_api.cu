@@ -34,8 +34,8 @@ inline bool use_tensor_cores(sbp_dtype dt, uint32_t flags, int64_t M, int64_t M_
 }
 
 // fp32 layers: the tensor cores take the products in three bf16 parts each where that is quicker than the CUDA cores
-inline bool use_split(sbp_dtype dt, uint32_t flags, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx) {
-    return dt == SBP_F32 && !(flags & SBP_FLAG_PLAIN_FMA) && split_backward_supported(M_keep_cap, C_in, C_out, want_dx);
+inline bool use_split(sbp_dtype dt, uint32_t flags, bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
+    return dt == SBP_F32 && !(flags & SBP_FLAG_PLAIN_FMA) && split_backward_quicker(w_out_in, M_keep_cap, C_in, C_out, want_dw, want_dx);
 }
 
 // Weights stored [C_out, C_in]: whether the products read W and write dW in place, or work on transposed copies in the
@@ -275,7 +275,7 @@ sbp_status backward_direct(sbp_dtype dt, bool w_out_in, bool fresh_dw, const voi
                                                 dw_accumulate, dX, db_rides ? db : nullptr, accumulate, w_out_in, ws_dw, ws_db,
                                                 status_word, stream);
         if (s != SBP_OK) return s;
-    } else if ((dW != nullptr || dX != nullptr) && use_split(dt, flags, M_keep_cap, C_in, C_out, dX != nullptr)) {
+    } else if ((dW != nullptr || dX != nullptr) && use_split(dt, flags, w_out_in, M_keep_cap, C_in, C_out, dW != nullptr, dX != nullptr)) {
         if (launch_split_backward((const float*)X_keep, (const float*)dY, (const float*)W, w_out_in, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap,
                                   C_in, C_out, dW, db_rides ? db : nullptr, dw_accumulate, accumulate, (float*)dX, ws_dw, status_word,
                                   stream) != cudaSuccess)
@@ -345,7 +345,7 @@ int sbp_linear_backward_kernel_count(sbp_dtype dt, int64_t M, int64_t M_keep_cap
     if (want_db && !db_rides) n += 2;                      // strip partials + fixed-order reduce
     if (tc) return n + tc_backward_kernel_count(M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0, db_rides,
                                                 (flags & SBP_FLAG_DY_COMPACT) != 0);
-    if (use_split(dt, flags, M_keep_cap, C_in, C_out, want_dX != 0))
+    if (use_split(dt, flags, direct, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0))
         return n + split_backward_kernel_count(direct, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0);
     return n + fma_backward_kernel_count(dt, direct, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0);
 }

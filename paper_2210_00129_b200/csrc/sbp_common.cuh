@@ -164,6 +164,7 @@ cudaError_t launch_reduce_partials_pair(const float* partials_a, int splits_a, i
 // dy_rows / dx_rows: row m of the product reads row dy_rows[m] of dY and writes row dx_rows[m] of dX
 // (nullptr = m itself); M = rows of dX
 size_t fma_dw_workspace_bytes(sbp_dtype dt, int64_t M_keep_cap, int64_t C_in, int64_t C_out);
+double fma_backward_us(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);      // fp32, estimated
 int    fma_backward_kernel_count(sbp_dtype dt, bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY, const void* W, bool w_out_in, const int32_t* dy_rows,
                                 const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
@@ -172,7 +173,8 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
 
 // the same products of fp32 layers on the tensor cores, each operand as a sum of three bf16 numbers
 bool   split_forward_supported(int64_t M, int64_t C_in, int64_t C_out);
-bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx);
+bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx);        // room for them in the workspace
+bool   split_backward_quicker(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
 int    split_backward_kernel_count(bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,

@@ -769,7 +769,7 @@ constexpr double kKbUs = 1.4, kItemUs = 2.5;                               // us
 
 int64_t tiles_of(int64_t rows, int64_t cols) { return ceil_div(rows, 2 * kTile) * ceil_div(cols, kTile); }
 
-int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, bool want_dx) {
+int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, bool want_dx, double* list_us = nullptr) {
     int best = 1;
     double best_us = 0.0;
     const int64_t w_kb = ceil_div(M_keep_cap, kBK), x_kb = ceil_div(C_out, kBK);
@@ -781,6 +781,7 @@ int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, boo
                           (s > 1 ? 2.0 + (double)s * (double)C_in * (double)C_out * 8.0 / 4e6 : 0.0);
         if (best_us == 0.0 || us < best_us * 0.99) { best_us = us; best = (int)s; }
     }
+    if (list_us != nullptr) *list_us = best_us;
     return best;
 }
 
@@ -791,17 +792,33 @@ int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, boo
 // 1839 and 184 10.4, 9.4, 152 with 2597 and 104 11.8, 10.6; 88 with 3193 and 264 9.4, 10.2, 64 with 3339 and 1232 20.6, 13.7, 32 with
 // 21611 and 168 11.1, 15.2; 232 with 164 and 128 10.8, 11.4, 296 with 162 and 72 13.7, 12.4, 304 with 103 and 32 13.3, 11.3.
 // dW + db + dX: 104 kept rows of 128 -> 144 11.5, 12.7 us, 649 of 152 -> 104 13.7, 12.1, 942 of 472 -> 48 15.9, 13.7; 6770 of 32 -> 72
-// 13.1, 13.7; few rows behind deep sums of dX 95 of 80 -> 376 16.2, 12.0, 72 of 32 -> 720 30.5, 21.9 (dW + db alone 16 of 1024 -> 3072
-// 7.7, 12.0, 500 of 40 -> 256 8.1, 10.2).
+// 13.1, 13.7; few rows behind deep sums of dX 95 of 80 -> 376 16.2, 12.0, 72 of 32 -> 720 30.5, 21.9.
 bool split_forward_supported(int64_t M, int64_t C_in, int64_t C_out) {
     if (M < 32 || C_in < 32 || C_out < 32) return false;
     const int64_t work = M * C_in * C_out;
-    return C_in >= 288 || (C_in >= 96 && work >= 36000000) || (C_in >= 56 && work >= 100000000) || (C_in >= 40 && work >= 400000000);
+    return C_in >= 288 || (C_in >= 96 && work >= 50000000) || (C_in >= 56 && work >= 100000000) || (C_in >= 40 && work >= 400000000);
 }
 bool split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx) {
     if (M_keep_cap < 16 || C_in < 32 || C_out < 32) return false;
     const int64_t work = M_keep_cap * C_in * C_out;
     return (want_dx && C_out >= 256) || (C_in >= 40 && C_out >= 40 && work >= 20000000) || work >= 80000000;
+}
+// Calls for dW, or dX, alone have half the work for the same start, and the CUDA cores cut dW into more pieces: there both times are
+// estimated (fits to 6500 shapes of 32 to 3072 channels and 16 to 60000 kept rows, 6 and 8 % off on average).  dW + db, CUDA cores and here: 32
+// kept rows of 2992 -> 352 5.7, 8.4 us, 131 of 2264 -> 100 8.7, 11.0, 1081 of 164 -> 156 11.0, 13.6, 1712 of 152 -> 248 13.8, 11.6; dX: 254 of
+// 1844 -> 72 6.3, 10.1, 613 of 732 -> 52 5.4, 8.5.  (The lines above alone took 522 of 3886 calls for dW + db that are more than 5 % slower
+// here, by up to 56 %, and 131 of 4786 for dX; 158 and 15 are left.)
+bool split_backward_quicker(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
+    if (!split_backward_supported(M_keep_cap, C_in, C_out, want_dx)) return false;
+    if (want_dw == want_dx) return true;
+    double us = 0.0;
+    if (want_dw) {
+        split_plan(M_keep_cap, C_in, C_out, out_in, false, &us);
+        us = 3.8 + 1.03 * us;
+    } else {
+        us = 4.5 + 0.85 * list_time(tiles_of(M_keep_cap, C_in), (double)ceil_div(C_out, kBK) * kKbUs + kItemUs, 0, 0.0, kPairs);
+    }
+    return us < fma_backward_us(out_in, M_keep_cap, C_in, C_out, want_dw, want_dx);
 }
 
 cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,

@@ -253,3 +253,42 @@ def test_bias_sums_of_one_piece_are_rounded_once(kept, padding, C_in, C_out, out
     # half a unit in the last place, and what the sums of the rounding errors lose: each below 2^-24 of an error of 2^-24 of a partial sum
     bound = 2.0 ** -24 * want.abs() + valid * 2.0 ** -48 * kept_dY.abs().sum(0)
     assert bool(((db.double() - want).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("out_in", [False, True])
+@pytest.mark.parametrize("wanted", ["dW", "dX", "dW db", "dX db", "dW dX", "db", "dW db dX"])
+@pytest.mark.parametrize("M,kept,padding,C_in,C_out,on_cuda_cores", [
+    (64, 32, 0, 2992, 352, {"dW", "dW db"}), (500, 254, 0, 1844, 72, {"dX", "dX db"}), (2000, 1081, 30, 164, 156, {"dW", "dW db", "dX", "dX db"}),
+    (6000, 5000, 100, 260, 388, set()), (1500, 700, 0, 508, 516, set()),
+])
+def test_calls_for_some_of_the_outputs(M, kept, padding, C_in, C_out, on_cuda_cores, wanted, out_in):
+    """dW or dX alone have a line of their own against the CUDA cores; every combination of outputs against the oracle, accumulated."""
+    X, Wt, dY = synth.layer_inputs("f32", M, C_in, C_out, 95)
+    keep = np.sort(np.random.default_rng(8).permutation(M)[:kept]).astype(np.int32)
+    valid = keep[:kept - padding]
+    rows, count = torch.from_numpy(keep).cuda(), torch.tensor([len(valid)], dtype=torch.int32, device="cuda")
+    want = oracle.linear_backward(synth.to_f64(X[valid], "f32"), synth.to_f64(dY, "f32"), synth.to_f64(Wt, "f32"), valid)
+    Xk, dY_d, W = dev(X[keep], "f32"), dev(dY, "f32"), dev(np.ascontiguousarray(Wt.T) if out_in else Wt, "f32")
+    nb = sbp.sbp_linear_backward_workspace_bytes(sbp.SBP_F32, M, kept, C_in, C_out)
+    results = []
+    for extra in (0, sbp.SBP_FLAG_PLAIN_FMA):
+        ws = torch.full((nb,), 0xff, dtype=torch.uint8, device="cuda")
+        out = dict(dW=torch.full_like(W, 0.25), db=torch.full((C_out,), 0.25, device="cuda"), dX=torch.full((M, C_in), float("nan"), device="cuda"))
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        sbp.sbp_linear_backward(sbp.SBP_F32, Xk, dY_d, W, rows, count, M, kept, C_in, C_out, *(out[n] if n in wanted.split() else None for n in ("dW", "db", "dX")),
+                                (sbp.SBP_FLAG_W_OUT_IN if out_in else 0) | sbp.SBP_FLAG_ACCUMULATE | extra, ws, nb, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        results.append(out)
+    got, plain = results
+    for name in wanted.split():
+        g = host((got[name].t() if out_in and name == "dW" else got[name]).contiguous()).astype(np.float64)
+        exact = want[name] + (0.0 if name == "dX" else 0.25)
+        assert np.linalg.norm(g - exact) <= (1e-6 if wanted in on_cuda_cores else REL) * np.linalg.norm(exact), name
+        same = torch.equal(got[name], plain[name])
+        if name != "db":
+            assert same == (wanted in on_cuda_cores), name
+    for name in set(got) - set(wanted.split()):
+        assert bool((got[name] == 0.25).all()) if name != "dX" else bool(got[name].isnan().all())
+    if "dX" in wanted:
+        assert not host(got["dX"])[np.setdiff1d(np.arange(M), valid)].view(np.uint8).any()
