@@ -350,7 +350,7 @@ int sbp_linear_backward_kernel_count(sbp_dtype dt, int64_t M, int64_t M_keep_cap
     return n + fma_backward_kernel_count(dt, direct, M_keep_cap, C_in, C_out, want_dW != 0, want_dX != 0);
 }
 
-int64_t sbp_plan_search_count(void) { return tc_plan_searches(); }
+int64_t sbp_plan_search_count(void) { return tc_plan_searches() + split_plan_searches(); }
 
 sbp_status sbp_act_backward(sbp_dtype dt, sbp_activation act, const void* Z_keep, const void* dH, const int32_t* M_keep_dev,
                             int64_t M_keep_cap, int64_t C, void* dZ, int32_t* status_word, void* stream) {

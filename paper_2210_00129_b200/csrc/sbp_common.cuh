@@ -176,6 +176,7 @@ bool   split_forward_supported(int64_t M, int64_t C_in, int64_t C_out);
 bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx);        // room for them in the workspace
 bool   split_backward_quicker(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out);
+int64_t split_plan_searches();           // shapes whose plans have been searched so far in this process
 int    split_backward_kernel_count(bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);
 cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, const float* bias, int64_t M, int64_t C_in, int64_t C_out,
                                  float* Y, int32_t* status_word, cudaStream_t stream);

@@ -21,6 +21,8 @@
 // stage's loads behind each conversion the registers spill.)  Measured on B200, 768 -> 3072, 3136 rows with 1568 kept, CUDA cores -> here: forward
 // 299 -> 87 us, dW + db + dX 395 -> 100; relative errors against 64-bit sums Y 2.5e-7 -> 0.8e-7, dW 5.0e-7 -> 1.2e-7, dX 7.0e-7 -> 1.5e-7,
 // db 0.7e-7 -> 0.6e-7.  Over 260 shapes of 32 to 2900 channels and 64 to 65536 rows no Y, dW or dX was further off than the CUDA cores'.
+#include <map>
+#include <tuple>
 #include <type_traits>
 
 #include "tc_ptx.cuh"
@@ -769,7 +771,9 @@ constexpr double kKbUs = 1.4, kItemUs = 2.5;                               // us
 
 int64_t tiles_of(int64_t rows, int64_t cols) { return ceil_div(rows, 2 * kTile) * ceil_div(cols, kTile); }
 
-int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, bool want_dx, double* list_us = nullptr) {
+struct SplitPlan { int splits; double us; };                               // us: of the tiles and the reduce launch
+
+SplitPlan search_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, bool want_dx) {
     int best = 1;
     double best_us = 0.0;
     const int64_t w_kb = ceil_div(M_keep_cap, kBK), x_kb = ceil_div(C_out, kBK);
@@ -781,8 +785,23 @@ int split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, boo
                           (s > 1 ? 2.0 + (double)s * (double)C_in * (double)C_out * 8.0 / 4e6 : 0.0);
         if (best_us == 0.0 || us < best_us * 0.99) { best_us = us; best = (int)s; }
     }
-    if (list_us != nullptr) *list_us = best_us;
-    return best;
+    return SplitPlan{best, best_us};
+}
+
+// Remembered for the life of the process, as the bf16 plans are (tc_backward.cu): the four plans of a shape are one search.
+struct ShapePlans { SplitPlan of[2][2]; };                                 // [out_in][want_dx]
+std::mutex g_shape_mutex;
+std::map<std::tuple<int64_t, int64_t, int64_t>, ShapePlans> g_shape_plans;
+
+SplitPlan split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_in, bool want_dx) {
+    const auto key = std::make_tuple(M_keep_cap, C_in, C_out);
+    std::lock_guard<std::mutex> lock(g_shape_mutex);
+    const auto it = g_shape_plans.find(key);
+    if (it != g_shape_plans.end()) return it->second.of[out_in][want_dx];
+    ShapePlans plans;
+    for (int v = 0; v < 4; ++v) plans.of[v & 1][v >> 1] = search_plan(M_keep_cap, C_in, C_out, (v & 1) != 0, (v & 2) != 0);
+    g_shape_plans[key] = plans;
+    return plans.of[out_in][want_dx];
 }
 
 }  // namespace
@@ -811,13 +830,8 @@ bool split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, b
 bool split_backward_quicker(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
     if (!split_backward_supported(M_keep_cap, C_in, C_out, want_dx)) return false;
     if (want_dw == want_dx) return true;
-    double us = 0.0;
-    if (want_dw) {
-        split_plan(M_keep_cap, C_in, C_out, out_in, false, &us);
-        us = 3.8 + 1.03 * us;
-    } else {
-        us = 4.5 + 0.85 * list_time(tiles_of(M_keep_cap, C_in), (double)ceil_div(C_out, kBK) * kKbUs + kItemUs, 0, 0.0, kPairs);
-    }
+    const double us = want_dw ? 3.8 + 1.03 * split_plan(M_keep_cap, C_in, C_out, out_in, false).us
+                              : 4.5 + 0.85 * list_time(tiles_of(M_keep_cap, C_in), (double)ceil_div(C_out, kBK) * kKbUs + kItemUs, 0, 0.0, kPairs);
     return us < fma_backward_us(out_in, M_keep_cap, C_in, C_out, want_dw, want_dx);
 }
 
@@ -838,10 +852,15 @@ cudaError_t launch_split_forward(const float* X, const float* W, bool w_out_in, 
     return launch(prm, stream);
 }
 
+int64_t split_plan_searches() {
+    std::lock_guard<std::mutex> lock(g_shape_mutex);
+    return (int64_t)g_shape_plans.size();
+}
+
 size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
     int most = 1;
     for (int v = 0; v < 4; ++v) {
-        const int s = split_plan(M_keep_cap, C_in, C_out, (v & 1) != 0, (v & 2) != 0);
+        const int s = split_plan(M_keep_cap, C_in, C_out, (v & 1) != 0, (v & 2) != 0).splits;
         if (s > most) most = s;
     }
     return most > 1 ? (size_t)most * (size_t)(C_in + 1) * (size_t)C_out * sizeof(float) : 0;
@@ -849,7 +868,7 @@ size_t split_workspace_bytes(int64_t M_keep_cap, int64_t C_in, int64_t C_out) {
 
 int split_backward_kernel_count(bool w_out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx) {
     if (!want_dw && !want_dx) return 0;
-    const int splits = want_dw ? split_plan(M_keep_cap, C_in, C_out, w_out_in, want_dx) : 1;
+    const int splits = want_dw ? split_plan(M_keep_cap, C_in, C_out, w_out_in, want_dx).splits : 1;
     const int64_t nx = want_dx ? tiles_of(M_keep_cap, C_in) : 0, nw = want_dw ? (w_out_in ? tiles_of(C_out, C_in) : tiles_of(C_in, C_out)) * splits : 0;
     return (int)launches_of(nx + nw) + (splits > 1 ? 1 : 0);
 }
@@ -858,7 +877,7 @@ cudaError_t launch_split_backward(const float* X_keep, const float* dY, const fl
                                   const int32_t* dx_rows, const int32_t* M_keep_dev, int64_t M, int64_t M_keep_cap, int64_t C_in,
                                   int64_t C_out, float* dW, float* db, bool dw_accumulate, bool db_accumulate, float* dX, float* workspace,
                                   int32_t* status_word, cudaStream_t stream) {
-    const int splits = dW != nullptr ? split_plan(M_keep_cap, C_in, C_out, w_out_in, dX != nullptr) : 1;
+    const int splits = dW != nullptr ? split_plan(M_keep_cap, C_in, C_out, w_out_in, dX != nullptr).splits : 1;
     const bool pieces = dW != nullptr && splits > 1;
     float* ws_db = workspace;                                              // [splits, C_out], then [splits, C_in * C_out]
     float* ws_dw = workspace + (int64_t)splits * C_out;

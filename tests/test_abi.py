@@ -109,6 +109,20 @@ def test_split_plans_are_searched_once_per_shape(lib):
     assert sbp.sbp_plan_search_count() == seen
 
 
+def test_fp32_split_plans_are_searched_once_per_shape(lib):
+    shapes = [(12544, 768, 3072), (12544, 3072, 768), (3136, 772, 516), (100352, 128, 512), (2400, 256, 260)]
+    before = sbp.sbp_plan_search_count()
+    for M, ci, co in shapes:
+        sbp.sbp_linear_backward_workspace_bytes(0, M, M // 2, ci, co)
+    seen = sbp.sbp_plan_search_count()
+    assert seen == before + len(shapes)
+    for M, ci, co in shapes:
+        sbp.sbp_linear_backward_workspace_bytes(0, M, M // 2, ci, co)
+        for want_dw, want_dx, flags in ((1, 1, 0), (1, 0, 0), (0, 1, 0), (1, 1, 64), (1, 0, 64)):
+            sbp.sbp_linear_backward_kernel_count(0, M, M // 2, ci, co, want_dw, 1, want_dx, flags)
+    assert sbp.sbp_plan_search_count() == seen
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(sbp, "_lib", None)
     monkeypatch.setattr(sbp, "LIB_PATH", str(tmp_path / "nope.so"))
