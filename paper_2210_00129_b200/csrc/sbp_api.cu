@@ -173,7 +173,7 @@ sbp_status sbp_linear_forward(sbp_dtype dt, const void* X, const void* W, const 
             return SBP_ERR_CUDA;
         return SBP_OK;
     }
-    const bool split = dt == SBP_F32 && !(flags & SBP_FLAG_PLAIN_FMA) && split_forward_supported(M, C_in, C_out);
+    const bool split = dt == SBP_F32 && !(flags & SBP_FLAG_PLAIN_FMA) && split_forward_supported(M, C_in, C_out) && split_can_run();
     if ((split ? launch_split_forward((const float*)X, (const float*)W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, (float*)Y,
                                       status_word, stream)
                : launch_fma_forward(dt, X, W, (flags & SBP_FLAG_W_OUT_IN) != 0, bias, M, C_in, C_out, Y, status_word, stream)) != cudaSuccess)
@@ -275,7 +275,7 @@ sbp_status backward_direct(sbp_dtype dt, bool w_out_in, bool fresh_dw, const voi
                                                 dw_accumulate, dX, db_rides ? db : nullptr, accumulate, w_out_in, ws_dw, ws_db,
                                                 status_word, stream);
         if (s != SBP_OK) return s;
-    } else if ((dW != nullptr || dX != nullptr) && use_split(dt, flags, w_out_in, M_keep_cap, C_in, C_out, dW != nullptr, dX != nullptr)) {
+    } else if ((dW != nullptr || dX != nullptr) && use_split(dt, flags, w_out_in, M_keep_cap, C_in, C_out, dW != nullptr, dX != nullptr) && split_can_run()) {
         if (launch_split_backward((const float*)X_keep, (const float*)dY, (const float*)W, w_out_in, dy_rows, dx_rows, M_keep_dev, M_dx, M_keep_cap,
                                   C_in, C_out, dW, db_rides ? db : nullptr, dw_accumulate, accumulate, (float*)dX, ws_dw, status_word,
                                   stream) != cudaSuccess)

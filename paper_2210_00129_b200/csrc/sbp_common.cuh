@@ -172,6 +172,7 @@ cudaError_t launch_fma_backward(sbp_dtype dt, const void* X_keep, const void* dY
                                 float* workspace, const int32_t* status_word, cudaStream_t stream);
 
 // the same products of fp32 layers on the tensor cores, each operand as a sum of three bf16 numbers
+bool   split_can_run();                  // to be asked before a launch
 bool   split_forward_supported(int64_t M, int64_t C_in, int64_t C_out);
 bool   split_backward_supported(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dx);        // room for them in the workspace
 bool   split_backward_quicker(bool out_in, int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool want_dw, bool want_dx);

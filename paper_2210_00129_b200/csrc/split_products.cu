@@ -21,6 +21,7 @@
 // stage's loads behind each conversion the registers spill.)  Measured on B200, 768 -> 3072, 3136 rows with 1568 kept, CUDA cores -> here: forward
 // 299 -> 87 us, dW + db + dX 395 -> 100; relative errors against 64-bit sums Y 2.5e-7 -> 0.8e-7, dW 5.0e-7 -> 1.2e-7, dX 7.0e-7 -> 1.5e-7,
 // db 0.7e-7 -> 0.6e-7.  Over 260 shapes of 32 to 2900 channels and 64 to 65536 rows no Y, dW or dX was further off than the CUDA cores'.
+#include <atomic>
 #include <map>
 #include <tuple>
 #include <type_traits>
@@ -729,12 +730,6 @@ int64_t launches_of(int64_t items) { return ceil_div(items, kMaxRounds * kPairs)
 cudaError_t launch(SplitParams prm, cudaStream_t stream) {
     const cudaError_t opt = opt_in_dynamic_smem<split_products_kernel>((int)kSmemBytes);
     if (opt != cudaSuccess) return opt;
-    // the roles' registers come out of those that the block is launched with: a build that gives it fewer must not run
-    static const bool enough = [] {
-        cudaFuncAttributes a;
-        return cudaFuncGetAttributes(&a, split_products_kernel) == cudaSuccess && a.numRegs >= kLaunchRegs;
-    }();
-    if (!enough) return cudaErrorLaunchOutOfResources;
     const int64_t items = (int64_t)prm.items[0] + prm.items[1];
     for (int64_t first = 0; first < items; first += kMaxRounds * kPairs) {
         const int64_t count = items - first < kMaxRounds * kPairs ? items - first : kMaxRounds * kPairs;
@@ -805,6 +800,18 @@ SplitPlan split_plan(int64_t M_keep_cap, int64_t C_in, int64_t C_out, bool out_i
 }
 
 }  // namespace
+
+// The roles' registers come out of those that the block is launched with: a build that gives it fewer must not run, and its callers take the
+// CUDA cores.  So they do where the question itself fails (it is asked again then; the launch there says what is wrong).
+bool split_can_run() {
+    static std::atomic<int> known{0};                                      // 1: yes, 2: no
+    if (known.load(std::memory_order_relaxed) == 0) {
+        cudaFuncAttributes a;
+        if (cudaFuncGetAttributes(&a, split_products_kernel) != cudaSuccess) return false;
+        known.store(a.numRegs >= kLaunchRegs ? 1 : 2, std::memory_order_relaxed);
+    }
+    return known.load(std::memory_order_relaxed) == 1;
+}
 
 // The lines against the CUDA cores, which start in 3 us where this kernel takes 8 (a cluster of whole SMs, one deep stage), but whose
 // blocks take 4 us for every 100 of depth.  Forward, CUDA cores and here: depth 128 with 491 rows and 376 columns 6.9, 9.2 us, 104 with
