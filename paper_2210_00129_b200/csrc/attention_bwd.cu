@@ -80,7 +80,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-// Calls of one problem a block: zeros for the problem's own 64 columns in the rows of sample b that an ascending token list leaves out, with
+// Calls whose blocks have equal lists of problems: zeros for the problem's own 64 columns in the rows of sample b that an ascending token list leaves out, with
 // no look at memory (the walk's dependent loads are longer than the first products: 7.7 us here, 8.5 with it).  `glob` holds the
 // global row of every listed token of the sample (shared memory).  The z-th unlisted row lies behind g listed ones, with g
 // the first list position whose token has more than z unlisted rows in front of it: a search of at most eight steps.  Every
@@ -116,7 +116,7 @@ __device__ __forceinline__ void zero_unlisted_rows(__nv_bfloat16* out0, __nv_bfl
     }
 }
 
-// Calls of several: zeros for the rows that an ascending list of token rows leaves out, whole rows (all heads) of the outputs.  A warp walks a range of
+// Calls that leave blocks without a problem for a while: zeros for the rows that an ascending list of token rows leaves out, whole rows (all heads) of the outputs.  A warp walks a range of
 // rows of its own, a few unlisted ones at a time: the stores go out while the block waits for products, so that memory works then too.
 // (In front of the first products, an equal share of the problem's own rows a warp and 128 bytes of each, they took 3500 of a problem's
 // 17500 clocks with the products' 1000 underneath.)
@@ -154,19 +154,30 @@ __device__ __forceinline__ void start_walk(const AttnParams& p, ZeroWalk& z, int
 __device__ __forceinline__ void zero_rows(const AttnParams& p, ZeroWalk* walk, int warp, int warps, int lane, bool rest) {
     ZeroWalk z = *walk;
     const bool same = p.q_rows == p.k_rows && p.q_offs == p.k_offs;
+    const auto zero_line = [&](int64_t at) {
+        if (z.pass == 0) ptx::st_global_v4(p.dQ + at, 0u, 0u, 0u, 0u);
+        if (z.pass == 1 || same) {
+            ptx::st_global_v4(p.dK + at, 0u, 0u, 0u, 0u);
+            ptx::st_global_v4(p.dV + at, 0u, 0u, 0u, 0u);
+        }
+    };
     int most = rest ? 0x7fffffff : z.budget;
     while (most > 0 && z.pass < 2) {
         if (z.todo != 0u) {
-            const int64_t at = (int64_t)((uint64_t)(uint32_t)(z.base + __ffs(z.todo) - 1) * p.ld_out * 8u);
-            for (int c = lane * 8; c < p.heads * kD; c += 256) {
-                if (z.pass == 0) ptx::st_global_v4(p.dQ + at + c, 0u, 0u, 0u, 0u);
-                if (z.pass == 1 || same) {
-                    ptx::st_global_v4(p.dK + at + c, 0u, 0u, 0u, 0u);
-                    ptx::st_global_v4(p.dV + at + c, 0u, 0u, 0u, 0u);
-                }
+            if (p.heads > 2) {
+                const int64_t at = (int64_t)((uint64_t)(uint32_t)(z.base + __ffs(z.todo) - 1) * p.ld_out * 8u);
+                for (int c = lane * 8; c < p.heads * kD; c += 256) zero_line(at + c);
+                z.todo &= z.todo - 1u;
+                --most;
+            } else {
+                // four rows of one head, or two of two heads, at a time (one: 298 to 400 problems of one head 3 to 12 % slower)
+                const int per = p.heads == 1 ? 4 : 2;
+                uint32_t own = z.todo;
+                for (int k = lane * per / 32; k > 0; --k) own &= own - 1u;
+                if (own != 0u) zero_line((int64_t)((uint64_t)(uint32_t)(z.base + __ffs(own) - 1) * p.ld_out * 8u) + lane % (32 / per) * 8);
+                for (int k = 0; k < per; ++k) z.todo &= z.todo - 1u;
+                most -= per;
             }
-            z.todo &= z.todo - 1u;
-            --most;
         } else if (z.next < z.end) {                        // the next window of 32 rows
             const int d = z.p + lane < z.n ? __ldg((z.pass == 0 ? p.q_rows : p.k_rows) + z.p + lane) - z.next : 32;
             const uint32_t listed = __reduce_or_sync(0xffffffffu, (d >= 0 && d < 32) ? 1u << d : 0u);
@@ -298,7 +309,7 @@ __device__ __forceinline__ void store_rows(__nv_bfloat16* out, uint32_t ld, int 
     }
 }
 
-// kSeparate: dM has blocks of its own; kOwn: one problem a block at most, which clears its own unlisted rows
+// kSeparate: dM has blocks of its own; kOwn: each problem clears its own unlisted rows, instead of the walk
 template <int G, bool kSeparate, bool kOwn>
 __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(const __grid_constant__ AttnParams p) {
     constexpr int kThreads = 128 * G;
@@ -715,23 +726,35 @@ __global__ void __launch_bounds__(128 * G, G == 2 ? 2 : 1) attention_bwd_kernel(
 int round16(int64_t v) { return (int)((v + 15) / 16 * 16); }
 
 template <int G, bool kSeparate>
-cudaError_t launch_attention_kernel(const AttnParams& prm, uint32_t bytes, int most_bytes, cudaStream_t stream) {
+cudaError_t launch_attention_kernel(const AttnParams& prm, int64_t q_most, int64_t k_most, uint32_t bytes, int most_bytes, cudaStream_t stream) {
     const int64_t problems = (int64_t)prm.B * prm.heads, resident = G == 2 ? 2 * kNumSMs : kNumSMs;
     const int64_t grid = problems < resident ? problems : resident;
     const auto go = [&](auto kernel, cudaError_t opt, const AttnParams& q) {
         return opt != cudaSuccess ? opt : launch_pdl(kernel, dim3((unsigned)grid), dim3(128 * G), bytes, stream, q);
     };
-    if (problems <= resident)
-        return go(attention_bwd_kernel<G, kSeparate, true>, opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate, true>>(most_bytes), prm);
-    // Zeros: equal shares of the rows, less for the first blocks where these have a problem more than the others, by the rows that can be
-    // visited in a problem's time: some 7200 / (heads x outputs), half of them unlisted (Drop QKV, B = 128: 2400 60.0 us, 3600 58.9, 7200 58.5).
+    // The walk is worth its reads where it shortens the longest lists: blocks that are idle while `more` others have their last problem clear
+    // most of the rows.  A row costs a line of 128 bytes for each head and output that leaves it out, and some 6 lines to be found; an idle block
+    // clears `worth` lines in a problem's time (up to a quarter more it is given all of them: a small share for the others costs these more
+    // than it saves).  Both ways were timed on 700 calls.  12 heads, 196 tokens, half of them listed, each problem its own rows -> the walk:
+    // 312 problems 18.7 -> 18.4 us, 516 21.7 -> 21.0, 1536 63.4 -> 59.0; 576 on 296 blocks, few of them idle, 21.9 -> 23.2 (28.1, and 30.5 instead of
+    // 18.9 for problems of 128 tokens, with all rows for the idle ones).  One block an SM: the walk wins with few idle blocks too, and without
+    // any from three problems a block on (10 to 15 % of the time).
+    const int64_t rows = (int64_t)prm.B * prm.N, more = problems % grid, idle = grid - more;
+    const double find = prm.heads == 1 ? 1.5 : prm.heads == 2 ? 3.0 : 6.0;
+    const double outside_q = prm.q_rows == nullptr ? 0.0 : 1.0 - (double)q_most / (double)prm.N;
+    const double outside_k = prm.k_rows == nullptr ? 0.0 : 1.0 - (double)k_most / (double)prm.N;
+    const double lines = (double)rows * (prm.q_rows == prm.k_rows ? outside_q * (3.0 * prm.heads + find)
+                                                                  : outside_q * (prm.heads + find) + outside_k * (2.0 * prm.heads + find));
+    const double for_idle = lines / (double)idle, for_problem = lines / (double)problems;
+    const bool walk = problems > grid && (G == 2 ? more != 0 && for_idle <= 900.0 + 10.0 * for_problem
+                                                 : problems > 2 * grid || for_idle <= 8000.0 + 4.0 * for_problem);
+    if (!walk) return go(attention_bwd_kernel<G, kSeparate, true>, opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate, true>>(most_bytes), prm);
     AttnParams q = prm;
-    const int64_t rows = (int64_t)prm.B * prm.N, outs = prm.q_rows == nullptr ? 2 : prm.k_rows == prm.q_rows ? 3 : 1;
-    const int64_t more = problems % grid, worth = 7200 / (prm.heads * outs) + 1;
-    const int64_t spare = rows - (grid - more) * worth;
+    const double worth = G == 2 ? 15.0 * (double)(30 + (q_most > k_most ? q_most : k_most)) : q_most > 128 ? 3800.0 : 1900.0;
+    const double spare = for_idle <= 1.25 * worth ? 0.0 : (double)rows * (1.0 - worth / for_idle);      // rows that the idle blocks do not get to
     q.zero_blocks = (int)more;
-    q.zero_first = more == 0 || spare <= 0 ? 0 : (int)((spare + grid - 1) / grid);
-    q.zero_rest = (int)((rows - more * q.zero_first + (grid - more) - 1) / (grid - more));
+    q.zero_first = more == 0 || spare <= 0.0 ? 0 : (int)((int64_t)spare / grid + 1);
+    q.zero_rest = rows <= more * q.zero_first ? 0 : (int)((rows - more * q.zero_first + idle - 1) / idle);
     return go(attention_bwd_kernel<G, kSeparate, false>, opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate, false>>(most_bytes), q);
 }
 
@@ -768,8 +791,8 @@ cudaError_t launch_attention(AttnParams& prm, int64_t q_most, int64_t k_most, cu
     const uint32_t ends[2] = {prm.off_da + q_tiles * kTileB, G == 2 && prm.separate ? prm.off_v + kTileB : 0u};
     for (uint32_t end : ends) bytes = bytes < end ? end : bytes;
     if (bytes > kLimit) return cudaErrorInvalidValue;
-    return prm.separate ? launch_attention_kernel<G, true>(prm, bytes + 1024u, (int)kLimit + 1024, stream)
-                        : launch_attention_kernel<G, false>(prm, bytes + 1024u, (int)kLimit + 1024, stream);
+    return prm.separate ? launch_attention_kernel<G, true>(prm, q_most, k_most, bytes + 1024u, (int)kLimit + 1024, stream)
+                        : launch_attention_kernel<G, false>(prm, q_most, k_most, bytes + 1024u, (int)kLimit + 1024, stream);
 }
 
 }  // namespace
