@@ -69,3 +69,28 @@ def test_forward_on_cuda_cores(dtype, M, C_in, C_out, w_out_in):
                            flags=sbp.SBP_FLAG_PLAIN_FMA | (sbp.SBP_FLAG_W_OUT_IN if w_out_in else 0))
     torch.cuda.synchronize()
     _check(Y, want, dtype, True)
+
+
+@pytest.mark.parametrize("M,kept,valid,C_in,C_out,out_in", [
+    (1176, 294, 294, 68, 260, False), (1400, 700, 700, 1028, 1540, False), (1400, 700, 651, 1028, 1540, True),      # 64 x 128 tiles
+    (40000, 20000, 19990, 36, 68, False),                                                                          # the same, long and thin
+    (3000, 1500, 1500, 768, 100, True),
+])
+def test_fp32_backward_on_the_cuda_cores_by_request(M, kept, valid, C_in, C_out, out_in):
+    """Sizes that the tensor-core kernel takes by default: SBP_FLAG_PLAIN_FMA keeps them here."""
+    X, Wt, dY = synth.layer_inputs("f32", M, C_in, C_out, 63)
+    keep = np.sort(np.random.default_rng(9).permutation(M)[:kept]).astype(np.int32)
+    rows, count = torch.from_numpy(keep).cuda(), torch.tensor([valid], dtype=torch.int32, device="cuda")
+    want = oracle.linear_backward(synth.to_f64(X[keep[:valid]], "f32"), synth.to_f64(dY, "f32"), synth.to_f64(Wt, "f32"), keep[:valid])
+    W = dev(np.ascontiguousarray(Wt.T) if out_in else Wt, "f32")
+    nb = sbp.sbp_linear_backward_workspace_bytes(sbp.SBP_F32, M, kept, C_in, C_out)
+    ws, st = torch.empty(nb, dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    dW, db, dX = torch.full_like(W, float("nan")), torch.full((C_out,), float("nan"), device="cuda"), torch.full((M, C_in), float("nan"), device="cuda")
+    sbp.sbp_linear_backward(sbp.SBP_F32, dev(X[keep], "f32"), dev(dY, "f32"), W, rows, count, M, kept, C_in, C_out, dW, db, dX,
+                            sbp.SBP_FLAG_PLAIN_FMA | (sbp.SBP_FLAG_W_OUT_IN if out_in else 0), ws, nb, st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    _check(dW.t().contiguous() if out_in else dW, want["dW"], "f32", False)
+    _check(db, want["db"], "f32", False)
+    _check(dX, want["dX"], "f32", True)
+    assert not host(dX)[np.setdiff1d(np.arange(M), keep[:valid])].view(np.uint8).any()
