@@ -23,7 +23,7 @@
 //  - The next problem's rows are copied as soon as the last product has read the operands, under the read-out and the
 //    stores of this one.
 // Measured on B200, ViT-B/16 heads (12 x 64, 196 tokens), whole pass with the sampler: Drop QKV, half of the tokens, B = 128:
-// 99 us with a thread a row and copies behind the read-out, 64 with the zeros of a problem's own rows in front of its first wait, now 58;
+// 99 us with a thread a row and copies behind the read-out, 64 with the zeros of a problem's own rows in front of its first wait, now 59;
 // Drop Query only, B = 64: 94 -> 71 -> 61.  (One thread issuing the products instead of a whole warp with one lane elected: 70 and 78 us,
 // each instruction waiting for its operands to reach uniform registers.)  A problem's chain, some 17000 clocks with two blocks on an SM: wait
 // for the copies 900, first products and zeros 2300, softmax 5300, gradient products and zeros 3200, next copies 2900, read-out and stores 2400.
@@ -734,8 +734,8 @@ cudaError_t launch_attention_kernel(const AttnParams& prm, int64_t q_most, int64
     };
     // The walk is worth its reads where it shortens the longest lists: blocks that are idle while `more` others have their last problem clear
     // most of the rows.  A row costs a line of 128 bytes for each head and output that leaves it out, and some 6 lines to be found; an idle block
-    // clears `worth` lines in a problem's time (up to a quarter more it is given all of them: a small share for the others costs these more
-    // than it saves).  Both ways were timed on 700 calls.  12 heads, 196 tokens, half of them listed, each problem its own rows -> the walk:
+    // clears `worth` lines in a problem's time, twice as many where a problem has two query tiles (up to a quarter more it is given all of them: a
+    // small share for the others costs these more than it saves).  Both ways were timed on 700 calls.  12 heads, 196 tokens, half of them listed, each problem its own rows -> the walk:
     // 312 problems 18.7 -> 18.4 us, 516 21.7 -> 21.0, 1536 63.4 -> 59.0; 576 on 296 blocks, few of them idle, 21.9 -> 23.2 (28.1, and 30.5 instead of
     // 18.9 for problems of 128 tokens, with all rows for the idle ones).  One block an SM: the walk wins with few idle blocks too, and without
     // any from three problems a block on (10 to 15 % of the time).
@@ -746,11 +746,11 @@ cudaError_t launch_attention_kernel(const AttnParams& prm, int64_t q_most, int64
     const double lines = (double)rows * (prm.q_rows == prm.k_rows ? outside_q * (3.0 * prm.heads + find)
                                                                   : outside_q * (prm.heads + find) + outside_k * (2.0 * prm.heads + find));
     const double for_idle = lines / (double)idle, for_problem = lines / (double)problems;
-    const bool walk = problems > grid && (G == 2 ? more != 0 && for_idle <= 900.0 + 10.0 * for_problem
+    const bool walk = problems > grid && (G == 2 ? more != 0 && for_idle <= 700.0 + 10.0 * for_problem
                                                  : problems > 2 * grid || for_idle <= 8000.0 + 4.0 * for_problem);
     if (!walk) return go(attention_bwd_kernel<G, kSeparate, true>, opt_in_dynamic_smem<attention_bwd_kernel<G, kSeparate, true>>(most_bytes), prm);
     AttnParams q = prm;
-    const double worth = G == 2 ? 15.0 * (double)(30 + (q_most > k_most ? q_most : k_most)) : q_most > 128 ? 3800.0 : 1900.0;
+    const double worth = q_most > 128 ? 3800.0 : 1900.0;
     const double spare = for_idle <= 1.25 * worth ? 0.0 : (double)rows * (1.0 - worth / for_idle);      // rows that the idle blocks do not get to
     q.zero_blocks = (int)more;
     q.zero_first = more == 0 || spare <= 0.0 ? 0 : (int)((int64_t)spare / grid + 1);
