@@ -561,7 +561,8 @@ def run_cuda(args, w, name):
 
 
 def roofline_of(w, name, job, r):
-    """Roofline object of the dominant kernel (tc_backward_kernel; the CUDA-core kernels for fp32 / tiny shapes):
+    """Roofline object of the dominant kernel (tc_backward_kernel; the CUDA-core kernels for tiny shapes, among them the one
+    fp32 workload here, 32 -> 64, which is too small for split_products_kernel):
     algorithmic work of the backward calls of one step over their measured duration, against the measured peak."""
     peaks, peak_kind = load_peaks()
     M, M_keep = job.M, r["M_keep"]

@@ -211,9 +211,11 @@ size_t sbp_linear_backward_workspace_bytes(sbp_dtype dt, int64_t M, int64_t M_ke
  * error of dW against 64-bit sums: 1e-7 to 1e-5, growing with the number of kept
  * rows), dX rounded to bf16 (nearest even).  SBP_F32: fp32 FMA arithmetic, or, for
  * products large enough, six tensor-core products of operands in three bf16 parts each,
- * summed in fp32: no further from 64-bit sums than the FMAs (1e-7 against 2e-7 to 7e-7),
- * subnormal operands and sums included, infinities and NaNs as the FMAs have them;
- * SBP_FLAG_PLAIN_FMA keeps to the FMAs.
+ * summed in fp32: no further from 64-bit sums than the FMAs (relative error of Y and dX
+ * 1e-7 against 1e-7 to 7e-7, of dW, growing with the kept rows, up to 5e-7 against 3e-6,
+ * of db 1e-7 against 1e-7), subnormal operands and sums included, infinities and NaNs as
+ * the FMAs have them; sums that are not finite, or hold operands beyond 2^112, cost up to
+ * ten times a finite call.  SBP_FLAG_PLAIN_FMA keeps to the FMAs.
  * C_in and C_out must be multiples of 8 (bf16) / 4 (fp32), else SBP_ERR_UNSUPPORTED.
  *
  * flags: SBP_FLAG_ACCUMULATE adds into dW and db; SBP_FLAG_VALIDATE first checks
@@ -316,7 +318,8 @@ sbp_status sbp_patch_scatter(sbp_dtype dt, const void* dX_patches /* dev */, int
  * own base pointers, so the three slices of a fused [B*N, 3*heads*d] projection output can be passed with
  * ld = 3*heads*d; dA [B*N, ld_da] likewise.  q_rows / q_offsets (and kv_*) are lists as sbp_sample_keep writes them:
  * ascending global row ids b*N + n and B + 1 offsets; max_kept = the largest per-sample count any list may hold
- * (e.g. sbp_keep_count(...)), ignored when no list is given.
+ * (e.g. sbp_keep_count(...)), ignored when no list is given; tokens listed past it take no part, and their rows of the
+ * outputs may be left unwritten.
  * This build: SBP_BF16 with d = 64, at most 256 tokens of a sample on either side (N <= 256 where a side takes all
  * tokens), leading dimensions multiples of 8: otherwise SBP_ERR_UNSUPPORTED.  P = S and dM are rounded to bf16
  * between the products, accumulation is fp32.  SBP_ERR_INVALID_ARG for null / misaligned pointers and bad sizes.

@@ -735,7 +735,7 @@ cudaError_t launch_attention_kernel(const AttnParams& prm, int64_t q_most, int64
     // The walk is worth its reads where it shortens the longest lists: blocks that are idle while `more` others have their last problem clear
     // most of the rows.  A row costs a line of 128 bytes for each head and output that leaves it out, and some 6 lines to be found; an idle block
     // clears `worth` lines in a problem's time, twice as many where a problem has two query tiles (up to a quarter more it is given all of them: a
-    // small share for the others costs these more than it saves).  Both ways were timed on 700 calls.  12 heads, 196 tokens, half of them listed, each problem its own rows -> the walk:
+    // small share for the others costs these more than it saves).  Both ways were timed on 755 calls.  12 heads, 196 tokens, half of them listed, each problem its own rows -> the walk:
     // 312 problems 18.7 -> 18.4 us, 516 21.7 -> 21.0, 1536 63.4 -> 59.0; 576 on 296 blocks, few of them idle, 21.9 -> 23.2 (28.1, and 30.5 instead of
     // 18.9 for problems of 128 tokens, with all rows for the idle ones).  One block an SM: the walk wins with few idle blocks too, and without
     // any from three problems a block on (10 to 15 % of the time).

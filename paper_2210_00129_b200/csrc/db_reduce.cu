@@ -112,9 +112,9 @@ struct ReduceJob {
     int64_t n_vec;        // float4 elements per partial
     int splits;
     int accumulate;
-    int lanes;            // 1: one thread per float4, partials added in ascending order
+    int lanes;            // 1: one thread per float4, partials added to `out` (or 0) in ascending order
                           // Y = 4 or 32: 256/Y float4 columns x Y row lanes per block; lane y adds partials
-                          //    y, y+Y, ... in ascending order, the Y lane sums are then added in a fixed order
+                          //    y, y+Y, ... in ascending order, the Y lane sums are then added in a fixed order, `out` last
     int blocks;
 };
 

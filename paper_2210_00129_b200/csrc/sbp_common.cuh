@@ -149,7 +149,7 @@ cudaError_t launch_db(sbp_dtype dt, const void* dY, const int32_t* keep_rows, co
                       int64_t M_keep_cap, int64_t C_out, float* db, bool accumulate, float* workspace,
                       int max_splits, const int32_t* status_word, cudaStream_t stream);
 
-// out[i] = (accumulate ? out[i] : 0) + sum_s partials[s*n + i], summed in ascending s
+// out[i] = (accumulate ? out[i] : 0) + sum_s partials[s*n + i], in a fixed order (db_reduce.cu)
 cudaError_t launch_reduce_partials(const float* partials, int splits, int64_t n, float* out,
                                    bool accumulate, const int32_t* status_word, cudaStream_t stream);
 
